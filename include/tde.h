@@ -147,11 +147,14 @@ TDE_API int tde_eos_load_table(tde_ctx *ctx, int n_rho, int n_T, double log10_rh
 TDE_API int tde_eos_destroy(tde_eos *eos);
 
 /* Invert n cells (rho, e) -> (T, P, cs2), all cgs, device arrays of n doubles.
- * mode TDE_INVERT_BISECT: binary search of the interpolated log10 e column,
- * carried out in FP32 on a rounded copy of the table and confirmed by the FP64
- * bracket of the cell (FP64 bisection where FP32 cannot decide);
- * TDE_INVERT_BISECT_PLAIN: the same search entirely in FP64 (the plain form of
- * Sec. 4.2's runtime map).  Both give identical results.  T, P or cs2 may be NULL.  Inputs outside the table are clamped to its edge and
+ * The logarithms, interpolations and the solve are in 64-bit fixed point (55
+ * fraction bits of log2; finer than FP64 logarithms of this size); tables with
+ * an entry of magnitude 38 or more (log10) take FP64 instead.
+ * mode TDE_INVERT_BISECT: binary search of the interpolated log e column, on a
+ * rounded 32-bit copy of the part of the table that log e bounds, confirmed by
+ * the 64-bit bracket of the cell (64-bit bisection where it cannot decide);
+ * TDE_INVERT_BISECT_PLAIN: the same search of the whole column entirely in 64
+ * bits (the plain form of Sec. 4.2's runtime map).  Both give identical results.  T, P or cs2 may be NULL.  Inputs outside the table are clamped to its edge and
  * counted (counts may be NULL; reading it synchronises the stream). */
 TDE_API int tde_eos_invert(tde_eos *eos, int mode, int64_t n, const double *rho, const double *e,
                    double *T, double *P, double *cs2, tde_counts *counts);
@@ -164,8 +167,8 @@ TDE_API int tde_eos_invert(tde_eos *eos, int mode, int64_t n, const double *rho,
  * log10 P ranges (tde_eos_surrogate_norm).  Parameters, 4482 floats:
  *   W1[64][2], b1[64], W2[64][64], b2[64], W3[2][64], b3[2].
  * TDE_INVERT_SURROGATE uses the network (BF16 weights; the 64 x 64 layer on the
- * tensor cores, FP32 accumulation) to guess log10 T, takes one FP64 Newton step
- * on the interpolated log10 e column (linear inside a cell) from the guess's
+ * tensor cores, FP32 accumulation) to guess log10 T, takes one Newton step
+ * on the interpolated log e column (linear inside a cell) from the guess's
  * cell, and accepts the cell the step lands in iff the table brackets the root
  * there -- then the result equals bisection's exactly.  The cells it does not
  * settle are gathered (warp-aggregated queue) and inverted by bisection in a

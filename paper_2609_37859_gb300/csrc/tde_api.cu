@@ -26,6 +26,14 @@ void tde::fill_math_tables(MathTables *h) {
   for (int j = 0; j < 128; ++j) h->exp2j[j] = (double)exp2l(j / 128.0L);
 }
 
+void tde::fx_fill_math(FxMath *h) {
+  for (int j = 0; j < 256; ++j) {
+    h->c[j] = (unsigned)floorl(1024.0L / (1.0L + (j + 0.5L) / 256.0L) + 0.5L);
+    h->lg[j] = (fx)floorl(-log2l(h->c[j] / 1024.0L) * 36028797018963968.0L + 0.5L);
+    h->ex[j] = (unsigned long long)floorl(exp2l((j + 0.5L) / 256.0L) * 4611686018427387904.0L + 0.5L);
+  }
+}
+
 namespace {
 
 int fail(tde_ctx *c, int code, const char *msg) {
@@ -91,7 +99,7 @@ bool fill_phys(tde_mesh *m, const tde_params *pr, tde_eos *eos) {
   if (p.eos == EOS_TABLE) {
     if (!eos) return false;
     p.tab = eos->tab;
-    if (p.eos_mode == TDE_INVERT_BISECT_PLAIN) p.tab.le32 = nullptr;   // every step in FP64
+    if (p.eos_mode == TDE_INVERT_BISECT_PLAIN) p.tab.n32 = nullptr;   // every step in 64 bits
   }
   return true;
 }
@@ -164,6 +172,83 @@ extern "C" int tde_finalize(tde_ctx *ctx) {
 }
 
 // ============================================================= EOS ====
+
+// The fixed-point form of a loaded table (tde_fx.cuh), one allocation: the node
+// pairs, their 32-bit copies, the search buckets and the log2 / exp2 tables.  A
+// table with an entry outside the format keeps the axes only, and every cell
+// goes through the FP64 arrays.
+static cudaError_t load_fx_table(tde_eos *e, double lr_max, const double *le, const double *lp, const double *lc) {
+  DTable &t = e->tab;
+  const int nr = t.nr, nt = t.nt;
+  const size_t nn = (size_t)nr * nt, npair = (size_t)(nr - 1) * nt;
+  t.fa = fx_axes(nr, nt, t.lr0, lr_max, t.inv_dlr, t.lt0, t.dlt);
+  const double *src[3] = {le, lp, lc};
+  std::vector<fx> v[3];
+  bool ok = t.fa.valid;
+  for (int q = 0; q < 3; ++q) {
+    v[q].resize(nn);
+    for (size_t k = 0; k < nn; ++k) {
+      v[q][k] = fx_of_log10(src[q][k]);
+      ok = ok && v[q][k] != FX_BAD;
+    }
+  }
+  // bucket width: the smallest power of two that needs at most 8 nt buckets
+  fx y0 = v[0][0], y1 = v[0][0];
+  for (size_t k = 0; k < nn && ok; ++k) { y0 = std::min(y0, v[0][k]); y1 = std::max(y1, v[0][k]); }
+  int sh = 32;
+  while (((y1 - y0) >> sh) + 1 > 8LL * nt) ++sh;
+  const int nbk = ok ? (int)((y1 - y0) >> sh) + 1 : 0;
+  const bool buckets = ok && nt <= 65535;
+  std::vector<unsigned char> h(sizeof(FxMath));
+  fx_fill_math(reinterpret_cast<FxMath *>(h.data()));
+  size_t o_node = 0, o_n32 = 0, o_bk = 0;
+  auto part = [&](size_t bytes) {
+    const size_t o = (h.size() + 15) / 16 * 16;
+    h.resize(o + bytes);
+    return o;
+  };
+  if (ok) {
+    o_node = part(sizeof(longlong2) * 3 * npair);
+    o_n32 = part(sizeof(int2) * npair);
+    if (buckets) o_bk = part(sizeof(ushort2) * (size_t)(nr - 1) * nbk);
+    longlong2 *nd = reinterpret_cast<longlong2 *>(h.data() + o_node);
+    int2 *n32 = reinterpret_cast<int2 *>(h.data() + o_n32);
+    for (int i = 0; i + 1 < nr; ++i)
+      for (int j = 0; j < nt; ++j) {
+        const size_t k = (size_t)i * nt + j;
+        for (int q = 0; q < 3; ++q) nd[3 * k + q] = make_longlong2(v[q][k], v[q][k + nt]);
+        n32[k] = make_int2((int)(v[0][k] >> 32), (int)(v[0][k + nt] >> 32));
+      }
+    ushort2 *bk = reinterpret_cast<ushort2 *>(h.data() + o_bk);
+    for (int i = 0; i + 1 < nr && buckets; ++i) {
+      // an interpolated node lies between the two rows', so the cell of y lies
+      // between the rows' cells of the bucket's ends
+      int a[2] = {0, 0}, b[2] = {0, 0};
+      for (int q = 0; q < nbk; ++q) {
+        const fx ya = y0 + ((fx)q << sh), yb = ya + ((fx)1 << sh);
+        for (int r = 0; r < 2; ++r) {
+          const fx *col = v[0].data() + (size_t)(i + r) * nt;
+          while (a[r] < nt - 2 && col[a[r] + 1] <= ya) ++a[r];
+          while (b[r] < nt - 2 && col[b[r] + 1] <= yb) ++b[r];
+        }
+        bk[(size_t)i * nbk + q] = make_ushort2((unsigned short)std::min(a[0], a[1]), (unsigned short)std::max(b[0], b[1]));
+      }
+    }
+  }
+  cudaError_t err = cudaMalloc(&e->d_fx, h.size());
+  if (err == cudaSuccess) err = cudaMemcpy(e->d_fx, h.data(), h.size(), cudaMemcpyHostToDevice);
+  if (err != cudaSuccess) return err;
+  t.fm = reinterpret_cast<const FxMath *>(e->d_fx);
+  if (ok) {
+    t.node = reinterpret_cast<const longlong2 *>(e->d_fx + o_node);
+    t.n32 = reinterpret_cast<const int2 *>(e->d_fx + o_n32);
+    t.bk = buckets ? reinterpret_cast<const ushort2 *>(e->d_fx + o_bk) : nullptr;
+    t.y0 = y0;
+    t.bshift = sh;
+    t.nbk = nbk;
+  }
+  return cudaSuccess;
+}
 
 extern "C" int tde_eos_load_table(tde_ctx *ctx, int n_rho, int n_T, double lr_min, double lr_max,
                                   double lT_min, double lT_max, const double *log10_e,
@@ -250,6 +335,15 @@ extern "C" int tde_eos_load_table(tde_ctx *ctx, int n_rho, int n_T, double lr_mi
     }
     t.mt = e->d_mt;
   }
+  try {
+    err = load_fx_table(e, lr_max, log10_e, log10_P, log10_cs2);
+  } catch (const std::bad_alloc &) {
+    err = cudaErrorMemoryAllocation;
+  }
+  if (err != cudaSuccess) {
+    tde_eos_destroy(e);
+    return cuda_fail(ctx, err, "tde_eos_load_table: fixed-point table");
+  }
   *out = e;
   return TDE_OK;
 }
@@ -257,6 +351,7 @@ extern "C" int tde_eos_load_table(tde_ctx *ctx, int n_rho, int n_T, double lr_mi
 extern "C" int tde_eos_destroy(tde_eos *e) {
   if (!e) return TDE_EINVAL;
   cudaFree(e->d_mt);
+  cudaFree(e->d_fx);
   cudaFree(e->d_data);
   cudaFree(e->d_cnt);
   cudaFree(e->d_w);

@@ -12,6 +12,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "tde_fx.cuh"
+
 namespace tde {
 
 enum { EOS_IDEAL = 0, EOS_TABLE = 1 };
@@ -144,6 +146,20 @@ struct DTable {
   const double *__restrict__ lc;   // log10 cs^2
   const float *__restrict__ le32;  // log10 e rounded to FP32 (guides the search)
   const MathTables *__restrict__ mt;   // tables of fast_log10 / fast_exp10 (or null)
+  // fixed-point form (tde_fx.cuh; log2 units, Q55), built at load where every
+  // entry fits it.  node: per (density cell i, temperature node j) the pairs
+  // (row i, row i + 1) of log e, log P, log cs^2 in three 16-byte words, so an
+  // inversion's last lookups are two runs of 48 bytes; null: from the FP64
+  // arrays (caller-owned views, tables beyond the format)
+  FxAxes fa;
+  const FxMath *__restrict__ fm;       // tables of fx_log2 / fx_exp2
+  const longlong2 *__restrict__ node;  // [nr - 1][nt][3]
+  const int2 *__restrict__ n32;        // [nr - 1][nt] the log e pairs in Q23 (the search)
+  // per density cell and bucket of log e (2^bshift wide from y0): the first and
+  // last temperature cell the inversion can end in (null: search the column)
+  const ushort2 *__restrict__ bk;
+  fx y0;
+  int bshift, nbk;
 };
 
 __device__ __forceinline__ double tlog10(const DTable &t, double x) {
@@ -379,23 +395,25 @@ __device__ __forceinline__ double cell_log10T(const DTable &t, int j, double s) 
   return __fma_rn(__dadd_rn(dint(j), s), t.dlt, t.lt0);
 }
 
-// (rho, e) -> P, cs2 (cgs) by binary search of the interpolated log10 e column
-// at fixed density weight, then an exact linear solve inside the cell
-// (Sec. 4.2, runtime map).  Returns true if the input was clamped to the table
-// edge; then *e_used is the table's e at the clamped point.  WANT_CS2 = false
-// computes P only (cs2, T and e_used are left untouched).
-template <bool WANT_CS2 = true>
-__device__ __forceinline__ bool eos_invert(const DTable &t, double rho, double e, double &P,
-                                           double &cs2, double &e_used, double *T = nullptr) {
+// (rho, e) -> P, cs2 (cgs): the temperature cell of the interpolated log e column
+// at fixed density weight, then an exact linear solve inside it (Sec. 4.2, runtime
+// map).  Returns true if the input was clamped to the table edge; then *e_used is
+// the table's e at the clamped point.  WANT_CS2 = false computes P only (cs2, T
+// and e_used are left untouched).
+//
+// The FP64 form, for tables whose entries the fixed-point format does not take.
+template <bool WANT_CS2>
+__device__ __forceinline__ bool eos_invert_fp64(const DTable &t, double rho, double e, double &P,
+                                                double &cs2, double &e_used, double *T) {
   int i;
   double w;
   bool cl = rho_cell(t, rho, i, w);
   const int nt = t.nt;
   const double *__restrict__ a = t.le + (size_t)i * nt;
   const double *__restrict__ b = a + nt;
-  double glo = lerp_rn(w, __ldg(a), __ldg(b));
-  double ghi = lerp_rn(w, __ldg(a + nt - 1), __ldg(b + nt - 1));
-  double y = dgt0(e) ? tlog10(t, e) : -INFINITY;
+  const double glo = lerp_rn(w, __ldg(a), __ldg(b));
+  const double ghi = lerp_rn(w, __ldg(a + nt - 1), __ldg(b + nt - 1));
+  const double y = dgt0(e) ? tlog10(t, e) : -INFINITY;
   int j;
   double s;
   if (!dlt(glo, y)) {
@@ -403,39 +421,14 @@ __device__ __forceinline__ bool eos_invert(const DTable &t, double rho, double e
   } else if (dle(ghi, y)) {
     j = nt - 2; s = 1.0; cl = true;
   } else {
-    // search in FP32 (FP64 issues 55x slower on this part), then confirm the cell
-    // with the FP64 bracket the linear solve needs anyway; the cell with
-    // g_j <= y < g_{j+1} is unique, so a confirmed FP32 answer equals the FP64
-    // bisection's, and an unconfirmed one (y within FP32 rounding of a node)
-    // falls back to it
     int lo = 0, hi = nt - 1;
-    if (t.le32) {   // tables without the FP32 copy (caller-owned views) skip this
-      const float *__restrict__ a32 = t.le32 + (size_t)i * nt;
-      const float *__restrict__ b32 = a32 + nt;
-      const float w32 = d2f_guide(w), y32 = d2f_guide(y);
-      while (hi - lo > 1) {
-        const int mid = (lo + hi) >> 1;
-        const float a0 = __ldg(a32 + mid);
-        const float g = fmaf(w32, __ldg(b32 + mid) - a0, a0);
-        if (g <= y32) lo = mid; else hi = mid;
-      }
+    while (hi - lo > 1) {
+      const int mid = (lo + hi) >> 1;
+      const double g = lerp_rn(w, __ldg(a + mid), __ldg(b + mid));
+      if (dle(g, y)) lo = mid; else hi = mid;
     }
     j = lo;
-    double g0 = lerp_rn(w, __ldg(a + j), __ldg(b + j));
-    double g1 = lerp_rn(w, __ldg(a + j + 1), __ldg(b + j + 1));
-    if (!(dle(g0, y) && dlt(y, g1))) {
-      lo = 0;
-      hi = nt - 1;
-      while (hi - lo > 1) {
-        const int mid = (lo + hi) >> 1;
-        const double g = lerp_rn(w, __ldg(a + mid), __ldg(b + mid));
-        if (dle(g, y)) lo = mid; else hi = mid;
-      }
-      j = lo;
-      g0 = lerp_rn(w, __ldg(a + j), __ldg(b + j));
-      g1 = lerp_rn(w, __ldg(a + j + 1), __ldg(b + j + 1));
-    }
-    s = cell_solve(y, g0, g1);
+    s = cell_solve(y, lerp_rn(w, __ldg(a + j), __ldg(b + j)), lerp_rn(w, __ldg(a + j + 1), __ldg(b + j + 1)));
   }
   P = texp10(t, bilin(t.lp, nt, i, w, j, s));
   if (WANT_CS2) {
@@ -443,6 +436,142 @@ __device__ __forceinline__ bool eos_invert(const DTable &t, double rho, double e
     if (T) *T = texp10(t, cell_log10T(t, j, s));
     e_used = cl ? texp10(t, bilin(t.le, nt, i, w, j, s)) : e;
   }
+  return cl;
+}
+
+// The fixed-point form with every table value converted from the FP64 arrays as
+// it is read and the column searched in full: the same bits as eos_invert's, for
+// the entry that may allocate nothing and so has no prepared table.  Cells whose
+// lookups touch an entry outside the format take the FP64 form.
+__device__ __forceinline__ fx fx_ld(const double *__restrict__ f, size_t k, bool &ok) {
+  const fx v = fx_of_log10(__ldg(f + k));
+  ok = ok && v != FX_BAD;
+  return v;
+}
+template <bool WANT_CS2>
+__device__ __noinline__ bool eos_invert_views(const DTable &t, double rho, double e, double &P, double &cs2,
+                                              double &e_used, double *T) {
+  if (t.fa.valid && t.fm) {
+    int i;
+    ufx w;
+    bool cl = fx_rho_cell(t.fm, t.fa, t.nr, rho, i, w), ok = true;
+    const int nt = t.nt;
+    const size_t a = (size_t)i * nt, b = a + nt;
+    auto g = [&](const double *f, int j) { return fx_lerp(fx_ld(f, a + j, ok), fx_ld(f, b + j, ok), w); };
+    const fx glo = g(t.le, 0), ghi = g(t.le, nt - 1);
+    const fx y = dgt0(e) ? fx_log2(t.fm, e) : -FX_SAT;
+    int j;
+    ufx s;
+    if (y <= glo) {
+      j = 0; s = 0; cl = true;
+    } else if (y >= ghi) {
+      j = nt - 2; s = ~0ull; cl = true;
+    } else {
+      int lo = 0, hi = nt - 1;
+      while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (g(t.le, mid) <= y) lo = mid; else hi = mid;
+      }
+      j = lo;
+      const fx g0 = g(t.le, j), g1 = g(t.le, j + 1);
+      ok = ok && g0 <= y && y < g1;
+      s = ok ? fx_frac(y - g0, g1 - g0) : 0;
+    }
+    const fx lp = fx_lerp(g(t.lp, j), g(t.lp, j + 1), s);
+    fx lc = 0, lu = 0;
+    if (WANT_CS2) {
+      lc = fx_lerp(g(t.lc, j), g(t.lc, j + 1), s);
+      if (cl) lu = fx_lerp(g(t.le, j), g(t.le, j + 1), s);
+    }
+    if (ok) {
+      P = fx_exp2(t.fm, lp);
+      if (WANT_CS2) {
+        cs2 = fx_exp2(t.fm, lc);
+        if (T) *T = fx_exp2(t.fm, fx_log2T(t.fa, j, s));
+        e_used = cl ? fx_exp2(t.fm, lu) : e;
+      }
+      return cl;
+    }
+  }
+  return eos_invert_fp64<WANT_CS2>(t, rho, e, P, cs2, e_used, T);
+}
+
+// a pair (row i, row i + 1) of the prepared table interpolated in density
+__device__ __forceinline__ fx fx_pair(const longlong2 *__restrict__ q, ufx w) {
+  const longlong2 v = __ldg(q);
+  return fx_lerp(v.x, v.y, w);
+}
+
+// the results at fraction s of cell (i, j); nd = the cell's first node
+template <bool WANT_CS2>
+__device__ __forceinline__ void eos_at(const DTable &t, const longlong2 *__restrict__ nd, ufx w, int j, ufx s,
+                                       bool cl, double e, double &P, double &cs2, double &e_used, double *T) {
+  P = fx_exp2(t.fm, fx_lerp(fx_pair(nd + 1, w), fx_pair(nd + 4, w), s));
+  if (WANT_CS2) {
+    cs2 = fx_exp2(t.fm, fx_lerp(fx_pair(nd + 2, w), fx_pair(nd + 5, w), s));
+    if (T) *T = fx_exp2(t.fm, fx_log2T(t.fa, j, s));
+    e_used = cl ? fx_exp2(t.fm, fx_lerp(fx_pair(nd, w), fx_pair(nd + 3, w), s)) : e;
+  }
+}
+
+// The inversion on the prepared table.  The cell with g_j <= y < g_{j+1} is
+// unique, so any search that ends in a bracketing cell gives the same result: the
+// bucket of log e bounds it to a few cells, a bisection on the 32-bit pairs
+// picks one, the 64-bit bracket the solve needs anyway confirms it, and the rare
+// miss (log e within 2^-22 of a node) bisects the column in 64 bits.  What bounds
+// it for scattered inputs is the gathers (one 16-byte word per lane and load), so
+// the buckets (1 or 2 search loads instead of 8) and the node pairs (6 loads for
+// all of a cell's 12 values) matter as much as the arithmetic.
+template <bool WANT_CS2 = true>
+__device__ __forceinline__ bool eos_invert(const DTable &t, double rho, double e, double &P,
+                                           double &cs2, double &e_used, double *T = nullptr) {
+  if (!t.node) return eos_invert_views<WANT_CS2>(t, rho, e, P, cs2, e_used, T);   // uniform
+  int i;
+  ufx w;
+  bool cl = fx_rho_cell(t.fm, t.fa, t.nr, rho, i, w);
+  const int nt = t.nt;
+  const longlong2 *__restrict__ row = t.node + (size_t)i * nt * 3;
+  const fx y = dgt0(e) ? fx_log2(t.fm, e) : -FX_SAT;
+  int lo = 0, hi = nt - 1;
+  if (t.n32) {
+    if (t.bk) {
+      const fx q = (y - t.y0) >> t.bshift;
+      const int qi = q < 0 ? 0 : (q >= t.nbk ? t.nbk - 1 : (int)q);
+      const ushort2 r = __ldg(t.bk + (size_t)i * t.nbk + qi);
+      lo = r.x;
+      hi = r.y + 1;
+    }
+    const int2 *__restrict__ r32 = t.n32 + (size_t)i * nt;
+    const int y32 = (int)(y >> 32), w32 = (int)(w >> 33);
+    while (hi - lo > 1) {
+      const int mid = (lo + hi) >> 1;
+      const int2 v = __ldg(r32 + mid);
+      if (v.x + 2 * __mulhi(v.y - v.x, w32) <= y32) lo = mid; else hi = mid;
+    }
+  } else {   // every step in 64 bits
+    while (hi - lo > 1) {
+      const int mid = (lo + hi) >> 1;
+      if (fx_pair(row + 3 * mid, w) <= y) lo = mid; else hi = mid;
+    }
+  }
+  int j = lo;
+  fx g0 = fx_pair(row + 3 * j, w), g1 = fx_pair(row + 3 * j + 3, w);
+  ufx s;
+  for (;;) {   // at most twice
+    if (j == 0 && y <= g0) { s = 0; cl = true; break; }
+    if (j == nt - 2 && y >= g1) { s = ~0ull; cl = true; break; }
+    if (g0 <= y && y < g1) { s = fx_frac(y - g0, g1 - g0); break; }
+    lo = 0;
+    hi = nt - 1;
+    while (hi - lo > 1) {
+      const int mid = (lo + hi) >> 1;
+      if (fx_pair(row + 3 * mid, w) <= y) lo = mid; else hi = mid;
+    }
+    j = lo;
+    g0 = fx_pair(row + 3 * j, w);
+    g1 = fx_pair(row + 3 * j + 3, w);
+  }
+  eos_at<WANT_CS2>(t, row + 3 * j, w, j, s, cl, e, P, cs2, e_used, T);
   return cl;
 }
 

@@ -1,0 +1,254 @@
+// tde_fx.cuh -- 64-bit fixed-point arithmetic for the tabulated EOS: log2, exp2,
+// interpolation and the cell solve on the integer pipe.
+//
+// Why: the inversion is arithmetic on logarithms, whose absolute precision is
+// what counts, and sm_103a issues one FP64 warp instruction per 16 cycles and SM
+// against about 32 integer ones.  In FP64 an inversion takes about 100 such
+// slots (1600 cycles per warp); here it is a few hundred integer instructions
+// and no FP64 at all: 2^24 inversions of (T, P, cs^2) with densities and energies
+// scattered over the 256 x 256 table went from 3.10 ms to 0.63 ms (1.06 TB/s of
+// input and output), the learned-guess form on 6 million from 1.86 to 0.78 ms, a
+// step of the 8.4 M-cell star mesh from 25.6 to 21.4 ms.  A fixed-point logarithm of 55 fraction bits resolves
+// 2.8e-17 in log2, an FP64 one of size 40 (log10 of size 12) only 7e-15, so the
+// results are nearer to the exact ones than the FP64 form's.
+//
+// Format: Q55 in a signed 64-bit integer, in log2 units (values in (-128, 128));
+// weights and fractions are unsigned Q64.  Every step is a fixed sequence of
+// integer operations, so all kernels (and the host) get the same bits.
+//
+// Methods: log2 by a table of reciprocals c_j ~ 1/m of 10 bits (the product of
+// the 53-bit significand with c_j is exact in 64 bits) and the series of
+// ln(1 + r), |r| < 2^-8.4; exp2 by a table of 2^((j + 1/2)/256) and the series
+// of 2^g, |g| <= 2^-9 (both after the table-driven scheme of P. T. Tang, ACM
+// TOMS 15 and 16); the quotient from the FP32 reciprocal refined to second
+// order.
+#pragma once
+#include <stdint.h>
+#include <string.h>
+
+#ifdef __CUDACC__
+#define FX_HD __host__ __device__ __forceinline__
+#else
+#define FX_HD inline
+#endif
+
+namespace tde {
+
+typedef long long fx;              // Q55, log2 units
+typedef unsigned long long ufx;    // fractions, Q64
+
+constexpr int FX_Q = 55;
+constexpr fx FX_ONE = 1LL << FX_Q;
+constexpr fx FX_BAD = (fx)0x8000000000000000ull;   // a value outside the format
+constexpr fx FX_SAT = 128 * (FX_ONE - 1);          // |log2| of what lies beyond every table
+constexpr double FX_MAX_LOG10 = 38.0;              // |log10| of a table entry the format takes
+constexpr unsigned long long FX_LOG2_10 = 0xD49A784BCD1B8AFEull;   // log2(10), Q62
+
+struct FxMath {
+  fx lg[256];                    // -log2(c_j / 1024), Q55
+  unsigned long long ex[256];    // 2^((j + 1/2) / 256), Q62
+  unsigned c[256];               // 1024 / (1 + (j + 1/2) / 256), rounded
+};
+
+FX_HD fx fx_bits(double x) {
+#ifdef __CUDA_ARCH__
+  return __double_as_longlong(x);
+#else
+  fx b;
+  memcpy(&b, &x, 8);
+  return b;
+#endif
+}
+FX_HD double fx_double(fx b) {
+#ifdef __CUDA_ARCH__
+  return __longlong_as_double(b);
+#else
+  double x;
+  memcpy(&x, &b, 8);
+  return x;
+#endif
+}
+FX_HD ufx fx_umulhi(ufx a, ufx b) {
+#ifdef __CUDA_ARCH__
+  return __umul64hi(a, b);
+#else
+  return (ufx)(((unsigned __int128)a * b) >> 64);
+#endif
+}
+FX_HD fx fx_mulhi(fx a, fx b) {
+#ifdef __CUDA_ARCH__
+  return __mul64hi(a, b);
+#else
+  return (fx)(((__int128)a * b) >> 64);
+#endif
+}
+FX_HD int fx_mulhi32(int a, int b) {
+#ifdef __CUDA_ARCH__
+  return __mulhi(a, b);
+#else
+  return (int)(((fx)a * b) >> 32);
+#endif
+}
+FX_HD int fx_clz(ufx a) {
+#ifdef __CUDA_ARCH__
+  return __clzll((fx)a);
+#else
+  return __builtin_clzll(a);
+#endif
+}
+
+// log10 value v (a table entry, FP64) in Q55 log2 units, rounded to nearest;
+// FX_BAD if it is not below FX_MAX_LOG10 in magnitude (or not a number)
+FX_HD fx fx_of_log10(double v) {
+  const fx b = fx_bits(v), a = b & 0x7fffffffffffffffLL;
+  if (a >= fx_bits(FX_MAX_LOG10)) return FX_BAD;
+  const int e = (int)(a >> 52);   // 2^(e - 1023) <= |v|; subnormals round to 0 below
+  const ufx m = ((ufx)(a & 0xfffffffffffffLL) | 0x10000000000000ull) << 11;
+  // |v| log2(10) = m 2^(e - 1086) LOG2_10 2^-62 = h 2^(e - 1084), wanted times 2^55
+  const ufx h = fx_umulhi(m, FX_LOG2_10);
+  const int s = 1029 - e;         // >= 1 for |v| < 64
+  const fx q = s < 64 ? (fx)((h >> s) + ((h >> (s - 1)) & 1)) : 0;
+  return b < 0 ? -q : q;
+}
+
+// log2 of x > 0 in Q55.  x above 2^127 (or infinite, or a positive NaN)
+// saturates at FX_SAT, x below 2^-127 (or not positive) at -FX_SAT.
+FX_HD fx fx_log2(const FxMath *__restrict__ mt, double x) {
+  const fx b = fx_bits(x);
+  const int k = (int)(b >> 52) - 1023;   // negative x: far below -127
+  if (k < -126) return -FX_SAT;
+  if (k > 126) return FX_SAT;
+  const fx mant = b & 0xfffffffffffffLL;
+  const int j = (int)(mant >> 44);
+  // r = m c - 1, exact in Q62: |r| <= 2^-9 + 2^-10
+  const fx R = (fx)((ufx)(mant | 0x10000000000000LL) * mt->c[j]) - (1LL << 62);
+  const int p = (int)(R >> 23);          // 2^7 r in Q32 (r in Q39)
+  const int lo = (int)(R & 0x7fffff);
+  // ln(1 + r) = r - r^2/2 + r^2 (r s), s = 1/3 - r/4 + r^2/5 - r^3/6 (Q32; the
+  // next term, r^7/7, is below 2^-61)
+  int s = 52429 + fx_mulhi32(p, -341);   // 2^32 / (5 2^14), 2^32 / (6 2^21)
+  s = -8388608 + fx_mulhi32(p, s);       // 2^32 / (4 2^7)
+  s = 1431655765 + fx_mulhi32(p, s);     // 2^32 / 3
+  const int rs = fx_mulhi32(p, s);       // r s in Q39
+  const fx sq = (fx)p * p + (((fx)p * lo) >> 22);   // r^2 in Q78
+  const fx ln = R - (sq >> 17) + (((fx)(int)(sq >> 32) * rs) >> 23);   // Q62
+  // times log2(e) = 1 + 0.4427: Q62 -> Q55
+  const fx l2 = ln + fx_mulhi(ln, 0x71547652B82FE177LL);   // (log2(e) - 1) in Q64
+  return ((fx)k << FX_Q) + mt->lg[j] + ((l2 + 64) >> 7);
+}
+
+// 2^L, correctly rounded but for about 2^-55 relative
+FX_HD double fx_exp2(const FxMath *__restrict__ mt, fx L) {
+  const int n = (int)(L >> FX_Q), j = (int)(L >> 47) & 255;
+  const fx g = (L & ((1LL << 47) - 1)) - (1LL << 46);   // Q55, |g| <= 2^-9
+  const int q = (int)(g >> 15);                         // 2^8 g in Q32 (g in Q40)
+  // 2^g = 1 + g (c1 + g (c2 + g (c3 + g (c4 + g c5)))), c_k = ln(2)^k / k!
+  int h = 161365 + fx_mulhi32(q, 87);    // c4 2^32 / 2^8, c5 2^32 / 2^16
+  h = 238388332 + fx_mulhi32(q, h);      // c3 2^32
+  const fx h2 = 0x0F5FDEFFC162C754LL + (((fx)q * h) >> 10);              // c2 + .., Q62
+  const fx g71 = g << 16;                                                // g in Q71
+  const fx m1 = 0x2C5C85FDF473DE6BLL + (fx_mulhi(g71, h2) >> 7);         // c1 + .., Q62
+  const fx m2 = fx_mulhi(g71, m1);                                       // 2^g - 1, Q69
+  const ufx T = mt->ex[j];
+  const ufx V = T + (ufx)(fx_mulhi((fx)T, m2 << 3) >> 8);                // Q62, in [1, 2]
+  return fx_double(((fx)(n + 1022) << 52) + (fx)((V + 512) >> 10));
+}
+
+// a + w (b - a), w in Q64
+FX_HD fx fx_lerp(fx a, fx b, ufx w) { return a + (fx_mulhi(b - a, (fx)(w >> 1)) << 1); }
+
+// the fraction num / den in Q64, 0 <= num < den (< 1; error below 2^-50)
+FX_HD ufx fx_frac(fx num, fx den) {
+  const int z = fx_clz((ufx)den);
+  const ufx D = (ufx)den << z, N = (ufx)num << z;   // D in [1/2, 1) of 2^64
+  // FP32 reciprocal of D's 24 leading bits: R0 in Q23, (1, 2)
+  float rf;
+#ifdef __CUDA_ARCH__
+  rf = __frcp_rn(__uint_as_float(0x3f000000u | ((unsigned)(D >> 40) & 0x7fffffu)));
+  const unsigned rb = __float_as_uint(fminf(rf, 1.99999988f));
+#else
+  const unsigned db = 0x3f000000u | ((unsigned)(D >> 40) & 0x7fffffu);
+  float df;
+  memcpy(&df, &db, 4);
+  rf = 1.0f / df;
+  if (rf > 1.99999988f) rf = 1.99999988f;
+  unsigned rb;
+  memcpy(&rb, &rf, 4);
+#endif
+  const unsigned R = (rb & 0x7fffffu) | 0x800000u;
+  // 1/D = R (1 + e + e^2), e = 1 - D R in Q55, |e| < 2^-21
+  const fx e = FX_ONE - (fx)((ufx)(unsigned)(D >> 32) * R + (((ufx)(unsigned)D * R) >> 32));
+  const int e53 = (int)(e >> 2);
+  const fx c = e + (((fx)e53 * e53) >> 51);
+  const fx q = (fx)((ufx)(unsigned)(N >> 32) * R + (((ufx)(unsigned)N * R) >> 32));   // N R, Q55
+  fx s = q + (((fx)(int)(q >> 26) * (fx)(int)(c >> 2)) >> 27);   // Q29 x Q53
+  s = s < 0 ? 0 : (s > FX_ONE - 1 ? FX_ONE - 1 : s);
+  return (ufx)s << 9;
+}
+
+// The table's axes in fixed point (the same function of the FP64 axes for every
+// caller).  valid: the format takes them.
+struct FxAxes {
+  int valid;
+  int sh;              // x (cell units along log rho) has sh fraction bits after the scaling
+  fx L0, Dmax, tol;    // log2 of the lowest density, the range, half an FP64 ulp of log10 rho there
+  ufx G;               // 1 / (cell width), 64-bit significand
+  fx lt0, dlt;         // log2 T of the coldest node, cell width (Q55)
+  unsigned dlt_lo;     // its next 32 bits
+};
+
+inline FxAxes fx_axes(int nr, int nt, double lr0, double lr1, double inv_dlr, double lt0, double dlt) {
+  FxAxes a;
+  memset(&a, 0, sizeof a);
+  a.L0 = fx_of_log10(lr0);
+  const fx l1 = fx_of_log10(lr1);
+  a.lt0 = fx_of_log10(lt0);
+  const fx lt1 = fx_of_log10(lt0 + (nt - 1) * dlt);
+  if (a.L0 == FX_BAD || l1 == FX_BAD || a.lt0 == FX_BAD || lt1 == FX_BAD || !(inv_dlr > 0x1p-8 && inv_dlr < 0x1p20) ||
+      !(dlt < 32.0) || nr > (1 << 24) || nt > (1 << 24))
+    return a;
+  a.Dmax = l1 - a.L0;
+  const double m = (lr0 < 0 ? -lr0 : lr0) > (lr1 < 0 ? -lr1 : lr1) ? (lr0 < 0 ? -lr0 : lr0) : (lr1 < 0 ? -lr1 : lr1);
+  int ex = 0;
+  while ((double)(1u << (ex + 1)) <= m) ++ex;      // 2^ex <= largest |log10 rho| (or 1)
+  a.tol = (fx)(3.3219 * (double)(1u << (ex + 1))); // half an ulp of it: 2^(ex - 53) log2(10) 2^55
+  // 1 / (cell width in log2 units), by integer arithmetic: cells / range
+  const long double G = (long double)inv_dlr * 0.30102999566398119521373889472449302677L;   // log10(2)
+  int eg = 0;
+  long double f = G;
+  while (f >= 2.0L) { f /= 2.0L; ++eg; }
+  while (f < 1.0L) { f *= 2.0L; --eg; }
+  a.G = (ufx)(f * 9223372036854775808.0L);         // in [2^63, 2^64)
+  a.sh = 54 - eg;
+  const long double d2 = (long double)dlt * 3.3219280948873623478703194294893901759L * 36028797018963968.0L;   // Q55
+  a.dlt = (fx)d2;
+  a.dlt_lo = (unsigned)((d2 - (long double)a.dlt) * 4294967296.0L);
+  a.valid = 1;
+  return a;
+}
+
+// Density cell i and weight w (Q64) of rho; true if clamped to the table.  As in
+// FP64, a density within the rounding of the table's edge is not clamped.
+FX_HD bool fx_rho_cell(const FxMath *__restrict__ mt, const FxAxes &A, int nr, double rho, int &i, ufx &w) {
+  fx D = fx_log2(mt, rho) - A.L0;
+  bool cl = false;
+  if (D < 0) { cl = D < -A.tol; D = 0; }
+  const fx b = fx_bits(rho);
+  if ((b & 0x7fffffffffffffffLL) > 0x7ff0000000000000LL) { cl = true; D = 0; }   // not a number
+  if (D > A.Dmax) { cl = cl || D > A.Dmax + A.tol; D = A.Dmax; }
+  const ufx x = fx_umulhi((ufx)D, A.G);
+  i = (int)(x >> A.sh);
+  w = x << (64 - A.sh);
+  if (i > nr - 2) { i = nr - 2; w = ~0ull; }
+  return cl;
+}
+
+// log2 T at fraction s (Q64) of temperature cell j
+FX_HD fx fx_log2T(const FxAxes &A, int j, ufx s) {
+  return A.lt0 + (fx)j * A.dlt + (fx)(((ufx)(unsigned)j * A.dlt_lo) >> 32) + (fx)fx_umulhi((ufx)A.dlt, s);
+}
+
+// tables of fx_log2 and fx_exp2 (host, extended precision)
+void fx_fill_math(FxMath *h);
+
+}  // namespace tde

@@ -1,7 +1,7 @@
 // tde_mlp.cu -- the learned EOS guess: a 2 -> 64 -> 64 -> 2 SiLU network that maps
 // normalised (log10 rho, log10 e) to normalised (log10 T, log10 P).  The paper
 // has no learned component; the network only chooses the temperature cell in
-// which one FP64 Newton step on the interpolated log10 e column is taken, and
+// which one Newton step on the interpolated log e column is taken, and
 // table bisection stays both the fallback and the judge (Sec. 4.2 runtime map).
 //
 //  * Training: FP32 forward/backward kernels on BF16-rounded weights (the
@@ -12,7 +12,7 @@
 //    cores, the 64 x 64 layer on the 5th-generation tensor cores
 //    (tcgen05.mma kind::f16, BF16 operands from shared memory, FP32 accumulator
 //    in tensor memory, read back with tcgen05.ld), layer 3 in FP32, then the
-//    FP64 Newton step with the bisection fallback.
+//    Newton step (64-bit fixed point, as the bisection's) with its fallback.
 #include <cuda_bf16.h>
 #include <math.h>
 #include <string.h>
@@ -309,59 +309,53 @@ __device__ __forceinline__ void cm_split(const CellMap &cm, long long t, long lo
   first = (long long)((unsigned)t - q * (unsigned)per) * size;
 }
 
-// One FP64 Newton step from the guessed log10 T, judged by the table bracket.
+// One Newton step from the guessed log10 T, judged by the table bracket.
 // The column g is linear inside a temperature cell, so the step from the
-// guess's cell j lands on x = j + s with s the cell solve; if the root is in
+// guess's cell j lands on x = j + (y - g_j) / (g_{j+1} - g_j); if the root is in
 // cell j that is the root itself, otherwise x lies in the cell j' the linear
-// extension points to, and the root is taken there when j' brackets it.  An
-// accepted cell is the one bisection finds (g_j <= y < g_{j+1} is unique) and the
-// state is evaluated with the same formulas, so the result is the bisection
-// result bit for bit.  Returns false for the cells left to bisection (clamped
-// inputs, a step that misses).
+// extension points to (FP32 decides which), and the root is taken there when j'
+// brackets it.  An accepted cell is the one bisection finds (g_j <= y < g_{j+1}
+// is unique) and the state is evaluated with the same formulas (eos_at), so the
+// result is the bisection result bit for bit.  Returns false for the cells left
+// to bisection (clamped inputs, a step that misses, a table without the
+// prepared form).
 __device__ __forceinline__ bool newton_cell(const DTable &t, double rho_c, double e, float lTg, float idlt,
                                             long long c, double *T, double *P, double *cs2, double *eu) {
+  if (!t.node || !dgt0(e)) return false;
   const int nt = t.nt;
   int i;
-  double w;
-  const bool cl = rho_cell(t, rho_c, i, w);
-  // the decisions below compare on the integer pipe (dgt0, dle, dlt: the
-  // same outcomes as the FP64 comparisons for every non-NaN value)
-  const bool pos = dgt0(e);
-  if (cl || !pos) return false;
-  const double ly = tlog10(t, e);
-  const double *__restrict__ ra = t.le + (size_t)i * nt;
-  const double *__restrict__ rb = ra + nt;
+  ufx w;
+  if (fx_rho_cell(t.fm, t.fa, t.nr, rho_c, i, w)) return false;
+  const fx y = fx_log2(t.fm, e);
+  const longlong2 *__restrict__ row = t.node + (size_t)i * nt * 3;
   const float xg = (lTg - (float)t.lt0) * idlt;
   int j = (int)floorf(fminf(fmaxf(xg, 0.f), (float)(nt - 2)));
   j = min(max(j, 0), nt - 2);
-  double g0 = lerp_rn(w, __ldg(ra + j), __ldg(rb + j));
-  double g1 = lerp_rn(w, __ldg(ra + j + 1), __ldg(rb + j + 1));
-  double sc = cell_solve(ly, g0, g1);
-  bool in = dle(g0, ly) && dlt(ly, g1);
+  fx g0 = fx_pair(row + 3 * j, w), g1 = fx_pair(row + 3 * j + 3, w);
+  bool in = g0 <= y && y < g1;
   if (!in) {
-    const double xn = __dadd_rn(dint(j), sc);   // the Newton result, in cell units
-    if (dge0(xn) && dlt(xn, dint(nt - 1))) {
-      const int j2 = ifloor_nonneg(xn);
-      if (j2 != j) {
-        j = j2;
-        g0 = lerp_rn(w, __ldg(ra + j), __ldg(rb + j));
-        g1 = lerp_rn(w, __ldg(ra + j + 1), __ldg(rb + j + 1));
-        in = dle(g0, ly) && dlt(ly, g1);
-        if (in) sc = cell_solve(ly, g0, g1);
-      }
+    // (the top 32 bits are enough to choose a cell)
+    const float xn = (float)j + __fdividef((float)(int)((y - g0) >> 32), (float)max((int)((g1 - g0) >> 32), 1));
+    if (xn >= 0.f && xn < (float)(nt - 1)) {
+      j = (int)xn;
+      g0 = fx_pair(row + 3 * j, w);
+      g1 = fx_pair(row + 3 * j + 3, w);
+      in = g0 <= y && y < g1;
     }
   }
   // at the coldest node bisection clamps (y <= g_0): leave that to it
-  if (!(in && (j > 0 || dlt(g0, ly)))) return false;
-  if (P) P[c] = texp10(t, bilin(t.lp, nt, i, w, j, sc));
-  if (cs2) cs2[c] = texp10(t, bilin(t.lc, nt, i, w, j, sc));
-  if (T) T[c] = texp10(t, cell_log10T(t, j, sc));
+  if (!(in && (j > 0 || g0 < y))) return false;
+  double Pv, cv, ev, Tv;
+  eos_at<true>(t, row + 3 * j, w, j, fx_frac(y - g0, g1 - g0), false, e, Pv, cv, ev, T ? &Tv : nullptr);
+  if (P) P[c] = Pv;
+  if (cs2) cs2[c] = cv;
+  if (T) T[c] = Tv;
   if (eu) eu[c] = 0.0;   // inside the table
   return true;
 }
 
 // The learned guess.  NEWTON = 0: the network alone (raw outputs, the guess);
-// NEWTON = 1: the guess goes straight into the FP64 Newton step in the same
+// NEWTON = 1: the guess goes straight into the Newton step in the same
 // thread (newton_cell), accepted cells are written and the rest queued for
 // k_eos_fallback (one atomic per tile reserves the tile's queue slots; the
 // accepted count is added once per CTA).
@@ -426,7 +420,7 @@ __global__ void __launch_bounds__(IT, 8) k_eos_surrogate(SurrogateArgs a) {
     float y0 = 0.f, y1 = 0.f;
     if (!s_abort) {
       // ---- inputs and layer 1, FP32 only: the network needs log10 rho and the
-      // position z of log10 e in its column to FP32 accuracy (the FP64 work of
+      // position z of log10 e in its column to FP32 accuracy (the exact work of
       // the inversion is newton_cell's)
       float x0 = 0.f, x1 = 0.f;
       if (live) {
@@ -523,7 +517,7 @@ __global__ void __launch_bounds__(IT, 8) k_eos_surrogate(SurrogateArgs a) {
     const bool have = !s_abort;   // uniform: set before the last barrier
     if (!NEWTON && !have) break;
     if (NEWTON) {
-      // the FP64 Newton step from this thread's guess; misses are queued
+      // the Newton step from this thread's guess; misses are queued
       const bool ok = live ? (have && newton_cell(a.t, a.rho[c], a.e[c], a.nm.cT + a.nm.sT * y0, a.nm.idlt, c,
                                                   a.T, a.P, a.cs2, a.eu))
                            : true;
@@ -736,7 +730,7 @@ cudaError_t launch_surrogate_newton(tde_eos *e, const CellMap &cm, long long n, 
 }
 
 // The learned-guess inversion of the cells of cm (n = largest block's cell
-// count, or the array length): guess, FP64 Newton with queueing, bisection of
+// count, or the array length): guess, Newton step with queueing, bisection of
 // the queue.  The same inputs give the bisection results bit for bit.
 cudaError_t surrogate_run(tde_eos *e, const CellMap &cm, long long n, const double *rho,
                           const double *en, double *T, double *P, double *cs2, double *eu,

@@ -39,10 +39,12 @@ static __device__ __align__(256) NAScratch g_noalloc_scratch;
 // Tables of the table-driven log10 / exp10 that the mesh path's EOS lookups use
 // (4.6 KB, constant: written once per device at set-up, never by a kernel).
 static __device__ __align__(256) MathTables g_noalloc_mt;
+static __device__ __align__(256) FxMath g_noalloc_fm;   // and of fx_log2 / fx_exp2 (5 KB)
 
 // device addresses of the two arrays, looked up once per device
 NAScratch *g_scratch_ptr[64] = {};
 const MathTables *g_mt_ptr[64] = {};
+const FxMath *g_fm_ptr[64] = {};
 
 __device__ __forceinline__ void na_bh_pos(const BH &bh, double t, double r[3]) {
   const double s = t - bh.t0;
@@ -200,18 +202,23 @@ extern "C" int tde_compute_dt_noalloc(tde_ctx *ctx, int nblocks, const tde_block
     return na_fail(ctx, TDE_EINVAL, "tde_compute_dt_noalloc: grid (N >= 1, ghost width 0..8)");
 
   // one-time set-up per device (the first call on a device does it; that first
-  // call should therefore come before any stream capture): the two arrays'
-  // device addresses, and the log10 / exp10 tables copied into the second
+  // call should therefore come before any stream capture): the arrays'
+  // device addresses, and the log10 / exp10 tables copied into the others
   cudaError_t err = cudaSetDevice(ctx->device);
   if (err == cudaSuccess && !g_scratch_ptr[ctx->device]) {
     MathTables h;
     fill_math_tables(&h);
-    void *ps = nullptr, *pm = nullptr;
+    FxMath hf;
+    fx_fill_math(&hf);
+    void *ps = nullptr, *pm = nullptr, *pf = nullptr;
     err = cudaMemcpyToSymbol(g_noalloc_mt, &h, sizeof h);
+    if (err == cudaSuccess) err = cudaMemcpyToSymbol(g_noalloc_fm, &hf, sizeof hf);
+    if (err == cudaSuccess) err = cudaGetSymbolAddress(&pf, g_noalloc_fm);
     if (err == cudaSuccess) err = cudaGetSymbolAddress(&pm, g_noalloc_mt);
     if (err == cudaSuccess) err = cudaGetSymbolAddress(&ps, g_noalloc_scratch);
     if (err == cudaSuccess) {
       g_mt_ptr[ctx->device] = static_cast<const MathTables *>(pm);
+      g_fm_ptr[ctx->device] = static_cast<const FxMath *>(pf);
       g_scratch_ptr[ctx->device] = static_cast<NAScratch *>(ps);
     }
   }
@@ -246,6 +253,8 @@ extern "C" int tde_compute_dt_noalloc(tde_ctx *ctx, int nblocks, const tde_block
     p.tab.lp = table->log10_P;
     p.tab.lc = table->log10_cs2;
     p.tab.mt = g_mt_ptr[ctx->device];
+    p.tab.fm = g_fm_ptr[ctx->device];
+    p.tab.fa = fx_axes(p.tab.nr, p.tab.nt, p.tab.lr0, table->log10_rho_max, p.tab.inv_dlr, p.tab.lt0, p.tab.dlt);
   }
   p.dxmin = INFINITY;
   for (int a = 0; a < 3; ++a) {

@@ -30,7 +30,21 @@ enum { RIEMANN_HLLC = 0, RIEMANN_HLLE = 1 };
 // For NaN operands they are not the IEEE predicates; the kernels count
 // non-finite states rather than rely on comparisons with NaN.
 
-__device__ __forceinline__ long long dbits(double x) { return __double_as_longlong(x); }
+// The bits through an opaque move: the compiler recognises sign and magnitude
+// masks and comparisons of a double's bits and turns them back into FP64
+// instructions (a magnitude into an FP64 addition: 28 of them per cell in an
+// eight-variable PPM sweep).
+__device__ __forceinline__ long long dbits(double x) {
+  long long b;
+  asm("mov.b64 %0, %1;" : "=l"(b) : "d"(x));
+  return b;
+}
+__device__ __forceinline__ double dfrom(long long b) {
+  double x;
+  asm("mov.b64 %0, %1;" : "=d"(x) : "l"(b));
+  return x;
+}
+__device__ __forceinline__ long long dmag(double x) { return dbits(x) & 0x7fffffffffffffffLL; }   // bits of |x|
 // order key: key(a) < key(b) iff a < b for non-NaN a, b (except -0 < +0)
 __device__ __forceinline__ long long dkey(double x) {
   const long long b = dbits(x);
@@ -50,6 +64,9 @@ __device__ __forceinline__ bool dle(double a, double b) { return dkey(a) <= dkey
 __device__ __forceinline__ double dmin(double a, double b) { return dkey(a) <= dkey(b) ? a : b; }
 __device__ __forceinline__ double dmax(double a, double b) { return dkey(a) >= dkey(b) ? a : b; }
 __device__ __forceinline__ bool dfinite(double x) { return ((dbits(x) >> 52) & 0x7ff) != 0x7ff; }
+// -x and |x| by the sign bit
+__device__ __forceinline__ double dneg(double x) { return dfrom(dbits(x) ^ (long long)0x8000000000000000ull); }
+__device__ __forceinline__ double dabs(double x) { return dfrom(dmag(x)); }
 // the double value of a small integer |k| < 2^51, by one FP64 add
 __device__ __forceinline__ double dint(long long k) {
   return __longlong_as_double(0x4338000000000000LL + k) - 6755399441055744.0;
@@ -211,7 +228,7 @@ __host__ __device__ __forceinline__ double exp2i(int e) {
 // x 2^e for a normal x whose result is normal: an integer add on the exponent
 // field (exact, and no FP64 instruction)
 __device__ __forceinline__ double scale2i(double x, int e) {
-  return __longlong_as_double(__double_as_longlong(x) + ((long long)e << 52));
+  return dfrom(dbits(x) + ((long long)e << 52));
 }
 
 // cell width, its reciprocal and the grid size along a on block B's level
@@ -244,42 +261,36 @@ __device__ __forceinline__ double rsqrt_seed(double d) {
   return r;
 }
 
-// 1/d from the seed r: with e = 1 - d r, 1/d = r / (1 - e) = r (1 + e + e^2 +
-// e^3 + ...); keeping the terms through e^2 (two FMAs after the residual)
-// leaves a truncation error ~e^3 < 2^-59, far below the FP64 rounding, so the
-// result is within one ulp of 1/d.  For normal d whose reciprocal is normal
-// (every use below: sums of same-signed slopes, wave-speed differences,
-// densities, Gamma_e - 1).
-__device__ __forceinline__ double rcp_nr(double d) {
+// 1/d within 0.51 ulp by integer arithmetic (fx_rcp) for normal d whose reciprocal
+// is normal; otherwise (zero, infinite, not a number, at the ends of the range)
+// from the hardware seed r: with e = 1 - d r, 1/d = r (1 + e + e^2 + ...).
+// (The rare forms are calls: inlined, the compiler would evaluate them for every
+// thread and select, on the FP64 pipe.)
+static __device__ __noinline__ double rcp_fp64(double d) {
   const double r = rcp_seed(d);
   const double e = fma(-d, r, 1.0);
   return fma(r, fma(e, e, e), r);
 }
-
-// sqrt(a / b) for a, b > 0 as a / sqrt(a b): y = seed of 1/sqrt(t), t = a b,
-// e = 1 - t y^2, 1/sqrt(t) = y (1 - e)^(-1/2) = y (1 + e/2 + 3 e^2/8 + ...);
-// the truncation error ~(5/16) e^3 is below 2^-61, and the roundings of t, y^2
-// and the final product keep the result within about two ulps of the correctly
-// rounded sqrt(a / b).  Replaces a division and a square root (the wave-speed
-// estimates of the Riemann solver and of the time-step condition).  Where a b
-// leaves the range in which the seed and y^2 are normal (floor states of
-// 1e-300 give a b ~ 1e-600) the IEEE form is used instead.
-__device__ __forceinline__ double sqrt_ratio(double a, double b) {
-  const double t = a * b;
-  if ((unsigned long long)(((dbits(t) >> 52) & 0x7ff) - 2) >= 0x7fcull) return sqrt(a / b);
-  const double y = rsqrt_seed(t);
-  const double e = fma(-t, y * y, 1.0);
-  const double y1 = fma(y, e * fma(e, 0.375, 0.5), y);
-  return a * y1;
+__device__ __forceinline__ double rcp_nr(double d) {
+  const long long b = dbits(d);
+  return fx_rcp_ok(b) ? fx_rcp(b) : rcp_fp64(d);
 }
 
-// 1/sqrt(t) for t > 0: the hardware seed refined to second order as in
-// sqrt_ratio, within about two ulps; the IEEE form outside the seed's normal range
+// sqrt(a / b) for a, b > 0 within 0.52 ulp by integer arithmetic (the wave speeds
+// of the Riemann solver and of the time-step condition); the IEEE form where a or
+// b is not a positive normal number.
+static __device__ __noinline__ double sqrt_ratio_ieee(double a, double b) { return sqrt(a / b); }
+__device__ __forceinline__ double sqrt_ratio(double a, double b) {
+  const long long ka = dbits(a), kb = dbits(b);
+  if (fx_pos_ok(ka) && fx_pos_ok(kb)) return fx_sqrt_ratio(ka, kb);
+  return sqrt_ratio_ieee(a, b);
+}
+
+// 1/sqrt(t) for t > 0, likewise
+static __device__ __noinline__ double rsqrt_ieee(double t) { return 1.0 / sqrt(t); }
 __device__ __forceinline__ double rsqrt_nr(double t) {
-  if ((unsigned long long)(((dbits(t) >> 52) & 0x7ff) - 2) >= 0x7fcull) return 1.0 / sqrt(t);
-  const double y = rsqrt_seed(t);
-  const double e = fma(-t, y * y, 1.0);
-  return fma(y, e * fma(e, 0.375, 0.5), y);
+  const long long k = dbits(t);
+  return fx_pos_ok(k) ? fx_rsqrt(k) : rsqrt_ieee(t);
 }
 
 // sqrt(r2) < r for r2 >= 0, decided as with the correctly rounded square root:
@@ -670,46 +681,72 @@ __device__ __forceinline__ void cons_to_prim(const Phys &p, const double *u, dou
 }
 
 // ------------------------------------------------------- reconstruction ----
+//
+// Both schemes work on the differences D of neighbouring cells along a pencil; a
+// thread walks a run of cells of one variable, so each cell value is read once
+// and each difference formed once.
 
-// PLM, van Leer limiter: half-slope h = dl dr / (dl + dr) if dl dr > 0; faces q -+ h
-__device__ __forceinline__ void plm(double qm, double q0, double qp, double &left, double &right) {
-  double dl = q0 - qm, dr = qp - q0;
-  double pr = dl * dr;
-  double h = dgt0(pr) ? pr * rcp_nr(dl + dr) : 0.0;
-  left = q0 - h;
-  right = q0 + h;
+// PLM, van Leer limiter, cell q0 with the differences dl, dr to its neighbours:
+// half-slope h = dl dr / (dl + dr) if dl dr > 0; faces q0 -+ h.  (Where a product
+// is added to something, the rounding is spelt out here and in the Riemann
+// solvers, so that every kernel they are compiled into gives the same bits.)
+__device__ __forceinline__ void plm(double q0, double dl, double dr, double &left, double &right) {
+  const double pr = __dmul_rn(dl, dr);
+  left = q0;
+  right = q0;
+  if (dgt0(pr)) {
+    const double ir = rcp_nr(__dadd_rn(dl, dr));
+    left = __fma_rn(-pr, ir, q0);
+    right = __fma_rn(pr, ir, q0);
+  }
 }
 
-// PPM: 4th-order interface value between q0 and q1, clipped to [q0, q1]
-__device__ __forceinline__ double ppm_iface(double qm1, double q0, double q1, double q2) {
-  double a = (7.0 / 12.0) * (q0 + q1) - (1.0 / 12.0) * (qm1 + q2);
-  double lo = dmin(q0, q1), hi = dmax(q0, q1);
-  return dmin(dmax(a, lo), hi);
+// PPM interface between cells q0 and q1 = q0 + D1, with D0 and D2 the differences
+// below and above: the 4th-order value 7/12 (q0 + q1) - 1/12 (qm1 + q2) is
+// q0 + T/2 with T = D1 + (D0 - D2)/6; clipped to [q0, q1] (T to between 0 and
+// 2 D1, by its sign and magnitude on the integer pipe).  Returns the value and
+// twice its distance from q0 (T) and from q1 (V = 2 D1 - T).
+__device__ __forceinline__ double ppm_iface(double q0, double q1, double D0, double D1, double D2, double &T,
+                                            double &V) {
+  double t = fma(D0 - D2, 1.0 / 6.0, D1);
+  const long long bt = dbits(t), b1 = dbits(D1);
+  const long long m1 = b1 & 0x7fffffffffffffffLL;
+  const bool over = (bt & 0x7fffffffffffffffLL) > m1 + 0x10000000000000LL && (bt ^ b1) >= 0;   // |t| > 2 |D1|
+  if ((bt ^ b1) < 0 || m1 < 0x10000000000000LL) t = 0.0;   // the other sign, or D1 = 0
+  T = t;
+  V = fma(2.0, D1, -t);
+  double a = fma(0.5, t, q0);
+  if (over && m1 >= 0x10000000000000LL) {
+    T = scale2i(D1, 1);
+    V = 0.0;
+    a = q1;
+  }
+  return a;
 }
 
-// Colella-Woodward (1984) monotonicity constraints on the parabola (aL, q0, aR).
-// The textbook tests (aR - q0)(q0 - aL) <= 0, da^2 < da q6 and da q6 < -da^2
-// (da = aR - aL, q6 = 6 (q0 - (aL + aR) / 2)) are taken in equivalent forms that
-// need no FP64 product: q0 not strictly between aL and aR; aL on the far side of
-// 3 q0 - 2 aR; aR on the far side of 3 q0 - 2 aL ("far" along the sign of da,
-// by which the textbook inequalities divide).  The comparisons run on the
-// integer pipe; the forms agree with the products except within rounding of a
-// tie, where both branches give the same interface value up to rounding (at the
-// tie of the second test 3 q0 - 2 aR equals aL), and for products that
-// underflow.  Three FP64 operations per variable and cell instead of about ten.
-__device__ __forceinline__ void ppm_limit(double q0, double &aL, double &aR) {
-  const long long kL = dkey0(aL), kR = dkey0(aR), kq = dkey0(q0);
-  const bool up = kL < kR;
-  if (up ? !(kL < kq && kq < kR) : !(kR < kq && kq < kL)) {
+// Colella-Woodward (1984) monotonicity constraints on the parabola (aL, q0, aR),
+// given V = 2 (q0 - aL) and T = 2 (aR - q0).  The textbook tests
+// (aR - q0)(q0 - aL) <= 0, da^2 < da q6 and da q6 < -da^2 (da = aR - aL,
+// q6 = 6 (q0 - (aL + aR) / 2)) read, in these distances: V and T of opposite
+// sign or zero; |V| > 2 |T|; |T| > 2 |V|.  All on the integer pipe; the limited
+// values 3 q0 - 2 aR = q0 - T and 3 q0 - 2 aL = q0 + V take one FP64 operation
+// where a limit acts.
+__device__ __forceinline__ void ppm_limit(double q0, double V, double T, double &aL, double &aR) {
+  const long long bv = dbits(V), bt = dbits(T);
+  const long long mv = bv & 0x7fffffffffffffffLL, mt = bt & 0x7fffffffffffffffLL;
+  const bool flat = (bv ^ bt) < 0 || mv == 0 || mt == 0;
+  const bool low = !flat && mv > mt + 0x10000000000000LL, high = !flat && mt > mv + 0x10000000000000LL;
+  if (flat) {
     aL = q0;
     aR = q0;
-    return;
   }
-  const double t3 = 3.0 * q0;
-  const double nL = fma(-2.0, aR, t3), nR = fma(-2.0, aL, t3);
-  const long long knL = dkey0(nL), knR = dkey0(nR);
-  if (up ? kL < knL : knL < kL) aL = nL;
-  else if (up ? knR < kR : kR < knR) aR = nR;
+  // (a vote, so that the addition is skipped where no lane of the warp needs it
+  // rather than evaluated and selected)
+  if (__any_sync(__activemask(), low || high)) {
+    const double x = q0 + (low ? dneg(T) : V);
+    if (low) aL = x;
+    if (high) aR = x;
+  }
 }
 
 // ------------------------------------------------------------------ HLLC ----
@@ -723,56 +760,55 @@ struct FState {
 // Davis wave-speed estimates; F[0..4] = mass, momentum, energy; F[5] = U_aux
 // flux (Eq. dual-flux); vf = face velocity (Eq. dual-face-velocity).  The wave
 // pattern is selected without branching on it.
+//
+// Every speed enters relative to the chosen side's gas (sigma = S - u,
+// w = S_M - u), which keeps the contact's distance from the gas to full precision
+// in flows far faster than sound, and the star state's flux is written by its
+// contact: mass m = r chi S_M with chi = sigma / (S - S_M), momentum m v plus
+// P* = P + r sigma w, energy (E* + P*) S_M, auxiliary A chi S_M, instead of
+// F_K + S (U*_K - U_K).  Outside the wave fan chi = 1, w = 0 and S_M = u give the
+// side's own flux by the same expressions.  About 40 FP64 operations a face
+// instead of 73 (the square roots and reciprocals are integer arithmetic).
 template <int D, int EOSK, int DUAL>
 __device__ __forceinline__ void hllc(const Phys &p, const FState &L, const FState &R, double *F,
                                      double &vf) {
   const int t1 = D == 0 ? 1 : 0, t2 = D == 2 ? 1 : 2;
-  double ul = L.v[D], ur = R.v[D];
-  double cl = sqrt_ratio(L.g1 * L.P, L.r), cr = sqrt_ratio(R.g1 * R.P, R.r);
-  double SL = dmin(ul - cl, ur - cr);
-  double SR = dmax(ul + cl, ur + cr);
-  double al = L.r * (SL - ul), ar = R.r * (SR - ur);
-  double SM = (R.P - L.P + al * ul - ar * ur) * rcp_nr(al - ar);
-  bool supL = dge0(SL), supR = dle0(SR);
-  bool useL = supL || (!supR && dge0(SM));
-  // chosen side K; its total energy only (the other side's enters no flux)
-  double r = useL ? L.r : R.r, un = useL ? ul : ur, P = useL ? L.P : R.P;
-  const double vK0 = useL ? L.v[0] : R.v[0], vK1 = useL ? L.v[1] : R.v[1], vK2 = useL ? L.v[2] : R.v[2];
-  const double UK = EOSK == EOS_IDEAL ? P * p.inv_gm1 : P * rcp_nr((useL ? L.ge : R.ge) - 1.0);
-  double E = UK + 0.5 * r * (vK0 * vK0 + vK1 * vK1 + vK2 * vK2);
-  double vt1 = useL ? L.v[t1] : R.v[t1], vt2 = useL ? L.v[t2] : R.v[t2];
-  double S = useL ? SL : SR;
-  double Seff = (supL || supR) ? 0.0 : S;
-  double den = S - SM;
-  if (dzero(den)) den = 1.0;   // only reachable when Seff == 0
-  double rS = useL ? al : ar;   // r (S - u) of side K: the same product as al / ar
-  double inv = rcp_nr(den);
-  double fac = rS * inv;
-  double mflux = r * un;
-  // U*_K - U_K and F_K in the (normal, t1, t2) frame
-  double d0 = fac - r;
-  double dn = fac * SM - mflux;
-  double d1 = (fac - r) * vt1;
-  double d2 = (fac - r) * vt2;
-  // E*_K - E_K = [E (S - u) + (SM - u)(rS SM + P)] / (S - SM) - E
-  //            = (SM - u)(E + P + rS SM) / (S - SM): no cancellation, two fewer FP64 ops
-  const double EP = E + P;
-  double dE = (SM - un) * fma(rS, SM, EP) * inv;
-  F[0] = mflux + Seff * d0;
-  double Fn = mflux * un + P + Seff * dn;
-  double F1 = mflux * vt1 + Seff * d1;
-  double F2 = mflux * vt2 + Seff * d2;
-  F[1 + D] = Fn;
-  F[1 + t1] = F1;
-  F[1 + t2] = F2;
-  F[4] = EP * un + Seff * dE;
+  const double ul = L.v[D], ur = R.v[D];
+  const double cl = sqrt_ratio(L.g1 * L.P, L.r), cr = sqrt_ratio(R.g1 * R.P, R.r);
+  // S_L - u_L = min(-c_L, du - c_R), S_R - u_R = max(c_R, c_L - du), du = u_R - u_L
+  const double du = ur - ul;
+  const double sl = dmin(dneg(cl), du - cr), sr = dmax(cr, cl - du);
+  const double al = __dmul_rn(L.r, sl), ar = __dmul_rn(R.r, sr);
+  // S_M - u_L = (P_R - P_L - a_R du) / (a_L - a_R)
+  const double wl = __dmul_rn(fma(-ar, du, R.P - L.P), rcp_nr(__dsub_rn(al, ar)));
+  const double SM = __dadd_rn(ul, wl);
+  const bool supL = dle(dneg(ul), sl), supR = dle(sr, dneg(ur));   // S_L >= 0, S_R <= 0
+  const bool useL = supL || (!supR && dge0(SM)), sup = supL || supR;
+  const double r = useL ? L.r : R.r, un = useL ? ul : ur, P = useL ? L.P : R.P;
+  const double v0 = useL ? L.v[0] : R.v[0], v1 = useL ? L.v[1] : R.v[1], v2 = useL ? L.v[2] : R.v[2];
+  const double vt1 = useL ? L.v[t1] : R.v[t1], vt2 = useL ? L.v[t2] : R.v[t2];
+  const double sg = useL ? sl : sr, rs = useL ? al : ar;
+  // E + P
+  const double ig = EOSK == EOS_IDEAL ? p.inv_gm1 : rcp_nr((useL ? L.ge : R.ge) - 1.0);
+  const double EP = fma(0.5 * r, fma(v2, v2, fma(v1, v1, v0 * v0)), fma(P, ig, P));
+  const double wk = useL ? wl : __dsub_rn(wl, du);
+  double den = __dsub_rn(sg, wk);
+  if (dzero(den)) den = 1.0;   // only outside the fan
+  const double inv = rcp_nr(den);
+  const double uf = sup ? un : SM, w = sup ? 0.0 : wk;
+  const double q = sup ? uf : (sg * inv) * uf;   // chi times the face's normal velocity
+  // E* + P* = E + P + w ((E + P + r sigma S_M) / (S - S_M) + r sigma)
+  const double H = fma(w, fma(fma(rs, uf, EP), inv, rs), EP);
+  const double m = r * q;
+  F[0] = m;
+  F[1 + D] = fma(m, uf, fma(rs, w, P));
+  F[1 + t1] = m * vt1;
+  F[1 + t2] = m * vt2;
+  F[4] = H * uf;
   if (DUAL) {
-    double f = F[0];
-    bool up = dgt0(f);
-    double ru = up ? L.r : R.r, Au = up ? L.A : R.A;
-    double iru = rcp_nr(ru);
-    F[5] = !dzero(f) ? f * (Au * iru) : 0.0;
-    vf = !dzero(f) ? f * iru : 0.0;
+    // the chosen side is the upwind one of the mass flux
+    F[5] = q * (useL ? L.A : R.A);
+    vf = q;
   } else {
     F[5] = 0.0;
     vf = 0.0;
@@ -782,32 +818,35 @@ __device__ __forceinline__ void hllc(const Phys &p, const FState &L, const FStat
 // HLLE flux across a face normal to direction D (Harten, Lax and van Leer with
 // Einfeldt's two-wave form; the production solver of Table 1) with the same
 // Davis wave-speed bounds as hllc: b- = min(S_L, 0), b+ = max(S_R, 0),
-// F = (b+ F_L - b- F_R + b+ b- (U_R - U_L)) / (b+ - b-); F[5] and vf follow the
-// sign of the mass flux as for hllc.
+// F = (b+ F_L - b- F_R + b+ b- (U_R - U_L)) / (b+ - b-), written by what each
+// side carries: with alpha = b+ / (b+ - b-) and beta = 1 - alpha, side L enters
+// with the velocity a_L = alpha (u_L - b-) and the pressure share alpha P_L, side R
+// with a_R = beta (u_R - b+) and beta P_R (about 45 FP64 operations instead of
+// 90); F[5] and vf follow the sign of the mass flux as for hllc.
 template <int D, int EOSK, int DUAL>
 __device__ __forceinline__ void hlle(const Phys &p, const FState &L, const FState &R, double *F,
                                      double &vf) {
-  double ul = L.v[D], ur = R.v[D];
-  double cl = sqrt_ratio(L.g1 * L.P, L.r), cr = sqrt_ratio(R.g1 * R.P, R.r);
-  double Ul = EOSK == EOS_IDEAL ? L.P * p.inv_gm1 : L.P * rcp_nr(L.ge - 1.0);
-  double Ur = EOSK == EOS_IDEAL ? R.P * p.inv_gm1 : R.P * rcp_nr(R.ge - 1.0);
-  double El = Ul + 0.5 * L.r * (L.v[0] * L.v[0] + L.v[1] * L.v[1] + L.v[2] * L.v[2]);
-  double Er = Ur + 0.5 * R.r * (R.v[0] * R.v[0] + R.v[1] * R.v[1] + R.v[2] * R.v[2]);
+  const double ul = L.v[D], ur = R.v[D];
+  const double cl = sqrt_ratio(L.g1 * L.P, L.r), cr = sqrt_ratio(R.g1 * R.P, R.r);
+  const double igl = EOSK == EOS_IDEAL ? p.inv_gm1 : rcp_nr(L.ge - 1.0);
+  const double igr = EOSK == EOS_IDEAL ? p.inv_gm1 : rcp_nr(R.ge - 1.0);
+  const double El = fma(0.5 * L.r, fma(L.v[2], L.v[2], fma(L.v[1], L.v[1], L.v[0] * L.v[0])), __dmul_rn(L.P, igl));
+  const double Er = fma(0.5 * R.r, fma(R.v[2], R.v[2], fma(R.v[1], R.v[1], R.v[0] * R.v[0])), __dmul_rn(R.P, igr));
   const double bm = dmin(dmin(ul - cl, ur - cr), 0.0);
   const double bp = dmax(dmax(ul + cl, ur + cr), 0.0);
   double den = bp - bm;
   if (dzero(den)) den = 1.0;   // both fluxes vanish there
-  const double inv = rcp_nr(den), bpm = bp * bm;
-  const double ml = L.r * ul, mr = R.r * ur;
-  // mass, momentum (x, y, z), energy: physical fluxes and conserved states
-  F[0] = (bp * ml - bm * mr + bpm * (R.r - L.r)) * inv;
+  const double inv = rcp_nr(den), al = __dmul_rn(bp, inv), be = __dmul_rn(dneg(bm), inv);
+  const double cL = __dmul_rn(al, __dsub_rn(ul, bm)), cR = __dmul_rn(be, __dsub_rn(ur, bp));
+  const double ml = __dmul_rn(cL, L.r), mr = __dmul_rn(cR, R.r);
+  const double pl = __dmul_rn(al, L.P), pr = __dmul_rn(be, R.P);
+  F[0] = __dadd_rn(ml, mr);
 #pragma unroll
   for (int q = 0; q < 3; ++q) {
-    const double fl = ml * L.v[q] + (q == D ? L.P : 0.0);
-    const double fr = mr * R.v[q] + (q == D ? R.P : 0.0);
-    F[1 + q] = (bp * fl - bm * fr + bpm * (R.r * R.v[q] - L.r * L.v[q])) * inv;
+    const double f = __fma_rn(ml, L.v[q], __dmul_rn(mr, R.v[q]));
+    F[1 + q] = q == D ? __dadd_rn(f, __dadd_rn(pl, pr)) : f;
   }
-  F[4] = (bp * ((El + L.P) * ul) - bm * ((Er + R.P) * ur) + bpm * (Er - El)) * inv;
+  F[4] = fma(El, cL, fma(pl, ul, fma(Er, cR, __dmul_rn(pr, ur))));
   if (DUAL) {
     double f = F[0];
     bool up = dgt0(f);

@@ -144,7 +144,7 @@ __global__ void __launch_bounds__(NT) k_c2p(Phys p, BH bh, TimeArgs ta,
         double rate = 0.0;
 #pragma unroll
         for (int a = 0; a < 3; ++a)
-          if (p.active[a]) rate = dmax(rate, (fabs(w[1 + a]) + cs) * block_idx(p, B, a));
+          if (p.active[a]) rate = dmax(rate, (dabs(w[1 + a]) + cs) * block_idx(p, B, a));
         best = dmin(best, rcp_nr(rate));
       }
     }
@@ -820,14 +820,13 @@ cudaError_t build_sweep_tmaps(tde_mesh *m) {
 }
 
 // shared memory of one sweep CTA (doubles, then the excision bytes): the
-// staging / flux union, the face values, the PPM interface scratch, the
-// potential and the density of the tile's cells
+// staging / flux union, the face values, the potential and the density of the
+// tile's cells
 static size_t sweep_smem(const Phys &p, int D, int PD, int NF, int M) {
   const int NV = p.nwv;
   int LS, XO;
   sweep_lane_layout(p, D, M, LS, XO);
-  size_t nd = (size_t)sweep_union_len(D, NV, PD, NF, M, LS) + 2 * (size_t)NV * NF * M +
-              (p.recon == PPM ? 4 * (size_t)(NF + 1) * M : 0) + 2 * (size_t)NF * M;
+  size_t nd = (size_t)sweep_union_len(D, NV, PD, NF, M, LS) + 2 * (size_t)NV * NF * M + 2 * (size_t)NF * M;
   // then the excision flags (NF M bytes, rounded up to doubles) and the TMA barrier
   return (nd + ((size_t)NF * M + 7) / 8 + 1) * sizeof(double);
 }

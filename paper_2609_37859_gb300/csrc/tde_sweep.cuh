@@ -112,7 +112,7 @@ __device__ __forceinline__ bool sweep_wait(uint32_t mbar, uint32_t parity) {
 
 // Shared memory of a sweep tile, in doubles (then the excision bytes):
 // the staged primitives, later reused for the fluxes; the face values; the
-// PPM interface scratch; the potential and the density of the tile's cells.
+// potential and the density of the tile's cells.
 __host__ __device__ __forceinline__ int sweep_stage_len(int D, int NV, int PD, int M, int LS) {
   return D == 0 ? NV * PD * M : NV * PD * LS;
 }
@@ -123,10 +123,9 @@ __host__ __device__ __forceinline__ int sweep_union_len(int D, int NV, int PD, i
 
 // the TMA completion barrier of a sweep CTA: 8-byte aligned after the excision
 // flags (the last part of the tile's shared memory)
-template <int D, int RECON, int NV, int M>
+template <int D, int NV, int M>
 __device__ __forceinline__ unsigned long long *sweep_mbar(double *sm, int PD, int NF, int LS) {
-  double *Rh = sm + sweep_union_len(D, NV, PD, NF, M, LS) + 2 * NV * NF * M +
-               (RECON == PPM ? 4 * (NF + 1) * M : 0) + NF * M;
+  double *Rh = sm + sweep_union_len(D, NV, PD, NF, M, LS) + 2 * NV * NF * M + NF * M;
   return reinterpret_cast<unsigned long long *>(Rh + NF * M + (NF * M + 7) / 8);
 }
 
@@ -173,8 +172,7 @@ __device__ __forceinline__ bool sweep_tile(const SweepArgs &a, int qb, int tile,
   double *Fl = sm;
   double *FMs = sm + sweep_union_len(D, NV, PD, NF, M, LS);   // [NV][NF][M]  low face of cells g-1 .. g+nd
   double *FPs = FMs + NV * NF * M;       // [NV][NF][M]  high face
-  double *If = FPs + NV * NF * M;        // PPM: [4][NF + 1][M] interface values
-  double *Ph = If + (RECON == PPM ? 4 * (NF + 1) * M : 0);   // [NF][M] potential of cells g-1 .. g+nd
+  double *Ph = FPs + NV * NF * M;        // [NF][M] potential of cells g-1 .. g+nd
   double *Rh = Ph + NF * M;              // [NF][M] density of the same cells (gravity source)
   unsigned char *Ex = reinterpret_cast<unsigned char *>(Rh + NF * M);   // [NF][M] excised
 
@@ -300,72 +298,71 @@ __device__ __forceinline__ bool sweep_tile(const SweepArgs &a, int qb, int tile,
 
   // ---- B: face values of every cell adjacent to a face of the tile; the
   // density of those cells kept for the gravity source (the staged primitives
-  // become the flux area after this phase)
-  if (grav) {
-    for (int e = threadIdx.x; e < (nd + 2) * M; e += NTS) {
-      int c, lane;
-      split(e, nd + 2, c, lane);
-      if (lane >= nlane) continue;
-      Rh[D == 0 ? lane * NF + c : c * M + lane] = Wt[sw(0, g - 1 + c, lane)];
-    }
-  }
-  if (RECON == PLM) {
-    for (int e = threadIdx.x; e < (nd + 2) * M; e += NTS) {
-      int c, lane;
-      split(e, nd + 2, c, lane);
-      if (lane >= nlane) continue;
-      const int pos = g - 1 + c;
-#pragma unroll
-      for (int v = 0; v < NV; ++v) {
-        double lo, hi;
-        plm(Wt[sw(v, pos - 1, lane)], Wt[sw(v, pos, lane)], Wt[sw(v, pos + 1, lane)], lo, hi);
-        FMs[sf(v, c, lane)] = lo;
-        FPs[sf(v, c, lane)] = hi;
-      }
-    }
-    __syncthreads();
-  } else {
-    // PPM: the interpolated value of each of the nd + 3 interfaces once (a cell's
-    // upper interface is its neighbour's lower one), four variables at a time,
-    // then the monotonicity limits per cell
-    const int NI = NF + 1, nfc = nd + 3;
-    auto si = [&](int vv, int f, int lane) {
-      return D == 0 ? (vv * M + lane) * NI + f : (vv * NI + f) * M + lane;
-    };
-#pragma unroll
-    for (int h = 0; h < NV; h += 4) {
-      for (int e = threadIdx.x; e < nfc * M; e += NTS) {
-        int f, lane;
-        split(e, nfc, f, lane);
-        if (lane >= nlane) continue;
-        const int p0 = g - 3 + f;   // interface f lies between cells p0 + 1 and p0 + 2
-#pragma unroll
-        for (int vv = 0; vv < 4; ++vv) {
-          if (h + vv >= NV) break;
-          const int v = h + vv;
-          If[si(vv, f, lane)] = ppm_iface(Wt[sw(v, p0, lane)], Wt[sw(v, p0 + 1, lane)],
-                                          Wt[sw(v, p0 + 2, lane)], Wt[sw(v, p0 + 3, lane)]);
+  // become the flux area after this phase).  A thread takes a run of cells of one
+  // variable and lane, so every cell value is read once and every difference and
+  // interface value formed once (but for those at a run's start), with no barrier
+  // before the Riemann solves.  A PPM run starts with seven extra FP64 operations
+  // (of seven a cell) and a PLM run with one (of six), while a few warps keep the
+  // FP64 pipe busy: PPM takes two runs a pencil (an x sweep of 2 M cells: 513 /
+  // 486 / 498 / 506 us with 1 / 2 / 3 / 4 runs), PLM four (a step of the 128^3
+  // wave: 2.84 / 2.66 / 2.63 / 2.62 ms).
+  {
+    constexpr int NRUN = RECON == PPM ? 2 : 4;
+    const int RL = (nd + 2 + NRUN - 1) / NRUN;
+    const int ws = D == 0 ? 1 : LS, fs = D == 0 ? 1 : M;
+    for (int e = threadIdx.x; e < NV * NRUN * M; e += NTS) {
+      const int lane = e % M, v = e / (M * NRUN);
+      const int c0 = (e / M % NRUN) * RL, c1 = min(c0 + RL, nd + 2);
+      if (lane >= nlane || c0 >= c1) continue;
+      const double *w = Wt + sw(v, g - 1 + c0, lane);
+      double *fm = FMs + sf(v, c0, lane), *fp = FPs + sf(v, c0, lane);
+      double *rh = Rh + (D == 0 ? lane * NF + c0 : c0 * M + lane);
+      const bool keep = grav && v == 0;
+      double q0 = w[0], q1 = w[ws];
+      if (RECON == PLM) {
+        double dl = q0 - w[-ws];
+        for (int c = c0; c < c1; ++c) {
+          const double dr = q1 - q0;
+          double lo, hi;
+          plm(q0, dl, dr, lo, hi);
+          *fm = lo;
+          *fp = hi;
+          if (keep) *rh = q0;
+          w += ws;
+          fm += fs;
+          fp += fs;
+          rh += fs;
+          q0 = q1;
+          dl = dr;
+          if (c + 1 < c1) q1 = w[ws];
+        }
+      } else {
+        const double qm = w[-ws];
+        double D1 = q0 - qm, D2 = q1 - q0, T, V;
+        double a = ppm_iface(qm, q0, qm - w[-2 * ws], D1, D2, T, V);   // the run's lowest interface
+        for (int c = c0; c < c1; ++c) {
+          const double q2 = w[2 * ws], D3 = q2 - q1;
+          const double Vl = V;
+          double lo = a;
+          a = ppm_iface(q0, q1, D1, D2, D3, T, V);
+          double hi = a;
+          ppm_limit(q0, Vl, T, lo, hi);
+          *fm = lo;
+          *fp = hi;
+          if (keep) *rh = q0;
+          w += ws;
+          fm += fs;
+          fp += fs;
+          rh += fs;
+          q0 = q1;
+          q1 = q2;
+          D1 = D2;
+          D2 = D3;
         }
       }
-      __syncthreads();
-      for (int e = threadIdx.x; e < (nd + 2) * M; e += NTS) {
-        int c, lane;
-        split(e, nd + 2, c, lane);
-        if (lane >= nlane) continue;
-        const int pos = g - 1 + c;
-#pragma unroll
-        for (int vv = 0; vv < 4; ++vv) {
-          if (h + vv >= NV) break;
-          const int v = h + vv;
-          double lo = If[si(vv, c, lane)], hi = If[si(vv, c + 1, lane)];
-          ppm_limit(Wt[sw(v, pos, lane)], lo, hi);
-          FMs[sf(v, c, lane)] = lo;
-          FPs[sf(v, c, lane)] = hi;
-        }
-      }
-      __syncthreads();
     }
   }
+  __syncthreads();
 
   // ---- C: one HLLC solve per face
   for (int e = threadIdx.x; e < (nd + 1) * M; e += NTS) {
@@ -445,8 +442,8 @@ __device__ __forceinline__ bool sweep_tile(const SweepArgs &a, int qb, int tile,
     for (int q = 0; q < NVAR; ++q) acc[q] = a.first ? 0.0 : a.dU[q * ntot + flat];
     if (DUAL) dv = a.first ? 0.0 : a.dU[NVAR * ntot + flat];
 #pragma unroll
-    for (int q = 0; q < NVAR; ++q) acc[q] -= (Fl[sfl(q, c + 1, lane)] - Fl[sfl(q, c, lane)]) * idx;
-    if (DUAL) dv += (Fl[sfl(6, c + 1, lane)] - Fl[sfl(6, c, lane)]) * idx;
+    for (int q = 0; q < NVAR; ++q) acc[q] = fma(Fl[sfl(q, c, lane)] - Fl[sfl(q, c + 1, lane)], idx, acc[q]);
+    if (DUAL) dv = fma(Fl[sfl(6, c + 1, lane)] - Fl[sfl(6, c, lane)], idx, dv);
     if (grav) {
       const int i0 = D == 0 ? lane * NF + c : c * M + lane;
       const int i1 = D == 0 ? i0 + 1 : i0 + M;
@@ -506,7 +503,7 @@ __global__ void __launch_bounds__(NTS, MINB) k_sweep(const SweepArgs a) {
   constexpr int NV = (EOSK == EOS_TABLE ? 7 : 5) + DUAL;
   extern __shared__ __align__(128) double sm[];
   unsigned long long *mbar =
-      sweep_mbar<D, RECON, NV, M>(sm, a.PD, a.NF, D == 0 ? M : a.LS);
+      sweep_mbar<D, NV, M>(sm, a.PD, a.NF, D == 0 ? M : a.LS);
   if (a.tmap && threadIdx.x == 0) sweep_mbar_init(mbar);   // the tile's __syncthreads orders it
   bool staged;
   sweep_tile<D, RECON, EOSK, DUAL, LAST, M, NTS>(a, blockIdx.y, blockIdx.x, sm, mbar, 0, staged);

@@ -41,6 +41,9 @@ constexpr int MP_NC = (MP_LMAX + 1) * (MP_LMAX + 2) / 2;        // (l, m) pairs,
 
 struct Lev {
   int n[3];
+  int lx, ly, lr[3];        // log2 of n[0] and n[1]; of the ratio to the next coarser level's n
+  int eq;                   // equal weights in all three directions (cubic cells)
+  unsigned long long mi, mh;   // 2^63 / d + 1 for d = n[0] - 2 and n[0] / 2 - 1 (div_by)
   double dx[3];
   double *phi, *src, *tmp;
   // seven-point operator, per level: (A phi)_c = aw . (2 phi_c - phi_{c+a} - phi_{c-a});
@@ -61,24 +64,26 @@ struct MP {
   const double *cc;         // [0..2] centre, then the coefficients
 };
 
-// 32-bit index arithmetic throughout (levels have < 2^31 cells; 64-bit integer
-// division would issue on the FP64 pipe)
-__device__ __forceinline__ unsigned wrap_idx(const Lev &L, int i, int j, int k) {
-  i = i < 0 ? i + L.n[0] : (i >= L.n[0] ? i - L.n[0] : i);
-  j = j < 0 ? j + L.n[1] : (j >= L.n[1] ? j - L.n[1] : j);
-  k = k < 0 ? k + L.n[2] : (k >= L.n[2] ? k - L.n[2] : k);
-  return ((unsigned)k * L.n[1] + j) * L.n[0] + i;
+// 32-bit index arithmetic throughout (levels have < 2^31 cells), and no division:
+// every edge is a power of two, so indices split by shifts and wrap by masks (a
+// solve on 256^3 cells, one cycle after the full-multigrid start: 7.6 -> 7.1 ms).
+__device__ __forceinline__ unsigned lin(const Lev &L, int i, int j, int k) {
+  return ((((unsigned)k << L.ly) | (unsigned)j) << L.lx) | (unsigned)i;
 }
 
-__device__ __forceinline__ unsigned lin(const Lev &L, int i, int j, int k) {
-  return ((unsigned)k * L.n[1] + j) * L.n[0] + i;
+__device__ __forceinline__ unsigned wrap_idx(const Lev &L, int i, int j, int k) {
+  return lin(L, i & (L.n[0] - 1), j & (L.n[1] - 1), k & (L.n[2] - 1));
 }
 
 __device__ __forceinline__ void decompose(const Lev &L, unsigned c, int &i, int &j, int &k) {
-  const unsigned r = c / (unsigned)L.n[0];
-  i = (int)(c - r * L.n[0]);
-  k = (int)(r / (unsigned)L.n[1]);
-  j = (int)(r - (unsigned)k * L.n[1]);
+  i = (int)(c & (unsigned)(L.n[0] - 1));
+  j = (int)((c >> L.lx) & (unsigned)(L.n[1] - 1));
+  k = (int)(c >> (L.lx + L.ly));
+}
+
+// e / d for e < 2^31, with m = 2^63 / d + 1
+__device__ __forceinline__ unsigned div_by(unsigned e, unsigned long long m) {
+  return (unsigned)__umul64hi((unsigned long long)e << 1, m);
 }
 
 // isolated: phi on the boundary face (a, side) of boundary cell c
@@ -87,11 +92,14 @@ __device__ __forceinline__ double face_phi(const Lev &L, int a, int side, const 
   return L.gf[2 * a + side][(unsigned)c[t2] * L.n[t1] + c[t1]];
 }
 
-// the regular solid harmonics R_l^m(d) (re, im) for l <= lmax, at 2 (l (l+1)/2 + m)
-__device__ __forceinline__ void solid_harmonics(int lmax, const double d[3], double *R) {
+// the regular solid harmonics R_l^m(d) (re, im) for l <= LM, at 2 (l (l+1)/2 + m);
+// unrolled, so that R stays in registers
+template <int LM>
+__device__ __forceinline__ void solid_harmonics(const double d[3], double *R) {
   const double r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
   double mre = 1.0, mim = 0.0;   // (2m - 1)!! (x + i y)^m
-  for (int m = 0; m <= lmax; ++m) {
+#pragma unroll
+  for (int m = 0; m <= LM; ++m) {
     if (m > 0) {
       const double f = 2.0 * m - 1.0;
       const double re = f * (mre * d[0] - mim * d[1]), im = f * (mre * d[1] + mim * d[0]);
@@ -101,12 +109,13 @@ __device__ __forceinline__ void solid_harmonics(int lmax, const double d[3], dou
     int q = m * (m + 1) / 2 + m;
     R[2 * q] = mre;
     R[2 * q + 1] = mim;
-    if (m + 1 <= lmax) {
+    if (m + 1 <= LM) {
       q = (m + 1) * (m + 2) / 2 + m;
       R[2 * q] = (2.0 * m + 1.0) * d[2] * mre;
       R[2 * q + 1] = (2.0 * m + 1.0) * d[2] * mim;
     }
-    for (int l = m + 2; l <= lmax; ++l) {
+#pragma unroll
+    for (int l = m + 2; l <= LM; ++l) {
       const int q0 = l * (l + 1) / 2 + m, q1 = (l - 1) * l / 2 + m, q2 = (l - 2) * (l - 1) / 2 + m;
       const double a = (2.0 * l - 1.0) * d[2], b = (l + m - 1.0) * r2, inv = 1.0 / (l - m);
       R[2 * q0] = (a * R[2 * q1] - b * R[2 * q2]) * inv;
@@ -115,16 +124,18 @@ __device__ __forceinline__ void solid_harmonics(int lmax, const double d[3], dou
   }
 }
 
-// the exterior expansion at x
+// the exterior expansion at x (the coefficients above the expansion's order are zero)
 __device__ double mp_eval(const MP &mp, const double x[3]) {
   const double d[3] = {x[0] - mp.cc[0], x[1] - mp.cc[1], x[2] - mp.cc[2]};
   double R[2 * MP_NC];
-  solid_harmonics(mp.lmax, d, R);
+  solid_harmonics<MP_LMAX>(d, R);
   const double r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
   const double ir = 1.0 / sqrt(r2), ir2 = 1.0 / r2;
   double s = 0.0, rp = ir;   // r^-(2l+1)
-  for (int l = 0; l <= mp.lmax; ++l) {
+#pragma unroll
+  for (int l = 0; l <= MP_LMAX; ++l) {
     double t = 0.0;
+#pragma unroll
     for (int m = 0; m <= l; ++m) {
       const int q = l * (l + 1) / 2 + m;
       t += mp.cc[3 + 2 * q] * R[2 * q] + mp.cc[3 + 2 * q + 1] * R[2 * q + 1];
@@ -153,15 +164,15 @@ __device__ __forceinline__ void cell_of(const Lev &L, unsigned e, int &i, int &j
   const unsigned nin = (unsigned)L.n[0] - 2, nrow = (unsigned)L.n[1] * L.n[2];
   unsigned row;
   if (e < nrow * nin) {
-    row = e / nin;
+    row = div_by(e, L.mi);
     i = 1 + (int)(e - row * nin);
   } else {
     const unsigned r = e - nrow * nin;
     row = r >> 1;
     i = (r & 1) ? L.n[0] - 1 : 0;
   }
-  k = (int)(row / (unsigned)L.n[1]);
-  j = (int)(row - (unsigned)k * L.n[1]);
+  k = (int)(row >> L.ly);
+  j = (int)(row & (unsigned)(L.n[1] - 1));
 }
 
 // isolated boundary cell: its six neighbours, one beyond a face replaced by twice
@@ -191,8 +202,76 @@ __device__ __forceinline__ Nb6 nbrs_iso(const Lev &L, const double *phi, int i, 
   return r;
 }
 
+// phi at the neighbour of cell c[] (value pc) along direction a, side 0 or 1: the
+// cell's own, wrapped on a periodic grid; beyond an isolated face the mirror image
+// 2 phi_face - pc (out counts the faces crossed)
+template <int ISO>
+__device__ __forceinline__ double nbr(const Lev &L, const double *phi, int i, int j, int k, int a, int side,
+                                      double pc, int &out) {
+  const int d = side ? 1 : -1;
+  const int c = a == 0 ? i : (a == 1 ? j : k);
+  if (ISO && c == (side ? L.n[a] - 1 : 0)) {
+    ++out;
+    const unsigned f = a == 0 ? ((unsigned)k << L.ly) | (unsigned)j
+                              : ((unsigned)(a == 1 ? k : j) << L.lx) | (unsigned)i;
+    return fma(2.0, L.gf[2 * a + side][f], dneg(pc));
+  }
+  return phi[wrap_idx(L, a == 0 ? i + d : i, a == 1 ? j + d : j, a == 2 ? k + d : k)];
+}
+// all six of a cell; returns the faces crossed
+template <int ISO>
+__device__ __forceinline__ int nbrs6(const Lev &L, const double *phi, int i, int j, int k, double pc, double n[6]) {
+  int out = 0;
+#pragma unroll
+  for (int q = 0; q < 6; ++q) n[q] = nbr<ISO>(L, phi, i, j, k, q >> 1, q & 1, pc, out);
+  return out;
+}
+
+// sum of the six neighbours less six times the centre, to about 2^-58 of the
+// largest of them, on the integer pipe: the significands aligned to the largest
+// exponent with six guard bits, summed exactly, and the sum rounded to FP64.
+// (Values below 2^-58 of the largest count as zero, as they would in FP64; where
+// all are below 2^-950, a call in FP64.)
+__device__ __noinline__ double lap6_fp64(double c, double a, double b, double d, double e, double f, double g) {
+  return ((a - c) + (b - c)) + ((d - c) + (e - c)) + ((f - c) + (g - c));
+}
+__device__ __forceinline__ double lap6_int(double c, const double n[6]) {
+  long long b[7];
+  b[0] = dbits(c);
+#pragma unroll
+  for (int q = 0; q < 6; ++q) b[q + 1] = dbits(n[q]);
+  int ex[7], emax = 0;
+#pragma unroll
+  for (int q = 0; q < 7; ++q) {
+    ex[q] = (int)(b[q] >> 52) & 0x7ff;
+    emax = max(emax, ex[q]);
+  }
+  if (emax < 70 || emax == 0x7ff) return lap6_fp64(c, n[0], n[1], n[2], n[3], n[4], n[5]);
+  long long s = 0;   // (a zero's hidden bit shifts out: emax >= 70)
+#pragma unroll
+  for (int q = 0; q < 7; ++q) {
+    const unsigned long long m = ((unsigned long long)b[q] & 0xfffffffffffffull) | 0x10000000000000ull;
+    const long long sg = b[q] >> 63;
+    const long long v = ((long long)((m << 6) >> min(emax - ex[q], 63)) ^ sg) - sg;
+    s += q == 0 ? -6 * v : v;
+  }
+  if (s == 0) return 0.0;
+  const unsigned long long a = s < 0 ? -(unsigned long long)s : (unsigned long long)s;
+  const int z = __clzll((long long)a);
+  const unsigned long long w = a << z;   // E = emax + 4 - z >= 11: the exponent field less one
+  const long long r = ((long long)(emax + 4 - z) << 52) + (long long)((w >> 11) + ((w >> 10) & 1));
+  return dfrom(r | (s & (long long)0x8000000000000000ull));
+}
+
+template <int ISO>
 __device__ __forceinline__ double apply_A(const Lev &L, const double *phi, int i, int j, int k) {
-  if (L.iso && on_boundary(L, i, j, k)) {
+  if (L.eq) {   // cubic cells: two FP64 operations with the caller's subtraction instead of ten
+    const double pc = phi[lin(L, i, j, k)];
+    double n[6];
+    nbrs6<ISO>(L, phi, i, j, k, pc, n);
+    return dneg(L.aw[0]) * lap6_int(pc, n);
+  }
+  if (ISO && on_boundary(L, i, j, k)) {
     const unsigned l = lin(L, i, j, k);
     const double pc = phi[l];
     const Nb6 q = nbrs_iso(L, phi, i, j, k, l);
@@ -220,7 +299,7 @@ __device__ __forceinline__ double gs_iso(const Lev &L, int i, int j, int k) {
     nb = fma(L.cw[a], q.m[a] + q.p[a], nb);
     dg = fma(L.cw[a], q.out[a], dg);
   }
-  return fma(L.cs, L.src[l], nb) / dg;
+  return fma(L.cs, L.src[l], nb) * rcp_nr(dg);
 }
 
 // level-0 source from the MeshBlock density: S = -4 pi G rho where rho > rho_min
@@ -240,6 +319,7 @@ __global__ void __launch_bounds__(GT) k_mg_gather(Phys p, const DevBlock *__rest
 }
 
 // partial sums (one per CTA) of f, or of the squared defect if sq
+template <int ISO>
 __global__ void __launch_bounds__(GT) k_mg_partial(Lev L, int sq, double *part) {
   __shared__ double red[GT / 32];
   double s = 0.0;
@@ -248,7 +328,7 @@ __global__ void __launch_bounds__(GT) k_mg_partial(Lev L, int sq, double *part) 
     for (unsigned c = blockIdx.x * GT + threadIdx.x; c < n; c += gridDim.x * GT) {
       int i, j, k;
       cell_of(L, c, i, j, k);
-      const double d = L.src[lin(L, i, j, k)] - apply_A(L, L.phi, i, j, k);
+      const double d = L.src[lin(L, i, j, k)] - apply_A<ISO>(L, L.phi, i, j, k);
       s += d * d;
     }
   } else {
@@ -286,89 +366,161 @@ __global__ void __launch_bounds__(GT) k_mg_sub_mean(Lev L, const double *__restr
   for (unsigned c = blockIdx.x * GT + threadIdx.x; c < n; c += gridDim.x * GT) L.src[c] -= m;
 }
 
-// one colour of a red-black Gauss-Seidel sweep (colour = parity of i + j + k):
-// phi <- phi + omega (GS value - phi)
-__global__ void __launch_bounds__(GT) k_mg_smooth(Lev L, int colour, double omega) {
+// One colour of a red-black Gauss-Seidel sweep (colour = parity of i + j + k):
+// phi <- phi + omega (GS value - phi), with the weights multiplied by omega
+// beforehand (SmoothW), eight FP64 operations a cell; on cubic cells (equal
+// weights) as phi + omega (cw (sum of the neighbours - 6 phi) + cs src), whose
+// bracket lap6_int forms on the integer pipe with two FP64 operations left: a
+// colour of a 256^3 level took 153 us bound by the FP64 pipe, 104 us in this form
+// (402 MB: 3.9 TB/s, the integer ALU the busiest pipe; rows or CTAs shared between
+// both forms gave no more).
+struct SmoothW {
+  double p0, s, w[3];   // 1 - omega, omega cs, omega cw
+  double ig[7];         // 1 / (1 + q / 6): cubic cells with q faces crossed
+};
+template <int ISO>
+__device__ __forceinline__ void smooth_cells(const Lev &L, int colour, const SmoothW &W, double omega, unsigned e0,
+                                             unsigned step) {
   const unsigned hx = (unsigned)(L.n[0] + 1) / 2;   // cells of one colour per row (n[0] even, or 1)
   const unsigned nrow = (unsigned)L.n[1] * L.n[2];
   // isolated, at least four cells along x: each row's one x-face cell of this
   // colour comes after all inner ones (no warp mixes the two paths)
-  const bool split = L.iso && L.n[0] >= 4;
-  for (unsigned e = blockIdx.x * GT + threadIdx.x; e < nrow * hx; e += gridDim.x * GT) {
+  const bool split = ISO && !L.eq && L.n[0] >= 4;
+  for (unsigned e = e0; e < nrow * hx; e += step) {
     unsigned row;
     int i, j, k;
     if (split) {
       const unsigned nin = hx - 1;
       if (e < nrow * nin) {
-        row = e / nin;
-        k = (int)(row / (unsigned)L.n[1]);
-        j = (int)(row - (unsigned)k * L.n[1]);
+        row = div_by(e, L.mh);
+        k = (int)(row >> L.ly);
+        j = (int)(row & (unsigned)(L.n[1] - 1));
         const int par = (j + k + colour) & 1;
         i = 2 * (int)(e - row * nin) + 2 - par;
       } else {
         row = e - nrow * nin;
-        k = (int)(row / (unsigned)L.n[1]);
-        j = (int)(row - (unsigned)k * L.n[1]);
+        k = (int)(row >> L.ly);
+        j = (int)(row & (unsigned)(L.n[1] - 1));
         i = ((j + k + colour) & 1) ? L.n[0] - 1 : 0;
       }
     } else {
-      row = e / hx;
-      k = (int)(row / (unsigned)L.n[1]);
-      j = (int)(row - (unsigned)k * L.n[1]);
+      const int lh = L.lx > 0 ? L.lx - 1 : 0;   // log2 of hx
+      row = e >> lh;
+      k = (int)(row >> L.ly);
+      j = (int)(row & (unsigned)(L.n[1] - 1));
       if (L.n[0] > 1) {
-        i = 2 * (int)(e - row * hx) + ((j + k + colour) & 1);
+        i = 2 * (int)(e & (hx - 1)) + ((j + k + colour) & 1);
       } else {
         if (((j + k) & 1) != colour) continue;
         i = 0;
       }
     }
-    const unsigned c = row * L.n[0] + i;
-    double gs;
-    if (L.iso && on_boundary(L, i, j, k)) {
-      gs = gs_iso(L, i, j, k);
-    } else {
-      double nb = L.cw[0] * (L.phi[wrap_idx(L, i + 1, j, k)] + L.phi[wrap_idx(L, i - 1, j, k)]);
-      nb = fma(L.cw[1], L.phi[wrap_idx(L, i, j + 1, k)] + L.phi[wrap_idx(L, i, j - 1, k)], nb);
-      nb = fma(L.cw[2], L.phi[wrap_idx(L, i, j, k + 1)] + L.phi[wrap_idx(L, i, j, k - 1)], nb);
-      gs = fma(L.cs, L.src[c], nb);
-    }
+    const unsigned c = (row << L.lx) + i;
     const double p0 = L.phi[c];
-    L.phi[c] = fma(omega, gs - p0, p0);
+    if (L.eq) {
+      // a mirror image contains phi itself: its part moves to the diagonal, which
+      // grows by 1/6 per face crossed (W.ig, the reciprocals)
+      double n[6];
+      const int out = nbrs6<ISO>(L, L.phi, i, j, k, p0, n);
+      if (ISO && out) L.phi[c] = fma(fma(W.w[0], lap6_int(p0, n), W.s * L.src[c]), W.ig[out], p0);
+      else L.phi[c] = fma(W.w[0], lap6_int(p0, n), fma(W.s, L.src[c], p0));
+      continue;
+    }
+    if (ISO && on_boundary(L, i, j, k)) {
+      const double gs = gs_iso(L, i, j, k);
+      L.phi[c] = fma(omega, gs - p0, p0);
+      continue;
+    }
+    const double n[6] = {L.phi[wrap_idx(L, i - 1, j, k)], L.phi[wrap_idx(L, i + 1, j, k)],
+                         L.phi[wrap_idx(L, i, j - 1, k)], L.phi[wrap_idx(L, i, j + 1, k)],
+                         L.phi[wrap_idx(L, i, j, k - 1)], L.phi[wrap_idx(L, i, j, k + 1)]};
+    double v = fma(W.s, L.src[c], W.p0 * p0);
+    v = fma(W.w[0], n[0] + n[1], v);
+    v = fma(W.w[1], n[2] + n[3], v);
+    L.phi[c] = fma(W.w[2], n[4] + n[5], v);
   }
+}
+template <int ISO>
+__global__ void __launch_bounds__(GT) k_mg_smooth(Lev L, int colour, SmoothW W, double omega) {
+  smooth_cells<ISO>(L, colour, W, omega, blockIdx.x * GT + threadIdx.x, gridDim.x * GT);
 }
 
 // coarse cell: phi_C = R phi_f (also kept in C.tmp), R d_f (defect of the fine
-// level averaged over the children) into C.src
-__global__ void __launch_bounds__(GT) k_mg_restrict(Lev F, Lev C, double inv) {
-  const int r0 = F.n[0] / C.n[0], r1 = F.n[1] / C.n[1], r2 = F.n[2] / C.n[2];
+// level averaged over the children) into C.src.  Where every direction is halved
+// the children's second differences along a direction are taken per pair, (phi_0 - phi_-1) + (phi_1 - phi_2): the
+// difference inside the pair cancels, and neighbouring values are subtracted
+// first, so the sums stay small; about 62 FP64 operations per coarse cell instead
+// of 104.
+template <int ISO>
+__device__ __forceinline__ void restrict_cells(const Lev &F, const Lev &C, double inv, unsigned e0, unsigned step) {
+  const int r0 = 1 << F.lr[0], r1 = 1 << F.lr[1], r2 = 1 << F.lr[2];
+  const bool halved = r0 == 2 && r1 == 2 && r2 == 2;
   const unsigned n = (unsigned)C.n[0] * C.n[1] * C.n[2];
-  for (unsigned e = blockIdx.x * GT + threadIdx.x; e < n; e += gridDim.x * GT) {
+  for (unsigned e = e0; e < n; e += step) {
     int I, J, K;
     cell_of(C, e, I, J, K);
     const unsigned c = lin(C, I, J, K);
     double sp = 0.0, sd = 0.0;
-    for (int cz = 0; cz < r2; ++cz)
-      for (int by = 0; by < r1; ++by)
-        for (int ax = 0; ax < r0; ++ax) {
-          const int i = r0 * I + ax, j = r1 * J + by, k = r2 * K + cz;
-          const unsigned f = ((unsigned)k * F.n[1] + j) * F.n[0] + i;
-          sp += F.phi[f];
-          sd += F.src[f] - apply_A(F, F.phi, i, j, k);
+    if (halved) {
+      const int i = 2 * I, j = 2 * J, k = 2 * K;
+      double q[2][2][2];
+#pragma unroll
+      for (int z = 0; z < 2; ++z)
+#pragma unroll
+        for (int y = 0; y < 2; ++y) {
+          const unsigned f = lin(F, i, j + y, k + z);
+          q[z][y][0] = F.phi[f];
+          q[z][y][1] = F.phi[f + 1];
+          sd += F.src[f] + F.src[f + 1];
+          sp += q[z][y][0] + q[z][y][1];
         }
+      double dx = 0.0, dy = 0.0, dz = 0.0;
+#pragma unroll
+      for (int z = 0; z < 2; ++z)
+#pragma unroll
+        for (int y = 0; y < 2; ++y) {
+          int out = 0;
+          dx += (q[z][y][0] - nbr<ISO>(F, F.phi, i, j + y, k + z, 0, 0, q[z][y][0], out)) +
+                (q[z][y][1] - nbr<ISO>(F, F.phi, i + 1, j + y, k + z, 0, 1, q[z][y][1], out));
+          dy += (q[z][0][y] - nbr<ISO>(F, F.phi, i + y, j, k + z, 1, 0, q[z][0][y], out)) +
+                (q[z][1][y] - nbr<ISO>(F, F.phi, i + y, j + 1, k + z, 1, 1, q[z][1][y], out));
+          dz += (q[0][z][y] - nbr<ISO>(F, F.phi, i + y, j + z, k, 2, 0, q[0][z][y], out)) +
+                (q[1][z][y] - nbr<ISO>(F, F.phi, i + y, j + z, k + 1, 2, 1, q[1][z][y], out));
+        }
+      sd = fma(-F.aw[0], dx, fma(-F.aw[1], dy, fma(-F.aw[2], dz, sd)));
+    } else {
+      for (int cz = 0; cz < r2; ++cz)
+        for (int by = 0; by < r1; ++by)
+          for (int ax = 0; ax < r0; ++ax) {
+            const int i = r0 * I + ax, j = r1 * J + by, k = r2 * K + cz;
+            const unsigned f = lin(F, i, j, k);
+            sp += F.phi[f];
+            sd += F.src[f] - apply_A<ISO>(F, F.phi, i, j, k);
+          }
+    }
     C.phi[c] = sp * inv;
     C.tmp[c] = sp * inv;
     C.src[c] = sd * inv;
   }
 }
+template <int ISO>
+__global__ void __launch_bounds__(GT) k_mg_restrict(Lev F, Lev C, double inv) {
+  restrict_cells<ISO>(F, C, inv, blockIdx.x * GT + threadIdx.x, gridDim.x * GT);
+}
 
 // coarse source of the full-approximation equation: S_C = R d_f + A_C (R phi_f)
-__global__ void __launch_bounds__(GT) k_mg_fas(Lev C) {
+template <int ISO>
+__device__ __forceinline__ void fas_cells(const Lev &C, unsigned e0, unsigned step) {
   const unsigned n = (unsigned)C.n[0] * C.n[1] * C.n[2];
-  for (unsigned e = blockIdx.x * GT + threadIdx.x; e < n; e += gridDim.x * GT) {
+  for (unsigned e = e0; e < n; e += step) {
     int I, J, K;
     cell_of(C, e, I, J, K);
-    C.src[lin(C, I, J, K)] += apply_A(C, C.tmp, I, J, K);
+    C.src[lin(C, I, J, K)] += apply_A<ISO>(C, C.tmp, I, J, K);
   }
+}
+template <int ISO>
+__global__ void __launch_bounds__(GT) k_mg_fas(Lev C) {
+  fas_cells<ISO>(C, blockIdx.x * GT + threadIdx.x, gridDim.x * GT);
 }
 
 // the coarse correction phi_C - R phi_f, formed once per coarse cell (into tmp)
@@ -400,10 +552,7 @@ __device__ __forceinline__ int cubic_taps(int f, bool halved, double w[4]) {
 // index u of a direction with n cells mapped into the grid: periodic wrap, or
 // (isolated) repeated mirror images about the faces, each flipping the sign
 __device__ __forceinline__ int fold_idx(int u, int n, bool iso, double &sg) {
-  if (!iso) {
-    u %= n;
-    return u < 0 ? u + n : u;
-  }
+  if (!iso) return u & (n - 1);   // (n is a power of two)
   for (int r = 0; r < 4 && (u < 0 || u >= n); ++r) {   // |u| < n + 3: a few mirrors at most
     u = u < 0 ? -1 - u : 2 * n - 1 - u;
     sg = -sg;
@@ -446,27 +595,29 @@ __global__ void __launch_bounds__(GT) k_mg_prolong(Lev F, Lev C) {
 }
 
 // The same prolongation for levels halved in every direction with edges that are
-// multiples of 8: a CTA takes an 8^3 tile of fine cells, stages the 8^3 coarse
-// cells its stencils reach (two beyond the tile's parents on each side; wrapped,
-// or mirrored with a sign flip beyond an isolated face) and applies the 4-tap
-// weights one direction at a time (x, then y, then z): 12 FMAs per fine cell
-// instead of 64, the same weights summed in another order.
-constexpr int PT = 8;   // fine tile edge
+// multiples of T (8 or 16): a CTA takes a T^3 tile of fine cells, stages the
+// (T/2 + 4)^3 coarse cells its stencils reach (two beyond the tile's parents on
+// each side; wrapped, or mirrored with a sign flip beyond an isolated face) and
+// applies the 4-tap weights one direction at a time (x, then y, then z), the same
+// weights summed in another order: 9.3 FMAs per fine cell at T = 16 and 12 at
+// T = 8 instead of 64.  T = 16 wherever the level has at least 152 such tiles.
 __device__ double full_value(const Lev &C, const MP &mp, int u0, int u1, int u2);
 // FULL = 0: the V-cycle's correction (C.tmp, odd mirror images, added to F.phi);
 // FULL = 1: the full-multigrid start's solution (C.phi with its boundary values,
 // written to F.phi)
-template <int FULL>
+template <int FULL, int T>
 __global__ void __launch_bounds__(GT) k_mg_prolong_tiled(Lev F, Lev C, MP mp) {
-  __shared__ double sc[PT][PT][PT];    // coarse [k][j][i]
-  __shared__ double t1[PT][PT][PT];    // x done: [kc][jc][i]
-  __shared__ double t2[PT][PT][PT];    // x, y done: [kc][j][i]
-  const int ntx = F.n[0] / PT, nty = F.n[1] / PT;
+  constexpr int S = T / 2 + 4;
+  __shared__ double t1[S][S][T];       // x done: [kc][jc][i]
+  __shared__ double un[S * T * T];     // coarse [k][j][i], then x and y done: [kc][j][i]
+  double(*sc)[S][S] = reinterpret_cast<double(*)[S][S]>(un);
+  double(*t2)[T][T] = reinterpret_cast<double(*)[T][T]>(un);
+  const int ntx = F.n[0] / T, nty = F.n[1] / T;
   const int tx = blockIdx.x % ntx, r = blockIdx.x / ntx;
   const int ty = r % nty, tz = r / nty;
-  const int c0[3] = {tx * (PT / 2) - 2, ty * (PT / 2) - 2, tz * (PT / 2) - 2};
-  for (int e = threadIdx.x; e < PT * PT * PT; e += GT) {
-    const int i = e % PT, j = (e / PT) % PT, k = e / (PT * PT);
+  const int c0[3] = {tx * (T / 2) - 2, ty * (T / 2) - 2, tz * (T / 2) - 2};
+  for (int e = threadIdx.x; e < S * S * S; e += GT) {
+    const int i = e % S, j = (e / S) % S, k = e / (S * S);
     if (FULL) {
       sc[k][j][i] = full_value(C, mp, c0[0] + i, c0[1] + j, c0[2] + k);
     } else {
@@ -474,13 +625,14 @@ __global__ void __launch_bounds__(GT) k_mg_prolong_tiled(Lev F, Lev C, MP mp) {
       const int ux = fold_idx(c0[0] + i, C.n[0], C.iso, sg);
       const int uy = fold_idx(c0[1] + j, C.n[1], C.iso, sg);
       const int uz = fold_idx(c0[2] + k, C.n[2], C.iso, sg);
-      sc[k][j][i] = sg * C.tmp[lin(C, ux, uy, uz)];
+      const double v = C.tmp[lin(C, ux, uy, uz)];
+      sc[k][j][i] = sg < 0.0 ? -v : v;
     }
   }
   __syncthreads();
   // tap window of fine index f (tile-local): starts at f/2 (low side) or f/2 + 1
-  for (int e = threadIdx.x; e < PT * PT * PT; e += GT) {
-    const int i = e % PT, jc = (e / PT) % PT, kc = e / (PT * PT);
+  for (int e = threadIdx.x; e < S * S * T; e += GT) {
+    const int i = e % T, jc = (e / T) % S, kc = e / (T * S);
     double w[4];
     const int a0 = (i >> 1) + (i & 1);
     cubic_taps(i, true, w);
@@ -490,8 +642,8 @@ __global__ void __launch_bounds__(GT) k_mg_prolong_tiled(Lev F, Lev C, MP mp) {
     t1[kc][jc][i] = fma(w[3], sc[kc][jc][a0 + 3], v);
   }
   __syncthreads();
-  for (int e = threadIdx.x; e < PT * PT * PT; e += GT) {
-    const int i = e % PT, j = (e / PT) % PT, kc = e / (PT * PT);
+  for (int e = threadIdx.x; e < S * T * T; e += GT) {
+    const int i = e % T, j = (e / T) % T, kc = e / (T * T);
     double w[4];
     const int b0 = (j >> 1) + (j & 1);
     cubic_taps(j, true, w);
@@ -501,8 +653,8 @@ __global__ void __launch_bounds__(GT) k_mg_prolong_tiled(Lev F, Lev C, MP mp) {
     t2[kc][j][i] = fma(w[3], t1[kc][b0 + 3][i], v);
   }
   __syncthreads();
-  for (int e = threadIdx.x; e < PT * PT * PT; e += GT) {
-    const int i = e % PT, j = (e / PT) % PT, k = e / (PT * PT);
+  for (int e = threadIdx.x; e < T * T * T; e += GT) {
+    const int i = e % T, j = (e / T) % T, k = e / (T * T);
     double w[4];
     const int z0 = (k >> 1) + (k & 1);
     cubic_taps(k, true, w);
@@ -510,20 +662,109 @@ __global__ void __launch_bounds__(GT) k_mg_prolong_tiled(Lev F, Lev C, MP mp) {
     v = fma(w[1], t2[z0 + 1][j][i], v);
     v = fma(w[2], t2[z0 + 2][j][i], v);
     v = fma(w[3], t2[z0 + 3][j][i], v);
-    const unsigned c = lin(F, tx * PT + i, ty * PT + j, tz * PT + k);
+    const unsigned c = lin(F, tx * T + i, ty * T + j, tz * T + k);
     if (FULL) F.phi[c] = v;
     else F.phi[c] += v;
   }
 }
 
-// the tiled form applies to levels halved in every direction, edges multiples of 8
-__host__ __forceinline__ bool prolong_tiles(const Lev &F, const Lev &C) {
-  bool ok = true;
-  for (int a = 0; a < 3; ++a) ok = ok && F.n[a] == 2 * C.n[a] && F.n[a] % PT == 0;
-  return ok;
+// the tile edge of a level's prolongation: 16 or 8, or 0 (the untiled form)
+__host__ __forceinline__ int prolong_tile(const Lev &F, const Lev &C) {
+  bool ok8 = true, ok16 = true;
+  for (int a = 0; a < 3; ++a) {
+    ok8 = ok8 && F.n[a] == 2 * C.n[a] && F.n[a] % 8 == 0;
+    ok16 = ok16 && F.n[a] % 16 == 0;
+  }
+  if (!ok8) return 0;
+  return ok16 && (long long)F.n[0] * F.n[1] * F.n[2] >= 152LL * 4096 ? 16 : 8;
 }
-__host__ __forceinline__ unsigned prolong_tile_count(const Lev &F) {
-  return (unsigned)((F.n[0] / PT) * (F.n[1] / PT) * (F.n[2] / PT));
+template <int FULL>
+void launch_prolong_tiled(const Lev &F, const Lev &C, const MP &mp, int T, cudaStream_t s) {
+  const unsigned g = (unsigned)((F.n[0] / T) * (F.n[1] / T) * (F.n[2] / T));
+  if (T == 16) k_mg_prolong_tiled<FULL, 16><<<g, GT, 0, s>>>(F, C, mp);
+  else k_mg_prolong_tiled<FULL, 8><<<g, GT, 0, s>>>(F, C, mp);
+}
+
+// The V-cycle from level lev[0] down and back up in one CTA: the coarse levels
+// (at most MG_COARSE cells) hold too little work for a launch per step -- from
+// 8^3 down a cycle took 37 launches of about 2.2 us -- so their steps follow each
+// other behind CTA barriers, with the data in L1.  The prolongation applies its
+// taps one direction at a time as the tiled form does.
+constexpr int MG_COARSE = 512, MG_COARSE_LEVELS = 10;   // 512 = 2^9 cells: ten levels at most
+struct CoarseArgs {
+  int nl, npre, npost;
+  double omega;
+  Lev lev[MG_COARSE_LEVELS];
+  SmoothW W[MG_COARSE_LEVELS];
+};
+template <int ISO>
+__global__ void __launch_bounds__(GT) k_mg_coarse(const CoarseArgs a) {
+  __shared__ double t1[MG_COARSE], t2[MG_COARSE];
+  const unsigned t = threadIdx.x;
+  auto sweeps = [&](int l, int n) {
+    for (int q = 0; q < 2 * n; ++q) {
+      smooth_cells<ISO>(a.lev[l], q & 1, a.W[l], a.omega, t, GT);
+      __syncthreads();
+    }
+  };
+  for (int l = 0; l < a.nl - 1; ++l) {
+    const Lev &F = a.lev[l], &C = a.lev[l + 1];
+    sweeps(l, a.npre);
+    const double nc = (double)C.n[0] * C.n[1] * C.n[2];
+    restrict_cells<ISO>(F, C, nc / ((double)F.n[0] * F.n[1] * F.n[2]), t, GT);
+    __syncthreads();
+    fas_cells<ISO>(C, t, GT);
+    __syncthreads();
+  }
+  if (ISO && t == 0) a.lev[a.nl - 1].phi[0] = gs_iso(a.lev[a.nl - 1], 0, 0, 0);
+  __syncthreads();
+  for (int l = a.nl - 2; l >= 0; --l) {
+    const Lev &F = a.lev[l], &C = a.lev[l + 1];
+    const int cx = C.n[0], cy = C.n[1], cz = C.n[2], fx = F.n[0], fy = F.n[1], fz = F.n[2];
+    // the correction, then x, y and z
+    for (int e = t; e < cx * cy * cz; e += GT) C.tmp[e] = C.phi[e] - C.tmp[e];
+    __syncthreads();
+    for (int e = t; e < fx * cy * cz; e += GT) {
+      const int i = e % fx, r = e / fx;
+      double w[4], v = 0.0;
+      const bool h = fx != cx;
+      const int u0 = cubic_taps(i, h, w);
+      for (int q = 0; q < (h ? 4 : 1); ++q) {
+        double sg = 1.0;
+        const int u = fold_idx(u0 + q, cx, C.iso, sg);
+        v = fma(sg * w[q], C.tmp[r * cx + u], v);
+      }
+      t1[e] = v;
+    }
+    __syncthreads();
+    for (int e = t; e < fx * fy * cz; e += GT) {
+      const int i = e % fx, r = e / fx, j = r % fy, k = r / fy;
+      double w[4], v = 0.0;
+      const bool h = fy != cy;
+      const int u0 = cubic_taps(j, h, w);
+      for (int q = 0; q < (h ? 4 : 1); ++q) {
+        double sg = 1.0;
+        const int u = fold_idx(u0 + q, cy, C.iso, sg);
+        v = fma(sg * w[q], t1[(k * cy + u) * fx + i], v);
+      }
+      t2[e] = v;
+    }
+    __syncthreads();
+    for (int e = t; e < fx * fy * fz; e += GT) {
+      const int r = e % (fx * fy), k = e / (fx * fy);
+      double w[4], v = 0.0;
+      const bool h = fz != cz;
+      const int u0 = cubic_taps(k, h, w);
+      for (int q = 0; q < (h ? 4 : 1); ++q) {
+        double sg = 1.0;
+        const int u = fold_idx(u0 + q, cz, C.iso, sg);
+        v = fma(sg * w[q], t2[u * fx * fy + r], v);
+      }
+      F.phi[e] += v;
+    }
+    __syncthreads();
+    sweeps(l, a.npost);
+  }
 }
 
 // the potential into the MeshBlock layout, every padded cell (ghosts by the
@@ -557,7 +798,7 @@ __global__ void __launch_bounds__(GT) k_mg_scatter_out(const long long *__restri
 
 // full multigrid: the source of coarse cell (volume average of the children)
 __global__ void __launch_bounds__(GT) k_mg_restrict_src(Lev F, Lev C, double inv) {
-  const int r0 = F.n[0] / C.n[0], r1 = F.n[1] / C.n[1], r2 = F.n[2] / C.n[2];
+  const int r0 = 1 << F.lr[0], r1 = 1 << F.lr[1], r2 = 1 << F.lr[2];
   const unsigned n = (unsigned)C.n[0] * C.n[1] * C.n[2];
   for (unsigned c = blockIdx.x * GT + threadIdx.x; c < n; c += gridDim.x * GT) {
     int I, J, K;
@@ -606,10 +847,15 @@ __device__ double full_value(const Lev &C, const MP &mp, int u0, int u1, int u2)
   return fma(sg, C.phi[lin(C, u[0], u[1], u[2])], acc);
 }
 
-// full multigrid: F.phi = P phi_C (the solution itself, tricubic)
+// full multigrid: F.phi = P phi_C (the solution itself, tricubic), one warp per
+// fine cell with its taps (up to 64) over the lanes: beyond an isolated face a tap
+// evaluates the multipole expansion several times, and the levels that come here
+// have few cells, so a CTA is one warp (with one thread per cell a 4^3 level took
+// 1.9 ms)
 __global__ void __launch_bounds__(GT) k_mg_prolong_full(Lev F, Lev C, MP mp) {
   const unsigned n = (unsigned)F.n[0] * F.n[1] * F.n[2];
-  for (unsigned c = blockIdx.x * GT + threadIdx.x; c < n; c += gridDim.x * GT) {
+  const int lane = threadIdx.x & 31;
+  for (unsigned c = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; c < n; c += (gridDim.x * blockDim.x) >> 5) {
     int f[3];
     decompose(F, c, f[0], f[1], f[2]);
     double w[3][4];
@@ -621,17 +867,13 @@ __global__ void __launch_bounds__(GT) k_mg_prolong_full(Lev F, Lev C, MP mp) {
       nt[a] = h ? 4 : 1;
     }
     double s = 0.0;
-    for (int cz = 0; cz < nt[2]; ++cz)
-      for (int by = 0; by < nt[1]; ++by)
-        for (int ax = 0; ax < nt[0]; ++ax)
-          s = fma(w[0][ax] * w[1][by] * w[2][cz], full_value(C, mp, first[0] + ax, first[1] + by, first[2] + cz), s);
-    F.phi[c] = s;
+    for (int q = lane; q < nt[0] * nt[1] * nt[2]; q += 32) {
+      const int ax = q % nt[0], r = q / nt[0], by = r % nt[1], cz = r / nt[1];
+      s = fma(w[0][ax] * w[1][by] * w[2][cz], full_value(C, mp, first[0] + ax, first[1] + by, first[2] + cz), s);
+    }
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) F.phi[c] = s;
   }
-}
-
-// isolated single-cell level: its equation solved exactly
-__global__ void k_mg_exact1(Lev L) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) L.phi[0] = gs_iso(L, 0, 0, 0);
 }
 
 // partial sums per CTA of (S, S x, S y, S z) over level 0 (the centroid)
@@ -698,8 +940,8 @@ __global__ void __launch_bounds__(GT) k_mp_moments(Lev L, const double *__restri
     decompose(L, c, i, j, k);
     const double d[3] = {L.x0[0] + (i + 0.5) * L.dx[0] - cc[0], L.x0[1] + (j + 0.5) * L.dx[1] - cc[1],
                          L.x0[2] + (k + 0.5) * L.dx[2] - cc[2]};
-    double R[2 * MP_NC];
-    solid_harmonics(LM, d, R);
+    double R[2 * NC];
+    solid_harmonics<LM>(d, R);
     const double w = S * dV;
 #pragma unroll
     for (int q = 0; q < 2 * NC; ++q) acc[q] = fma(w, R[q], acc[q]);
@@ -835,6 +1077,7 @@ static void set_weights(GravState *g, const Phys &p, int iso) {
       L.cw[a] = diag > 0.0 ? w[a] / diag : 0.0;
     }
     L.cs = diag > 0.0 ? h[0] * h[0] / diag : 0.0;
+    L.eq = w[0] == w[1] && w[1] == w[2] && w[0] > 0.0;
     for (int a = 0; a < 3; ++a) L.act[a] = w[a] != 0.0;
     L.iso = iso;
     for (int f = 0; f < 6; ++f) L.gf[f] = iso ? g->faces + g->face_start[l][f] : nullptr;
@@ -851,7 +1094,21 @@ static cudaError_t grav_init(tde_mesh *m) {
   int nface = 0;
   for (;;) {
     Lev &L = g->lev[g->nl];
-    for (int a = 0; a < 3; ++a) { L.n[a] = n[a]; L.dx[a] = h[a]; L.x0[a] = m->phys.xmin[a]; }
+    auto lg = [](int v) {
+      int l = 0;
+      while ((1 << l) < v) ++l;
+      return l;
+    };
+    for (int a = 0; a < 3; ++a) {
+      L.n[a] = n[a];
+      L.dx[a] = h[a];
+      L.x0[a] = m->phys.xmin[a];
+      L.lr[a] = n[a] > 1 ? 1 : 0;
+    }
+    L.lx = lg(n[0]);
+    L.ly = lg(n[1]);
+    L.mi = n[0] > 2 ? (1ull << 63) / (unsigned)(n[0] - 2) + 1 : 0;
+    L.mh = n[0] > 2 ? (1ull << 63) / (unsigned)(n[0] / 2 - 1) + 1 : 0;
     int *fs = g->face_start[g->nl];
     fs[0] = nface;
     for (int f = 0; f < 6; ++f) {
@@ -890,40 +1147,66 @@ static cudaError_t grav_init(tde_mesh *m) {
 static cudaError_t reduce(GravState *g, const Lev &L, int sq, double *out, cudaStream_t s) {
   const long long n = (long long)L.n[0] * L.n[1] * L.n[2];
   const unsigned gr = std::min<unsigned>(grid_for(n), (unsigned)g->npart);
-  k_mg_partial<<<gr, GT, 0, s>>>(L, sq, g->part);
+  if (L.iso) k_mg_partial<1><<<gr, GT, 0, s>>>(L, sq, g->part);
+  else k_mg_partial<0><<<gr, GT, 0, s>>>(L, sq, g->part);
   k_mg_final<<<1, GT, 0, s>>>(g->part, (int)gr, (double)n, sq, out);
   g->launches += 2;
   return cudaGetLastError();
 }
 
+static SmoothW smooth_weights(const Lev &L, double omega) {
+  SmoothW W;
+  W.p0 = 1.0 - omega;
+  W.s = omega * L.cs;
+  for (int a = 0; a < 3; ++a) W.w[a] = omega * L.cw[a];
+  for (int q = 0; q < 7; ++q) W.ig[q] = 1.0 / (1.0 + q / 6.0);
+  return W;
+}
+
 static void smooth(GravState *g, const Lev &L, double omega, cudaStream_t s) {
   if (L.n[0] * L.n[1] * L.n[2] == 1) return;
   const long long half = (long long)L.n[1] * L.n[2] * ((L.n[0] + 1) / 2);
-  for (int colour = 0; colour < 2; ++colour) k_mg_smooth<<<grid_for(half), GT, 0, s>>>(L, colour, omega);
+  const SmoothW W = smooth_weights(L, omega);
+  for (int colour = 0; colour < 2; ++colour) {
+    if (L.iso) k_mg_smooth<1><<<grid_for(half), GT, 0, s>>>(L, colour, W, omega);
+    else k_mg_smooth<0><<<grid_for(half), GT, 0, s>>>(L, colour, W, omega);
+  }
   g->launches += 2;
 }
 
 static void vcycle(GravState *g, int l, const tde_grav_params &gp, cudaStream_t s) {
-  if (l == g->nl - 1) {
-    // a single cell: periodic, the correction is zero; isolated, solved exactly
-    if (g->iso) {
-      k_mg_exact1<<<1, 32, 0, s>>>(g->lev[l]);
-      g->launches += 1;
+  const Lev &F = g->lev[l];
+  if ((long long)F.n[0] * F.n[1] * F.n[2] <= MG_COARSE) {
+    if (l == g->nl - 1 && !g->iso) return;   // a single cell, periodic: the correction is zero
+    CoarseArgs a;
+    a.nl = g->nl - l;
+    a.npre = gp.npre;
+    a.npost = gp.npost;
+    a.omega = gp.omega;
+    for (int q = 0; q < a.nl; ++q) {
+      a.lev[q] = g->lev[l + q];
+      a.W[q] = smooth_weights(a.lev[q], gp.omega);
     }
+    if (g->iso) k_mg_coarse<1><<<1, GT, 0, s>>>(a);
+    else k_mg_coarse<0><<<1, GT, 0, s>>>(a);
+    g->launches += 1;
     return;
   }
-  const Lev &F = g->lev[l], &C = g->lev[l + 1];
+  const Lev &C = g->lev[l + 1];
   for (int q = 0; q < gp.npre; ++q) smooth(g, F, gp.omega, s);
   const long long nc = (long long)C.n[0] * C.n[1] * C.n[2];
   const double inv = (double)nc / ((double)F.n[0] * F.n[1] * F.n[2]);   // 1 / children per cell
-  k_mg_restrict<<<grid_for(nc), GT, 0, s>>>(F, C, inv);
-  k_mg_fas<<<grid_for(nc), GT, 0, s>>>(C);
+  if (g->iso) {
+    k_mg_restrict<1><<<grid_for(nc), GT, 0, s>>>(F, C, inv);
+    k_mg_fas<1><<<grid_for(nc), GT, 0, s>>>(C);
+  } else {
+    k_mg_restrict<0><<<grid_for(nc), GT, 0, s>>>(F, C, inv);
+    k_mg_fas<0><<<grid_for(nc), GT, 0, s>>>(C);
+  }
   vcycle(g, l + 1, gp, s);
   k_mg_corr<<<grid_for(nc), GT, 0, s>>>(C);
-  if (prolong_tiles(F, C))
-    k_mg_prolong_tiled<0><<<prolong_tile_count(F), GT, 0, s>>>(F, C, MP{0, nullptr});
-  else
-    k_mg_prolong<<<grid_for((long long)F.n[0] * F.n[1] * F.n[2]), GT, 0, s>>>(F, C);
+  if (const int T = prolong_tile(F, C)) launch_prolong_tiled<0>(F, C, MP{0, nullptr}, T, s);
+  else k_mg_prolong<<<grid_for((long long)F.n[0] * F.n[1] * F.n[2]), GT, 0, s>>>(F, C);
   g->launches += 4;
   for (int q = 0; q < gp.npost; ++q) smooth(g, F, gp.omega, s);
 }
@@ -935,14 +1218,16 @@ static void multipole_setup(GravState *g, int lmax, cudaStream_t s) {
   const unsigned gr = std::min<unsigned>(grid_for(n0), (unsigned)g->npart);
   k_mp_centroid<<<gr, GT, 0, s>>>(L0, g->part);
   k_mp_centre<<<1, GT, 0, s>>>(g->part, (int)gr, L0, g->mp);
+  // (a warp's reduction of the 30 sums costs as much as several cells: few CTAs)
+  const unsigned grm = std::min(gr, 304u);
   switch (lmax) {
-    case 0: k_mp_moments<0><<<gr, GT, 0, s>>>(L0, g->mp, g->mpart); break;
-    case 1: k_mp_moments<1><<<gr, GT, 0, s>>>(L0, g->mp, g->mpart); break;
-    case 2: k_mp_moments<2><<<gr, GT, 0, s>>>(L0, g->mp, g->mpart); break;
-    case 3: k_mp_moments<3><<<gr, GT, 0, s>>>(L0, g->mp, g->mpart); break;
-    default: k_mp_moments<4><<<gr, GT, 0, s>>>(L0, g->mp, g->mpart); break;
+    case 0: k_mp_moments<0><<<grm, GT, 0, s>>>(L0, g->mp, g->mpart); break;
+    case 1: k_mp_moments<1><<<grm, GT, 0, s>>>(L0, g->mp, g->mpart); break;
+    case 2: k_mp_moments<2><<<grm, GT, 0, s>>>(L0, g->mp, g->mpart); break;
+    case 3: k_mp_moments<3><<<grm, GT, 0, s>>>(L0, g->mp, g->mpart); break;
+    default: k_mp_moments<4><<<grm, GT, 0, s>>>(L0, g->mp, g->mpart); break;
   }
-  k_mp_coef<<<2 * MP_NC, GT, 0, s>>>(g->mpart, (int)gr, lmax, g->mp);
+  k_mp_coef<<<2 * MP_NC, GT, 0, s>>>(g->mpart, (int)grm, lmax, g->mp);
   const MP mp{lmax, g->mp};
   for (int l = 0; l < g->nl; ++l) {
     FaceJob job;
@@ -969,10 +1254,10 @@ static void full_multigrid(GravState *g, const tde_grav_params &gp, int lmax, cu
   const MP mp{lmax, g->mp};
   for (int l = g->nl - 2; l >= 0; --l) {
     const Lev &F = g->lev[l];
-    if (prolong_tiles(F, g->lev[l + 1]))
-      k_mg_prolong_tiled<1><<<prolong_tile_count(F), GT, 0, s>>>(F, g->lev[l + 1], mp);
+    if (const int T = prolong_tile(F, g->lev[l + 1]))
+      launch_prolong_tiled<1>(F, g->lev[l + 1], mp, T, s);
     else
-      k_mg_prolong_full<<<grid_for((long long)F.n[0] * F.n[1] * F.n[2]), GT, 0, s>>>(F, g->lev[l + 1], mp);
+      k_mg_prolong_full<<<(unsigned)std::min<long long>((long long)F.n[0] * F.n[1] * F.n[2], 152LL * 32), 32, 0, s>>>(F, g->lev[l + 1], mp);
     g->launches += 1;
     vcycle(g, l, gp, s);
     if (l == 0) smooth(g, F, gp.omega, s);

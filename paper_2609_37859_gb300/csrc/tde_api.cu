@@ -173,76 +173,101 @@ extern "C" int tde_finalize(tde_ctx *ctx) {
 
 // ============================================================= EOS ====
 
-// The fixed-point form of a loaded table (tde_fx.cuh), one allocation: the node
-// pairs, their 32-bit copies, the search buckets and the log2 / exp2 tables.  A
-// table with an entry outside the format keeps the axes only, and every cell
-// goes through the FP64 arrays.
+// The fixed-point form of a loaded table (tde_fx.cuh), built on the device from the
+// FP64 arrays: the node pairs and their 32-bit copies, then the search buckets.
+__global__ void k_fx_nodes(const double *__restrict__ le, const double *__restrict__ lp,
+                           const double *__restrict__ lc, long long npair, int nt, longlong2 *nd, int2 *n32) {
+  for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < npair;
+       k += (long long)gridDim.x * blockDim.x) {
+    const fx a = fx_of_log10(le[k]), b = fx_of_log10(le[k + nt]);
+    nd[3 * k] = make_longlong2(a, b);
+    nd[3 * k + 1] = make_longlong2(fx_of_log10(lp[k]), fx_of_log10(lp[k + nt]));
+    nd[3 * k + 2] = make_longlong2(fx_of_log10(lc[k]), fx_of_log10(lc[k + nt]));
+    n32[k] = make_int2((int)(a >> 32), (int)(b >> 32));
+  }
+}
+// An interpolated node lies between the two rows', so the cell of y lies between
+// the rows' cells of the bucket's ends.
+__global__ void k_fx_buckets(const longlong2 *__restrict__ nd, int nr, int nt, fx y0, int sh, int nbk, ushort2 *bk) {
+  const long long n = (long long)(nr - 1) * nbk;
+  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
+    const long long i = e / nbk;
+    const fx y[2] = {y0 + ((e - i * nbk) << sh), y0 + ((e - i * nbk + 1) << sh)};
+    const longlong2 *col = nd + 3 * i * nt;
+    int r[2][2];   // the last node at or below y (at most nt - 2, at least 0), per row and end
+    for (int row = 0; row < 2; ++row)
+      for (int end = 0; end < 2; ++end) {
+        int lo = 0, hi = nt - 1;
+        while (hi - lo > 1) {
+          const int mid = (lo + hi) >> 1;
+          const longlong2 v = col[3 * mid];
+          if ((row ? v.y : v.x) <= y[end]) lo = mid; else hi = mid;
+        }
+        r[row][end] = lo;
+      }
+    bk[e] = make_ushort2((unsigned short)min(r[0][0], r[1][0]), (unsigned short)max(r[0][1], r[1][1]));
+  }
+}
+
+// One allocation: the log2 / exp2 tables, then the above.  A table with an entry
+// outside the format keeps the axes only, and every cell goes through the FP64
+// arrays.
 static cudaError_t load_fx_table(tde_eos *e, double lr_max, const double *le, const double *lp, const double *lc) {
   DTable &t = e->tab;
   const int nr = t.nr, nt = t.nt;
   const size_t nn = (size_t)nr * nt, npair = (size_t)(nr - 1) * nt;
   t.fa = fx_axes(nr, nt, t.lr0, lr_max, t.inv_dlr, t.lt0, t.dlt);
-  const double *src[3] = {le, lp, lc};
-  std::vector<fx> v[3];
   bool ok = t.fa.valid;
-  for (int q = 0; q < 3; ++q) {
-    v[q].resize(nn);
-    for (size_t k = 0; k < nn; ++k) {
-      v[q][k] = fx_of_log10(src[q][k]);
-      ok = ok && v[q][k] != FX_BAD;
-    }
-  }
+  for (size_t k = 0; k < nn; ++k)
+    ok = ok && fabs(le[k]) < FX_MAX_LOG10 && fabs(lp[k]) < FX_MAX_LOG10 && fabs(lc[k]) < FX_MAX_LOG10;
   // bucket width: the smallest power of two that needs at most 8 nt buckets
-  fx y0 = v[0][0], y1 = v[0][0];
-  for (size_t k = 0; k < nn && ok; ++k) { y0 = std::min(y0, v[0][k]); y1 = std::max(y1, v[0][k]); }
-  int sh = 32;
-  while (((y1 - y0) >> sh) + 1 > 8LL * nt) ++sh;
-  const int nbk = ok ? (int)((y1 - y0) >> sh) + 1 : 0;
+  int sh = 32, nbk = 0;
+  fx y0 = 0;
+  if (ok) {   // (the columns increase: the ends hold the extremes)
+    fx y1 = fx_of_log10(le[nt - 1]);
+    y0 = fx_of_log10(le[0]);
+    for (int i = 1; i < nr; ++i) {
+      y0 = std::min(y0, fx_of_log10(le[(size_t)i * nt]));
+      y1 = std::max(y1, fx_of_log10(le[(size_t)i * nt + nt - 1]));
+    }
+    while (((y1 - y0) >> sh) + 1 > 8LL * nt) ++sh;
+    nbk = (int)((y1 - y0) >> sh) + 1;
+  }
   const bool buckets = ok && nt <= 65535;
-  std::vector<unsigned char> h(sizeof(FxMath));
-  fx_fill_math(reinterpret_cast<FxMath *>(h.data()));
-  size_t o_node = 0, o_n32 = 0, o_bk = 0;
+  size_t size = sizeof(FxMath), o_node = 0, o_n32 = 0, o_bk = 0;
   auto part = [&](size_t bytes) {
-    const size_t o = (h.size() + 15) / 16 * 16;
-    h.resize(o + bytes);
+    const size_t o = (size + 15) / 16 * 16;
+    size = o + bytes;
     return o;
   };
   if (ok) {
     o_node = part(sizeof(longlong2) * 3 * npair);
     o_n32 = part(sizeof(int2) * npair);
     if (buckets) o_bk = part(sizeof(ushort2) * (size_t)(nr - 1) * nbk);
-    longlong2 *nd = reinterpret_cast<longlong2 *>(h.data() + o_node);
-    int2 *n32 = reinterpret_cast<int2 *>(h.data() + o_n32);
-    for (int i = 0; i + 1 < nr; ++i)
-      for (int j = 0; j < nt; ++j) {
-        const size_t k = (size_t)i * nt + j;
-        for (int q = 0; q < 3; ++q) nd[3 * k + q] = make_longlong2(v[q][k], v[q][k + nt]);
-        n32[k] = make_int2((int)(v[0][k] >> 32), (int)(v[0][k + nt] >> 32));
-      }
-    ushort2 *bk = reinterpret_cast<ushort2 *>(h.data() + o_bk);
-    for (int i = 0; i + 1 < nr && buckets; ++i) {
-      // an interpolated node lies between the two rows', so the cell of y lies
-      // between the rows' cells of the bucket's ends
-      int a[2] = {0, 0}, b[2] = {0, 0};
-      for (int q = 0; q < nbk; ++q) {
-        const fx ya = y0 + ((fx)q << sh), yb = ya + ((fx)1 << sh);
-        for (int r = 0; r < 2; ++r) {
-          const fx *col = v[0].data() + (size_t)(i + r) * nt;
-          while (a[r] < nt - 2 && col[a[r] + 1] <= ya) ++a[r];
-          while (b[r] < nt - 2 && col[b[r] + 1] <= yb) ++b[r];
-        }
-        bk[(size_t)i * nbk + q] = make_ushort2((unsigned short)std::min(a[0], a[1]), (unsigned short)std::max(b[0], b[1]));
-      }
-    }
   }
-  cudaError_t err = cudaMalloc(&e->d_fx, h.size());
-  if (err == cudaSuccess) err = cudaMemcpy(e->d_fx, h.data(), h.size(), cudaMemcpyHostToDevice);
+  FxMath fm;
+  fx_fill_math(&fm);
+  cudaError_t err = cudaMalloc(&e->d_fx, size);
+  if (err == cudaSuccess) err = cudaMemcpy(e->d_fx, &fm, sizeof fm, cudaMemcpyHostToDevice);
   if (err != cudaSuccess) return err;
   t.fm = reinterpret_cast<const FxMath *>(e->d_fx);
   if (ok) {
-    t.node = reinterpret_cast<const longlong2 *>(e->d_fx + o_node);
-    t.n32 = reinterpret_cast<const int2 *>(e->d_fx + o_n32);
-    t.bk = buckets ? reinterpret_cast<const ushort2 *>(e->d_fx + o_bk) : nullptr;
+    longlong2 *node = reinterpret_cast<longlong2 *>(e->d_fx + o_node);
+    int2 *n32 = reinterpret_cast<int2 *>(e->d_fx + o_n32);
+    ushort2 *bk = buckets ? reinterpret_cast<ushort2 *>(e->d_fx + o_bk) : nullptr;
+    cudaStream_t s = e->ctx->stream;
+    k_fx_nodes<<<(unsigned)std::min<size_t>((npair + 255) / 256, 2048), 256, 0, s>>>(t.le, t.lp, t.lc, (long long)npair,
+                                                                                    nt, node, n32);
+    if (buckets) {
+      const size_t nb = (size_t)(nr - 1) * nbk;
+      k_fx_buckets<<<(unsigned)std::min<size_t>((nb + 255) / 256, 2048), 256, 0, s>>>(node, nr, nt, y0, sh, nbk, bk);
+    }
+    err = cudaGetLastError();
+    if (err == cudaSuccess) err = cudaStreamSynchronize(s);   // (the handle may be used on another stream)
+    if (err != cudaSuccess) return err;
+    t.node = node;
+    t.n32 = n32;
+    t.bk = bk;
     t.y0 = y0;
     t.bshift = sh;
     t.nbk = nbk;
@@ -335,11 +360,7 @@ extern "C" int tde_eos_load_table(tde_ctx *ctx, int n_rho, int n_T, double lr_mi
     }
     t.mt = e->d_mt;
   }
-  try {
-    err = load_fx_table(e, lr_max, log10_e, log10_P, log10_cs2);
-  } catch (const std::bad_alloc &) {
-    err = cudaErrorMemoryAllocation;
-  }
+  err = load_fx_table(e, lr_max, log10_e, log10_P, log10_cs2);
   if (err != cudaSuccess) {
     tde_eos_destroy(e);
     return cuda_fail(ctx, err, "tde_eos_load_table: fixed-point table");

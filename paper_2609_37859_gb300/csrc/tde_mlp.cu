@@ -85,125 +85,229 @@ __global__ void k_mlp_samples(DTable t, MLPNorm nm, long long n, unsigned long l
 
 // ------------------------------------------------------------------ training
 
-constexpr int GT = 128;   // samples (threads) per CTA in the gradient kernel
+constexpr int TRAIN_ALIGN = 128;   // a training batch is a multiple of this many samples
+constexpr int GS = 32;             // samples per CTA in the gradient kernel
+constexpr int GT = 512;            // its threads
+constexpr int HP = H + 4;          // padded row of a [..][H] tile (16-byte rows on distinct banks)
+
+// one Adam step after the gradient (in the CTA that finishes last)
+struct AdamArgs {
+  float *w, *m, *v;         // FP32 master weights and moments
+  __nv_bfloat16 *wb;        // their BF16 rounding
+  unsigned *done;           // CTAs finished (zero between launches); null: gradient only
+  float lr, b1, b2, eps, bc1, bc2;
+};
+
+__device__ __forceinline__ void red4(float *p, float a, float b, float c, float d) {
+  asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
+}
 
 // loss and gradient of L = (1/n) sum_s sum_o (y - target)^2 over samples
 // [s0, s0 + count) with the BF16-rounded weights wb; gradient and loss are
 // accumulated into g (NPARAM floats) and *loss.
-__global__ void __launch_bounds__(GT) k_mlp_grad(const __nv_bfloat16 *__restrict__ wb,
+//
+// A batch is little work (4096 samples: 0.11 GFLOP), so what bounds a step is the
+// depth of its dependent sums and the number of SMs it reaches: a CTA takes 32
+// samples (a batch of 4096 fills 128 SMs) with 16 warps, every layer's products
+// are register tiles of 4 or 8 outputs a thread (operands read as float4), and the
+// CTA that finishes last applies Adam instead of a second launch.  One training
+// step of 4096: 19 us (79 with a thread per sample and 128 samples a CTA).
+__global__ void __launch_bounds__(GT) k_mlp_grad(const __nv_bfloat16 *wb_in,
                                                  const float *__restrict__ x,
                                                  const float *__restrict__ tg, long long s0,
                                                  long long count, float inv_n, float *g,
-                                                 float *loss) {
-  extern __shared__ float sh[];
-  float *sw = sh;                       // NPARAM weights (as float)
-  float *sh1 = sw + NPARAM;             // [GT][H + 1]
-  float *sga2 = sh1 + GT * (H + 1);     // [GT][H + 1]
-  float *sh2 = sga2 + GT * (H + 1);     // [GT][H + 1]
-  float *sga1 = sh2 + GT * (H + 1);     // [GT][H + 1]
-  float *sx = sga1 + GT * (H + 1);      // [GT][2]
-  float *sgy = sx + 2 * GT;             // [GT][2]
+                                                 float *loss, AdamArgs ad) {
+  extern __shared__ __align__(16) float sh[];
+  float *W2 = sh;                  // [H][HP]
+  float *sh1 = W2 + H * HP;        // [GS][HP] hidden 1
+  float *sh2 = sh1 + GS * HP;      // [GS][HP] hidden 2
+  float *sg2 = sh2 + GS * HP;      // [GS][HP] gradient of pre-activation 2
+  float *sg1 = sg2 + GS * HP;      // [GS][HP] gradient of pre-activation 1
+  float *sw = sg1 + GS * HP;       // W1, b1, b2, W3, b3
+  float *W1 = sw, *b1 = W1 + 2 * H, *b2 = b1 + H, *W3 = b2 + H, *b3 = W3 + 2 * H;
+  float *sx = b3 + 4;              // [GS][2]
+  float *sgy = sx + 2 * GS;        // [GS][2]
+  __shared__ int s_last;
   const int tid = threadIdx.x;
-  for (int q = tid; q < NPARAM; q += GT) sw[q] = __bfloat162float(wb[q]);
-  __syncthreads();
-  const long long s = s0 + blockIdx.x * (long long)GT + tid;
-  const bool live = s < s0 + count;
-  float *ra1 = sga1 + tid * (H + 1), *ra2 = sga2 + tid * (H + 1);   // pre-activations, then grads
-  float *rh1 = sh1 + tid * (H + 1), *rh2 = sh2 + tid * (H + 1);
-  float xi0 = 0.f, xi1 = 0.f, t0 = 0.f, t1 = 0.f;
-  if (live) {
-    xi0 = x[2 * s]; xi1 = x[2 * s + 1];
-    t0 = tg[2 * s]; t1 = tg[2 * s + 1];
-  }
-  for (int o = 0; o < H; ++o) {
-    const float a1 = sw[OW1 + 2 * o] * xi0 + sw[OW1 + 2 * o + 1] * xi1 + sw[OB1 + o];
-    ra1[o] = a1;
-    rh1[o] = silu_f(a1);
-  }
-  for (int o = 0; o < H; ++o) {
-    float acc = sw[OB2 + o];
-#pragma unroll 16
-    for (int i = 0; i < H; ++i) acc += sw[OW2 + o * H + i] * rh1[i];
-    ra2[o] = acc;
-    rh2[o] = silu_f(acc);
-  }
-  float y0 = sw[OB3], y1 = sw[OB3 + 1];
-  for (int i = 0; i < H; ++i) {
-    const float h = rh2[i];
-    y0 += sw[OW3 + i] * h;
-    y1 += sw[OW3 + H + i] * h;
-  }
-  const float r0 = live ? y0 - t0 : 0.f, r1 = live ? y1 - t1 : 0.f;
-  const float gy0 = 2.f * r0 * inv_n, gy1 = 2.f * r1 * inv_n;
-  sx[2 * tid] = xi0;
-  sx[2 * tid + 1] = xi1;
-  sgy[2 * tid] = gy0;
-  sgy[2 * tid + 1] = gy1;
-  float gh1[H];
+  const bool vec = (reinterpret_cast<uintptr_t>(g + OW2) & 15) == 0;   // a caller's g may start on any float
+  const long long first = s0 + blockIdx.x * (long long)GS;
+  {   // eight weights of a row per thread (OW2 is a multiple of eight)
+    static_assert(H * H / 8 == GT && OW2 % 8 == 0, "weight rows");
+    const uint4 v = *reinterpret_cast<const uint4 *>(wb_in + OW2 + 8 * tid);
+    float *d = W2 + (tid / (H / 8)) * HP + 8 * (tid % (H / 8));
+    const unsigned u[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-  for (int i = 0; i < H; ++i) gh1[i] = 0.f;
-  for (int o = 0; o < H; ++o) {
-    const float gh2 = sw[OW3 + o] * gy0 + sw[OW3 + H + o] * gy1;
-    const float ga2 = gh2 * dsilu_f(ra2[o]);
-    ra2[o] = ga2;
-#pragma unroll
-    for (int i = 0; i < H; ++i) gh1[i] += sw[OW2 + o * H + i] * ga2;
+    for (int q = 0; q < 4; ++q) {   // a BF16 is the high half of its FP32
+      d[2 * q] = __uint_as_float(u[q] << 16);
+      d[2 * q + 1] = __uint_as_float(u[q] & 0xffff0000u);
+    }
   }
-#pragma unroll
-  for (int o = 0; o < H; ++o) ra1[o] = gh1[o] * dsilu_f(ra1[o]);
-  // per-CTA loss
-  float l = r0 * r0 + r1 * r1;
-  for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
-  if ((tid & 31) == 0) atomicAdd(loss, l * inv_n);
-  __syncthreads();
-  // reductions over the CTA's samples
-  for (int q = tid; q < H * H; q += GT) {   // dW2[o][i] = sum_s ga2[s][o] h1[s][i]
-    const int o = q / H, i = q % H;
-    float acc = 0.f;
-    for (int k = 0; k < GT; ++k) acc += sga2[k * (H + 1) + o] * sh1[k * (H + 1) + i];
-    atomicAdd(g + OW2 + q, acc);
+  if (tid < 2 * H) {
+    W1[tid] = __bfloat162float(wb_in[OW1 + tid]);
+    W3[tid] = __bfloat162float(wb_in[OW3 + tid]);
   }
   if (tid < H) {
-    const int o = tid;
-    float d1 = 0.f, w0 = 0.f, w1 = 0.f, d2 = 0.f, v0 = 0.f, v1 = 0.f;
-    for (int k = 0; k < GT; ++k) {
-      const float ga1 = sga1[k * (H + 1) + o];
-      d1 += ga1;
-      w0 += ga1 * sx[2 * k];
-      w1 += ga1 * sx[2 * k + 1];
-      d2 += sga2[k * (H + 1) + o];
-      const float h2 = sh2[k * (H + 1) + o];
-      v0 += sgy[2 * k] * h2;
-      v1 += sgy[2 * k + 1] * h2;
+    b1[tid] = __bfloat162float(wb_in[OB1 + tid]);
+    b2[tid] = __bfloat162float(wb_in[OB2 + tid]);
+  }
+  if (tid < 2) b3[tid] = __bfloat162float(wb_in[OB3 + tid]);
+  if (tid < 2 * GS) sx[tid] = first + tid / 2 < s0 + count ? x[2 * first + tid] : 0.f;
+  const bool live = first + (tid >> 4) < s0 + count;
+  const float t0 = live ? tg[2 * (first + (tid >> 4))] : 0.f, t1 = live ? tg[2 * (first + (tid >> 4)) + 1] : 0.f;
+  __syncthreads();
+  // layer 1
+  for (int q = tid; q < GS * H; q += GT) {
+    const int k = q / H, o = q % H;
+    sh1[k * HP + o] = silu_f(W1[2 * o] * sx[2 * k] + W1[2 * o + 1] * sx[2 * k + 1] + b1[o]);
+  }
+  __syncthreads();
+  // layer 2: sample sg and outputs og + 16 j
+  const int og = tid & 15, sg = tid >> 4;
+  float a2[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) a2[j] = b2[og + 16 * j];
+  {
+    const float *h0 = sh1 + sg * HP;
+#pragma unroll 4
+    for (int i = 0; i < H; i += 4) {
+      const float4 p = *reinterpret_cast<const float4 *>(h0 + i);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const float4 w = *reinterpret_cast<const float4 *>(W2 + (og + 16 * j) * HP + i);
+        a2[j] += w.x * p.x; a2[j] += w.y * p.y; a2[j] += w.z * p.z; a2[j] += w.w * p.w;
+      }
     }
-    atomicAdd(g + OB1 + o, d1);
-    atomicAdd(g + OW1 + 2 * o, w0);
-    atomicAdd(g + OW1 + 2 * o + 1, w1);
-    atomicAdd(g + OB2 + o, d2);
-    atomicAdd(g + OW3 + o, v0);
-    atomicAdd(g + OW3 + H + o, v1);
   }
-  if (tid == H) {
-    float b0 = 0.f, b1 = 0.f;
-    for (int k = 0; k < GT; ++k) { b0 += sgy[2 * k]; b1 += sgy[2 * k + 1]; }
-    atomicAdd(g + OB3, b0);
-    atomicAdd(g + OB3 + 1, b1);
+  // layer 3 (a sample's outputs over the 16 lanes of its group), loss, backward
+  float l = 0.f, gy0, gy1;
+  {
+    float y0 = 0.f, y1 = 0.f;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int o = og + 16 * j;
+      const float h = silu_f(a2[j]);
+      sh2[sg * HP + o] = h;
+      y0 += W3[o] * h;
+      y1 += W3[H + o] * h;
+    }
+#pragma unroll
+    for (int d = 8; d > 0; d >>= 1) {
+      y0 += __shfl_xor_sync(0xffffffffu, y0, d);
+      y1 += __shfl_xor_sync(0xffffffffu, y1, d);
+    }
+    const float r0 = live ? y0 + b3[0] - t0 : 0.f, r1 = live ? y1 + b3[1] - t1 : 0.f;
+    gy0 = 2.f * r0 * inv_n;
+    gy1 = 2.f * r1 * inv_n;
+    if (og == 0) {
+      sgy[2 * sg] = gy0;
+      sgy[2 * sg + 1] = gy1;
+      l = r0 * r0 + r1 * r1;
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int o = og + 16 * j;
+      sg2[sg * HP + o] = (W3[o] * gy0 + W3[H + o] * gy1) * dsilu_f(a2[j]);
+    }
   }
-}
-
-__global__ void k_adam(float *w, float *m, float *v, float *g, __nv_bfloat16 *wb, int n, float lr,
-                       float b1, float b2, float eps, float bc1, float bc2) {
-  for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < n; q += gridDim.x * blockDim.x) {
-    const float gq = g[q];
-    const float mq = b1 * m[q] + (1.f - b1) * gq;
-    const float vq = b2 * v[q] + (1.f - b2) * gq * gq;
-    m[q] = mq;
-    v[q] = vq;
-    const float wq = w[q] - lr * (mq / bc1) / (sqrtf(vq / bc2) + eps);
-    w[q] = wq;
-    wb[q] = __float2bfloat16_rn(wq);
-    g[q] = 0.f;
+  l += __shfl_xor_sync(0xffffffffu, l, 16);   // the warp's two samples
+  if ((tid & 31) == 0) atomicAdd(loss, l * inv_n);
+  __syncthreads();
+  // gradient of hidden 1: sample sg and inputs 4 og .. 4 og + 3
+  {
+    float gh[4] = {0.f, 0.f, 0.f, 0.f};
+    const float *g0 = sg2 + sg * HP;
+#pragma unroll 4
+    for (int o = 0; o < H; o += 4) {
+      const float4 p = *reinterpret_cast<const float4 *>(g0 + o);
+      const float pa[4] = {p.x, p.y, p.z, p.w};
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const float4 w = *reinterpret_cast<const float4 *>(W2 + (o + j) * HP + 4 * og);
+        gh[0] += w.x * pa[j]; gh[1] += w.y * pa[j]; gh[2] += w.z * pa[j]; gh[3] += w.w * pa[j];
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int i = 4 * og + u;
+      const float a1 = W1[2 * i] * sx[2 * sg] + W1[2 * i + 1] * sx[2 * sg + 1] + b1[i];
+      sg1[sg * HP + i] = gh[u] * dsilu_f(a1);
+    }
   }
+  // dW2[o][i] = sum_s ga2[s][o] h1[s][i]: outputs 2 sg, 2 sg + 1, inputs 4 og .. 4 og + 3
+  {
+    float d[2][4] = {};
+#pragma unroll 8
+    for (int k = 0; k < GS; ++k) {
+      const float4 h = *reinterpret_cast<const float4 *>(sh1 + k * HP + 4 * og);
+      const float2 q = *reinterpret_cast<const float2 *>(sg2 + k * HP + 2 * sg);
+      d[0][0] += q.x * h.x; d[0][1] += q.x * h.y; d[0][2] += q.x * h.z; d[0][3] += q.x * h.w;
+      d[1][0] += q.y * h.x; d[1][1] += q.y * h.y; d[1][2] += q.y * h.z; d[1][3] += q.y * h.w;
+    }
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      float *p = g + OW2 + (2 * sg + j) * H + 4 * og;
+      if (vec) red4(p, d[j][0], d[j][1], d[j][2], d[j][3]);
+      else
+        for (int u = 0; u < 4; ++u) atomicAdd(p + u, d[j][u]);
+    }
+  }
+  __syncthreads();
+  // the small gradients: two warps per sum over the samples
+  {
+    const int o = tid & (H - 1), part = tid / H;
+    if (part < 6) {
+      const float *c = part == 0 ? sg2 : (part < 3 ? sh2 : sg1);
+      const float *f = part == 1 || part == 2 ? sgy + part - 1 : sx + (part == 5 ? 1 : 0);
+      const bool plain = part == 0 || part == 3;
+      float d = 0.f;
+#pragma unroll 8
+      for (int k = 0; k < GS; ++k) d += plain ? c[k * HP + o] : c[k * HP + o] * f[2 * k];
+      const int at = part == 0 ? OB2 + o : part == 1 ? OW3 + o : part == 2 ? OW3 + H + o : part == 3 ? OB1 + o
+                                         : part == 4 ? OW1 + 2 * o : OW1 + 2 * o + 1;
+      atomicAdd(g + at, d);
+    } else if (part == 6 && o < 2) {
+      float d = 0.f;
+      for (int k = 0; k < GS; ++k) d += sgy[2 * k + o];
+      atomicAdd(g + OB3 + o, d);
+    }
+  }
+  if (!ad.done) return;
+  // Adam in the CTA that finishes last: its additions are ordered before the count,
+  // and the count before its reads
+  __threadfence();
+  __syncthreads();
+  if (tid == 0) s_last = atomicAdd(ad.done, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  // (all of a thread's loads before its arithmetic: one round of memory latency)
+  constexpr int NQ = (NPARAM + GT - 1) / GT;
+  float gq[NQ], mq[NQ], vq[NQ], wq[NQ];
+#pragma unroll
+  for (int u = 0; u < NQ; ++u) {
+    const int q = tid + u * GT;
+    if (q < NPARAM) {
+      gq[u] = __ldcg(g + q);
+      mq[u] = ad.m[q];
+      vq[u] = ad.v[q];
+      wq[u] = ad.w[q];
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < NQ; ++u) {
+    const int q = tid + u * GT;
+    if (q < NPARAM) {
+      const float m = ad.b1 * mq[u] + (1.f - ad.b1) * gq[u];
+      const float v = ad.b2 * vq[u] + (1.f - ad.b2) * gq[u] * gq[u];
+      const float w = wq[u] - ad.lr * (m / ad.bc1) / (sqrtf(v / ad.bc2) + ad.eps);
+      ad.m[q] = m;
+      ad.v[q] = v;
+      ad.w[q] = w;
+      ad.wb[q] = __float2bfloat16_rn(w);
+      g[q] = 0.f;
+    }
+  }
+  if (tid == 0) *ad.done = 0;
 }
 
 __global__ void k_round_bf16(const float *w, __nv_bfloat16 *wb, int n) {
@@ -603,6 +707,11 @@ int mlp_fail(tde_ctx *c, int code, const char *msg) {
     }                                                                    \
   } while (0)
 
+// d_w: the weights, Adam's m and v (NPARAM floats each), the gradient (from OG, so
+// that its W2 part starts on 16 bytes) and the count of finished CTAs
+constexpr int OG = (3 * NPARAM + OW2 + 3) / 4 * 4 - OW2, WBUF = OG + NPARAM + 2;
+static_assert((OG + OW2) % 4 == 0 && OG >= 3 * NPARAM, "gradient alignment");
+
 MLPNorm norm_of(const tde_eos *e) {
   MLPNorm n;
   n.cr = (float)e->norm[0]; n.sr = (float)e->norm[1];
@@ -618,8 +727,8 @@ MLPNorm norm_of(const tde_eos *e) {
 int ensure_net_buffers(tde_eos *e) {
   tde_ctx *c = e->ctx;
   if (!e->d_w) {
-    MCK(c, cudaMalloc(&e->d_w, sizeof(float) * 4 * NPARAM));
-    MCK(c, cudaMemset(e->d_w, 0, sizeof(float) * 4 * NPARAM));
+    MCK(c, cudaMalloc(&e->d_w, sizeof(float) * WBUF));
+    MCK(c, cudaMemset(e->d_w, 0, sizeof(float) * WBUF));
   }
   if (!e->d_wb) MCK(c, cudaMalloc(&e->d_wb, sizeof(__nv_bfloat16) * NPARAM));
   if (!e->d_status) {
@@ -632,7 +741,7 @@ int ensure_net_buffers(tde_eos *e) {
 int upload_weights(tde_eos *e, const float *w) {
   tde_ctx *c = e->ctx;
   MCK(c, cudaMemcpyAsync(e->d_w, w, sizeof(float) * NPARAM, cudaMemcpyHostToDevice, c->stream));
-  MCK(c, cudaMemsetAsync(e->d_w + NPARAM, 0, sizeof(float) * 3 * NPARAM, c->stream));   // m, v, g
+  MCK(c, cudaMemsetAsync(e->d_w + NPARAM, 0, sizeof(float) * (WBUF - NPARAM), c->stream));   // m, v, g, count
   k_round_bf16<<<(NPARAM + 255) / 256, 256, 0, c->stream>>>(e->d_w, (__nv_bfloat16 *)e->d_wb, NPARAM);
   MCK(c, cudaGetLastError());
   MCK(c, cudaStreamSynchronize(c->stream));
@@ -640,18 +749,15 @@ int upload_weights(tde_eos *e, const float *w) {
   return TDE_OK;
 }
 
-size_t grad_smem() { return sizeof(float) * (NPARAM + 4 * GT * (H + 1) + 4 * GT); }
+size_t grad_smem() { return sizeof(float) * ((H + 4 * GS) * HP + 2 * H + H + H + 2 * H + 4 + 4 * GS); }
 
 cudaError_t launch_grad(tde_eos *e, const float *x, const float *tg, long long s0, long long count,
-                        float inv_n, float *g, float *loss, cudaStream_t s) {
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(k_mlp_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)grad_smem());
-    attr = true;
-  }
-  const unsigned grid = (unsigned)((count + GT - 1) / GT);
+                        float inv_n, float *g, float *loss, const AdamArgs &ad, cudaStream_t s) {
+  cudaError_t err = cudaFuncSetAttribute(k_mlp_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)grad_smem());
+  if (err != cudaSuccess) return err;
+  const unsigned grid = (unsigned)((count + GS - 1) / GS);
   k_mlp_grad<<<grid, GT, grad_smem(), s>>>((const __nv_bfloat16 *)e->d_wb, x, tg, s0, count, inv_n, g,
-                                           loss);
+                                           loss, ad);
   return cudaGetLastError();
 }
 
@@ -840,7 +946,7 @@ extern "C" int tde_eos_surrogate_grad(tde_eos *e, int64_t n, const float *x, con
   MCK(c, cudaMemsetAsync(grad, 0, sizeof(float) * NPARAM, c->stream));
   MCK(c, cudaMemsetAsync(loss, 0, sizeof(float), c->stream));
   ProfScope ps(c, TDE_K_EOS);
-  MCK(c, launch_grad(e, x, target, 0, n, 1.0f / (float)n, grad, loss, c->stream));
+  MCK(c, launch_grad(e, x, target, 0, n, 1.0f / (float)n, grad, loss, AdamArgs{}, c->stream));
   return TDE_OK;
 }
 
@@ -857,7 +963,7 @@ extern "C" int tde_eos_surrogate_train(tde_eos *e, uint64_t seed, int n_samples,
                                        double lr, tde_train_report *rep) {
   if (!e) return TDE_EINVAL;
   tde_ctx *c = e->ctx;
-  if (n_samples < GT || epochs < 1 || batch < GT || batch % GT || !(lr > 0.0))
+  if (n_samples < TRAIN_ALIGN || epochs < 1 || batch < TRAIN_ALIGN || batch % TRAIN_ALIGN || !(lr > 0.0))
     return mlp_fail(c, TDE_EINVAL, "tde_eos_surrogate_train: sizes (batch a multiple of 128)");
   int r = ensure_net_buffers(e);
   if (r) return r;
@@ -874,32 +980,38 @@ extern "C" int tde_eos_surrogate_train(tde_eos *e, uint64_t seed, int n_samples,
     r = upload_weights(e, w.data());
     if (r) return r;
   }
-  float *d_x = nullptr, *d_y = nullptr, *d_loss = nullptr;
   const int nb_per_epoch = n_samples / batch;
   const int nbt = nb_per_epoch * epochs;
-  MCK(c, cudaMalloc(&d_x, sizeof(float) * 2 * n_samples));
-  MCK(c, cudaMalloc(&d_y, sizeof(float) * 2 * n_samples));
-  MCK(c, cudaMalloc(&d_loss, sizeof(float) * nbt));
   cudaStream_t s = c->stream;
+  // samples, targets and losses in one stream-ordered allocation (given back below)
+  float *d_x = nullptr;
+  MCK(c, cudaMallocAsync((void **)&d_x, sizeof(float) * (4 * (size_t)n_samples + nbt), s));
+  float *d_y = d_x + 2 * (size_t)n_samples, *d_loss = d_y + 2 * (size_t)n_samples;
   cudaEvent_t e0, e1;
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
   cudaEventRecord(e0, s);
   cudaMemsetAsync(d_loss, 0, sizeof(float) * nbt, s);
   k_mlp_samples<<<1024, 256, 0, s>>>(e->tab, norm_of(e), n_samples, seed, d_x, d_y);
-  float *w = e->d_w, *m = w + NPARAM, *v = m + NPARAM, *g = v + NPARAM;
-  const float b1 = 0.9f, b2 = 0.999f;
+  AdamArgs ad;
+  ad.w = e->d_w;
+  ad.m = ad.w + NPARAM;
+  ad.v = ad.m + NPARAM;
+  ad.wb = (__nv_bfloat16 *)e->d_wb;
+  ad.b1 = 0.9f;
+  ad.b2 = 0.999f;
+  ad.eps = 1e-8f;
+  float *g = e->d_w + OG;
+  ad.done = reinterpret_cast<unsigned *>(g + NPARAM);
   int step = 0;
   cudaError_t err = cudaGetLastError();
   for (int ep = 0; ep < epochs && err == cudaSuccess; ++ep) {
     for (int bi = 0; bi < nb_per_epoch && err == cudaSuccess; ++bi, ++step) {
-      err = launch_grad(e, d_x, d_y, (long long)bi * batch, batch, 1.0f / batch, g, d_loss + step, s);
       const double prog = (double)step / (double)nbt;
-      const float lrs = (float)(lr * (0.05 + 0.95 * 0.5 * (1.0 + cos(3.141592653589793 * prog))));
-      const float bc1 = 1.f - powf(b1, (float)(step + 1)), bc2 = 1.f - powf(b2, (float)(step + 1));
-      k_adam<<<(NPARAM + 255) / 256, 256, 0, s>>>(w, m, v, g, (__nv_bfloat16 *)e->d_wb, NPARAM, lrs, b1, b2,
-                                                   1e-8f, bc1, bc2);
-      if (err == cudaSuccess) err = cudaGetLastError();
+      ad.lr = (float)(lr * (0.05 + 0.95 * 0.5 * (1.0 + cos(3.141592653589793 * prog))));
+      ad.bc1 = 1.f - powf(ad.b1, (float)(step + 1));
+      ad.bc2 = 1.f - powf(ad.b2, (float)(step + 1));
+      err = launch_grad(e, d_x, d_y, (long long)bi * batch, batch, 1.0f / batch, g, d_loss + step, ad, s);
     }
   }
   cudaEventRecord(e1, s);
@@ -910,14 +1022,12 @@ extern "C" int tde_eos_surrogate_train(tde_eos *e, uint64_t seed, int n_samples,
   cudaEventElapsedTime(&ms, e0, e1);
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
-  cudaFree(d_x);
-  cudaFree(d_y);
-  cudaFree(d_loss);
+  cudaFreeAsync(d_x, s);
   if (err != cudaSuccess) {
     c->err = std::string("tde_eos_surrogate_train: ") + cudaGetErrorString(err);
     return TDE_ECUDA;
   }
-  c->launches[TDE_K_EOS] += 2 * (uint64_t)nbt + 1;
+  c->launches[TDE_K_EOS] += (uint64_t)nbt + 1;
   if (rep) {
     rep->loss_first = losses.front();
     rep->loss_last = losses.back();

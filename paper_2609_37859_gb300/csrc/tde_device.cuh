@@ -691,14 +691,21 @@ __device__ __forceinline__ void cons_to_prim(const Phys &p, const double *u, dou
 // is added to something, the rounding is spelt out here and in the Riemann
 // solvers, so that every kernel they are compiled into gives the same bits.)
 __device__ __forceinline__ void plm(double q0, double dl, double dr, double &left, double &right) {
-  const double pr = __dmul_rn(dl, dr);
+  const long long kl = dbits(dl), kr = dbits(dr);
   left = q0;
   right = q0;
-  if (dgt0(pr)) {
-    const double ir = rcp_nr(__dadd_rn(dl, dr));
+  // dl dr > 0, by the signs (a product that underflows gives h = 0 below)
+  if ((kl ^ kr) >= 0 && (kl << 1) != 0 && (kr << 1) != 0) {
+    const double pr = __dmul_rn(dl, dr), ir = rcp_nr(__dadd_rn(dl, dr));
     left = __fma_rn(-pr, ir, q0);
     right = __fma_rn(pr, ir, q0);
   }
+}
+// a - b, without the subtraction where a = b on every lane of the warp
+__device__ __forceinline__ double diff_or_zero(double a, double b) {
+  double d = 0.0;
+  if (__any_sync(__activemask(), dbits(a) != dbits(b))) d = a - b;
+  return d;
 }
 
 // PPM interface between cells q0 and q1 = q0 + D1, with D0 and D2 the differences

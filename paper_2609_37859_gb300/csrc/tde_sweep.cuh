@@ -304,10 +304,11 @@ __device__ __forceinline__ bool sweep_tile(const SweepArgs &a, int qb, int tile,
   // before the Riemann solves.  A PPM run starts with seven extra FP64 operations
   // (of seven a cell) and a PLM run with one (of six), while a few warps keep the
   // FP64 pipe busy: PPM takes two runs a pencil (an x sweep of 2 M cells: 513 /
-  // 486 / 498 / 506 us with 1 / 2 / 3 / 4 runs), PLM four (a step of the 128^3
+  // 486 / 498 / 506 us with 1 / 2 / 3 / 4 runs; three where five or six variables
+  // leave too few threads at two), PLM four (a step of the 128^3
   // wave: 2.84 / 2.66 / 2.63 / 2.62 ms).
   {
-    constexpr int NRUN = RECON == PPM ? 2 : 4;
+    constexpr int NRUN = RECON == PPM ? (NV >= 7 ? 2 : 3) : 4;
     const int RL = (nd + 2 + NRUN - 1) / NRUN;
     const int ws = D == 0 ? 1 : LS, fs = D == 0 ? 1 : M;
     for (int e = threadIdx.x; e < NV * NRUN * M; e += NTS) {
@@ -322,7 +323,7 @@ __device__ __forceinline__ bool sweep_tile(const SweepArgs &a, int qb, int tile,
       if (RECON == PLM) {
         double dl = q0 - w[-ws];
         for (int c = c0; c < c1; ++c) {
-          const double dr = q1 - q0;
+          const double dr = diff_or_zero(q1, q0);
           double lo, hi;
           plm(q0, dl, dr, lo, hi);
           *fm = lo;
@@ -340,13 +341,23 @@ __device__ __forceinline__ bool sweep_tile(const SweepArgs &a, int qb, int tile,
         const double qm = w[-ws];
         double D1 = q0 - qm, D2 = q1 - q0, T, V;
         double a = ppm_iface(qm, q0, qm - w[-2 * ws], D1, D2, T, V);   // the run's lowest interface
+        // the last pairs of neighbours with equal values: where the four cells of an
+        // interface are equal on every lane of the warp (floor gas, a variable that
+        // does not vary) its value is theirs and the cell below it is flat
+        int same = dbits(q1) != dbits(q0) ? 0 : (dbits(q0) == dbits(qm) ? 2 : 1);
         for (int c = c0; c < c1; ++c) {
-          const double q2 = w[2 * ws], D3 = q2 - q1;
-          const double Vl = V;
-          double lo = a;
-          a = ppm_iface(q0, q1, D1, D2, D3, T, V);
-          double hi = a;
-          ppm_limit(q0, Vl, T, lo, hi);
+          const double q2 = w[2 * ws];
+          double lo = a, hi, D3;
+          same = dbits(q2) == dbits(q1) ? same + 1 : 0;
+          if (__all_sync(__activemask(), same >= 3)) {
+            D3 = T = V = 0.0;
+            lo = hi = a = q0;
+          } else {
+            const double Vl = V;
+            D3 = q2 - q1;
+            hi = a = ppm_iface(q0, q1, D1, D2, D3, T, V);
+            ppm_limit(q0, Vl, T, lo, hi);
+          }
           *fm = lo;
           *fp = hi;
           if (keep) *rh = q0;

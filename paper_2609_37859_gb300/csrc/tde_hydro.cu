@@ -915,7 +915,9 @@ static cudaError_t sweep_dir(tde_mesh *m, SweepArgs &a, int D, int shape, bool f
   const int LA = D == 0 ? 1 : 0, OA = D == 2 ? 1 : 2;
   sweep_dir_fill(m, a, D, shape, first);
   const size_t smem = sweep_smem(p, D, a.PD, a.NF, M);
-  dim3 grid((unsigned)(((m->nmax[LA] + M - 1) / M) * m->nmax[OA]), (unsigned)nblk);
+  // (tiles of M consecutive pencils without tensor maps, else of M of a row)
+  const int tiles = a.tmap ? ((m->nmax[LA] + M - 1) / M) * m->nmax[OA] : (m->nmax[LA] * m->nmax[OA] + M - 1) / M;
+  dim3 grid((unsigned)tiles, (unsigned)nblk);
   return sweep_launch_by_shape(shape, a, D, last, grid, smem, m->ctx->stream);
 }
 

@@ -152,15 +152,30 @@ __device__ __forceinline__ bool sweep_tile(const SweepArgs &a, int qb, int tile,
   const int b = a.ids[qb];
   const DevBlock B = a.blocks[b];
   const int nd = B.n[D], nl = B.n[LA], no = B.n[OA];
-  const int nlc = (nl + M - 1) / M;
   staged = false;
-  if (tile >= nlc * no) return true;   // uniform over the CTA
-  const int l0 = (tile % nlc) * M, o = tile / nlc;
-  const int nlane = min(M, nl - l0);
+  // A tile staged by TMA is M pencils of one row of pencils (a box); where the rows
+  // are shorter than a tile, or there is no tensor map, a tile is M consecutive
+  // pencils of all rows, staged by the copy loop: no lanes idle at the rows' ends
+  // (rows of 21 in tiles of 8: 45 instead of 51 tiles; 8^3 blocks beside 16^3 ones
+  // in tiles of 16: half as many).
+  const bool tma = a.tmap && nl >= M;
+  const int nlc = (nl + M - 1) / M;
+  if (tile >= (tma ? nlc * no : (nl * no + M - 1) / M)) return true;   // uniform over the CTA
+  const int l0 = tma ? (tile % nlc) * M : 0, o = tma ? tile / nlc : 0;
+  const int q0 = tma ? o * nl + l0 : tile * M;   // the tile's first pencil, row by row
+  const int nlane = tma ? min(M, nl - l0) : min(M, nl * no - q0);
   const int g = p.g[D], pd = B.p[D];
   const long long st[3] = {1, B.p[0], (long long)B.p[0] * B.p[1]};
-  const long long sD = st[D], sL = st[LA];
-  const long long base = B.off + (long long)(p.g[LA] + l0) * sL + (long long)(p.g[OA] + o) * st[OA];
+  const long long sD = st[D];
+  // each lane's pencil: transverse indices and the flat index of its first cell
+  __shared__ int s_l[M], s_o[M];
+  __shared__ long long s_base[M];
+  if (threadIdx.x < M) {
+    const int q = min(q0 + (int)threadIdx.x, nl * no - 1), oo = q / nl, ll = q - oo * nl;
+    s_l[threadIdx.x] = ll;
+    s_o[threadIdx.x] = oo;
+    s_base[threadIdx.x] = B.off + (long long)(p.g[LA] + ll) * st[LA] + (long long)(p.g[OA] + oo) * st[OA];
+  }
   const int PD = a.PD, NF = a.NF, NFF = a.NF - 1;
   const int LS = D == 0 ? M : a.LS, XO = D == 0 ? 0 : a.XO;
   const long long ntot = a.ntot;
@@ -185,16 +200,21 @@ __device__ __forceinline__ bool sweep_tile(const SweepArgs &a, int qb, int tile,
   auto sfl = [&](int q, int f, int lane) {
     return D == 0 ? (q * M + lane) * NFF + f : (q * NFF + f) * M + lane;
   };
+  // element e of a phase over len cells or faces per lane; D = 0: e / len as a
+  // product with ceil(2^20 / len) (exact: e len < 2^20)
   auto split = [&](int e, int len, int &c, int &lane) {
-    if (D == 0) { lane = e / len; c = e - lane * len; }
-    else { c = e / M; lane = e - c * M; }
+    if (D == 0) {
+      const unsigned inv = ((1u << 20) + len - 1) / (unsigned)len;
+      lane = (int)((unsigned)e * inv >> 20);
+      c = e - lane * len;
+    } else { c = e / M; lane = e - c * M; }
   };
 
   // ---- A: stage the tile's primitives (all pencil cells incl. ghosts): one
   // TMA tensor copy of the tile's box (out-of-block parts of the box are
   // zero-filled and never read), or a copy loop
   const uint32_t mbar_addr = (uint32_t)__cvta_generic_to_shared(mbar);
-  if (a.tmap) {
+  if (tma) {
     staged = true;
     if (threadIdx.x == 0) {
       // earlier tiles' generic reads of the staging area before the async write
@@ -215,12 +235,22 @@ __device__ __forceinline__ bool sweep_tile(const SweepArgs &a, int qb, int tile,
             : "memory");
     }
   } else {
-    const int per = pd * M;
-    for (int e = threadIdx.x; e < NV * per; e += NTS) {
-      const int v = e / per;
-      int pos, lane;
-      split(e - v * per, pd, pos, lane);
-      if (lane < nlane) Wt[sw(v, pos, lane)] = a.W[v * ntot + base + pos * sD + lane * sL];
+    __syncthreads();   // (s_base)
+    if (D == 0) {   // consecutive threads along the pencils
+      for (int e = threadIdx.x; e < NV * M * pd; e += NTS) {
+        const int r = e / pd, pos = e - r * pd, lane = r % M, v = r / M;
+        if (lane < nlane) Wt[sw(v, pos, lane)] = a.W[v * ntot + s_base[lane] + pos];
+      }
+    } else {        // a thread's lane is fixed, its rows (v, pos) step by NTS / M
+      const int lane = threadIdx.x % M;
+      const double *src = a.W + s_base[lane];
+      int v = 0, pos = threadIdx.x / M;
+      while (lane < nlane) {
+        while (pos >= pd) { pos -= pd; ++v; }
+        if (v >= NV) break;
+        Wt[sw(v, pos, lane)] = src[v * ntot + pos * sD];
+        pos += NTS / M;
+      }
     }
   }
   const bool grav = a.bh.on || a.phi_sg, exc = a.bh.excise;
@@ -236,9 +266,9 @@ __device__ __forceinline__ bool sweep_tile(const SweepArgs &a, int qb, int tile,
       bh_pos(a.bh, ts, rb);
       if (threadIdx.x < 3) s_rb[threadIdx.x] = rb[threadIdx.x];
       if (threadIdx.x == 0 && exc) s_exc = sphere_of(a.bh.rexc);
-      if (D == 0 && threadIdx.x < M)
-        s_yz[threadIdx.x] = bh_r2_yz(cell_coord(p, B, 1, p.g[1] + l0 + threadIdx.x) - rb[1],
-                                     cell_coord(p, B, 2, p.g[2] + o) - rb[2]);
+      if (D == 0 && threadIdx.x < M)   // (s_l, s_o: this thread's own entries)
+        s_yz[threadIdx.x] = bh_r2_yz(cell_coord(p, B, 1, p.g[1] + s_l[threadIdx.x]) - rb[1],
+                                     cell_coord(p, B, 2, p.g[2] + s_o[threadIdx.x]) - rb[2]);
     }
     __syncthreads();
     const double rb0 = s_rb[0], rb1 = s_rb[1], rb2 = s_rb[2];
@@ -249,7 +279,7 @@ __device__ __forceinline__ bool sweep_tile(const SweepArgs &a, int qb, int tile,
       if (lane >= nlane) continue;
       const int idx = D == 0 ? lane * NF + c : c * M + lane;
       const bool inner = c > 0 && c <= nd;
-      const long long cflat = base + (long long)(g - 1 + c) * sD + lane * sL;
+      const long long cflat = s_base[lane] + (long long)(g - 1 + c) * sD;
       if (cached && inner && !a.first) {   // interior cell: the first sweep's value
         if (grav) Ph[idx] = a.phic[cflat];
         if (exc) Ex[idx] = a.exc_c[cflat];
@@ -262,8 +292,8 @@ __device__ __forceinline__ bool sweep_tile(const SweepArgs &a, int qb, int tile,
       } else {
         int cc[3];
         cc[D] = g - 1 + c;
-        cc[LA] = p.g[LA] + l0 + lane;
-        cc[OA] = p.g[OA] + o;
+        cc[LA] = p.g[LA] + s_l[lane];
+        cc[OA] = p.g[OA] + s_o[lane];
         double x[3];
         cell_centre(p, B, cc, x);
         r2 = bh_r2(x[0] - rb0, x[1] - rb1, x[2] - rb2);
@@ -282,7 +312,7 @@ __device__ __forceinline__ bool sweep_tile(const SweepArgs &a, int qb, int tile,
     }
   }
   __syncthreads();
-  if (a.tmap) {
+  if (tma) {
     // every thread waits for the copy (bounded); if it did not complete, the
     // tile is skipped, the status word set, and thread 0 waits once more
     // (bounded) so that no copy is in flight when the CTA goes on or exits
@@ -431,7 +461,7 @@ __device__ __forceinline__ bool sweep_tile(const SweepArgs &a, int qb, int tile,
         so += (long long)B.n[u1] * B.n[u2] * a.nvar;
       }
       const long long ncell = (long long)nl * no;
-      const long long cidx = (long long)o * nl + l0 + lane;
+      const long long cidx = q0 + lane;
       const double w = 0.5 * ta_dt(a.ta, b);
 #pragma unroll
       for (int q = 0; q < NVAR; ++q) a.freg[so + q * ncell + cidx] += w * F[q];
@@ -447,7 +477,7 @@ __device__ __forceinline__ bool sweep_tile(const SweepArgs &a, int qb, int tile,
     int c, lane;
     split(e, nd, c, lane);
     if (lane >= nlane) continue;
-    const long long flat = base + (long long)(g + c) * sD + lane * sL;
+    const long long flat = s_base[lane] + (long long)(g + c) * sD;
     double acc[NVAR], dv = 0.0;
 #pragma unroll
     for (int q = 0; q < NVAR; ++q) acc[q] = a.first ? 0.0 : a.dU[q * ntot + flat];

@@ -20,6 +20,16 @@ enum { EOS_IDEAL = 0, EOS_TABLE = 1 };
 enum { PLM = 0, PPM = 1 };
 enum { RIEMANN_HLLC = 0, RIEMANN_HLLE = 1 };
 
+// The first statement of every kernel launched by pdl_launch: waits until the
+// kernels before this one have completed and their writes are visible.  Nothing may
+// be read before it that an earlier kernel writes; such pointers are not
+// __restrict__ (a load through one may be moved over the wait).  The kernels do not
+// release their successors early (griddepcontrol.launch_dependents): CTAs placed
+// during a kernel wait on its registers and shared memory, which cost more than the
+// launch latency it hides (a step of a 32^3 mesh: 134 us with ordinary launches, 177
+// with the early release, 103 without it).
+__device__ __forceinline__ void pdl_begin() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // ------------------------------------- comparisons on the integer pipe ----
 //
 // A double's bit pattern, read as a signed 64-bit integer, orders positive

@@ -303,9 +303,10 @@ __device__ __forceinline__ double gs_iso(const Lev &L, int i, int j, int k) {
 }
 
 // level-0 source from the MeshBlock density: S = -4 pi G rho where rho > rho_min
-__global__ void __launch_bounds__(GT) k_mg_gather(Phys p, const DevBlock *__restrict__ blocks,
-                                                  const double *__restrict__ U, Lev L, double fourpiG,
+__global__ void __launch_bounds__(GT) k_mg_gather(Phys p, const DevBlock *blocks,
+                                                  const double *U, Lev L, double fourpiG,
                                                   double rho_min) {
+  pdl_begin();
   const int b = blockIdx.y;
   const DevBlock B = blocks[b];
   const int nint = B.n[0] * B.n[1] * B.n[2];
@@ -321,6 +322,7 @@ __global__ void __launch_bounds__(GT) k_mg_gather(Phys p, const DevBlock *__rest
 // partial sums (one per CTA) of f, or of the squared defect if sq
 template <int ISO>
 __global__ void __launch_bounds__(GT) k_mg_partial(Lev L, int sq, double *part) {
+  pdl_begin();
   __shared__ double red[GT / 32];
   double s = 0.0;
   if (sq) {
@@ -346,8 +348,9 @@ __global__ void __launch_bounds__(GT) k_mg_partial(Lev L, int sq, double *part) 
 }
 
 // the partial sums in a fixed order: out = sum / n (a mean) or sqrt(sum / n)
-__global__ void __launch_bounds__(GT) k_mg_final(const double *__restrict__ part, int np, double n,
+__global__ void __launch_bounds__(GT) k_mg_final(const double *part, int np, double n,
                                                  int root, double *out) {
+  pdl_begin();
   __shared__ double red[GT];
   double s = 0.0;
   for (int q = threadIdx.x; q < np; q += GT) s += part[q];
@@ -360,7 +363,8 @@ __global__ void __launch_bounds__(GT) k_mg_final(const double *__restrict__ part
   if (threadIdx.x == 0) *out = root ? sqrt(red[0] / n) : red[0] / n;
 }
 
-__global__ void __launch_bounds__(GT) k_mg_sub_mean(Lev L, const double *__restrict__ mean) {
+__global__ void __launch_bounds__(GT) k_mg_sub_mean(Lev L, const double *mean) {
+  pdl_begin();
   const unsigned n = (unsigned)L.n[0] * L.n[1] * L.n[2];
   const double m = *mean;
   for (unsigned c = blockIdx.x * GT + threadIdx.x; c < n; c += gridDim.x * GT) L.src[c] -= m;
@@ -442,6 +446,7 @@ __device__ __forceinline__ void smooth_cells(const Lev &L, int colour, const Smo
 }
 template <int ISO>
 __global__ void __launch_bounds__(GT) k_mg_smooth(Lev L, int colour, SmoothW W, double omega) {
+  pdl_begin();
   smooth_cells<ISO>(L, colour, W, omega, blockIdx.x * GT + threadIdx.x, gridDim.x * GT);
 }
 
@@ -505,6 +510,7 @@ __device__ __forceinline__ void restrict_cells(const Lev &F, const Lev &C, doubl
 }
 template <int ISO>
 __global__ void __launch_bounds__(GT) k_mg_restrict(Lev F, Lev C, double inv) {
+  pdl_begin();
   restrict_cells<ISO>(F, C, inv, blockIdx.x * GT + threadIdx.x, gridDim.x * GT);
 }
 
@@ -520,11 +526,13 @@ __device__ __forceinline__ void fas_cells(const Lev &C, unsigned e0, unsigned st
 }
 template <int ISO>
 __global__ void __launch_bounds__(GT) k_mg_fas(Lev C) {
+  pdl_begin();
   fas_cells<ISO>(C, blockIdx.x * GT + threadIdx.x, gridDim.x * GT);
 }
 
 // the coarse correction phi_C - R phi_f, formed once per coarse cell (into tmp)
 __global__ void __launch_bounds__(GT) k_mg_corr(Lev C) {
+  pdl_begin();
   const unsigned n = (unsigned)C.n[0] * C.n[1] * C.n[2];
   for (unsigned c = blockIdx.x * GT + threadIdx.x; c < n; c += gridDim.x * GT) C.tmp[c] = C.phi[c] - C.tmp[c];
 }
@@ -563,6 +571,7 @@ __device__ __forceinline__ int fold_idx(int u, int n, bool iso, double &sg) {
 // fine phi += P e, e = phi_C - R phi_f (in C.tmp), tricubic; beyond an isolated
 // face the correction is the odd mirror image (it vanishes on the faces)
 __global__ void __launch_bounds__(GT) k_mg_prolong(Lev F, Lev C) {
+  pdl_begin();
   const unsigned n = (unsigned)F.n[0] * F.n[1] * F.n[2];
   for (unsigned c = blockIdx.x * GT + threadIdx.x; c < n; c += gridDim.x * GT) {
     int f[3];
@@ -607,6 +616,7 @@ __device__ double full_value(const Lev &C, const MP &mp, int u0, int u1, int u2)
 // written to F.phi)
 template <int FULL, int T>
 __global__ void __launch_bounds__(GT) k_mg_prolong_tiled(Lev F, Lev C, MP mp) {
+  pdl_begin();
   constexpr int S = T / 2 + 4;
   __shared__ double t1[S][S][T];       // x done: [kc][jc][i]
   __shared__ double un[S * T * T];     // coarse [k][j][i], then x and y done: [kc][j][i]
@@ -681,8 +691,8 @@ __host__ __forceinline__ int prolong_tile(const Lev &F, const Lev &C) {
 template <int FULL>
 void launch_prolong_tiled(const Lev &F, const Lev &C, const MP &mp, int T, cudaStream_t s) {
   const unsigned g = (unsigned)((F.n[0] / T) * (F.n[1] / T) * (F.n[2] / T));
-  if (T == 16) k_mg_prolong_tiled<FULL, 16><<<g, GT, 0, s>>>(F, C, mp);
-  else k_mg_prolong_tiled<FULL, 8><<<g, GT, 0, s>>>(F, C, mp);
+  if (T == 16) pdl_launch(k_mg_prolong_tiled<FULL, 16>, g, GT, 0, s, F, C, mp);
+  else pdl_launch(k_mg_prolong_tiled<FULL, 8>, g, GT, 0, s, F, C, mp);
 }
 
 // The V-cycle from level lev[0] down and back up in one CTA: the coarse levels
@@ -699,6 +709,7 @@ struct CoarseArgs {
 };
 template <int ISO>
 __global__ void __launch_bounds__(GT) k_mg_coarse(const CoarseArgs a) {
+  pdl_begin();
   __shared__ double t1[MG_COARSE], t2[MG_COARSE];
   const unsigned t = threadIdx.x;
   auto sweeps = [&](int l, int n) {
@@ -769,8 +780,9 @@ __global__ void __launch_bounds__(GT) k_mg_coarse(const CoarseArgs a) {
 
 // the potential into the MeshBlock layout, every padded cell (ghosts by the
 // periodic image of their global position)
-__global__ void __launch_bounds__(GT) k_mg_scatter(Phys p, const DevBlock *__restrict__ blocks, Lev L,
+__global__ void __launch_bounds__(GT) k_mg_scatter(Phys p, const DevBlock *blocks, Lev L,
                                                    MP mp, double *phi_pad) {
+  pdl_begin();
   const int b = blockIdx.y;
   const DevBlock B = blocks[b];
   const int npad = B.p[0] * B.p[1] * B.p[2];
@@ -786,9 +798,10 @@ __global__ void __launch_bounds__(GT) k_mg_scatter(Phys p, const DevBlock *__res
 
 // isolated: the ghost cells beyond the boundary (a list built once per mesh)
 // take the expansion at their centres
-__global__ void __launch_bounds__(GT) k_mg_scatter_out(const long long *__restrict__ flat,
-                                                       const int *__restrict__ gidx, int n, Lev L, MP mp,
+__global__ void __launch_bounds__(GT) k_mg_scatter_out(const long long *flat,
+                                                       const int *gidx, int n, Lev L, MP mp,
                                                        double *phi_pad) {
+  pdl_begin();
   for (int e = blockIdx.x * GT + threadIdx.x; e < n; e += gridDim.x * GT) {
     double x[3];
     for (int a = 0; a < 3; ++a) x[a] = L.x0[a] + (gidx[3 * e + a] + 0.5) * L.dx[a];
@@ -798,6 +811,7 @@ __global__ void __launch_bounds__(GT) k_mg_scatter_out(const long long *__restri
 
 // full multigrid: the source of coarse cell (volume average of the children)
 __global__ void __launch_bounds__(GT) k_mg_restrict_src(Lev F, Lev C, double inv) {
+  pdl_begin();
   const int r0 = 1 << F.lr[0], r1 = 1 << F.lr[1], r2 = 1 << F.lr[2];
   const unsigned n = (unsigned)C.n[0] * C.n[1] * C.n[2];
   for (unsigned c = blockIdx.x * GT + threadIdx.x; c < n; c += gridDim.x * GT) {
@@ -853,6 +867,7 @@ __device__ double full_value(const Lev &C, const MP &mp, int u0, int u1, int u2)
 // have few cells, so a CTA is one warp (with one thread per cell a 4^3 level took
 // 1.9 ms)
 __global__ void __launch_bounds__(GT) k_mg_prolong_full(Lev F, Lev C, MP mp) {
+  pdl_begin();
   const unsigned n = (unsigned)F.n[0] * F.n[1] * F.n[2];
   const int lane = threadIdx.x & 31;
   for (unsigned c = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; c < n; c += (gridDim.x * blockDim.x) >> 5) {
@@ -878,6 +893,7 @@ __global__ void __launch_bounds__(GT) k_mg_prolong_full(Lev F, Lev C, MP mp) {
 
 // partial sums per CTA of (S, S x, S y, S z) over level 0 (the centroid)
 __global__ void __launch_bounds__(GT) k_mp_centroid(Lev L, double *part) {
+  pdl_begin();
   __shared__ double red[4][GT / 32];
   const unsigned n = (unsigned)L.n[0] * L.n[1] * L.n[2];
   double s[4] = {0.0, 0.0, 0.0, 0.0};
@@ -905,7 +921,8 @@ __global__ void __launch_bounds__(GT) k_mp_centroid(Lev L, double *part) {
 
 // the centroid from the partial sums (a fixed-order tree over GT threads; the
 // domain centre for a source summing to zero)
-__global__ void __launch_bounds__(GT) k_mp_centre(const double *__restrict__ part, int np, Lev L, double *cc) {
+__global__ void __launch_bounds__(GT) k_mp_centre(const double *part, int np, Lev L, double *cc) {
+  pdl_begin();
   __shared__ double red[4][GT];
   double t[4] = {0.0, 0.0, 0.0, 0.0};
   for (int b = threadIdx.x; b < np; b += GT)
@@ -925,7 +942,8 @@ __global__ void __launch_bounds__(GT) k_mp_centre(const double *__restrict__ par
 
 // partial moments per CTA: sum S dV R_l^m(x - c), 2 MP_NC values
 template <int LM>
-__global__ void __launch_bounds__(GT) k_mp_moments(Lev L, const double *__restrict__ cc, double *part) {
+__global__ void __launch_bounds__(GT) k_mp_moments(Lev L, const double *cc, double *part) {
+  pdl_begin();
   constexpr int NC = (LM + 1) * (LM + 2) / 2;
   __shared__ double red[2 * NC][GT / 32];
   const unsigned n = (unsigned)L.n[0] * L.n[1] * L.n[2];
@@ -962,7 +980,8 @@ __global__ void __launch_bounds__(GT) k_mp_moments(Lev L, const double *__restri
 
 // coefficients (A_lm, B_lm) = (2 - delta_m0) (l-m)! / (l+m)! / (4 pi) x the
 // moments; one CTA per coefficient, a fixed-order tree over the partial sums
-__global__ void __launch_bounds__(GT) k_mp_coef(const double *__restrict__ part, int np, int lmax, double *cc) {
+__global__ void __launch_bounds__(GT) k_mp_coef(const double *part, int np, int lmax, double *cc) {
+  pdl_begin();
   __shared__ double red[GT];
   const int q = blockIdx.x;
   double t = 0.0;
@@ -990,6 +1009,7 @@ struct FaceJob {
   int start[7];   // entries of the faces x-, x+, ..., z+ of this level
 };
 __global__ void __launch_bounds__(GT) k_mp_faces(FaceJob job, MP mp, double *out) {
+  pdl_begin();
   const Lev &L = job.L;
   for (int e = blockIdx.x * GT + threadIdx.x; e < job.start[6]; e += gridDim.x * GT) {
     int f = 0;
@@ -1147,9 +1167,9 @@ static cudaError_t grav_init(tde_mesh *m) {
 static cudaError_t reduce(GravState *g, const Lev &L, int sq, double *out, cudaStream_t s) {
   const long long n = (long long)L.n[0] * L.n[1] * L.n[2];
   const unsigned gr = std::min<unsigned>(grid_for(n), (unsigned)g->npart);
-  if (L.iso) k_mg_partial<1><<<gr, GT, 0, s>>>(L, sq, g->part);
-  else k_mg_partial<0><<<gr, GT, 0, s>>>(L, sq, g->part);
-  k_mg_final<<<1, GT, 0, s>>>(g->part, (int)gr, (double)n, sq, out);
+  if (L.iso) pdl_launch(k_mg_partial<1>, gr, GT, 0, s, L, sq, g->part);
+  else pdl_launch(k_mg_partial<0>, gr, GT, 0, s, L, sq, g->part);
+  pdl_launch(k_mg_final, 1, GT, 0, s, g->part, (int)gr, (double)n, sq, out);
   g->launches += 2;
   return cudaGetLastError();
 }
@@ -1168,8 +1188,8 @@ static void smooth(GravState *g, const Lev &L, double omega, cudaStream_t s) {
   const long long half = (long long)L.n[1] * L.n[2] * ((L.n[0] + 1) / 2);
   const SmoothW W = smooth_weights(L, omega);
   for (int colour = 0; colour < 2; ++colour) {
-    if (L.iso) k_mg_smooth<1><<<grid_for(half), GT, 0, s>>>(L, colour, W, omega);
-    else k_mg_smooth<0><<<grid_for(half), GT, 0, s>>>(L, colour, W, omega);
+    if (L.iso) pdl_launch(k_mg_smooth<1>, grid_for(half), GT, 0, s, L, colour, W, omega);
+    else pdl_launch(k_mg_smooth<0>, grid_for(half), GT, 0, s, L, colour, W, omega);
   }
   g->launches += 2;
 }
@@ -1187,8 +1207,8 @@ static void vcycle(GravState *g, int l, const tde_grav_params &gp, cudaStream_t 
       a.lev[q] = g->lev[l + q];
       a.W[q] = smooth_weights(a.lev[q], gp.omega);
     }
-    if (g->iso) k_mg_coarse<1><<<1, GT, 0, s>>>(a);
-    else k_mg_coarse<0><<<1, GT, 0, s>>>(a);
+    if (g->iso) pdl_launch(k_mg_coarse<1>, 1, GT, 0, s, a);
+    else pdl_launch(k_mg_coarse<0>, 1, GT, 0, s, a);
     g->launches += 1;
     return;
   }
@@ -1197,16 +1217,16 @@ static void vcycle(GravState *g, int l, const tde_grav_params &gp, cudaStream_t 
   const long long nc = (long long)C.n[0] * C.n[1] * C.n[2];
   const double inv = (double)nc / ((double)F.n[0] * F.n[1] * F.n[2]);   // 1 / children per cell
   if (g->iso) {
-    k_mg_restrict<1><<<grid_for(nc), GT, 0, s>>>(F, C, inv);
-    k_mg_fas<1><<<grid_for(nc), GT, 0, s>>>(C);
+    pdl_launch(k_mg_restrict<1>, grid_for(nc), GT, 0, s, F, C, inv);
+    pdl_launch(k_mg_fas<1>, grid_for(nc), GT, 0, s, C);
   } else {
-    k_mg_restrict<0><<<grid_for(nc), GT, 0, s>>>(F, C, inv);
-    k_mg_fas<0><<<grid_for(nc), GT, 0, s>>>(C);
+    pdl_launch(k_mg_restrict<0>, grid_for(nc), GT, 0, s, F, C, inv);
+    pdl_launch(k_mg_fas<0>, grid_for(nc), GT, 0, s, C);
   }
   vcycle(g, l + 1, gp, s);
-  k_mg_corr<<<grid_for(nc), GT, 0, s>>>(C);
+  pdl_launch(k_mg_corr, grid_for(nc), GT, 0, s, C);
   if (const int T = prolong_tile(F, C)) launch_prolong_tiled<0>(F, C, MP{0, nullptr}, T, s);
-  else k_mg_prolong<<<grid_for((long long)F.n[0] * F.n[1] * F.n[2]), GT, 0, s>>>(F, C);
+  else pdl_launch(k_mg_prolong, grid_for((long long)F.n[0] * F.n[1] * F.n[2]), GT, 0, s, F, C);
   g->launches += 4;
   for (int q = 0; q < gp.npost; ++q) smooth(g, F, gp.omega, s);
 }
@@ -1216,25 +1236,25 @@ static void multipole_setup(GravState *g, int lmax, cudaStream_t s) {
   const Lev &L0 = g->lev[0];
   const long long n0 = (long long)L0.n[0] * L0.n[1] * L0.n[2];
   const unsigned gr = std::min<unsigned>(grid_for(n0), (unsigned)g->npart);
-  k_mp_centroid<<<gr, GT, 0, s>>>(L0, g->part);
-  k_mp_centre<<<1, GT, 0, s>>>(g->part, (int)gr, L0, g->mp);
+  pdl_launch(k_mp_centroid, gr, GT, 0, s, L0, g->part);
+  pdl_launch(k_mp_centre, 1, GT, 0, s, g->part, (int)gr, L0, g->mp);
   // (a warp's reduction of the 30 sums costs as much as several cells: few CTAs)
   const unsigned grm = std::min(gr, 304u);
   switch (lmax) {
-    case 0: k_mp_moments<0><<<grm, GT, 0, s>>>(L0, g->mp, g->mpart); break;
-    case 1: k_mp_moments<1><<<grm, GT, 0, s>>>(L0, g->mp, g->mpart); break;
-    case 2: k_mp_moments<2><<<grm, GT, 0, s>>>(L0, g->mp, g->mpart); break;
-    case 3: k_mp_moments<3><<<grm, GT, 0, s>>>(L0, g->mp, g->mpart); break;
-    default: k_mp_moments<4><<<grm, GT, 0, s>>>(L0, g->mp, g->mpart); break;
+    case 0: pdl_launch(k_mp_moments<0>, grm, GT, 0, s, L0, g->mp, g->mpart); break;
+    case 1: pdl_launch(k_mp_moments<1>, grm, GT, 0, s, L0, g->mp, g->mpart); break;
+    case 2: pdl_launch(k_mp_moments<2>, grm, GT, 0, s, L0, g->mp, g->mpart); break;
+    case 3: pdl_launch(k_mp_moments<3>, grm, GT, 0, s, L0, g->mp, g->mpart); break;
+    default: pdl_launch(k_mp_moments<4>, grm, GT, 0, s, L0, g->mp, g->mpart); break;
   }
-  k_mp_coef<<<2 * MP_NC, GT, 0, s>>>(g->mpart, (int)grm, lmax, g->mp);
+  pdl_launch(k_mp_coef, 2 * MP_NC, GT, 0, s, g->mpart, (int)grm, lmax, g->mp);
   const MP mp{lmax, g->mp};
   for (int l = 0; l < g->nl; ++l) {
     FaceJob job;
     job.L = g->lev[l];
     for (int f = 0; f < 7; ++f) job.start[f] = g->face_start[l][f] - g->face_start[l][0];
     if (job.start[6] == 0) continue;
-    k_mp_faces<<<grid_for(job.start[6]), GT, 0, s>>>(job, mp, g->faces + g->face_start[l][0]);
+    pdl_launch(k_mp_faces, grid_for(job.start[6]), GT, 0, s, job, mp, g->faces + g->face_start[l][0]);
     g->launches += 1;
   }
   g->launches += 4;
@@ -1246,7 +1266,7 @@ static void full_multigrid(GravState *g, const tde_grav_params &gp, int lmax, cu
   for (int l = 1; l < g->nl; ++l) {
     const Lev &F = g->lev[l - 1], &C = g->lev[l];
     const long long nc = (long long)C.n[0] * C.n[1] * C.n[2];
-    k_mg_restrict_src<<<grid_for(nc), GT, 0, s>>>(F, C, (double)nc / ((double)F.n[0] * F.n[1] * F.n[2]));
+    pdl_launch(k_mg_restrict_src, grid_for(nc), GT, 0, s, F, C, (double)nc / ((double)F.n[0] * F.n[1] * F.n[2]));
     g->launches += 1;
   }
   cudaMemsetAsync(g->lev[g->nl - 1].phi, 0, sizeof(double), s);
@@ -1257,7 +1277,7 @@ static void full_multigrid(GravState *g, const tde_grav_params &gp, int lmax, cu
     if (const int T = prolong_tile(F, g->lev[l + 1]))
       launch_prolong_tiled<1>(F, g->lev[l + 1], mp, T, s);
     else
-      k_mg_prolong_full<<<(unsigned)std::min<long long>((long long)F.n[0] * F.n[1] * F.n[2], 152LL * 32), 32, 0, s>>>(F, g->lev[l + 1], mp);
+      pdl_launch(k_mg_prolong_full, (unsigned)std::min<long long>((long long)F.n[0] * F.n[1] * F.n[2], 152LL * 32), 32, 0, s, F, g->lev[l + 1], mp);
     g->launches += 1;
     vcycle(g, l, gp, s);
     if (l == 0) smooth(g, F, gp.omega, s);
@@ -1277,14 +1297,14 @@ cudaError_t gravity_solve(tde_mesh *m, const tde_grav_params &gp, int *cycles, d
   {
     ProfScope ps(c, TDE_K_GRAV, false);
     dim3 grid((unsigned)std::min<int64_t>((m->max_interior + GT - 1) / GT, 64), (unsigned)m->nb);
-    k_mg_gather<<<grid, GT, 0, s>>>(m->phys, m->d_blocks, m->U, L0, 4.0 * M_PI * gp.G, gp.rho_min);
+    pdl_launch(k_mg_gather, grid, GT, 0, s, m->phys, m->d_blocks, m->U, L0, 4.0 * M_PI * gp.G, gp.rho_min);
     if (!gp.warm || gp.fmg) cudaMemsetAsync(L0.phi, 0, sizeof(double) * n0, s);
     if (iso) {
       multipole_setup(g, gp.lmax, s);
     } else {
       for (int pass = 0; pass < 2; ++pass) {   // the source's mean, removed in two passes
         reduce(g, L0, 0, g->scal, s);
-        k_mg_sub_mean<<<grid_for(n0), GT, 0, s>>>(L0, g->scal);
+        pdl_launch(k_mg_sub_mean, grid_for(n0), GT, 0, s, L0, g->scal);
       }
       g->launches += 2;
     }
@@ -1376,9 +1396,9 @@ cudaError_t gravity_solve(tde_mesh *m, const tde_grav_params &gp, int *cycles, d
     ProfScope ps(c, TDE_K_GRAV, false);
     dim3 grid((unsigned)std::min<int64_t>((m->max_interior + GT - 1) / GT, 64), (unsigned)m->nb);
     const MP mp{gp.lmax, g->mp};
-    k_mg_scatter<<<grid, GT, 0, s>>>(m->phys, m->d_blocks, L0, mp, m->d_phi_sg);
+    pdl_launch(k_mg_scatter, grid, GT, 0, s, m->phys, m->d_blocks, L0, mp, m->d_phi_sg);
     if (iso && g->nout > 0) {
-      k_mg_scatter_out<<<grid_for(g->nout), GT, 0, s>>>(g->out_flat, g->out_g, g->nout, L0, mp, m->d_phi_sg);
+      pdl_launch(k_mg_scatter_out, grid_for(g->nout), GT, 0, s, g->out_flat, g->out_g, g->nout, L0, mp, m->d_phi_sg);
       g->launches += 1;
     }
   }

@@ -103,11 +103,12 @@ __device__ __forceinline__ void cta_bh_info(const BH &bh, double t, double dx, c
 // FP64 instructions of single warps -- is shared by 1024 cells).
 template <int EOSK, int DUAL, int EOSB = 0>
 __global__ void __launch_bounds__(NT) k_c2p(Phys p, BH bh, TimeArgs ta,
-                                            const DevBlock *__restrict__ blocks,
-                                            const int32_t *__restrict__ ids,
-                                            const double *__restrict__ U, double *__restrict__ W,
+                                            const DevBlock *blocks,
+                                            const int32_t *ids,
+                                            const double *U, double *W,
                                             long long ntot, Counters *cnt, int want_dt,
                                             unsigned long long *dtbits, EOSBuf eb) {
+  pdl_begin();
   const int b = ids[blockIdx.y];
   const DevBlock B = blocks[b];
   const int nint = B.n[0] * B.n[1] * B.n[2];
@@ -192,11 +193,12 @@ __global__ void __launch_bounds__(NT) k_c2p(Phys p, BH bh, TimeArgs ta,
 // advances, so the ghost layer cannot be copied from freshly converted
 // neighbours); events are counted on interior cells only
 template <int EOSK, int DUAL, int EOSB = 0>
-__global__ void __launch_bounds__(NT) k_c2p_padded(Phys p, const DevBlock *__restrict__ blocks,
-                                                   const int32_t *__restrict__ ids,
-                                                   const double *__restrict__ U,
-                                                   double *__restrict__ W, long long ntot,
+__global__ void __launch_bounds__(NT) k_c2p_padded(Phys p, const DevBlock *blocks,
+                                                   const int32_t *ids,
+                                                   const double *U,
+                                                   double *W, long long ntot,
                                                    Counters *cnt, EOSBuf eb) {
+  pdl_begin();
   const int b = ids[blockIdx.y];
   const DevBlock B = blocks[b];
   const int npad = B.p[0] * B.p[1] * B.p[2];
@@ -219,9 +221,10 @@ __global__ void __launch_bounds__(NT) k_c2p_padded(Phys p, const DevBlock *__res
 // primitives of listed cells (LAT ghost cells whose conserved values were
 // interpolated in time, restricted or prolonged; nothing counted: ghost cells)
 template <int EOSK, int DUAL, int EOSB = 0>
-__global__ void __launch_bounds__(NT) k_c2p_list(Phys p, const int32_t *__restrict__ list, int n,
-                                                 const double *__restrict__ U, double *__restrict__ W,
+__global__ void __launch_bounds__(NT) k_c2p_list(Phys p, const int32_t *list, int n,
+                                                 const double *U, double *W,
                                                  long long ntot, EOSBuf eb) {
+  pdl_begin();
   for (int e = blockIdx.x * NT + threadIdx.x; e < n; e += gridDim.x * NT) {
     const long long flat = list[e];
     double u[6], w[8];
@@ -239,10 +242,11 @@ __global__ void __launch_bounds__(NT) k_c2p_list(Phys p, const int32_t *__restri
 // closure inside k_c2p, for the learned-guess inversion's launches; nothing is
 // counted here (k_c2p counts when it takes the results).
 template <int DUAL, int PADDED>
-__global__ void __launch_bounds__(NT) k_c2p_eosin(Phys p, const DevBlock *__restrict__ blocks,
-                                                  const int32_t *__restrict__ ids,
-                                                  const double *__restrict__ U, double *rho_in,
+__global__ void __launch_bounds__(NT) k_c2p_eosin(Phys p, const DevBlock *blocks,
+                                                  const int32_t *ids,
+                                                  const double *U, double *rho_in,
                                                   double *e_in, long long ntot) {
+  pdl_begin();
   const int b = ids[blockIdx.y];
   const DevBlock B = blocks[b];
   const int n = PADDED ? B.p[0] * B.p[1] * B.p[2] : B.n[0] * B.n[1] * B.n[2];
@@ -269,9 +273,10 @@ __global__ void __launch_bounds__(NT) k_c2p_eosin(Phys p, const DevBlock *__rest
 
 // table inputs of listed cells (the learned-guess closure over a cell list)
 template <int DUAL>
-__global__ void __launch_bounds__(NT) k_c2p_eosin_list(Phys p, const int32_t *__restrict__ list, int n,
-                                                       const double *__restrict__ U, double *rho_in,
+__global__ void __launch_bounds__(NT) k_c2p_eosin_list(Phys p, const int32_t *list, int n,
+                                                       const double *U, double *rho_in,
                                                        double *e_in, long long ntot) {
+  pdl_begin();
   for (int e = blockIdx.x * NT + threadIdx.x; e < n; e += gridDim.x * NT) {
     const long long flat = list[e];
     double u[6];
@@ -291,6 +296,7 @@ __global__ void __launch_bounds__(1024) k_dt_finalize(int nb, double cfl,
                                                       unsigned long long *dtbits,
                                                       double *dt_block, double *dt_min,
                                                       double *scal) {
+  pdl_begin();
   __shared__ double red[32];
   double m = INFINITY;
   for (int b = threadIdx.x; b < nb; b += blockDim.x) {
@@ -320,11 +326,12 @@ __global__ void __launch_bounds__(1024) k_dt_finalize(int nb, double cfl,
 // is stored (the sources are interior cells, the destinations ghost cells, so
 // they never overlap), which lets the loads of a cell overlap in flight
 constexpr int GHOST_NF_MAX = 8;
-__global__ void __launch_bounds__(NT) k_ghost(const int32_t *__restrict__ map,
-                                              const int32_t *__restrict__ gstart,
-                                              const int32_t *__restrict__ gend,
-                                              const int32_t *__restrict__ ids, double *f, int nf,
+__global__ void __launch_bounds__(NT) k_ghost(const int32_t *map,
+                                              const int32_t *gstart,
+                                              const int32_t *gend,
+                                              const int32_t *ids, double *f, int nf,
                                               long long ntot) {
+  pdl_begin();
   const int b = ids[blockIdx.y];
   const int s0 = gstart[b], s1 = gend ? gend[b] : gstart[b + 1];
   for (int e = s0 + blockIdx.x * NT + threadIdx.x; e < s1; e += gridDim.x * NT) {
@@ -348,9 +355,10 @@ __global__ void __launch_bounds__(NT) k_ghost(const int32_t *__restrict__ map,
 // skipped, so the per-cell test (which decides as before) runs only near the
 // point mass.
 __global__ void __launch_bounds__(NT) k_excise(Phys p, BH bh, TimeArgs ta,
-                                               const DevBlock *__restrict__ blocks,
-                                               const int32_t *__restrict__ ids, double *U,
+                                               const DevBlock *blocks,
+                                               const int32_t *ids, double *U,
                                                long long ntot, Counters *cnt) {
+  pdl_begin();
   __shared__ int s_far;
   __shared__ double s_rb[3];
   const int b = ids[blockIdx.y];
@@ -389,9 +397,10 @@ __global__ void __launch_bounds__(NT) k_excise(Phys p, BH bh, TimeArgs ta,
   }
 }
 
-__global__ void __launch_bounds__(NT) k_sync(Phys p, const DevBlock *__restrict__ blocks,
-                                             const int32_t *__restrict__ ids, double *U,
+__global__ void __launch_bounds__(NT) k_sync(Phys p, const DevBlock *blocks,
+                                             const int32_t *ids, double *U,
                                              long long ntot, double eta2, Counters *cnt) {
+  pdl_begin();
   const int b = ids[blockIdx.y];
   const DevBlock B = blocks[b];
   const int nint = B.n[0] * B.n[1] * B.n[2];
@@ -473,14 +482,17 @@ __global__ void __launch_bounds__(NT) k_prim2cons(Phys p, const DevBlock *__rest
 
 // ------------------------------------------------------------- scalars ----
 
-__global__ void k_advance_time(double *scal) { scal[0] += scal[1]; }
-__global__ void k_set_dt(double *scal, double dt) { scal[1] = dt; scal[2] = dt; }
+__global__ void k_advance_time(double *scal) {
+  pdl_begin(); scal[0] += scal[1]; }
+__global__ void k_set_dt(double *scal, double dt) {
+  pdl_begin(); scal[1] = dt; scal[2] = dt; }
 
 // ---------------------------------------------------------- EOS batch ----
 
-__global__ void __launch_bounds__(NT) k_eos_invert(DTable t, long long n, const double *__restrict__ rho,
-                                                   const double *__restrict__ en, double *T,
+__global__ void __launch_bounds__(NT) k_eos_invert(DTable t, long long n, const double *rho,
+                                                   const double *en, double *T,
                                                    double *P, double *cs2, Counters *cnt) {
+  pdl_begin();
   for (long long e = blockIdx.x * (long long)NT + threadIdx.x; e < n; e += (long long)gridDim.x * NT) {
     double Pv, cv, eu, Tv;
     bool cl = eos_invert(t, rho[e], en[e], Pv, cv, eu, &Tv);
@@ -631,11 +643,11 @@ static cudaError_t surrogate_table_pass(tde_mesh *m, const double *Uin, int nblk
   if (!m->sb.rho || !m->eos || !m->eos->has_net) return cudaErrorInvalidValue;
   const long long nt = (long long)m->ntot;
   if (padded) {
-    if (p.dual) k_c2p_eosin<1, 1><<<grid, NT, 0, s>>>(p, m->d_blocks, ids, Uin, m->sb.rho, m->sb.e, nt);
-    else k_c2p_eosin<0, 1><<<grid, NT, 0, s>>>(p, m->d_blocks, ids, Uin, m->sb.rho, m->sb.e, nt);
+    if (p.dual) pdl_launch(k_c2p_eosin<1, 1>, grid, NT, 0, s, p, m->d_blocks, ids, Uin, m->sb.rho, m->sb.e, nt);
+    else pdl_launch(k_c2p_eosin<0, 1>, grid, NT, 0, s, p, m->d_blocks, ids, Uin, m->sb.rho, m->sb.e, nt);
   } else {
-    if (p.dual) k_c2p_eosin<1, 0><<<grid, NT, 0, s>>>(p, m->d_blocks, ids, Uin, m->sb.rho, m->sb.e, nt);
-    else k_c2p_eosin<0, 0><<<grid, NT, 0, s>>>(p, m->d_blocks, ids, Uin, m->sb.rho, m->sb.e, nt);
+    if (p.dual) pdl_launch(k_c2p_eosin<1, 0>, grid, NT, 0, s, p, m->d_blocks, ids, Uin, m->sb.rho, m->sb.e, nt);
+    else pdl_launch(k_c2p_eosin<0, 0>, grid, NT, 0, s, p, m->d_blocks, ids, Uin, m->sb.rho, m->sb.e, nt);
   }
   cudaError_t err = cudaGetLastError();
   if (err != cudaSuccess) return err;
@@ -665,14 +677,14 @@ cudaError_t launch_c2p(tde_mesh *m, const double *Uin, int nblk, const int32_t *
 #define C2P_ARGS p, bh, ta, m->d_blocks, ids, Uin, m->d_W, (long long)m->ntot, m->d_cnt, \
                  (int)want_dt, m->d_dtbits, eb
   if (p.eos == EOS_IDEAL) {
-    if (p.dual) k_c2p<EOS_IDEAL, 1><<<grid, NT, 0, m->ctx->stream>>>(C2P_ARGS);
-    else k_c2p<EOS_IDEAL, 0><<<grid, NT, 0, m->ctx->stream>>>(C2P_ARGS);
+    if (p.dual) pdl_launch(k_c2p<EOS_IDEAL, 1>, grid, NT, 0, m->ctx->stream, C2P_ARGS);
+    else pdl_launch(k_c2p<EOS_IDEAL, 0>, grid, NT, 0, m->ctx->stream, C2P_ARGS);
   } else if (surrogate_closure(m)) {
-    if (p.dual) k_c2p<EOS_TABLE, 1, 1><<<grid, NT, 0, m->ctx->stream>>>(C2P_ARGS);
-    else k_c2p<EOS_TABLE, 0, 1><<<grid, NT, 0, m->ctx->stream>>>(C2P_ARGS);
+    if (p.dual) pdl_launch(k_c2p<EOS_TABLE, 1, 1>, grid, NT, 0, m->ctx->stream, C2P_ARGS);
+    else pdl_launch(k_c2p<EOS_TABLE, 0, 1>, grid, NT, 0, m->ctx->stream, C2P_ARGS);
   } else {
-    if (p.dual) k_c2p<EOS_TABLE, 1><<<grid, NT, 0, m->ctx->stream>>>(C2P_ARGS);
-    else k_c2p<EOS_TABLE, 0><<<grid, NT, 0, m->ctx->stream>>>(C2P_ARGS);
+    if (p.dual) pdl_launch(k_c2p<EOS_TABLE, 1>, grid, NT, 0, m->ctx->stream, C2P_ARGS);
+    else pdl_launch(k_c2p<EOS_TABLE, 0>, grid, NT, 0, m->ctx->stream, C2P_ARGS);
   }
 #undef C2P_ARGS
   return cudaGetLastError();
@@ -691,14 +703,14 @@ cudaError_t launch_c2p_padded(tde_mesh *m, const double *Uin, int nblk, const in
   }
 #define C2PP_ARGS p, m->d_blocks, ids, Uin, m->d_W, (long long)m->ntot, m->d_cnt, eb
   if (p.eos == EOS_IDEAL) {
-    if (p.dual) k_c2p_padded<EOS_IDEAL, 1><<<grid, NT, 0, m->ctx->stream>>>(C2PP_ARGS);
-    else k_c2p_padded<EOS_IDEAL, 0><<<grid, NT, 0, m->ctx->stream>>>(C2PP_ARGS);
+    if (p.dual) pdl_launch(k_c2p_padded<EOS_IDEAL, 1>, grid, NT, 0, m->ctx->stream, C2PP_ARGS);
+    else pdl_launch(k_c2p_padded<EOS_IDEAL, 0>, grid, NT, 0, m->ctx->stream, C2PP_ARGS);
   } else if (surrogate_closure(m)) {
-    if (p.dual) k_c2p_padded<EOS_TABLE, 1, 1><<<grid, NT, 0, m->ctx->stream>>>(C2PP_ARGS);
-    else k_c2p_padded<EOS_TABLE, 0, 1><<<grid, NT, 0, m->ctx->stream>>>(C2PP_ARGS);
+    if (p.dual) pdl_launch(k_c2p_padded<EOS_TABLE, 1, 1>, grid, NT, 0, m->ctx->stream, C2PP_ARGS);
+    else pdl_launch(k_c2p_padded<EOS_TABLE, 0, 1>, grid, NT, 0, m->ctx->stream, C2PP_ARGS);
   } else {
-    if (p.dual) k_c2p_padded<EOS_TABLE, 1><<<grid, NT, 0, m->ctx->stream>>>(C2PP_ARGS);
-    else k_c2p_padded<EOS_TABLE, 0><<<grid, NT, 0, m->ctx->stream>>>(C2PP_ARGS);
+    if (p.dual) pdl_launch(k_c2p_padded<EOS_TABLE, 1>, grid, NT, 0, m->ctx->stream, C2PP_ARGS);
+    else pdl_launch(k_c2p_padded<EOS_TABLE, 0>, grid, NT, 0, m->ctx->stream, C2PP_ARGS);
   }
 #undef C2PP_ARGS
   return cudaGetLastError();
@@ -713,8 +725,8 @@ cudaError_t launch_c2p_list(tde_mesh *m, const double *Uin, const int32_t *list,
   EOSBuf eb{m->sb.P, m->sb.cs2, m->sb.eu};
   if (surrogate_closure(m)) {
     if (!m->sb.rho || !m->eos || !m->eos->has_net) return cudaErrorInvalidValue;
-    if (p.dual) k_c2p_eosin_list<1><<<grid, NT, 0, s>>>(p, list, n, Uin, m->sb.rho, m->sb.e, (long long)m->ntot);
-    else k_c2p_eosin_list<0><<<grid, NT, 0, s>>>(p, list, n, Uin, m->sb.rho, m->sb.e, (long long)m->ntot);
+    if (p.dual) pdl_launch(k_c2p_eosin_list<1>, grid, NT, 0, s, p, list, n, Uin, m->sb.rho, m->sb.e, (long long)m->ntot);
+    else pdl_launch(k_c2p_eosin_list<0>, grid, NT, 0, s, p, list, n, Uin, m->sb.rho, m->sb.e, (long long)m->ntot);
     cudaError_t err = cudaGetLastError();
     if (err != cudaSuccess) return err;
     m->ctx->launches[TDE_K_C2P] += 3;   // table inputs, guess + Newton, bisection of the misses
@@ -726,14 +738,14 @@ cudaError_t launch_c2p_list(tde_mesh *m, const double *Uin, const int32_t *list,
   }
 #define C2PL_ARGS p, list, n, Uin, m->d_W, (long long)m->ntot, eb
   if (p.eos == EOS_IDEAL) {
-    if (p.dual) k_c2p_list<EOS_IDEAL, 1><<<grid, NT, 0, s>>>(C2PL_ARGS);
-    else k_c2p_list<EOS_IDEAL, 0><<<grid, NT, 0, s>>>(C2PL_ARGS);
+    if (p.dual) pdl_launch(k_c2p_list<EOS_IDEAL, 1>, grid, NT, 0, s, C2PL_ARGS);
+    else pdl_launch(k_c2p_list<EOS_IDEAL, 0>, grid, NT, 0, s, C2PL_ARGS);
   } else if (surrogate_closure(m)) {
-    if (p.dual) k_c2p_list<EOS_TABLE, 1, 1><<<grid, NT, 0, s>>>(C2PL_ARGS);
-    else k_c2p_list<EOS_TABLE, 0, 1><<<grid, NT, 0, s>>>(C2PL_ARGS);
+    if (p.dual) pdl_launch(k_c2p_list<EOS_TABLE, 1, 1>, grid, NT, 0, s, C2PL_ARGS);
+    else pdl_launch(k_c2p_list<EOS_TABLE, 0, 1>, grid, NT, 0, s, C2PL_ARGS);
   } else {
-    if (p.dual) k_c2p_list<EOS_TABLE, 1><<<grid, NT, 0, s>>>(C2PL_ARGS);
-    else k_c2p_list<EOS_TABLE, 0><<<grid, NT, 0, s>>>(C2PL_ARGS);
+    if (p.dual) pdl_launch(k_c2p_list<EOS_TABLE, 1>, grid, NT, 0, s, C2PL_ARGS);
+    else pdl_launch(k_c2p_list<EOS_TABLE, 0>, grid, NT, 0, s, C2PL_ARGS);
   }
 #undef C2PL_ARGS
   return cudaGetLastError();
@@ -741,7 +753,7 @@ cudaError_t launch_c2p_list(tde_mesh *m, const double *Uin, const int32_t *list,
 
 cudaError_t launch_dt_finalize(tde_mesh *m, double cfl, double *dt_block, double *dt_min) {
   ProfScope _ps(m->ctx, TDE_K_DT);
-  k_dt_finalize<<<1, 1024, 0, m->ctx->stream>>>(m->nb, cfl, m->d_dtbits, dt_block, dt_min,
+  pdl_launch(k_dt_finalize, 1, 1024, 0, m->ctx->stream, m->nb, cfl, m->d_dtbits, dt_block, dt_min,
                                                 m->d_scal);
   return cudaGetLastError();
 }
@@ -751,7 +763,7 @@ cudaError_t launch_ghost(tde_mesh *m, double *field, int nf, int nblk, const int
   if (nf < 1 || nf > GHOST_NF_MAX) return cudaErrorInvalidValue;
   ProfScope _ps(m->ctx, TDE_K_GHOST);
   unsigned gx = (unsigned)min((m->max_ghosts + NT - 1) / NT, 64);
-  k_ghost<<<dim3(gx, (unsigned)nblk), NT, 0, m->ctx->stream>>>(m->d_ghost, m->d_gstart,
+  pdl_launch(k_ghost, dim3(gx, (unsigned)nblk), NT, 0, m->ctx->stream, m->d_ghost, m->d_gstart,
                                                                  sweep_only ? m->d_gend : nullptr, ids, field,
                                                                  nf, (long long)m->ntot);
   return cudaGetLastError();
@@ -1010,7 +1022,7 @@ cudaError_t launch_excise(tde_mesh *m, double *U, int nblk, const int32_t *ids, 
                           TimeArgs ta) {
   ProfScope _ps(m->ctx, TDE_K_EXCISE);
   dim3 grid((unsigned)std::min<int64_t>((m->max_interior + NT - 1) / NT, 8), (unsigned)nblk);
-  k_excise<<<grid, NT, 0, m->ctx->stream>>>(m->phys, bh, ta, m->d_blocks, ids, U,
+  pdl_launch(k_excise, grid, NT, 0, m->ctx->stream, m->phys, bh, ta, m->d_blocks, ids, U,
                                              (long long)m->ntot, m->d_cnt);
   return cudaGetLastError();
 }
@@ -1022,7 +1034,7 @@ cudaError_t launch_sync(tde_mesh *m, double *U, int nblk, const int32_t *ids, do
   if (err != cudaSuccess) return err;
   dim3 grid((unsigned)((m->max_interior + NT - 1) / NT), (unsigned)nblk);
   ProfScope _ps(m->ctx, TDE_K_SYNC);
-  k_sync<<<grid, NT, 0, m->ctx->stream>>>(m->phys, m->d_blocks, ids, U, (long long)m->ntot, eta2,
+  pdl_launch(k_sync, grid, NT, 0, m->ctx->stream, m->phys, m->d_blocks, ids, U, (long long)m->ntot, eta2,
                                            m->d_cnt);
   return cudaGetLastError();
 }
@@ -1036,13 +1048,13 @@ cudaError_t launch_prim2cons(tde_mesh *m, const double *W, double *U) {
 
 cudaError_t launch_advance_time(tde_mesh *m) {
   ProfScope _ps(m->ctx, TDE_K_SCALAR);
-  k_advance_time<<<1, 1, 0, m->ctx->stream>>>(m->d_scal);
+  pdl_launch(k_advance_time, 1, 1, 0, m->ctx->stream, m->d_scal);
   return cudaGetLastError();
 }
 
 cudaError_t launch_set_dt(tde_mesh *m, double dt) {
   ProfScope _ps(m->ctx, TDE_K_SCALAR);
-  k_set_dt<<<1, 1, 0, m->ctx->stream>>>(m->d_scal, dt);
+  pdl_launch(k_set_dt, 1, 1, 0, m->ctx->stream, m->d_scal, dt);
   return cudaGetLastError();
 }
 
@@ -1054,7 +1066,7 @@ cudaError_t launch_eos_invert(tde_eos *e, int64_t n, const double *rho, const do
   unsigned g = (unsigned)(blocks < 8LL * n_sm() ? blocks : 8LL * n_sm());
   DTable t = e->tab;
   if (plain) t.n32 = nullptr;   // no 32-bit guide: every bisection step in 64 bits
-  k_eos_invert<<<g, NT, 0, s>>>(t, (long long)n, rho, en, T, P, cs2, e->d_cnt);
+  pdl_launch(k_eos_invert, g, NT, 0, s, t, (long long)n, rho, en, T, P, cs2, e->d_cnt);
   return cudaGetLastError();
 }
 

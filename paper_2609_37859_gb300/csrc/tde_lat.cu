@@ -132,46 +132,51 @@ __global__ void __launch_bounds__(1024) k_lat_factors(int nb, const double *__re
 }
 
 // dt_b = f_b dt0 for the window
-__global__ void k_lat_prepare(int nb, const int32_t *__restrict__ f, double *dtb,
-                              const double *__restrict__ scal) {
+__global__ void k_lat_prepare(int nb, const int32_t *f, double *dtb,
+                              const double *scal) {
+  pdl_begin();
   for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < nb; b += gridDim.x * blockDim.x)
     dtb[b] = f[b] * scal[3];
 }
 
 // step start time of the listed blocks: t_window + tau dt0
-__global__ void k_lat_time(const int32_t *__restrict__ ids, int n, int tau, double *tstart,
-                           const double *__restrict__ scal) {
+__global__ void k_lat_time(const int32_t *ids, int n, int tau, double *tstart,
+                           const double *scal) {
+  pdl_begin();
   for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < n; q += gridDim.x * blockDim.x)
     tstart[ids[q]] = scal[0] + tau * scal[3];
 }
 
 // window end: t += f_max dt0
 __global__ void k_lat_advance(double *scal, int fmax) {
+  pdl_begin();
   scal[1] = fmax * scal[3];
   scal[0] += scal[1];
 }
 
 // copy the listed blocks (all padded cells, all fields) src -> dst
-__global__ void __launch_bounds__(LNT) k_copy_blocks(const DevBlock *__restrict__ blocks,
-                                                     const int32_t *__restrict__ ids,
-                                                     const double *__restrict__ src, double *dst,
+__global__ void __launch_bounds__(LNT) k_copy_blocks(const DevBlock *blocks,
+                                                     const int32_t *ids,
+                                                     const double *src, double *dst,
                                                      int nvar, long long ntot) {
+  pdl_begin();
   const DevBlock B = blocks[ids[blockIdx.y]];
   const long long n = (long long)B.p[0] * B.p[1] * B.p[2];
   for (long long e = blockIdx.x * (long long)LNT + threadIdx.x; e < n; e += (long long)gridDim.x * LNT)
     for (int v = 0; v < nvar; ++v) dst[v * ntot + B.off + e] = src[v * ntot + B.off + e];
 }
 
-__global__ void __launch_bounds__(LNT) k_ghost_lat(const int32_t *__restrict__ map,
-                                                   const int32_t *__restrict__ gstart,
-                                                   const int32_t *__restrict__ gend,
-                                                   const int32_t *__restrict__ gsrcb,
-                                                   const int32_t *__restrict__ ids,
-                                                   const int32_t *__restrict__ f, int flevel,
+__global__ void __launch_bounds__(LNT) k_ghost_lat(const int32_t *map,
+                                                   const int32_t *gstart,
+                                                   const int32_t *gend,
+                                                   const int32_t *gsrcb,
+                                                   const int32_t *ids,
+                                                   const int32_t *f, int flevel,
                                                    int tau, int stage, double *Udst,
-                                                   const double *__restrict__ Ucur,
-                                                   const double *__restrict__ Uold, int nvar,
+                                                   const double *Ucur,
+                                                   const double *Uold, int nvar,
                                                    long long ntot) {
+  pdl_begin();
   const int b = ids[blockIdx.y];
   const int s0 = gstart[b], s1 = gend[b];   // the ghost cells the sweeps read
   for (int e = s0 + blockIdx.x * LNT + threadIdx.x; e < s1; e += gridDim.x * LNT) {
@@ -260,9 +265,10 @@ __device__ __forceinline__ double minmod(double a, double b) {
   return fabs(a) < fabs(b) ? a : b;
 }
 
-__global__ void __launch_bounds__(LNT) k_ghost_amr(const AmrOp *__restrict__ ops, const int32_t *__restrict__ start,
-                                                   const int32_t *__restrict__ ids, const DevBlock *__restrict__ blocks,
+__global__ void __launch_bounds__(LNT) k_ghost_amr(const AmrOp *ops, const int32_t *start,
+                                                   const int32_t *ids, const DevBlock *blocks,
                                                    Phys p, AmrSrc S, double *Udst, int nvar) {
+  pdl_begin();
   const int b = ids[blockIdx.y];
   const int s0 = start[b], s1 = start[b + 1];
   for (int e = s0 + blockIdx.x * LNT + threadIdx.x; e < s1; e += gridDim.x * LNT) {
@@ -287,13 +293,14 @@ __global__ void __launch_bounds__(LNT) k_ghost_amr(const AmrOp *__restrict__ ops
 // source interior cell, converted in the same launch sequence (the conversion
 // is a function of the cell's conserved values alone, so the copy equals the
 // conversion of the copied conserved values bit for bit)
-__global__ void __launch_bounds__(LNT) k_ghost_w_lat(const int32_t *__restrict__ map,
-                                                     const int32_t *__restrict__ gstart,
-                                                     const int32_t *__restrict__ gend,
-                                                     const int32_t *__restrict__ gsrcb,
-                                                     const int32_t *__restrict__ ids,
-                                                     const int32_t *__restrict__ f, int flevel, double *W,
+__global__ void __launch_bounds__(LNT) k_ghost_w_lat(const int32_t *map,
+                                                     const int32_t *gstart,
+                                                     const int32_t *gend,
+                                                     const int32_t *gsrcb,
+                                                     const int32_t *ids,
+                                                     const int32_t *f, int flevel, double *W,
                                                      int nwv, long long ntot) {
+  pdl_begin();
   const int b = ids[blockIdx.y];
   const int s0 = gstart[b], s1 = gend[b];
   for (int e = s0 + blockIdx.x * LNT + threadIdx.x; e < s1; e += gridDim.x * LNT) {
@@ -349,12 +356,13 @@ __device__ __forceinline__ int owner_at(const OwnerLattice &ol, const Phys &p, i
 }
 
 __global__ void __launch_bounds__(LNT) k_reflux(Phys p, BH bh, OwnerLattice ol,
-                                                const DevBlock *__restrict__ blocks,
-                                                const int32_t *__restrict__ ids,
-                                                const int32_t *__restrict__ f, double *U,
+                                                const DevBlock *blocks,
+                                                const int32_t *ids,
+                                                const int32_t *f, double *U,
                                                 long long ntot, double *R,
-                                                const long long *__restrict__ fo, int nvar,
-                                                const double *__restrict__ scal, int tau, const double *__restrict__ phi_sg) {
+                                                const long long *fo, int nvar,
+                                                const double *scal, int tau, const double *phi_sg) {
+  pdl_begin();
   const int b = ids[blockIdx.x];
   const DevBlock B = blocks[b];
   const int fb = f[b];
@@ -469,7 +477,7 @@ cudaError_t launch_ghost_amr(tde_mesh *m, double *Udst, const double *Ucur, cons
   ProfScope ps(m->ctx, TDE_K_GHOST);
   const AmrSrc S{Udst, Ucur, Uold, f, flevel, tau, stage, (long long)m->ntot};
   const unsigned gx = (unsigned)std::max(1, std::min((m->max_amr + LNT - 1) / LNT, 64));
-  k_ghost_amr<<<dim3(gx, (unsigned)nblk), LNT, 0, m->ctx->stream>>>(m->d_amr, m->d_amr_start, ids, m->d_blocks,
+  pdl_launch(k_ghost_amr, dim3(gx, (unsigned)nblk), LNT, 0, m->ctx->stream, m->d_amr, m->d_amr_start, ids, m->d_blocks,
                                                                    m->phys, S, Udst, nvar);
   return cudaGetLastError();
 }
@@ -716,7 +724,7 @@ int lat_enqueue_window(tde_mesh *m, const BH &bh) {
   cudaStream_t s = c->stream;
   {
     ProfScope ps(c, TDE_K_SCALAR);
-    k_lat_prepare<<<(nb + 255) / 256, 256, 0, s>>>(nb, m->d_f, m->d_dtb, m->d_scal);
+    pdl_launch(k_lat_prepare, (nb + 255) / 256, 256, 0, s, nb, m->d_f, m->d_dtb, m->d_scal);
   }
   LCK(c, cudaMemsetAsync(m->d_freg, 0, sizeof(double) * m->freg_size, s));
   TimeArgs ta{m->d_dtb, 1, m->d_tstart, 1};
@@ -734,7 +742,7 @@ int lat_enqueue_window(tde_mesh *m, const BH &bh) {
       if (ncomp > 0) {
         {
           ProfScope ps(c, TDE_K_SCALAR);
-          k_reflux<<<ncomp, LNT, 0, s>>>(p, bh, ol, m->d_blocks, m->d_sorted, m->d_f, m->U, (long long)m->ntot,
+          pdl_launch(k_reflux, ncomp, LNT, 0, s, p, bh, ol, m->d_blocks, m->d_sorted, m->d_f, m->U, (long long)m->ntot,
                                          m->d_freg, m->d_fo, nvar, m->d_scal, tau,
                                          m->grav_on ? m->d_phi_sg : nullptr);
         }
@@ -757,15 +765,15 @@ int lat_enqueue_window(tde_mesh *m, const BH &bh) {
       }
       {
         ProfScope ps(c, TDE_K_SCALAR);
-        k_copy_blocks<<<dim3(gx_copy, n), LNT, 0, s>>>(m->d_blocks, ids, m->U, m->d_Uold, nvar,
+        pdl_launch(k_copy_blocks, dim3(gx_copy, n), LNT, 0, s, m->d_blocks, ids, m->U, m->d_Uold, nvar,
                                                        (long long)m->ntot);
-        k_lat_time<<<(n + 255) / 256, 256, 0, s>>>(ids, n, tau, m->d_tstart, m->d_scal);
+        pdl_launch(k_lat_time, (n + 255) / 256, 256, 0, s, ids, n, tau, m->d_tstart, m->d_scal);
       }
       for (int stage = 0; stage < 2; ++stage) {
         double *Udst = stage ? m->U1 : m->U;
         {
           ProfScope ps(c, TDE_K_GHOST);
-          k_ghost_lat<<<dim3(gx_ghost, n), LNT, 0, s>>>(m->d_ghost, m->d_gstart, m->d_gend, m->d_gsrcb, ids, m->d_f, f, tau,
+          pdl_launch(k_ghost_lat, dim3(gx_ghost, n), LNT, 0, s, m->d_ghost, m->d_gstart, m->d_gend, m->d_gsrcb, ids, m->d_f, f, tau,
                                                         stage, Udst, m->U, m->d_Uold, nvar, (long long)m->ntot);
         }
         LCK(c, cudaGetLastError());
@@ -776,7 +784,7 @@ int lat_enqueue_window(tde_mesh *m, const BH &bh) {
                                m->h_lat_glist_off[L + 1] - m->h_lat_glist_off[L]));
         {
           ProfScope ps(c, TDE_K_GHOST);
-          k_ghost_w_lat<<<dim3(gx_ghost, n), LNT, 0, s>>>(m->d_ghost, m->d_gstart, m->d_gend, m->d_gsrcb, ids, m->d_f, f,
+          pdl_launch(k_ghost_w_lat, dim3(gx_ghost, n), LNT, 0, s, m->d_ghost, m->d_gstart, m->d_gend, m->d_gsrcb, ids, m->d_f, f,
                                                           m->d_W, p.nwv, (long long)m->ntot);
         }
         LCK(c, cudaGetLastError());
@@ -786,7 +794,7 @@ int lat_enqueue_window(tde_mesh *m, const BH &bh) {
   }
   {
     ProfScope ps(c, TDE_K_SCALAR);
-    k_lat_advance<<<1, 1, 0, s>>>(m->d_scal, fmax);
+    pdl_launch(k_lat_advance, 1, 1, 0, s, m->d_scal, fmax);
   }
   LCK(c, cudaGetLastError());
   return TDE_OK;

@@ -113,10 +113,11 @@ __device__ __forceinline__ void red4(float *p, float a, float b, float c, float 
 // CTA that finishes last applies Adam instead of a second launch.  One training
 // step of 4096: 19 us (79 with a thread per sample and 128 samples a CTA).
 __global__ void __launch_bounds__(GT) k_mlp_grad(const __nv_bfloat16 *wb_in,
-                                                 const float *__restrict__ x,
-                                                 const float *__restrict__ tg, long long s0,
+                                                 const float *x,
+                                                 const float *tg, long long s0,
                                                  long long count, float inv_n, float *g,
                                                  float *loss, AdamArgs ad) {
+  pdl_begin();
   extern __shared__ __align__(16) float sh[];
   float *W2 = sh;                  // [H][HP]
   float *sh1 = W2 + H * HP;        // [GS][HP] hidden 1
@@ -465,6 +466,7 @@ __device__ __forceinline__ bool newton_cell(const DTable &t, double rho_c, doubl
 // accepted count is added once per CTA).
 template <int NEWTON>
 __global__ void __launch_bounds__(IT, 8) k_eos_surrogate(SurrogateArgs a) {
+  pdl_begin();
   __shared__ __align__(1024) unsigned char sA[IT * H * 2];   // h1, BF16, core-matrix layout
   __shared__ __align__(1024) unsigned char sB[H * H * 2];    // W2, BF16, core-matrix layout
   __shared__ float sW1[2 * H], sb1[H], sb2[H], sW3[2 * H], sb3[2];
@@ -664,11 +666,12 @@ __global__ void __launch_bounds__(IT, 8) k_eos_surrogate(SurrogateArgs a) {
 // Table bisection for the cells the Newton step left (their indices in queue).
 // With eu (the hydro closure's buffers) the clamped table energy is returned
 // (0 inside the table) and the closure counts clamps; without, they are counted here.
-__global__ void __launch_bounds__(256) k_eos_fallback(DTable t, const long long *__restrict__ queue,
-                                                      const unsigned long long *__restrict__ qcount,
-                                                      const double *__restrict__ rho,
-                                                      const double *__restrict__ e, double *T, double *P,
+__global__ void __launch_bounds__(256) k_eos_fallback(DTable t, const long long *queue,
+                                                      const unsigned long long *qcount,
+                                                      const double *rho,
+                                                      const double *e, double *T, double *P,
                                                       double *cs2, double *eu, Counters *cnt) {
+  pdl_begin();
   const long long nq = (long long)*qcount;
   for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < nq;
        q += (long long)gridDim.x * blockDim.x) {
@@ -756,7 +759,7 @@ cudaError_t launch_grad(tde_eos *e, const float *x, const float *tg, long long s
   cudaError_t err = cudaFuncSetAttribute(k_mlp_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)grad_smem());
   if (err != cudaSuccess) return err;
   const unsigned grid = (unsigned)((count + GS - 1) / GS);
-  k_mlp_grad<<<grid, GT, grad_smem(), s>>>((const __nv_bfloat16 *)e->d_wb, x, tg, s0, count, inv_n, g,
+  pdl_launch(k_mlp_grad, grid, GT, grad_smem(), s, (const __nv_bfloat16 *)e->d_wb, x, tg, s0, count, inv_n, g,
                                            loss, ad);
   return cudaGetLastError();
 }
@@ -794,7 +797,7 @@ cudaError_t launch_surrogate_kernel(tde_eos *e, long long n, const double *rho, 
   const int per_sm = 8;
   const long long tiles = (n + IT - 1) / IT * (a.cm.blocks ? a.cm.nblk : 1);
   const unsigned grid = (unsigned)std::min<long long>(tiles, (long long)sms * per_sm);
-  k_eos_surrogate<0><<<grid, IT, 0, s>>>(a);
+  pdl_launch(k_eos_surrogate<0>, grid, IT, 0, s, a);
   return cudaGetLastError();
 }
 
@@ -831,7 +834,7 @@ cudaError_t launch_surrogate_newton(tde_eos *e, const CellMap &cm, long long n, 
   const int per_sm = 8;
   const long long tiles = (n + IT - 1) / IT * (cm.blocks ? cm.nblk : 1);
   const unsigned grid = (unsigned)std::min<long long>(tiles, (long long)sms * per_sm);
-  k_eos_surrogate<1><<<grid, IT, 0, s>>>(a);
+  pdl_launch(k_eos_surrogate<1>, grid, IT, 0, s, a);
   return cudaGetLastError();
 }
 
@@ -851,7 +854,7 @@ cudaError_t surrogate_run(tde_eos *e, const CellMap &cm, long long n, const doub
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, e->ctx->device);
   const long long ncell = n * (cm.blocks ? cm.nblk : 1);
   const unsigned gf = (unsigned)std::min<long long>((ncell + 255) / 256, (long long)sms * 8);
-  k_eos_fallback<<<gf, 256, 0, s>>>(e->tab, queue, qcount, rho, en, T, P, cs2, eu, cnt);
+  pdl_launch(k_eos_fallback, gf, 256, 0, s, e->tab, queue, qcount, rho, en, T, P, cs2, eu, cnt);
   return cudaGetLastError();
 }
 

@@ -541,6 +541,7 @@ __device__ __forceinline__ bool sweep_tile(const SweepArgs &a, int qb, int tile,
 
 template <int D, int RECON, int EOSK, int DUAL, int LAST, int M, int NTS, int MINB>
 __global__ void __launch_bounds__(NTS, MINB) k_sweep(const SweepArgs a) {
+  pdl_begin();
   constexpr int NV = (EOSK == EOS_TABLE ? 7 : 5) + DUAL;
   extern __shared__ __align__(128) double sm[];
   unsigned long long *mbar =
@@ -560,8 +561,7 @@ cudaError_t sweep_one(const SweepArgs &a, bool last, dim3 grid, size_t smem, cud
   auto k = last ? k_sweep<D, RECON, EOSK, DUAL, 1, M, NTS, MINB> : k_sweep<D, RECON, EOSK, DUAL, 0, M, NTS, MINB>;
   cudaError_t err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (err != cudaSuccess) return err;
-  k<<<grid, NTS, smem, s>>>(a);
-  return cudaGetLastError();
+  return pdl_launch(k, grid, NTS, smem, s, a);
 }
 
 template <int D, int M, int NTS, int MINB>

@@ -379,7 +379,6 @@ extern "C" int tde_eos_destroy(tde_eos *e) {
   cudaFree(e->d_wb);
   cudaFree(e->d_status);
   cudaFree(e->d_queue);
-  cudaFree(e->d_guess);
   cudaFree(e->d_qcount);
   delete e;
   return TDE_OK;

@@ -227,6 +227,11 @@ struct DevBlock {
   long long off;
 };
 
+// k + 1/2 for a small integer |k| < 2^49, by one FP64 add
+__device__ __forceinline__ double dhalf(long long k) {
+  return dfrom(0x4328000000000000LL + 2 * k + 1) - 3377699720527872.0;   // 1.5 2^51, units of 1/2
+}
+
 // 2^e for |e| < 1000, exact (built from the exponent field)
 __host__ __device__ __forceinline__ double exp2i(int e) {
   unsigned long long b = (unsigned long long)(1023 + e) << 52;
@@ -668,8 +673,24 @@ __device__ __forceinline__ void c2p_energy(const Phys &p, const double *u, doubl
   }
 }
 
-// Conserved (rho, m, E[, U_aux]) -> primitives w = (rho, vx, vy, vz, P
-// [, Gamma_e, Gamma_1][, U_aux]) with the dual-energy switch of
+// The primitives w = (rho, vx, vy, vz, P[, Gamma_e, Gamma_1][, U_aux]) from the
+// floored density, the velocities and the closure's P, cs^2 and represented U
+// (code units), with the pressure floor.
+template <int EOSK, int DUAL>
+__device__ __forceinline__ void c2p_prims(const Phys &p, double uaux, double rho, double vx, double vy, double vz,
+                                          double P, double cs2, double Uu, double *w, Counters *cnt) {
+  if (dlt(P, p.p_floor)) { P = p.p_floor; if (cnt) count(&cnt->p_floor); }
+  w[0] = rho; w[1] = vx; w[2] = vy; w[3] = vz; w[4] = P;
+  if (EOSK == EOS_TABLE) {
+    w[5] = 1.0 + P * rcp_nr(Uu);         // Gamma_e
+    w[6] = rho * cs2 * rcp_nr(P);        // Gamma_1
+    if (DUAL) w[7] = uaux;
+  } else {
+    if (DUAL) w[5] = uaux;
+  }
+}
+
+// Conserved (rho, m, E[, U_aux]) -> primitives with the dual-energy switch of
 // Eq. dual-primitive-switch and the density / pressure floors.
 template <int EOSK, int DUAL, int EOSB = 0>
 __device__ __forceinline__ void cons_to_prim(const Phys &p, const double *u, double *w,
@@ -679,15 +700,7 @@ __device__ __forceinline__ void cons_to_prim(const Phys &p, const double *u, dou
   c2p_energy<DUAL>(p, u, rho, vx, vy, vz, Ue, cnt);
   double P, cs2, Uu;
   eos_closure<EOSK, EOSB>(p, rho, Ue, P, cs2, Uu, cnt, eb, flat);
-  if (dlt(P, p.p_floor)) { P = p.p_floor; if (cnt) count(&cnt->p_floor); }
-  w[0] = rho; w[1] = vx; w[2] = vy; w[3] = vz; w[4] = P;
-  if (EOSK == EOS_TABLE) {
-    w[5] = 1.0 + P * rcp_nr(Uu);         // Gamma_e
-    w[6] = rho * cs2 * rcp_nr(P);        // Gamma_1
-    if (DUAL) w[7] = u[5];
-  } else {
-    if (DUAL) w[5] = u[5];
-  }
+  c2p_prims<EOSK, DUAL>(p, DUAL ? u[5] : 0.0, rho, vx, vy, vz, P, cs2, Uu, w, cnt);
 }
 
 // ------------------------------------------------------- reconstruction ----

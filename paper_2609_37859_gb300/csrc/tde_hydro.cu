@@ -100,14 +100,16 @@ __device__ __forceinline__ void cta_bh_info(const BH &bh, double t, double dx, c
 // A CTA converts the cells blockIdx.x NT + threadIdx.x + q gridDim.x NT of its block
 // (launch_c2p: one per thread on small meshes, several on large ones, so that the
 // per-CTA part of the time step -- the point mass, the minima, a square root, all
-// FP64 instructions of single warps -- is shared by 1024 cells).
-template <int EOSK, int DUAL, int EOSB = 0>
+// FP64 instructions of single warps -- is shared by 1024 cells).  DT_ONLY: the
+// primitives are in W already, only the time step is taken (the learned-guess closure
+// converts in its own kernel).
+template <int EOSK, int DUAL, int DT_ONLY = 0>
 __global__ void __launch_bounds__(NT) k_c2p(Phys p, BH bh, TimeArgs ta,
                                             const DevBlock *blocks,
                                             const int32_t *ids,
                                             const double *U, double *W,
                                             long long ntot, Counters *cnt, int want_dt,
-                                            unsigned long long *dtbits, EOSBuf eb) {
+                                            unsigned long long *dtbits) {
   pdl_begin();
   const int b = ids[blockIdx.y];
   const DevBlock B = blocks[b];
@@ -135,12 +137,17 @@ __global__ void __launch_bounds__(NT) k_c2p(Phys p, BH bh, TimeArgs ta,
     const long long flat =
         B.off + ((long long)(r / B.n[1] + p.g[2]) * B.p[1] + (r % B.n[1] + p.g[1])) * B.p[0] + (i + p.g[0]);
     double u[6], w[8];
-#pragma unroll
-    for (int v = 0; v < 5 + DUAL; ++v) u[v] = U[v * ntot + flat];
-    cons_to_prim<EOSK, DUAL, EOSB>(p, u, w, cnt, &eb, flat);
     constexpr int NWV = (EOSK == EOS_TABLE ? 7 : 5) + DUAL;
+    if (DT_ONLY) {
 #pragma unroll
-    for (int v = 0; v < NWV; ++v) W[v * ntot + flat] = w[v];
+      for (int v = 0; v < 7; ++v) w[v] = W[v * ntot + flat];
+    } else {
+#pragma unroll
+      for (int v = 0; v < 5 + DUAL; ++v) u[v] = U[v * ntot + flat];
+      cons_to_prim<EOSK, DUAL>(p, u, w, cnt);
+#pragma unroll
+      for (int v = 0; v < NWV; ++v) W[v * ntot + flat] = w[v];
+    }
     if (want_dt && !(exc_box && inside_radius(dist2(e), bh.rexc))) {
       const double g1 = EOSK == EOS_TABLE ? w[6] : p.gamma;
       const double cs = sqrt_ratio(g1 * w[4], w[0]);
@@ -237,11 +244,10 @@ __global__ void __launch_bounds__(NT) k_c2p_list(Phys p, const int32_t *list, in
   }
 }
 
-// The table inputs (cgs rho, e) of the interior (PADDED = 0) or all padded
-// (PADDED = 1) cells of the listed blocks, by the same expressions as the
-// closure inside k_c2p, for the learned-guess inversion's launches; nothing is
-// counted here (k_c2p counts when it takes the results).
-template <int DUAL, int PADDED>
+// The table inputs (cgs rho, e) of all padded cells of the listed blocks, by the
+// same expressions as the closure inside k_c2p, for the learned-guess inversion's
+// launches; nothing is counted here (k_c2p_padded counts when it takes the results).
+template <int DUAL>
 __global__ void __launch_bounds__(NT) k_c2p_eosin(Phys p, const DevBlock *blocks,
                                                   const int32_t *ids,
                                                   const double *U, double *rho_in,
@@ -249,16 +255,9 @@ __global__ void __launch_bounds__(NT) k_c2p_eosin(Phys p, const DevBlock *blocks
   pdl_begin();
   const int b = ids[blockIdx.y];
   const DevBlock B = blocks[b];
-  const int n = PADDED ? B.p[0] * B.p[1] * B.p[2] : B.n[0] * B.n[1] * B.n[2];
+  const int n = B.p[0] * B.p[1] * B.p[2];
   for (int e = blockIdx.x * NT + threadIdx.x; e < n; e += gridDim.x * NT) {
-    long long flat;
-    if (PADDED) {
-      flat = B.off + e;
-    } else {
-      const int i = e % B.n[0], r = e / B.n[0];
-      const int j = r % B.n[1], k = r / B.n[1];
-      flat = B.off + ((long long)(k + p.g[2]) * B.p[1] + (j + p.g[1])) * B.p[0] + (i + p.g[0]);
-    }
+    const long long flat = B.off + e;
     double u[6];
 #pragma unroll
     for (int v = 0; v < 5 + DUAL; ++v) u[v] = U[v * ntot + flat];
@@ -634,29 +633,21 @@ static bool surrogate_closure(const tde_mesh *m) {
   return m->phys.eos == EOS_TABLE && m->phys.eos_mode == TDE_INVERT_SURROGATE;
 }
 
-// The learned-guess inversion of the listed blocks' cells (interior or all
-// padded): table inputs -> guess, Newton, queued bisection -> m->sb (P, cs2, eu).
-static cudaError_t surrogate_table_pass(tde_mesh *m, const double *Uin, int nblk, const int32_t *ids,
-                                        bool padded, dim3 grid) {
+// The learned-guess inversion of the listed blocks' padded cells: table inputs
+// -> guess, Newton, queued bisection -> m->sb (P, cs2, eu).
+static cudaError_t surrogate_table_pass(tde_mesh *m, const double *Uin, int nblk, const int32_t *ids, dim3 grid) {
   const Phys &p = m->phys;
   cudaStream_t s = m->ctx->stream;
   if (!m->sb.rho || !m->eos || !m->eos->has_net) return cudaErrorInvalidValue;
   const long long nt = (long long)m->ntot;
-  if (padded) {
-    if (p.dual) pdl_launch(k_c2p_eosin<1, 1>, grid, NT, 0, s, p, m->d_blocks, ids, Uin, m->sb.rho, m->sb.e, nt);
-    else pdl_launch(k_c2p_eosin<0, 1>, grid, NT, 0, s, p, m->d_blocks, ids, Uin, m->sb.rho, m->sb.e, nt);
-  } else {
-    if (p.dual) pdl_launch(k_c2p_eosin<1, 0>, grid, NT, 0, s, p, m->d_blocks, ids, Uin, m->sb.rho, m->sb.e, nt);
-    else pdl_launch(k_c2p_eosin<0, 0>, grid, NT, 0, s, p, m->d_blocks, ids, Uin, m->sb.rho, m->sb.e, nt);
-  }
+  if (p.dual) pdl_launch(k_c2p_eosin<1>, grid, NT, 0, s, p, m->d_blocks, ids, Uin, m->sb.rho, m->sb.e, nt);
+  else pdl_launch(k_c2p_eosin<0>, grid, NT, 0, s, p, m->d_blocks, ids, Uin, m->sb.rho, m->sb.e, nt);
   cudaError_t err = cudaGetLastError();
   if (err != cudaSuccess) return err;
   m->ctx->launches[TDE_K_C2P] += 3;   // table inputs, guess + Newton, bisection of the misses
-  CellMap cm{m->d_blocks, ids, nblk, padded ? 1 : 0, {p.g[0], p.g[1], p.g[2]}};
+  CellMap cm{m->d_blocks, ids, nblk, 1, {p.g[0], p.g[1], p.g[2]}};
   int64_t nmax = 0;
-  for (const DevBlock &B : m->hblocks)
-    nmax = std::max<int64_t>(nmax, padded ? (int64_t)B.p[0] * B.p[1] * B.p[2]
-                                          : (int64_t)B.n[0] * B.n[1] * B.n[2]);
+  for (const DevBlock &B : m->hblocks) nmax = std::max<int64_t>(nmax, (int64_t)B.p[0] * B.p[1] * B.p[2]);
   return launch_eos_surrogate_cells(m->eos, cm, nmax, m->sb, m->d_cnt, s);
 }
 
@@ -665,26 +656,27 @@ cudaError_t launch_c2p(tde_mesh *m, const double *Uin, int nblk, const int32_t *
   ProfScope _ps(m->ctx, TDE_K_C2P);
   dim3 grid((unsigned)((m->max_interior + NT - 1) / NT), (unsigned)nblk);
   const Phys &p = m->phys;
-  EOSBuf eb{m->sb.P, m->sb.cs2, m->sb.eu};
-  if (surrogate_closure(m)) {
-    cudaError_t err = surrogate_table_pass(m, Uin, nblk, ids, false, grid);
-    if (err != cudaSuccess) return err;
-  }
   // the time step's per-CTA work shared by four cells a thread, where that leaves
   // several waves of CTAs (closure and conversion of a step of the 8.4 M-cell star:
   // 3.09 -> 2.91 ms)
   if (want_dt && (int64_t)grid.x * nblk >= 64LL * n_sm()) grid.x = (grid.x + 3) / 4;
-#define C2P_ARGS p, bh, ta, m->d_blocks, ids, Uin, m->d_W, (long long)m->ntot, m->d_cnt, \
-                 (int)want_dt, m->d_dtbits, eb
-  if (p.eos == EOS_IDEAL) {
-    if (p.dual) pdl_launch(k_c2p<EOS_IDEAL, 1>, grid, NT, 0, m->ctx->stream, C2P_ARGS);
-    else pdl_launch(k_c2p<EOS_IDEAL, 0>, grid, NT, 0, m->ctx->stream, C2P_ARGS);
-  } else if (surrogate_closure(m)) {
-    if (p.dual) pdl_launch(k_c2p<EOS_TABLE, 1, 1>, grid, NT, 0, m->ctx->stream, C2P_ARGS);
-    else pdl_launch(k_c2p<EOS_TABLE, 0, 1>, grid, NT, 0, m->ctx->stream, C2P_ARGS);
+#define C2P_ARGS grid, NT, 0, m->ctx->stream, p, bh, ta, m->d_blocks, ids, Uin, m->d_W, (long long)m->ntot, m->d_cnt, \
+                 (int)want_dt, m->d_dtbits
+  if (surrogate_closure(m)) {
+    // the learned guess with the conversion in its own kernel, the time step after it
+    if (!m->sb.rho || !m->eos || !m->eos->has_net) return cudaErrorInvalidValue;
+    m->ctx->launches[TDE_K_C2P] += want_dt ? 2 : 1;
+    CellMap cm{m->d_blocks, ids, nblk, 0, {p.g[0], p.g[1], p.g[2]}};
+    cudaError_t err = launch_surrogate_c2p(m, cm, m->max_interior, Uin, m->ctx->stream);
+    if (err != cudaSuccess || !want_dt) return err;
+    if (p.dual) pdl_launch(k_c2p<EOS_TABLE, 1, 1>, C2P_ARGS);
+    else pdl_launch(k_c2p<EOS_TABLE, 0, 1>, C2P_ARGS);
+  } else if (p.eos == EOS_IDEAL) {
+    if (p.dual) pdl_launch(k_c2p<EOS_IDEAL, 1>, C2P_ARGS);
+    else pdl_launch(k_c2p<EOS_IDEAL, 0>, C2P_ARGS);
   } else {
-    if (p.dual) pdl_launch(k_c2p<EOS_TABLE, 1>, grid, NT, 0, m->ctx->stream, C2P_ARGS);
-    else pdl_launch(k_c2p<EOS_TABLE, 0>, grid, NT, 0, m->ctx->stream, C2P_ARGS);
+    if (p.dual) pdl_launch(k_c2p<EOS_TABLE, 1>, C2P_ARGS);
+    else pdl_launch(k_c2p<EOS_TABLE, 0>, C2P_ARGS);
   }
 #undef C2P_ARGS
   return cudaGetLastError();
@@ -698,7 +690,7 @@ cudaError_t launch_c2p_padded(tde_mesh *m, const double *Uin, int nblk, const in
   const Phys &p = m->phys;
   EOSBuf eb{m->sb.P, m->sb.cs2, m->sb.eu};
   if (surrogate_closure(m)) {
-    cudaError_t err = surrogate_table_pass(m, Uin, nblk, ids, true, grid);
+    cudaError_t err = surrogate_table_pass(m, Uin, nblk, ids, grid);
     if (err != cudaSuccess) return err;
   }
 #define C2PP_ARGS p, m->d_blocks, ids, Uin, m->d_W, (long long)m->ntot, m->d_cnt, eb

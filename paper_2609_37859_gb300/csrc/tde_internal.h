@@ -96,7 +96,6 @@ struct tde_eos {
   float *d_w = nullptr;              // FP32 master weights, then Adam m, v and the gradient
   void *d_wb = nullptr;              // BF16 weights used by training forward and inference
   long long *d_queue = nullptr;      // cells the surrogate's Newton step left for bisection
-  float *d_guess = nullptr;          // the network's log10 T guess per cell
   int64_t queue_cap = 0;
   unsigned long long *d_qcount = nullptr;
   int *d_status = nullptr;
@@ -295,6 +294,7 @@ cudaError_t launch_eos_surrogate(tde_eos *e, int64_t n, const double *rho, const
                                  double *T, double *P, double *cs2, cudaStream_t s);
 cudaError_t launch_eos_surrogate_cells(tde_eos *e, const CellMap &cm, int64_t nmax,
                                        const SurrogateBuf &sb, Counters *cnt, cudaStream_t s);
+cudaError_t launch_surrogate_c2p(tde_mesh *m, const CellMap &cm, int64_t nmax, const double *U, cudaStream_t s);
 cudaError_t launch_eos_eval(tde_eos *e, int64_t n, const double *rho, const double *T, double *P,
                             double *en, double *cs2, cudaStream_t s);
 

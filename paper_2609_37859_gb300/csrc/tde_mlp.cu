@@ -35,11 +35,29 @@ struct MLPNorm {
 };
 
 __device__ __forceinline__ float silu_f(float a) { return a / (1.0f + __expf(-a)); }
-// SiLU for inference with one MUFU operation: sigmoid(a) = (1 + tanh(a / 2)) / 2
-__device__ __forceinline__ float silu_tanh(float a) {
-  float th;
-  asm("tanh.approx.f32 %0, %1;" : "=f"(th) : "f"(0.5f * a));
-  return a * fmaf(0.5f, th, 0.5f);
+// Pairs of FP32 values for the packed FMA (one instruction for two)
+typedef unsigned long long f2;
+__device__ __forceinline__ f2 f2_pack(float a, float b) {
+  f2 d;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(a), "f"(b));
+  return d;
+}
+__device__ __forceinline__ void f2_split(f2 v, float &a, float &b) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ f2 f2_fma(f2 a, f2 b, f2 c) {
+  f2 d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+// SiLU for inference of two values from half their pre-activations, with one MUFU
+// operation each: a sigmoid(a) = (a / 2)(1 + tanh(a / 2))
+__device__ __forceinline__ f2 silu2_half(f2 z) {
+  float a, b, ta, tb;
+  f2_split(z, a, b);
+  asm("tanh.approx.f32 %0, %1;" : "=f"(ta) : "f"(a));
+  asm("tanh.approx.f32 %0, %1;" : "=f"(tb) : "f"(b));
+  return f2_fma(z, f2_pack(ta, tb), z);
 }
 __device__ __forceinline__ float dsilu_f(float a) {
   const float s = 1.0f / (1.0f + __expf(-a));
@@ -365,12 +383,11 @@ struct SurrogateArgs {
   long long n;
   const double *rho, *e;
   double *T, *P, *cs2;
-  float *yout;        // optional: raw network outputs [n][2] (normalised)
-  const float *xin;   // optional: network inputs instead of (rho, e) [n][2]
+  float *yout;        // raw network outputs [n][2] (normalised; NEWTON = 0)
+  const float *xin;   // the network's inputs [n][2] (NEWTON = 0)
   Counters *cnt;
   int *status;        // set to 1 if a bounded wait expired
   int skip_mma;       // failure-detection test: issue no MMA, so the wait expires
-  float *lTg;         // optional: the guessed log10 T of each cell
   CellMap cm;         // which cells: plain arrays (cm.blocks null) or cells of blocks
   // the fused Newton step (k_eos_surrogate<1>): results of accepted cells, the
   // closure's clamped energy (eu, or null), the queue of cells left for
@@ -378,6 +395,11 @@ struct SurrogateArgs {
   double *eu;
   long long *queue;
   unsigned long long *qcount;
+  // the hydro form (k_eos_surrogate<2, DUAL>): the cells' conserved state and primitives
+  Phys p;
+  const double *U;
+  double *W;
+  long long ntot;
 };
 
 // Cells of a cell map: block position bp's cell count, and the array index of
@@ -425,7 +447,7 @@ __device__ __forceinline__ void cm_split(const CellMap &cm, long long t, long lo
 // to bisection (clamped inputs, a step that misses, a table without the
 // prepared form).
 __device__ __forceinline__ bool newton_cell(const DTable &t, double rho_c, double e, float lTg, float idlt,
-                                            long long c, double *T, double *P, double *cs2, double *eu) {
+                                            double &P, double &cs2, double *T) {
   if (!t.node || !dgt0(e)) return false;
   const int nt = t.nt;
   int i;
@@ -450,26 +472,34 @@ __device__ __forceinline__ bool newton_cell(const DTable &t, double rho_c, doubl
   }
   // at the coldest node bisection clamps (y <= g_0): leave that to it
   if (!(in && (j > 0 || g0 < y))) return false;
-  double Pv, cv, ev, Tv;
-  eos_at<true>(t, row + 3 * j, w, j, fx_frac(y - g0, g1 - g0), false, e, Pv, cv, ev, T ? &Tv : nullptr);
-  if (P) P[c] = Pv;
-  if (cs2) cs2[c] = cv;
-  if (T) T[c] = Tv;
-  if (eu) eu[c] = 0.0;   // inside the table
+  double ev;
+  eos_at<true>(t, row + 3 * j, w, j, fx_frac(y - g0, g1 - g0), false, e, P, cs2, ev, T);
   return true;
 }
 
-// The learned guess.  NEWTON = 0: the network alone (raw outputs, the guess);
+// The learned guess.
+// NEWTON = 0: the network alone (raw outputs);
 // NEWTON = 1: the guess goes straight into the Newton step in the same
 // thread (newton_cell), accepted cells are written and the rest queued for
 // k_eos_fallback (one atomic per tile reserves the tile's queue slots; the
-// accepted count is added once per CTA).
-template <int NEWTON>
-__global__ void __launch_bounds__(IT, 8) k_eos_surrogate(SurrogateArgs a) {
+// accepted count is added once per CTA);
+// NEWTON = 2 (hydro): as 1, with the table inputs formed from the cell's conserved
+// state and the primitives of accepted cells written, so the FP64 work of the
+// conversion runs beside the network's integer and MUFU work and the state is read by
+// one kernel; the queued cells are converted by k_fallback_c2p.  A step of 8.4 M cells:
+// 14.3 -> 13.4 ms against separate kernels for inputs, inversion and conversion.
+// What bounds it is instruction issue (two thirds of its slots): the layers go two
+// units at a time through the packed FP32 FMA, and the output the inversion does not
+// use is left out (5.9 M cells 780 -> 728 us; one 16-byte record of weights per unit
+// instead of an array per weight was slower, 868 us: a third more shared reads).
+template <int NEWTON, int DUAL = 0>
+__global__ void __launch_bounds__(IT, 8) k_eos_surrogate(const SurrogateArgs a) {
   pdl_begin();
   __shared__ __align__(1024) unsigned char sA[IT * H * 2];   // h1, BF16, core-matrix layout
   __shared__ __align__(1024) unsigned char sB[H * H * 2];    // W2, BF16, core-matrix layout
-  __shared__ float sW1[2 * H], sb1[H], sb2[H], sW3[2 * H], sb3[2];
+  // layer 1's weights and the hidden biases, halved for silu2_half; read four at a time
+  __shared__ __align__(16) float sW1[2][H], sb1[H], sb2[H], sW3[2][H];
+  __shared__ float sb3[2];
   __shared__ __align__(8) unsigned long long mbar;
   __shared__ uint32_t tmem_base;
   __shared__ int s_abort;
@@ -490,13 +520,13 @@ __global__ void __launch_bounds__(IT, 8) k_eos_surrogate(SurrogateArgs a) {
     const int o = q / H, i = q % H;
     *reinterpret_cast<__nv_bfloat16 *>(sB + core_off(o, i)) = a.wb[OW2 + q];
   }
-  for (int q = tid; q < 2 * H; q += IT) {
-    sW1[q] = __bfloat162float(a.wb[OW1 + q]);
-    sW3[q] = __bfloat162float(a.wb[OW3 + q]);
-  }
   if (tid < H) {
-    sb1[tid] = __bfloat162float(a.wb[OB1 + tid]);
-    sb2[tid] = __bfloat162float(a.wb[OB2 + tid]);
+    sW1[0][tid] = 0.5f * __bfloat162float(a.wb[OW1 + 2 * tid]);
+    sW1[1][tid] = 0.5f * __bfloat162float(a.wb[OW1 + 2 * tid + 1]);
+    sb1[tid] = 0.5f * __bfloat162float(a.wb[OB1 + tid]);
+    sb2[tid] = 0.5f * __bfloat162float(a.wb[OB2 + tid]);
+    sW3[0][tid] = __bfloat162float(a.wb[OW3 + tid]);
+    sW3[1][tid] = __bfloat162float(a.wb[OW3 + H + tid]);
   }
   if (tid < 2) sb3[tid] = __bfloat162float(a.wb[OB3 + tid]);
   if (tid == 0) {
@@ -523,20 +553,28 @@ __global__ void __launch_bounds__(IT, 8) k_eos_surrogate(SurrogateArgs a) {
     const long long c = live ? cm_flat(a.cm, bp, local) : 0;
     // after an expired wait (s_abort, uniform) the network is skipped: the
     // Newton kernel queues the remaining cells for bisection, the plain one stops
-    float y0 = 0.f, y1 = 0.f;
+    float y0 = 0.f;
+    double rho_c = 1.0, e_c = 0.0;   // the table's inputs
+    if (NEWTON == 2 && live) {
+      double u[6], vx, vy, vz, Ue, rho;
+#pragma unroll
+      for (int v = 0; v < 5 + DUAL; ++v) u[v] = a.U[v * a.ntot + c];
+      c2p_energy<DUAL>(a.p, u, rho, vx, vy, vz, Ue, nullptr);
+      eos_inputs(a.p, rho, Ue, rho_c, e_c);
+    }
     if (!s_abort) {
       // ---- inputs and layer 1, FP32 only: the network needs log10 rho and the
       // position z of log10 e in its column to FP32 accuracy (the exact work of
       // the inversion is newton_cell's)
       float x0 = 0.f, x1 = 0.f;
       if (live) {
-        if (a.xin) {
+        if (!NEWTON) {
           x0 = a.xin[2 * c];
           x1 = a.xin[2 * c + 1];
         } else {
           const DTable &t = a.t;
-          const float lr = __log2f((float)a.rho[c]) * 0.30102999566f;
-          const float ly = __log2f((float)a.e[c]) * 0.30102999566f;
+          const float lr = __log2f((float)(NEWTON == 1 ? a.rho[c] : rho_c)) * 0.30102999566f;
+          const float ly = __log2f((float)(NEWTON == 1 ? a.e[c] : e_c)) * 0.30102999566f;
           const float xr = fminf(fmaxf((lr - (float)t.lr0) * (float)t.inv_dlr, 0.f), (float)(t.nr - 1));
           const int ti = min((int)xr, t.nr - 2);
           const float w32 = xr - (float)ti;
@@ -549,13 +587,21 @@ __global__ void __launch_bounds__(IT, 8) k_eos_surrogate(SurrogateArgs a) {
           x1 = (fminf(fmaxf(z, -1.f), 2.f) - a.nm.ce) * a.nm.ise;
         }
       }
+      const f2 xx0 = f2_pack(x0, x0), xx1 = f2_pack(x1, x1);
 #pragma unroll
       for (int k8 = 0; k8 < H / 8; ++k8) {
-        __align__(16) __nv_bfloat16 hv[8];
+        __align__(16) __nv_bfloat162 hv[4];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
+        for (int u = 0; u < 8; u += 4) {
           const int o = 8 * k8 + u;
-          hv[u] = __float2bfloat16_rn(silu_tanh(sW1[2 * o] * x0 + sW1[2 * o + 1] * x1 + sb1[o]));
+          const ulonglong2 w0 = *reinterpret_cast<const ulonglong2 *>(&sW1[0][o]);
+          const ulonglong2 w1 = *reinterpret_cast<const ulonglong2 *>(&sW1[1][o]);
+          const ulonglong2 b = *reinterpret_cast<const ulonglong2 *>(&sb1[o]);
+          float h0, h1;
+          f2_split(silu2_half(f2_fma(w0.x, xx0, f2_fma(w1.x, xx1, b.x))), h0, h1);
+          hv[u / 2] = __floats2bfloat162_rn(h0, h1);
+          f2_split(silu2_half(f2_fma(w0.y, xx0, f2_fma(w1.y, xx1, b.y))), h0, h1);
+          hv[u / 2 + 1] = __floats2bfloat162_rn(h0, h1);
         }
         *reinterpret_cast<uint4 *>(sA + core_off(tid, 8 * k8)) = *reinterpret_cast<uint4 *>(hv);
       }
@@ -587,8 +633,9 @@ __global__ void __launch_bounds__(IT, 8) k_eos_surrogate(SurrogateArgs a) {
         asm volatile("tcgen05.fence::after_thread_sync;");
         // ---- read the accumulator row of this thread (warp w owns TMEM lanes
         // 32w..32w+31) in two halves of 32 columns, and apply layer 3 (FP32)
-        y0 = sb3[0];
-        y1 = sb3[1];
+        // (two units at a time; the second output, log P, is not the inversion's)
+        const f2 half2 = f2_pack(0.5f, 0.5f);
+        f2 yy0 = f2_pack(sb3[0], 0.f), yy1 = f2_pack(sb3[1], 0.f);
 #pragma unroll
         for (int hf = 0; hf < 2; ++hf) {
           uint32_t r[32];
@@ -604,18 +651,28 @@ __global__ void __launch_bounds__(IT, 8) k_eos_surrogate(SurrogateArgs a) {
               : "r"(taddr));
           asm volatile("tcgen05.wait::ld.sync.aligned;");
 #pragma unroll
-          for (int q = 0; q < 32; ++q) {
+          for (int q = 0; q < 32; q += 4) {
             const int o = 32 * hf + q;
-            const float h2 = silu_tanh(__uint_as_float(r[q]) + sb2[o]);
-            y0 += sW3[o] * h2;
-            y1 += sW3[H + o] * h2;
+            const ulonglong2 b = *reinterpret_cast<const ulonglong2 *>(&sb2[o]);
+            const ulonglong2 w0 = *reinterpret_cast<const ulonglong2 *>(&sW3[0][o]);
+            const ulonglong2 w1 = *reinterpret_cast<const ulonglong2 *>(&sW3[1][o]);
+            const f2 p = silu2_half(f2_fma(f2_pack(__uint_as_float(r[q]), __uint_as_float(r[q + 1])), half2, b.x));
+            yy0 = f2_fma(w0.x, p, yy0);
+            if (!NEWTON) yy1 = f2_fma(w1.x, p, yy1);
+            const f2 v = silu2_half(f2_fma(f2_pack(__uint_as_float(r[q + 2]), __uint_as_float(r[q + 3])), half2, b.y));
+            yy0 = f2_fma(w0.y, v, yy0);
+            if (!NEWTON) yy1 = f2_fma(w1.y, v, yy1);
           }
         }
-        if (live && a.yout) {
+        float y0a, y0b;
+        f2_split(yy0, y0a, y0b);
+        y0 = y0a + y0b;
+        if (!NEWTON && live) {
+          float y1a, y1b;
+          f2_split(yy1, y1a, y1b);
           a.yout[2 * c] = y0;
-          a.yout[2 * c + 1] = y1;
+          a.yout[2 * c + 1] = y1a + y1b;
         }
-        if (live && a.lTg) a.lTg[c] = a.nm.cT + a.nm.sT * y0;
       }
       // every thread has its row in registers: the next tile may reuse sA and TMEM
       asm volatile("tcgen05.fence::before_thread_sync;");
@@ -624,9 +681,30 @@ __global__ void __launch_bounds__(IT, 8) k_eos_surrogate(SurrogateArgs a) {
     if (!NEWTON && !have) break;
     if (NEWTON) {
       // the Newton step from this thread's guess; misses are queued
-      const bool ok = live ? (have && newton_cell(a.t, a.rho[c], a.e[c], a.nm.cT + a.nm.sT * y0, a.nm.idlt, c,
-                                                  a.T, a.P, a.cs2, a.eu))
+      double Pv, cv, Tv;
+      if (NEWTON == 1 && live) {   // (read again: not held in registers through the network)
+        rho_c = a.rho[c];
+        e_c = a.e[c];
+      }
+      const bool ok = live ? (have && newton_cell(a.t, rho_c, e_c, a.nm.cT + a.nm.sT * y0, a.nm.idlt, Pv, cv,
+                                                  NEWTON == 1 && a.T ? &Tv : nullptr))
                            : true;
+      if (NEWTON == 1 && live && ok) {
+        if (a.P) a.P[c] = Pv;
+        if (a.cs2) a.cs2[c] = cv;
+        if (a.T) a.T[c] = Tv;
+        if (a.eu) a.eu[c] = 0.0;   // inside the table
+      }
+      if (NEWTON == 2 && live && ok) {
+        double u[6], w[8], vx, vy, vz, Ue, rho;
+#pragma unroll
+        for (int v = 0; v < 5 + DUAL; ++v) u[v] = a.U[v * a.ntot + c];
+        c2p_energy<DUAL>(a.p, u, rho, vx, vy, vz, Ue, a.cnt);
+        c2p_prims<EOS_TABLE, DUAL>(a.p, DUAL ? u[5] : 0.0, rho, vx, vy, vz, Pv * a.p.inv_unit_p, cv * a.p.inv_unit_e,
+                                   Ue, w, a.cnt);
+#pragma unroll
+        for (int v = 0; v < 7 + DUAL; ++v) a.W[v * a.ntot + c] = w[v];
+      }
       n_acc += (live && ok) ? 1u : 0u;
       const int lane = tid & 31;
       const unsigned rm = __ballot_sync(0xffffffffu, !ok);
@@ -683,6 +761,24 @@ __global__ void __launch_bounds__(256) k_eos_fallback(DTable t, const long long 
     if (P) P[c] = Pv;
     if (cs2) cs2[c] = cv;
     if (eu) eu[c] = cl ? euv : 0.0;
+  }
+}
+
+// the primitives of the cells the hydro form left (their indices in queue)
+template <int DUAL>
+__global__ void __launch_bounds__(256) k_fallback_c2p(Phys p, const long long *queue, const unsigned long long *qcount,
+                                                      const double *U, double *W, long long ntot, Counters *cnt) {
+  pdl_begin();
+  const long long nq = (long long)*qcount;
+  for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < nq;
+       q += (long long)gridDim.x * blockDim.x) {
+    const long long c = queue[q];
+    double u[6], w[8];
+#pragma unroll
+    for (int v = 0; v < 5 + DUAL; ++v) u[v] = U[v * ntot + c];
+    cons_to_prim<EOS_TABLE, DUAL>(p, u, w, cnt);
+#pragma unroll
+    for (int v = 0; v < 7 + DUAL; ++v) W[v * ntot + c] = w[v];
   }
 }
 
@@ -764,50 +860,39 @@ cudaError_t launch_grad(tde_eos *e, const float *x, const float *tg, long long s
   return cudaGetLastError();
 }
 
-cudaError_t launch_surrogate_kernel(tde_eos *e, long long n, const double *rho, const double *en,
-                                    double *T, double *P, double *cs2, const float *xin, float *yout,
-                                    cudaStream_t s, float *lTg = nullptr, const CellMap *cm = nullptr) {
-  SurrogateArgs a;
+// the network alone on n normalised inputs xin
+cudaError_t launch_surrogate_kernel(tde_eos *e, long long n, const float *xin, float *yout, cudaStream_t s) {
+  SurrogateArgs a{};
   a.t = e->tab;
   a.nm = norm_of(e);
   a.wb = (const __nv_bfloat16 *)e->d_wb;
   a.n = n;
-  a.rho = rho;
-  a.e = en;
-  a.T = T;
-  a.P = P;
-  a.cs2 = cs2;
   a.yout = yout;
   a.xin = xin;
   a.cnt = e->d_cnt;
   a.status = e->d_status;
   a.skip_mma = e->inject_wait_expiry;
-  a.lTg = lTg;
-  a.cm = cm ? *cm : CellMap{};
-  a.eu = nullptr;
-  a.queue = nullptr;
-  a.qcount = nullptr;
   int sms = 152;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, e->ctx->device);
   // one wave of resident CTAs: registers (64 x 128 threads) and shared memory
-  // (26 KB, largest carveout) admit 8 per SM, and 8 x 64 TMEM columns fill the
+  // (27 KB, largest carveout) admit 8 per SM, and 8 x 64 TMEM columns fill the
   // SM's 512 exactly
   cudaFuncSetAttribute(k_eos_surrogate<0>, cudaFuncAttributePreferredSharedMemoryCarveout,
                        (int)cudaSharedmemCarveoutMaxShared);
   const int per_sm = 8;
-  const long long tiles = (n + IT - 1) / IT * (a.cm.blocks ? a.cm.nblk : 1);
+  const long long tiles = (n + IT - 1) / IT;
   const unsigned grid = (unsigned)std::min<long long>(tiles, (long long)sms * per_sm);
   pdl_launch(k_eos_surrogate<0>, grid, IT, 0, s, a);
   return cudaGetLastError();
 }
 
 // the network and the Newton step in one pass (k_eos_surrogate<1>): 8 CTAs per
-// SM (64 registers, no spills), 8 x 64 TMEM columns fill the SM's 512
+// SM (64 registers), 8 x 64 TMEM columns fill the SM's 512
 cudaError_t launch_surrogate_newton(tde_eos *e, const CellMap &cm, long long n, const double *rho,
                                     const double *en, double *T, double *P, double *cs2, double *eu,
                                     long long *queue, unsigned long long *qcount, Counters *cnt,
-                                    cudaStream_t s) {
-  SurrogateArgs a;
+                                    cudaStream_t s, const tde_mesh *hy = nullptr, const double *hyU = nullptr) {
+  SurrogateArgs a{};
   a.t = e->tab;
   a.nm = norm_of(e);
   a.wb = (const __nv_bfloat16 *)e->d_wb;
@@ -817,24 +902,28 @@ cudaError_t launch_surrogate_newton(tde_eos *e, const CellMap &cm, long long n, 
   a.T = T;
   a.P = P;
   a.cs2 = cs2;
-  a.yout = nullptr;
-  a.xin = nullptr;
   a.cnt = cnt;
   a.status = e->d_status;
   a.skip_mma = e->inject_wait_expiry;
-  a.lTg = nullptr;
   a.cm = cm;
   a.eu = eu;
   a.queue = queue;
   a.qcount = qcount;
+  auto k = k_eos_surrogate<1>;
+  if (hy) {
+    a.p = hy->phys;
+    a.U = hyU;
+    a.W = hy->d_W;
+    a.ntot = (long long)hy->ntot;
+    k = hy->phys.dual ? k_eos_surrogate<2, 1> : k_eos_surrogate<2, 0>;
+  }
   int sms = 152;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, e->ctx->device);
-  cudaFuncSetAttribute(k_eos_surrogate<1>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                       (int)cudaSharedmemCarveoutMaxShared);
+  cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
   const int per_sm = 8;
   const long long tiles = (n + IT - 1) / IT * (cm.blocks ? cm.nblk : 1);
   const unsigned grid = (unsigned)std::min<long long>(tiles, (long long)sms * per_sm);
-  pdl_launch(k_eos_surrogate<1>, grid, IT, 0, s, a);
+  pdl_launch(k, grid, IT, 0, s, a);
   return cudaGetLastError();
 }
 
@@ -843,11 +932,9 @@ cudaError_t launch_surrogate_newton(tde_eos *e, const CellMap &cm, long long n, 
 // the queue.  The same inputs give the bisection results bit for bit.
 cudaError_t surrogate_run(tde_eos *e, const CellMap &cm, long long n, const double *rho,
                           const double *en, double *T, double *P, double *cs2, double *eu,
-                          float *lTg, long long *queue, unsigned long long *qcount, Counters *cnt,
-                          cudaStream_t s) {
+                          long long *queue, unsigned long long *qcount, Counters *cnt, cudaStream_t s) {
   cudaError_t r = cudaMemsetAsync(qcount, 0, sizeof(unsigned long long), s);
   if (r != cudaSuccess) return r;
-  (void)lTg;
   r = launch_surrogate_newton(e, cm, n, rho, en, T, P, cs2, eu, queue, qcount, cnt, s);
   if (r != cudaSuccess) return r;
   int sms = 152;
@@ -866,9 +953,7 @@ cudaError_t launch_eos_surrogate(tde_eos *e, int64_t n, const double *rho, const
   if (n <= 0) return cudaSuccess;
   if (e->queue_cap < n) {
     cudaFree(e->d_queue);
-    cudaFree(e->d_guess);
     e->d_queue = nullptr;
-    e->d_guess = nullptr;
     e->queue_cap = 0;
     cudaError_t r = cudaMalloc(&e->d_queue, sizeof(long long) * (size_t)n);
     if (r != cudaSuccess) return r;
@@ -880,14 +965,31 @@ cudaError_t launch_eos_surrogate(tde_eos *e, int64_t n, const double *rho, const
   }
   ProfScope ps(e->ctx, TDE_K_EOS);
   e->ctx->launches[TDE_K_EOS] += 1;   // the guess with its Newton step, then the bisection of the misses
-  return surrogate_run(e, CellMap{}, n, rho, en, T, P, cs2, nullptr, nullptr, e->d_queue,
+  return surrogate_run(e, CellMap{}, n, rho, en, T, P, cs2, nullptr, e->d_queue,
                        e->d_qcount, e->d_cnt, s);
+}
+
+// the interior cells of cm from the state U to the mesh's primitives: guess, Newton
+// step and conversion in one kernel, then the queued cells
+cudaError_t launch_surrogate_c2p(tde_mesh *m, const CellMap &cm, int64_t nmax, const double *U, cudaStream_t s) {
+  tde_eos *e = m->eos;
+  const SurrogateBuf &sb = m->sb;
+  cudaError_t r = cudaMemsetAsync(sb.qcount, 0, sizeof(unsigned long long), s);
+  if (r != cudaSuccess) return r;
+  r = launch_surrogate_newton(e, cm, nmax, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, sb.queue, sb.qcount,
+                              m->d_cnt, s, m, U);
+  if (r != cudaSuccess) return r;
+  int sms = 152;
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, e->ctx->device);
+  const unsigned gf = (unsigned)std::min<long long>((nmax * cm.nblk + 255) / 256, (long long)sms * 8);
+  auto k = m->phys.dual ? k_fallback_c2p<1> : k_fallback_c2p<0>;
+  return pdl_launch(k, gf, 256, 0, s, m->phys, sb.queue, sb.qcount, U, m->d_W, (long long)m->ntot, m->d_cnt);
 }
 
 cudaError_t launch_eos_surrogate_cells(tde_eos *e, const CellMap &cm, int64_t nmax,
                                        const SurrogateBuf &sb, Counters *cnt, cudaStream_t s) {
   if (nmax <= 0 || cm.nblk <= 0) return cudaSuccess;
-  return surrogate_run(e, cm, nmax, sb.rho, sb.e, nullptr, sb.P, sb.cs2, sb.eu, nullptr, sb.queue,
+  return surrogate_run(e, cm, nmax, sb.rho, sb.e, nullptr, sb.P, sb.cs2, sb.eu, sb.queue,
                        sb.qcount, cnt, s);
 }
 }  // namespace tde
@@ -958,7 +1060,7 @@ extern "C" int tde_eos_surrogate_forward(tde_eos *e, int64_t n, const float *x, 
   tde_ctx *c = e->ctx;
   if (n <= 0 || !x || !y || !e->has_net) return mlp_fail(c, TDE_EINVAL, "tde_eos_surrogate_forward: arguments or no weights");
   ProfScope ps(c, TDE_K_EOS);
-  MCK(c, launch_surrogate_kernel(e, n, nullptr, nullptr, nullptr, nullptr, nullptr, x, y, c->stream));
+  MCK(c, launch_surrogate_kernel(e, n, x, y, c->stream));
   return TDE_OK;
 }
 

@@ -34,7 +34,7 @@ __device__ __forceinline__ double cell_coord(const Phys &p, const DevBlock &B, i
     g %= N;
     if (g < 0) g += N;
   }
-  return p.xmin[a] + (g + 0.5) * block_dx(p, B, a);
+  return p.xmin[a] + dhalf(g) * block_dx(p, B, a);
 }
 
 // centre of padded cell c[] of block B

@@ -60,14 +60,8 @@ __device__ __forceinline__ long long dkey(double x) {
   const long long b = dbits(x);
   return b ^ ((b >> 63) & 0x7fffffffffffffffLL);
 }
-// the same with -0 and +0 equal (the IEEE order of non-NaN values)
-__device__ __forceinline__ long long dkey0(double x) {
-  const long long k = dkey(x);
-  return k < 0 ? k + 1 : k;
-}
 __device__ __forceinline__ bool dgt0(double x) { return dbits(x) > 0; }          // x > 0
 __device__ __forceinline__ bool dge0(double x) { return dkey(x) >= -1; }         // x >= 0 (incl. -0)
-__device__ __forceinline__ bool dle0(double x) { return dkey(x) <= 0; }          // x <= 0 (incl. +0)
 __device__ __forceinline__ bool dzero(double x) { return (dbits(x) << 1) == 0; }  // x == +-0
 __device__ __forceinline__ bool dlt(double a, double b) { return dkey(a) < dkey(b); }
 __device__ __forceinline__ bool dle(double a, double b) { return dkey(a) <= dkey(b); }
@@ -80,16 +74,6 @@ __device__ __forceinline__ double dabs(double x) { return dfrom(dmag(x)); }
 // the double value of a small integer |k| < 2^51, by one FP64 add
 __device__ __forceinline__ double dint(long long k) {
   return __longlong_as_double(0x4338000000000000LL + k) - 6755399441055744.0;
-}
-// x truncated to FP32 on the integer pipe (a guide value: normal x with
-// 2^-126 <= |x| < 2^128, or zero)
-__device__ __forceinline__ float d2f_guide(double x) {
-  const long long b = dbits(x);
-  const int e = (int)((b >> 52) & 0x7ff) - 1023 + 127;
-  if (e <= 0) return 0.0f;
-  const unsigned u = (unsigned)((b >> 32) & 0x80000000u) | ((unsigned)e << 23) |
-                     (unsigned)((b >> 29) & 0x7fffff);
-  return __uint_as_float(u);
 }
 
 // ------------------------------------------------ log10 / exp10 (FP64) ----
@@ -171,7 +155,7 @@ struct DTable {
   const double *__restrict__ le;   // log10 e
   const double *__restrict__ lp;   // log10 P
   const double *__restrict__ lc;   // log10 cs^2
-  const float *__restrict__ le32;  // log10 e rounded to FP32 (guides the search)
+  const float *__restrict__ le32;  // log10 e rounded to FP32 (the network's inputs)
   const MathTables *__restrict__ mt;   // tables of fast_log10 / fast_exp10 (or null)
   // fixed-point form (tde_fx.cuh; log2 units, Q55), built at load where every
   // entry fits it.  node: per (density cell i, temperature node j) the pairs
@@ -362,14 +346,6 @@ __device__ __forceinline__ double bh_dt2(double dxg, double r2, double rs2) {
 }
 
 // ---------------------------------------------------------------- EOS ----
-
-// floor(x) for 0 <= x < 2^31 (also -0) from the bit fields, on the integer pipe
-__device__ __forceinline__ int ifloor_nonneg(double x) {
-  const long long b = dbits(x);
-  const int e = (int)((b >> 52) & 0x7ff) - 1023;
-  if (e < 0) return 0;
-  return (int)(((b & 0xfffffffffffffLL) | 0x10000000000000LL) >> (52 - e));
-}
 
 // Density cell i and weight w of log10 rho (clamped to the table).
 __device__ __forceinline__ bool rho_cell(const DTable &t, double rho, int &i, double &w) {
@@ -717,11 +693,15 @@ __device__ __forceinline__ void plm(double q0, double dl, double dr, double &lef
   const long long kl = dbits(dl), kr = dbits(dr);
   left = q0;
   right = q0;
-  // dl dr > 0, by the signs (a product that underflows gives h = 0 below)
+  // dl dr > 0: by the signs, and by the product, which is zero where it underflows
+  // (differences of 1e-310, say, whose sum has no finite reciprocal)
   if ((kl ^ kr) >= 0 && (kl << 1) != 0 && (kr << 1) != 0) {
-    const double pr = __dmul_rn(dl, dr), ir = rcp_nr(__dadd_rn(dl, dr));
-    left = __fma_rn(-pr, ir, q0);
-    right = __fma_rn(pr, ir, q0);
+    const double pr = __dmul_rn(dl, dr);
+    if (!dzero(pr)) {
+      const double ir = rcp_nr(__dadd_rn(dl, dr));
+      left = __fma_rn(-pr, ir, q0);
+      right = __fma_rn(pr, ir, q0);
+    }
   }
 }
 // a - b, without the subtraction where a = b on every lane of the warp

@@ -23,7 +23,7 @@
 // test hook makes CTA 0 skip its first arrival, so that the first wait expires.
 //
 // Scope: 3-D meshes without refined-mesh ghost operations whose closure is the
-// ideal gas or the table inverted by bisection (plain or FP32-guided).  The
+// ideal gas or the table inverted by bisection (plain or with the 32-bit search).  The
 // learned-guess closure runs its tensor-core inference in kernels of its own,
 // so its levels stay on the launch sequence.
 #include <math.h>

@@ -392,21 +392,20 @@ def c2_section(ctx, eos, tde, torch, dev, args, fp64_peak, peaks):
 # capture.  They describe the kernels as captured: set KERNELS_AS_CAPTURED to
 # False (achieved, frac and traffic reported as null) whenever a sweep kernel
 # changes.
-FP64_FLOP_PER_CELL_SWEEP = {"sweep_x": 205.2, "sweep_y": 169.7, "sweep_z": 295.7}
-DRAM_BYTES_SWEEP = {"sweep_x": 268.5e6, "sweep_y": 402.6e6, "sweep_z": 545.1e6}
+FP64_FLOP_PER_CELL_SWEEP = {"sweep_x": 103.2, "sweep_y": 77.9, "sweep_z": 100.8}
+DRAM_BYTES_SWEEP = {"sweep_x": 266.9e6, "sweep_y": 398.8e6, "sweep_z": 588.0e6}
 # FP64-pipe issue slots (warp instructions x 32) per interior cell: a DADD or DMUL
 # holds the pipe as long as a DFMA, so the pipe's busy fraction is slots / peak.
-FP64_SLOTS_PER_CELL_SWEEP = {"sweep_x": 187.3, "sweep_y": 187.3, "sweep_z": 275.3}
+FP64_SLOTS_PER_CELL_SWEEP = {"sweep_x": 83.9, "sweep_y": 64.4, "sweep_z": 80.1}
 KERNELS_AS_CAPTURED = True
 # The same for the headline's sweeps (production-shaped mesh, PPM, point mass),
 # from ncu on the 8 x 8 x 4 MeshBlocks around the star of that mesh (8.4 M
 # cells, the same cells and scheme; the full mesh holds ~36 GB on the device,
 # too much for a multi-pass capture), two launches of each sweep averaged,
-# DRAM bytes scaled to the full mesh by its cells (x 8); a one-pass capture of
-# the full mesh gives the same FP64 slots per cell within 2 %.
-FP64_FLOP_PER_CELL_C5 = {"sweep_x": 240.7, "sweep_y": 224.8, "sweep_z": 355.3}
-FP64_SLOTS_PER_CELL_C5 = {"sweep_x": 185.5, "sweep_y": 174.9, "sweep_z": 268.0}
-DRAM_BYTES_C5 = {"sweep_x": 11.00e9, "sweep_y": 15.48e9, "sweep_z": 21.29e9}
+# DRAM bytes scaled to the full mesh by its cells (x 8).
+FP64_FLOP_PER_CELL_C5 = {"sweep_x": 162.8, "sweep_y": 157.4, "sweep_z": 181.0}
+FP64_SLOTS_PER_CELL_C5 = {"sweep_x": 118.2, "sweep_y": 115.5, "sweep_z": 131.9}
+DRAM_BYTES_C5 = {"sweep_x": 10.97e9, "sweep_y": 15.35e9, "sweep_z": 21.24e9}
 KERNELS_AS_CAPTURED_C5 = True
 C5_COUNTERS_NOTE = "profiles/k_sweep_c5_production_ncu.md (8x8x4-block case of the same mesh)"
 

@@ -287,6 +287,103 @@ FX_HD double fx_rsqrt(fx t) {
   return fx_double(((fx)(1021 - (e - odd) / 2) << 52) + (fx)((y + 512) >> 10));
 }
 
+// ------------------------------------------- sums of neighbours by integers ----
+//
+// The multigrid's second differences: significands aligned to the largest exponent of the
+// values, summed exactly, and the sum rounded to FP64.  Not where every value is below
+// 2^-950, nor from 2^1018 up (where a sum may overflow, or a value is infinite or not a
+// number): the sums are taken in FP64 there.
+
+FX_HD bool fx_sum_ok(int emax) { return emax >= 70 && emax <= 2040; }   // exponent field of the largest
+FX_HD int fx_min(int a, int b) {
+#ifdef __CUDA_ARCH__
+  return min(a, b);
+#else
+  return a < b ? a : b;
+#endif
+}
+FX_HD int fx_max(int a, int b) {
+#ifdef __CUDA_ARCH__
+  return max(a, b);
+#else
+  return a > b ? a : b;
+#endif
+}
+// as fx_double, opaque like fx_bits
+FX_HD double fx_value(fx b) {
+#ifdef __CUDA_ARCH__
+  double x;
+  asm("mov.b64 %0, %1;" : "=d"(x) : "l"(b));
+  return x;
+#else
+  return fx_double(b);
+#endif
+}
+
+// sum of the six neighbours n less six times the centre c, to about 2^-58 of the largest
+// of them, with six guard bits (values below that count as zero, as they would in FP64);
+// fp64(): the sum outside the range
+template <class F>
+FX_HD double fx_lap6(double c, const double n[6], F fp64) {
+  fx b[7];
+  b[0] = fx_bits(c);
+#pragma unroll
+  for (int q = 0; q < 6; ++q) b[q + 1] = fx_bits(n[q]);
+  int ex[7], emax = 0;
+#pragma unroll
+  for (int q = 0; q < 7; ++q) {
+    ex[q] = (int)(b[q] >> 52) & 0x7ff;
+    emax = fx_max(emax, ex[q]);
+  }
+  if (!fx_sum_ok(emax)) return fp64();
+  fx s = 0;   // (a zero's hidden bit shifts out: emax >= 70)
+#pragma unroll
+  for (int q = 0; q < 7; ++q) {
+    const ufx m = ((ufx)b[q] & 0xfffffffffffffull) | 0x10000000000000ull;
+    const fx sg = b[q] >> 63;
+    const fx v = ((fx)((m << 6) >> fx_min(emax - ex[q], 63)) ^ sg) - sg;
+    s += q == 0 ? -6 * v : v;
+  }
+  if (s == 0) return 0.0;
+  const ufx a = s < 0 ? -(ufx)s : (ufx)s;
+  const int z = fx_clz(a);               // at least 1
+  const ufx w = a << z;                  // the exponent field less one: 11 to 2043
+  const fx r = ((fx)(emax + 4 - z) << 52) + (fx)((w >> 11) + ((w >> 10) & 1));
+  return fx_value(r | (s & (fx)0x8000000000000000ull));
+}
+
+// sum of the 24 values o around a 2 x 2 x 2 group of cells less three times the eight
+// inside, q (the group's summed second differences: each cell is a neighbour of three
+// others), as fx_lap6 with four guard bits (48 units of the largest value fit); false where
+// it does not apply.  Values down to 1/16 of the largest enter exactly.
+FX_HD bool fx_lap_group(const double q[8], const double o[24], double &sum) {
+  int emax = 0;
+#pragma unroll
+  for (int u = 0; u < 8; ++u) emax = fx_max(emax, (int)(fx_bits(q[u]) >> 52) & 0x7ff);
+#pragma unroll
+  for (int u = 0; u < 24; ++u) emax = fx_max(emax, (int)(fx_bits(o[u]) >> 52) & 0x7ff);
+  if (!fx_sum_ok(emax)) return false;
+  auto part = [emax](double x) {   // (a zero's hidden bit shifts out: emax >= 70)
+    const fx b = fx_bits(x), sg = b >> 63;
+    const ufx m = ((ufx)b & 0xfffffffffffffull) | 0x10000000000000ull;
+    return ((fx)((m << 4) >> fx_min(emax - ((int)(b >> 52) & 0x7ff), 63)) ^ sg) - sg;
+  };
+  fx in = 0, s = 0;
+#pragma unroll
+  for (int u = 0; u < 8; ++u) in += part(q[u]);
+#pragma unroll
+  for (int u = 0; u < 24; ++u) s += part(o[u]);
+  s -= 3 * in;
+  sum = 0.0;
+  if (s == 0) return true;
+  const ufx a = s < 0 ? -(ufx)s : (ufx)s;
+  const int z = fx_clz(a);               // at least 1
+  const ufx w = a << z;                  // the exponent field less one: 13 to 2045
+  const fx r = ((fx)(emax + 6 - z) << 52) + (fx)((w >> 11) + ((w >> 10) & 1));
+  sum = fx_value(r | (s & (fx)0x8000000000000000ull));
+  return true;
+}
+
 // The table's axes in fixed point (the same function of the FP64 axes for every
 // caller).  valid: the format takes them.
 struct FxAxes {

@@ -227,72 +227,13 @@ __device__ __forceinline__ int nbrs6(const Lev &L, const double *phi, int i, int
   return out;
 }
 
-// sum of the six neighbours less six times the centre, to about 2^-58 of the
-// largest of them, on the integer pipe: the significands aligned to the largest
-// exponent with six guard bits, summed exactly, and the sum rounded to FP64.
-// (Values below 2^-58 of the largest count as zero, as they would in FP64; where
-// all are below 2^-950, a call in FP64.)
+// sum of the six neighbours less six times the centre on the integer pipe (fx_lap6), by a
+// call in FP64 outside its range
 __device__ __noinline__ double lap6_fp64(double c, double a, double b, double d, double e, double f, double g) {
   return ((a - c) + (b - c)) + ((d - c) + (e - c)) + ((f - c) + (g - c));
 }
 __device__ __forceinline__ double lap6_int(double c, const double n[6]) {
-  long long b[7];
-  b[0] = dbits(c);
-#pragma unroll
-  for (int q = 0; q < 6; ++q) b[q + 1] = dbits(n[q]);
-  int ex[7], emax = 0;
-#pragma unroll
-  for (int q = 0; q < 7; ++q) {
-    ex[q] = (int)(b[q] >> 52) & 0x7ff;
-    emax = max(emax, ex[q]);
-  }
-  if (emax < 70 || emax == 0x7ff) return lap6_fp64(c, n[0], n[1], n[2], n[3], n[4], n[5]);
-  long long s = 0;   // (a zero's hidden bit shifts out: emax >= 70)
-#pragma unroll
-  for (int q = 0; q < 7; ++q) {
-    const unsigned long long m = ((unsigned long long)b[q] & 0xfffffffffffffull) | 0x10000000000000ull;
-    const long long sg = b[q] >> 63;
-    const long long v = ((long long)((m << 6) >> min(emax - ex[q], 63)) ^ sg) - sg;
-    s += q == 0 ? -6 * v : v;
-  }
-  if (s == 0) return 0.0;
-  const unsigned long long a = s < 0 ? -(unsigned long long)s : (unsigned long long)s;
-  const int z = __clzll((long long)a);
-  const unsigned long long w = a << z;   // E = emax + 4 - z >= 11: the exponent field less one
-  const long long r = ((long long)(emax + 4 - z) << 52) + (long long)((w >> 11) + ((w >> 10) & 1));
-  return dfrom(r | (s & (long long)0x8000000000000000ull));
-}
-
-// sum of the 24 values around a 2 x 2 x 2 group of cells less three times the eight
-// inside (the group's summed second differences: each cell is a neighbour of three
-// others), as lap6_int with four guard bits (48 units of the largest value fit);
-// false where it does not apply.  Values down to 1/16 of the largest enter exactly.
-__device__ __forceinline__ bool lap_group_int(const double q[8], const double o[24], double &sum) {
-  int emax = 0;
-#pragma unroll
-  for (int u = 0; u < 8; ++u) emax = max(emax, (int)(dbits(q[u]) >> 52) & 0x7ff);
-#pragma unroll
-  for (int u = 0; u < 24; ++u) emax = max(emax, (int)(dbits(o[u]) >> 52) & 0x7ff);
-  if (emax < 70 || emax == 0x7ff) return false;
-  auto part = [emax](double x) {   // (a zero's hidden bit shifts out: emax >= 70)
-    const long long b = dbits(x), sg = b >> 63;
-    const unsigned long long m = ((unsigned long long)b & 0xfffffffffffffull) | 0x10000000000000ull;
-    return ((long long)((m << 4) >> min(emax - ((int)(b >> 52) & 0x7ff), 63)) ^ sg) - sg;
-  };
-  long long in = 0, s = 0;
-#pragma unroll
-  for (int u = 0; u < 8; ++u) in += part(q[u]);
-#pragma unroll
-  for (int u = 0; u < 24; ++u) s += part(o[u]);
-  s -= 3 * in;
-  sum = 0.0;
-  if (s == 0) return true;
-  const unsigned long long a = s < 0 ? -(unsigned long long)s : (unsigned long long)s;
-  const int z = __clzll((long long)a);
-  const unsigned long long w = a << z;
-  const long long r = ((long long)(emax + 6 - z) << 52) + (long long)((w >> 11) + ((w >> 10) & 1));
-  sum = dfrom(r | (s & (long long)0x8000000000000000ull));
-  return true;
+  return fx_lap6(c, n, [&] { return lap6_fp64(c, n[0], n[1], n[2], n[3], n[4], n[5]); });
 }
 
 template <int ISO>
@@ -525,7 +466,7 @@ __device__ __forceinline__ void restrict_cells(const Lev &F, const Lev &C, doubl
             o[8 + u] = nbr<ISO>(F, F.phi, i + y, j + side, k + z, 1, side, q[z][side][y], out);
             o[16 + u] = nbr<ISO>(F, F.phi, i + y, j + z, k + side, 2, side, q[side][z][y], out);
           }
-      if (F.eq && lap_group_int(&q[0][0][0], o, sum)) {
+      if (F.eq && fx_lap_group(&q[0][0][0], o, sum)) {
         sd = fma(F.aw[0], sum, sd);
       } else {
         double d[3] = {0.0, 0.0, 0.0};

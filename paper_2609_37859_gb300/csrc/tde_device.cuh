@@ -714,14 +714,19 @@ __device__ __forceinline__ double diff_or_zero(double a, double b) {
 // PPM interface between cells q0 and q1 = q0 + D1, with D0 and D2 the differences
 // below and above: the 4th-order value 7/12 (q0 + q1) - 1/12 (qm1 + q2) is
 // q0 + T/2 with T = D1 + (D0 - D2)/6; clipped to [q0, q1] (T to between 0 and
-// 2 D1, by its sign and magnitude on the integer pipe).  Returns the value and
-// twice its distance from q0 (T) and from q1 (V = 2 D1 - T).
+// 2 D1, by its sign and magnitude on the integer pipe).  At |T| = 2 |D1| the value is q1
+// itself, not q0 + D1: D1 is rounded, and where q1 is below half an ulp of q0 (a floor
+// beside a star) q0 + D1 is zero.  For smaller |T| the exact q0 + T/2 lies short of q1 --
+// T/2 is at least an FP64 step below D1, which is within half a step of q1 - q0 -- and
+// rounding keeps it in [q0, q1].  The limited values q0 - T and q0 + V of ppm_limit are
+// bounded by the neighbours in the same way.  Returns the value and twice its distance
+// from q0 (T) and from q1 (V = 2 D1 - T).
 __device__ __forceinline__ double ppm_iface(double q0, double q1, double D0, double D1, double D2, double &T,
                                             double &V) {
   double t = fma(D0 - D2, 1.0 / 6.0, D1);
   const long long bt = dbits(t), b1 = dbits(D1);
   const long long m1 = b1 & 0x7fffffffffffffffLL;
-  const bool over = (bt & 0x7fffffffffffffffLL) > m1 + 0x10000000000000LL && (bt ^ b1) >= 0;   // |t| > 2 |D1|
+  const bool over = (bt & 0x7fffffffffffffffLL) >= m1 + 0x10000000000000LL && (bt ^ b1) >= 0;   // |t| >= 2 |D1|
   if ((bt ^ b1) < 0 || m1 < 0x10000000000000LL) t = 0.0;   // the other sign, or D1 = 0
   T = t;
   V = fma(2.0, D1, -t);

@@ -409,7 +409,7 @@ inline FxAxes fx_axes(int nr, int nt, double lr0, double lr1, double inv_dlr, do
   const double m = (lr0 < 0 ? -lr0 : lr0) > (lr1 < 0 ? -lr1 : lr1) ? (lr0 < 0 ? -lr0 : lr0) : (lr1 < 0 ? -lr1 : lr1);
   int ex = 0;
   while ((double)(1u << (ex + 1)) <= m) ++ex;      // 2^ex <= largest |log10 rho| (or 1)
-  a.tol = (fx)(3.3219 * (double)(1u << (ex + 1))); // half an ulp of it: 2^(ex - 53) log2(10) 2^55
+  a.tol = (fx)(3.3219 * (double)(1u << (ex + 2))); // half an ulp of it: 2^(ex - 53) log2(10) 2^55
   // 1 / (cell width in log2 units), by integer arithmetic: cells / range
   const long double G = (long double)inv_dlr * 0.30102999566398119521373889472449302677L;   // log10(2)
   int eg = 0;

@@ -116,8 +116,8 @@ FX_HD fx fx_of_log10(double v) {
 // saturates at FX_SAT, x below 2^-127 (or not positive) at -FX_SAT.
 FX_HD fx fx_log2(const FxMath *__restrict__ mt, double x) {
   const fx b = fx_bits(x);
-  const int k = (int)(b >> 52) - 1023;   // negative x: far below -127
-  if (k < -126) return -FX_SAT;
+  const int k = (int)(b >> 52) - 1023;   // floor(log2 x); negative x: far below -127
+  if (k < -127) return -FX_SAT;
   if (k > 126) return FX_SAT;
   const fx mant = b & 0xfffffffffffffLL;
   const int j = (int)(mant >> 44);

@@ -1,6 +1,6 @@
 """The edges of the EOS table in the fixed-point inversion: a density counts as on the table
 up to half an FP64 ulp of log10 rho (of the axis's largest magnitude) beyond an edge, and as
-clamped further out."""
+clamped further out; and the lowest decade of the format."""
 import numpy as np
 import pytest
 
@@ -45,3 +45,21 @@ def test_clamped_densities(lrho):
         c0 = eos.counts()["table_clamp"]
         eos.invert(r, torch.full_like(r, 1e10), P=torch.empty_like(r))
         assert eos.counts()["table_clamp"] - c0 == want
+
+
+def test_lowest_decade_of_the_format(oracle):
+    """Densities and energies between 10^-38 and 2^-126, which a table may still hold."""
+    from paper_2609_37859_gb300 import tde
+    lrho = (-37.99, -37.0)
+    eos, le = _eos(tde, lrho, le0=-37.98)
+    ot = oracle.EOSTable(le.shape[0], le.shape[1], lrho, (2.0, 4.0), le, 0.9 * le, 0.95 * le)
+    rng = np.random.default_rng(3)
+    rho = 10.0 ** rng.uniform(-37.98, -37.9, 400)
+    e = 10.0 ** rng.uniform(-37.94, -37.0, 400)
+    o = [torch.empty(400, dtype=torch.float64, device="cuda") for _ in range(3)]
+    c = eos.invert(torch.from_numpy(rho).cuda(), torch.from_numpy(e).cuda(), T=o[0], P=o[1], cs2=o[2], counts=True)
+    want = np.array([ot.invert(r, x) for r, x in zip(rho, e)])
+    assert c.table_clamp == 0
+    # FP64 logarithms of size 38 are off by at most 2^-48; 1e3 times that covers the slopes
+    for k in range(3):
+        assert np.abs(o[k].cpu().numpy() / want[:, k] - 1).max() < 4e-12

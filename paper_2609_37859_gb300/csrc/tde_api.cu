@@ -99,7 +99,10 @@ bool fill_phys(tde_mesh *m, const tde_params *pr, tde_eos *eos) {
   if (p.eos == EOS_TABLE) {
     if (!eos) return false;
     p.tab = eos->tab;
-    if (p.eos_mode == TDE_INVERT_BISECT_PLAIN) p.tab.n32 = nullptr;   // every step in 64 bits
+    if (p.eos_mode == TDE_INVERT_BISECT_PLAIN) {   // every step in 64 bits
+      p.tab.n32 = nullptr;
+      p.tab.le32 = nullptr;
+    }
   }
   return true;
 }

@@ -71,6 +71,14 @@ __device__ __forceinline__ bool dfinite(double x) { return ((dbits(x) >> 52) & 0
 // -x and |x| by the sign bit
 __device__ __forceinline__ double dneg(double x) { return dfrom(dbits(x) ^ (long long)0x8000000000000000ull); }
 __device__ __forceinline__ double dabs(double x) { return dfrom(dmag(x)); }
+// x truncated to FP32 on the integer pipe (a guide value: normal x with
+// 2^-126 <= |x| < 2^128, or zero)
+__device__ __forceinline__ float dguide(double x) {
+  const long long b = dbits(x);
+  const int e = (int)((b >> 52) & 0x7ff) - 1023 + 127;
+  if (e <= 0) return 0.0f;
+  return __uint_as_float((unsigned)((b >> 32) & 0x80000000u) | ((unsigned)e << 23) | (unsigned)((b >> 29) & 0x7fffff));
+}
 // the double value of a small integer |k| < 2^51, by one FP64 add
 __device__ __forceinline__ double dint(long long k) {
   return __longlong_as_double(0x4338000000000000LL + k) - 6755399441055744.0;
@@ -155,20 +163,26 @@ struct DTable {
   const double *__restrict__ le;   // log10 e
   const double *__restrict__ lp;   // log10 P
   const double *__restrict__ lc;   // log10 cs^2
-  const float *__restrict__ le32;  // log10 e rounded to FP32 (the network's inputs)
+  const float *__restrict__ le32;  // log10 e rounded to FP32 (the network's inputs; the FP64 form's search)
   const MathTables *__restrict__ mt;   // tables of fast_log10 / fast_exp10 (or null)
   // fixed-point form (tde_fx.cuh; log2 units, Q55), built at load where every
   // entry fits it.  node: per (density cell i, temperature node j) the pairs
   // (row i, row i + 1) of log e, log P, log cs^2 in three 16-byte words, so an
   // inversion's last lookups are two runs of 48 bytes; null: from the FP64
-  // arrays (caller-owned views, tables beyond the format)
+  // arrays, in FP64 (a table with an entry outside the format) or, for arrays of a
+  // caller's own, in fixed point unless *outside says that they hold such an entry
   FxAxes fa;
   const FxMath *__restrict__ fm;       // tables of fx_log2 / fx_exp2
   const longlong2 *__restrict__ node;  // [nr - 1][nt][3]
   const int2 *__restrict__ n32;        // [nr - 1][nt] the log e pairs in Q23 (the search)
-  // per density cell and bucket of log e (2^bshift wide from y0): the first and
-  // last temperature cell the inversion can end in (null: search the column)
-  const ushort2 *__restrict__ bk;
+  union {   // (one word for both: the kernels' argument blocks keep their layout)
+    // node given: per density cell and bucket of log e (2^bshift wide from y0), the first
+    // and last temperature cell the inversion can end in (null: search the column)
+    const ushort2 *__restrict__ bk;
+    // node null: whether a caller's arrays hold an entry outside the format (null: a
+    // loaded table, which does)
+    const int *outside;
+  };
   fx y0;
   int bshift, nbk;
 };
@@ -403,7 +417,9 @@ __device__ __forceinline__ double cell_log10T(const DTable &t, int j, double s) 
 // the table's e at the clamped point.  WANT_CS2 = false computes P only (cs2, T
 // and e_used are left untouched).
 //
-// The FP64 form, for tables whose entries the fixed-point format does not take.
+// The FP64 form, for tables with an entry that the fixed-point format does not take:
+// every cell of such a table, so that the bits depend on the table alone.  The search
+// runs on the FP32 copy of log e (le32; null: in FP64), confirmed by the FP64 bracket.
 template <bool WANT_CS2>
 __device__ __forceinline__ bool eos_invert_fp64(const DTable &t, double rho, double e, double &P,
                                                 double &cs2, double &e_used, double *T) {
@@ -413,24 +429,40 @@ __device__ __forceinline__ bool eos_invert_fp64(const DTable &t, double rho, dou
   const int nt = t.nt;
   const double *__restrict__ a = t.le + (size_t)i * nt;
   const double *__restrict__ b = a + nt;
-  const double glo = lerp_rn(w, __ldg(a), __ldg(b));
-  const double ghi = lerp_rn(w, __ldg(a + nt - 1), __ldg(b + nt - 1));
+  auto g = [&](int j) { return lerp_rn(w, __ldg(a + j), __ldg(b + j)); };
   const double y = dgt0(e) ? tlog10(t, e) : -INFINITY;
   int j;
   double s;
-  if (!dlt(glo, y)) {
+  if (!dlt(g(0), y)) {
     j = 0; s = 0.0; cl = true;
-  } else if (dle(ghi, y)) {
+  } else if (dle(g(nt - 1), y)) {
     j = nt - 2; s = 1.0; cl = true;
   } else {
     int lo = 0, hi = nt - 1;
-    while (hi - lo > 1) {
-      const int mid = (lo + hi) >> 1;
-      const double g = lerp_rn(w, __ldg(a + mid), __ldg(b + mid));
-      if (dle(g, y)) lo = mid; else hi = mid;
+    if (t.le32) {
+      const float *__restrict__ a32 = t.le32 + (size_t)i * nt;
+      const float *__restrict__ b32 = a32 + nt;
+      const float w32 = dguide(w), y32 = dguide(y);
+      while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        const float a0 = __ldg(a32 + mid);
+        if (fmaf(w32, __ldg(b32 + mid) - a0, a0) <= y32) lo = mid; else hi = mid;
+      }
     }
     j = lo;
-    s = cell_solve(y, lerp_rn(w, __ldg(a + j), __ldg(b + j)), lerp_rn(w, __ldg(a + j + 1), __ldg(b + j + 1)));
+    double g0 = g(j), g1 = g(j + 1);
+    if (!(dle(g0, y) && dlt(y, g1))) {
+      lo = 0;
+      hi = nt - 1;
+      while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (dle(g(mid), y)) lo = mid; else hi = mid;
+      }
+      j = lo;
+      g0 = g(j);
+      g1 = g(j + 1);
+    }
+    s = cell_solve(y, g0, g1);
   }
   P = texp10(t, bilin(t.lp, nt, i, w, j, s));
   if (WANT_CS2) {
@@ -441,61 +473,56 @@ __device__ __forceinline__ bool eos_invert_fp64(const DTable &t, double rho, dou
   return cl;
 }
 
-// The fixed-point form with every table value converted from the FP64 arrays as
-// it is read and the column searched in full: the same bits as eos_invert's, for
-// the entry that may allocate nothing and so has no prepared table.  Cells whose
-// lookups touch an entry outside the format take the FP64 form.
-__device__ __forceinline__ fx fx_ld(const double *__restrict__ f, size_t k, bool &ok) {
-  const fx v = fx_of_log10(__ldg(f + k));
-  ok = ok && v != FX_BAD;
-  return v;
-}
+// Without the prepared table: the FP64 form, or, for the entry that may allocate nothing
+// (arrays of a caller's own, no entry outside the format), the fixed-point form with the
+// table values converted as they are read -- the same bits as eos_invert's.  The search
+// runs on their FP32 truncations (converting both values of each step put the time step of
+// a 32^3 mesh from 28 to 31 us), confirmed by the 64-bit bracket.
 template <bool WANT_CS2>
 __device__ __noinline__ bool eos_invert_views(const DTable &t, double rho, double e, double &P, double &cs2,
                                               double &e_used, double *T) {
-  if (t.fa.valid && t.fm) {
-    int i;
-    ufx w;
-    bool cl = fx_rho_cell(t.fm, t.fa, t.nr, rho, i, w), ok = true;
-    const int nt = t.nt;
-    const size_t a = (size_t)i * nt, b = a + nt;
-    auto g = [&](const double *f, int j) { return fx_lerp(fx_ld(f, a + j, ok), fx_ld(f, b + j, ok), w); };
-    const fx glo = g(t.le, 0), ghi = g(t.le, nt - 1);
-    const fx y = dgt0(e) ? fx_log2(t.fm, e) : -FX_SAT;
-    int j;
-    ufx s;
-    if (y <= glo) {
-      j = 0; s = 0; cl = true;
-    } else if (y >= ghi) {
-      j = nt - 2; s = ~0ull; cl = true;
-    } else {
-      int lo = 0, hi = nt - 1;
-      while (hi - lo > 1) {
-        const int mid = (lo + hi) >> 1;
-        if (g(t.le, mid) <= y) lo = mid; else hi = mid;
-      }
-      j = lo;
-      const fx g0 = g(t.le, j), g1 = g(t.le, j + 1);
-      ok = ok && g0 <= y && y < g1;
-      s = ok ? fx_frac(y - g0, g1 - g0) : 0;
-    }
-    const fx lp = fx_lerp(g(t.lp, j), g(t.lp, j + 1), s);
-    fx lc = 0, lu = 0;
-    if (WANT_CS2) {
-      lc = fx_lerp(g(t.lc, j), g(t.lc, j + 1), s);
-      if (cl) lu = fx_lerp(g(t.le, j), g(t.le, j + 1), s);
-    }
-    if (ok) {
-      P = fx_exp2(t.fm, lp);
-      if (WANT_CS2) {
-        cs2 = fx_exp2(t.fm, lc);
-        if (T) *T = fx_exp2(t.fm, fx_log2T(t.fa, j, s));
-        e_used = cl ? fx_exp2(t.fm, lu) : e;
-      }
-      return cl;
-    }
+  if (!t.outside || !t.fa.valid || *t.outside) return eos_invert_fp64<WANT_CS2>(t, rho, e, P, cs2, e_used, T);
+  int i;
+  ufx w;
+  bool cl = fx_rho_cell(t.fm, t.fa, t.nr, rho, i, w);
+  const int nt = t.nt;
+  const size_t a = (size_t)i * nt, b = a + nt;
+  auto g = [&](const double *f, int j) {
+    return fx_lerp(fx_of_log10(__ldg(f + a + j)), fx_of_log10(__ldg(f + b + j)), w);
+  };
+  const fx y = dgt0(e) ? fx_log2(t.fm, e) : -FX_SAT;
+  int lo = 0, hi = nt - 1;
+  // (log10 e from the high word, in units of 2^-23 log10(2))
+  const float w32 = (float)(unsigned)(w >> 32) * 2.3283064e-10f, y32 = (float)(int)(y >> 32) * 3.5885572e-8f;
+  while (hi - lo > 1) {
+    const int mid = (lo + hi) >> 1;
+    const float a0 = dguide(__ldg(t.le + a + mid));
+    if (fmaf(w32, dguide(__ldg(t.le + b + mid)) - a0, a0) <= y32) lo = mid; else hi = mid;
   }
-  return eos_invert_fp64<WANT_CS2>(t, rho, e, P, cs2, e_used, T);
+  int j = lo;
+  fx g0 = g(t.le, j), g1 = g(t.le, j + 1);
+  ufx s;
+  for (;;) {   // at most twice
+    if (j == 0 && y <= g0) { s = 0; cl = true; break; }
+    if (j == nt - 2 && y >= g1) { s = ~0ull; cl = true; break; }
+    if (g0 <= y && y < g1) { s = fx_frac(y - g0, g1 - g0); break; }
+    lo = 0;
+    hi = nt - 1;
+    while (hi - lo > 1) {
+      const int mid = (lo + hi) >> 1;
+      if (g(t.le, mid) <= y) lo = mid; else hi = mid;
+    }
+    j = lo;
+    g0 = g(t.le, j);
+    g1 = g(t.le, j + 1);
+  }
+  P = fx_exp2(t.fm, fx_lerp(g(t.lp, j), g(t.lp, j + 1), s));
+  if (WANT_CS2) {
+    cs2 = fx_exp2(t.fm, fx_lerp(g(t.lc, j), g(t.lc, j + 1), s));
+    if (T) *T = fx_exp2(t.fm, fx_log2T(t.fa, j, s));
+    e_used = cl ? fx_exp2(t.fm, fx_lerp(g(t.le, j), g(t.le, j + 1), s)) : e;
+  }
+  return cl;
 }
 
 // a pair (row i, row i + 1) of the prepared table interpolated in density

@@ -1079,7 +1079,10 @@ cudaError_t launch_eos_invert(tde_eos *e, int64_t n, const double *rho, const do
   long long blocks = (n + NT - 1) / NT;
   unsigned g = (unsigned)(blocks < 8LL * n_sm() ? blocks : 8LL * n_sm());
   DTable t = e->tab;
-  if (plain) t.n32 = nullptr;   // no 32-bit guide: every bisection step in 64 bits
+  if (plain) {   // no 32-bit guide: every bisection step in 64 bits
+    t.n32 = nullptr;
+    t.le32 = nullptr;
+  }
   pdl_launch(k_eos_invert, g, NT, 0, s, t, (long long)n, rho, en, T, P, cs2, e->d_cnt);
   return cudaGetLastError();
 }

@@ -444,12 +444,40 @@ __device__ __forceinline__ void cm_split(const CellMap &cm, long long t, long lo
 // brackets it.  An accepted cell is the one bisection finds (g_j <= y < g_{j+1}
 // is unique) and the state is evaluated with the same formulas (eos_at), so the
 // result is the bisection result bit for bit.  Returns false for the cells left
-// to bisection (clamped inputs, a step that misses, a table without the
-// prepared form).
+// to bisection (clamped inputs, a step that misses).  FX: on the prepared table; else in
+// FP64 (tables with an entry outside the fixed-point format).
+template <int FX>
 __device__ __forceinline__ bool newton_cell(const DTable &t, double rho_c, double e, float lTg, float idlt,
                                             double &P, double &cs2, double *T) {
-  if (!t.node || !dgt0(e)) return false;
+  if (!dgt0(e)) return false;
   const int nt = t.nt;
+  if (!FX) {
+    int i;
+    double w;
+    if (rho_cell(t, rho_c, i, w)) return false;
+    const double y = tlog10(t, e);
+    const double *__restrict__ ra = t.le + (size_t)i * nt;
+    const double *__restrict__ rb = ra + nt;
+    const float xg = (lTg - (float)t.lt0) * idlt;
+    int j = (int)floorf(fminf(fmaxf(xg, 0.f), (float)(nt - 2)));
+    j = min(max(j, 0), nt - 2);
+    double g0 = lerp_rn(w, __ldg(ra + j), __ldg(rb + j)), g1 = lerp_rn(w, __ldg(ra + j + 1), __ldg(rb + j + 1));
+    double s = cell_solve(y, g0, g1);
+    if (!(dle(g0, y) && dlt(y, g1))) {
+      const double xn = __dadd_rn(dint(j), s);   // the Newton result, in cell units
+      if (!(xn >= 0.0 && xn < (double)(nt - 1))) return false;
+      j = (int)xn;
+      g0 = lerp_rn(w, __ldg(ra + j), __ldg(rb + j));
+      g1 = lerp_rn(w, __ldg(ra + j + 1), __ldg(rb + j + 1));
+      if (!(dle(g0, y) && dlt(y, g1))) return false;
+      s = cell_solve(y, g0, g1);
+    }
+    if (j == 0 && !dlt(g0, y)) return false;   // (bisection clamps at the coldest node)
+    P = texp10(t, bilin(t.lp, nt, i, w, j, s));
+    cs2 = texp10(t, bilin(t.lc, nt, i, w, j, s));
+    if (T) *T = texp10(t, cell_log10T(t, j, s));
+    return true;
+  }
   int i;
   ufx w;
   if (fx_rho_cell(t.fm, t.fa, t.nr, rho_c, i, w)) return false;
@@ -492,8 +520,9 @@ __device__ __forceinline__ bool newton_cell(const DTable &t, double rho_c, doubl
 // units at a time through the packed FP32 FMA, and the output the inversion does not
 // use is left out (5.9 M cells 780 -> 728 us; one 16-byte record of weights per unit
 // instead of an array per weight was slower, 868 us: a third more shared reads).
-template <int NEWTON, int DUAL = 0>
-__global__ void __launch_bounds__(IT, 8) k_eos_surrogate(const SurrogateArgs a) {
+// FX: the table has the prepared form (newton_cell).
+template <int NEWTON, int DUAL = 0, int FX = 1>
+__global__ void __launch_bounds__(IT, FX ? 8 : 6) k_eos_surrogate(const SurrogateArgs a) {
   pdl_begin();
   __shared__ __align__(1024) unsigned char sA[IT * H * 2];   // h1, BF16, core-matrix layout
   __shared__ __align__(1024) unsigned char sB[H * H * 2];    // W2, BF16, core-matrix layout
@@ -686,8 +715,8 @@ __global__ void __launch_bounds__(IT, 8) k_eos_surrogate(const SurrogateArgs a) 
         rho_c = a.rho[c];
         e_c = a.e[c];
       }
-      const bool ok = live ? (have && newton_cell(a.t, rho_c, e_c, a.nm.cT + a.nm.sT * y0, a.nm.idlt, Pv, cv,
-                                                  NEWTON == 1 && a.T ? &Tv : nullptr))
+      const bool ok = live ? (have && newton_cell<FX>(a.t, rho_c, e_c, a.nm.cT + a.nm.sT * y0, a.nm.idlt, Pv, cv,
+                                                      NEWTON == 1 && a.T ? &Tv : nullptr))
                            : true;
       if (NEWTON == 1 && live && ok) {
         if (a.P) a.P[c] = Pv;
@@ -887,7 +916,8 @@ cudaError_t launch_surrogate_kernel(tde_eos *e, long long n, const float *xin, f
 }
 
 // the network and the Newton step in one pass (k_eos_surrogate<1>): 8 CTAs per
-// SM (64 registers), 8 x 64 TMEM columns fill the SM's 512
+// SM (64 registers), 8 x 64 TMEM columns fill the SM's 512 (six CTAs with the FP64
+// Newton step)
 cudaError_t launch_surrogate_newton(tde_eos *e, const CellMap &cm, long long n, const double *rho,
                                     const double *en, double *T, double *P, double *cs2, double *eu,
                                     long long *queue, unsigned long long *qcount, Counters *cnt,
@@ -909,18 +939,20 @@ cudaError_t launch_surrogate_newton(tde_eos *e, const CellMap &cm, long long n, 
   a.eu = eu;
   a.queue = queue;
   a.qcount = qcount;
-  auto k = k_eos_surrogate<1>;
+  const bool fx = e->tab.node != nullptr;
+  auto k = fx ? k_eos_surrogate<1> : k_eos_surrogate<1, 0, 0>;
   if (hy) {
     a.p = hy->phys;
     a.U = hyU;
     a.W = hy->d_W;
     a.ntot = (long long)hy->ntot;
-    k = hy->phys.dual ? k_eos_surrogate<2, 1> : k_eos_surrogate<2, 0>;
+    if (fx) k = hy->phys.dual ? k_eos_surrogate<2, 1> : k_eos_surrogate<2, 0>;
+    else k = hy->phys.dual ? k_eos_surrogate<2, 1, 0> : k_eos_surrogate<2, 0, 0>;
   }
   int sms = 152;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, e->ctx->device);
   cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
-  const int per_sm = 8;
+  const int per_sm = fx ? 8 : 6;
   const long long tiles = (n + IT - 1) / IT * (cm.blocks ? cm.nblk : 1);
   const unsigned grid = (unsigned)std::min<long long>(tiles, (long long)sms * per_sm);
   pdl_launch(k, grid, IT, 0, s, a);

@@ -27,11 +27,14 @@ using namespace tde;
 
 constexpr int NA_MAX_BLOCKS = 4096;   // largest block count one call accepts
 constexpr int NA_NT = 256;
+constexpr int NA_SCAN = 256;   // CTAs that look a table over
 
 struct NAScratch {
   tde_block_desc blocks[NA_MAX_BLOCKS];      // copy of the caller's block list
   long long off[NA_MAX_BLOCKS + 1];          // first padded cell of each block
   unsigned long long minbits[NA_MAX_BLOCKS]; // per-block CFL minima (IEEE bits)
+  int bad[NA_SCAN], outside;                 // a table entry outside the fixed-point format: per CTA, any
+  unsigned done;                             // CTAs finished (zero between calls)
 };
 
 // The only scratch of this entry point (about 176 KB per device).
@@ -52,8 +55,11 @@ __device__ __forceinline__ void na_bh_pos(const BH &bh, double t, double r[3]) {
   for (int a = 0; a < 3; ++a) r[a] = bh.x0[a] + bh.v0[a] * s + 0.5 * bh.a0[a] * s * s;
 }
 
-// padded sizes, offsets and the +inf initial minima of every block
-__global__ void k_na_setup(NAScratch *S, int nb, Phys p) {
+// padded sizes, offsets and the +inf initial minima of every block; whether the table in
+// the caller's arrays holds an entry outside the fixed-point format (then every cell takes
+// FP64, as with a loaded table)
+__global__ void __launch_bounds__(NA_NT) k_na_setup(NAScratch *S, int nb, Phys p) {
+  pdl_begin();
   if (threadIdx.x == 0 && blockIdx.x == 0) {
     long long o = 0;
     for (int b = 0; b < nb; ++b) {
@@ -65,14 +71,31 @@ __global__ void k_na_setup(NAScratch *S, int nb, Phys p) {
   }
   for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < nb; b += gridDim.x * blockDim.x)
     S->minbits[b] = (unsigned long long)__double_as_longlong(INFINITY);
+  if (p.eos != EOS_TABLE) return;
+  __shared__ int s_last;
+  const long long lim = dbits(FX_MAX_LOG10), n = (long long)p.tab.nr * p.tab.nt;
+  int bad = 0;
+  for (long long k = blockIdx.x * (long long)NA_NT + threadIdx.x; k < n; k += (long long)gridDim.x * NA_NT)
+    bad |= dmag(p.tab.le[k]) >= lim || dmag(p.tab.lp[k]) >= lim || dmag(p.tab.lc[k]) >= lim;
+  bad = __syncthreads_or(bad);
+  if (threadIdx.x == 0) {
+    S->bad[blockIdx.x] = bad;
+    __threadfence();
+    s_last = atomicInc(&S->done, gridDim.x - 1) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  bad = __syncthreads_or(threadIdx.x < gridDim.x && __ldcg(&S->bad[threadIdx.x]));
+  if (threadIdx.x == 0) S->outside = bad;
 }
 
 // The CFL minimum of tde_compute_dt (k_c2p's want_dt path) with the same
 // expressions, so that both entry points give the same bits.
 template <int EOSK, int DUAL>
 __global__ void __launch_bounds__(NA_NT) k_na_cfl(NAScratch *S, Phys p, BH bh,
-                                                  const double *__restrict__ U, long long ntot,
-                                                  const double *__restrict__ t_block) {
+                                                  const double *U, long long ntot, const double *t_block) {
+  pdl_begin();
   const int b = blockIdx.y;
   const tde_block_desc d = S->blocks[b];
   const int n[3] = {d.nx, d.ny, d.nz};
@@ -149,6 +172,7 @@ __global__ void __launch_bounds__(NA_NT) k_na_cfl(NAScratch *S, Phys p, BH bh,
 
 __global__ void __launch_bounds__(1024) k_na_finalize(NAScratch *S, int nb, double cfl,
                                                       double *dt_block, double *dt_min) {
+  pdl_begin();
   __shared__ double red[32];
   double m = INFINITY;
   for (int b = threadIdx.x; b < nb; b += blockDim.x) {
@@ -254,6 +278,7 @@ extern "C" int tde_compute_dt_noalloc(tde_ctx *ctx, int nblocks, const tde_block
     p.tab.lc = table->log10_cs2;
     p.tab.mt = g_mt_ptr[ctx->device];
     p.tab.fm = g_fm_ptr[ctx->device];
+    p.tab.outside = &S->outside;
     p.tab.fa = fx_axes(p.tab.nr, p.tab.nt, p.tab.lr0, table->log10_rho_max, p.tab.inv_dlr, p.tab.lt0, p.tab.dlt);
   }
   p.dxmin = INFINITY;
@@ -306,16 +331,17 @@ extern "C" int tde_compute_dt_noalloc(tde_ctx *ctx, int nblocks, const tde_block
     ctx->err = std::string("tde_compute_dt_noalloc: ") + cudaGetErrorString(err);
     return TDE_ECUDA;
   }
-  k_na_setup<<<(nblocks + 255) / 256, 256, 0, s>>>(S, nblocks, p);
-  dim3 grid_c((unsigned)((max_int + NA_NT - 1) / NA_NT), (unsigned)nblocks);
+  const unsigned gs = p.eos == TDE_EOS_TABLE ? NA_SCAN : (unsigned)((nblocks + NA_NT - 1) / NA_NT);
+  pdl_launch(k_na_setup, gs, NA_NT, 0, s, S, nblocks, p);
+  const dim3 gc((unsigned)((max_int + NA_NT - 1) / NA_NT), (unsigned)nblocks);
   if (p.eos == TDE_EOS_IDEAL) {
-    if (p.dual) k_na_cfl<EOS_IDEAL, 1><<<grid_c, NA_NT, 0, s>>>(S, p, bh, U, ntot, t_block);
-    else k_na_cfl<EOS_IDEAL, 0><<<grid_c, NA_NT, 0, s>>>(S, p, bh, U, ntot, t_block);
+    if (p.dual) pdl_launch(k_na_cfl<EOS_IDEAL, 1>, gc, NA_NT, 0, s, S, p, bh, U, ntot, t_block);
+    else pdl_launch(k_na_cfl<EOS_IDEAL, 0>, gc, NA_NT, 0, s, S, p, bh, U, ntot, t_block);
   } else {
-    if (p.dual) k_na_cfl<EOS_TABLE, 1><<<grid_c, NA_NT, 0, s>>>(S, p, bh, U, ntot, t_block);
-    else k_na_cfl<EOS_TABLE, 0><<<grid_c, NA_NT, 0, s>>>(S, p, bh, U, ntot, t_block);
+    if (p.dual) pdl_launch(k_na_cfl<EOS_TABLE, 1>, gc, NA_NT, 0, s, S, p, bh, U, ntot, t_block);
+    else pdl_launch(k_na_cfl<EOS_TABLE, 0>, gc, NA_NT, 0, s, S, p, bh, U, ntot, t_block);
   }
-  k_na_finalize<<<1, 1024, 0, s>>>(S, nblocks, cfl, dt_block, dt_min);
+  pdl_launch(k_na_finalize, 1, 1024, 0, s, S, nblocks, cfl, dt_block, dt_min);
   err = cudaGetLastError();
   if (err != cudaSuccess) {
     ctx->err = std::string("tde_compute_dt_noalloc: ") + cudaGetErrorString(err);

@@ -637,7 +637,7 @@ __global__ void __launch_bounds__(NT) k_boost(Phys p, const DevBlock *__restrict
 
 // ============================================================ launchers ====
 
-static int n_sm() {
+int n_sm() {
   static int n = 0;
   if (!n) {
     int dev = 0;

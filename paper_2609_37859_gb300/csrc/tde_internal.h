@@ -27,6 +27,8 @@ struct tde_ctx {
 namespace tde {
 // fills the tables of fast_log10 / fast_exp10 (host, extended precision)
 void fill_math_tables(MathTables *h);
+// SMs of the current device
+int n_sm();
 
 // Launches a kernel that begins with pdl_begin() (tde_device.cuh) with programmatic
 // stream serialisation: its launch is prepared while the kernel before it in the

@@ -267,9 +267,9 @@ __global__ void __launch_bounds__(RT) k_remap(RemapDst d, RemapSrc s, const doub
 
 // The same average for target cells at most twice as wide as the source's in every
 // direction (then at most three consecutive entries per direction): a thread walks
-// a column of target cells along z and keeps the x-y averages of the last three
-// source planes, so a plane is averaged once for all target cells that use it, with
-// the products of the x and y weights formed once per column.  The direct form is
+// zs cells of a column along z and keeps the x-y averages of the last three
+// source planes, so a plane is averaged once for all of them that use it, with
+// the products of the x and y weights formed once per run.  The direct form is
 // bound by the FP64 pipe (64 operations per cell of a twofold refinement); this one
 // needs 31: a 128^3 source onto 8.4 M cells went from 0.91 ms to 0.48 ms (the FP64
 // pipe still 86 % busy).
@@ -292,12 +292,13 @@ __device__ __forceinline__ void remap_plane(const double *__restrict__ g, const 
     }
 }
 __global__ void __launch_bounds__(RT, 4) k_remap_columns(RemapDst d, RemapSrc s, const double *__restrict__ G,
-                                                      const Axis *__restrict__ tab) {
+                                                      const Axis *__restrict__ tab, int zs) {
   const DevBlock B = d.blocks[blockIdx.y];
-  const int ncol = B.n[0] * B.n[1];
+  const int ncol = B.n[0] * B.n[1], nseg = (B.n[2] + zs - 1) / zs;
   const long long nc = (long long)s.N[0] * s.N[1] * s.N[2];
-  for (int e = blockIdx.x * RT + threadIdx.x; e < ncol; e += gridDim.x * RT) {
-    const int j = e / B.n[0], i = e - j * B.n[0];
+  for (int e = blockIdx.x * RT + threadIdx.x; e < ncol * nseg; e += gridDim.x * RT) {
+    const int seg = e / ncol, r = e - seg * ncol, j = r / B.n[0], i = r - j * B.n[0];
+    const int k0 = seg * zs, k1 = min(k0 + zs, B.n[2]);
     const Axis &X = tab[B.i0 + i], &Y = tab[d.N[0] + B.j0 + j];
     const int nx = X.n, ny = Y.n;
     double w[RC][RC];
@@ -320,8 +321,8 @@ __global__ void __launch_bounds__(RT, 4) k_remap_columns(RemapDst d, RemapSrc s,
       for (int q = 0; q < 5; ++q) v[p][q] = 0.0;
     const Axis *Zt = tab + d.N[0] + d.N[1] + B.k0;
     const long long plane = (long long)B.p[0] * B.p[1];
-    long long l = B.off + (long long)d.g[2] * plane + (long long)(j + d.g[1]) * B.p[0] + (i + d.g[0]);
-    for (int k = 0; k < B.n[2]; ++k, l += plane) {
+    long long l = B.off + (long long)(k0 + d.g[2]) * plane + (long long)(j + d.g[1]) * B.p[0] + (i + d.g[0]);
+    for (int k = k0; k < k1; ++k, l += plane) {
       const Axis &Z = Zt[k];
       const int nz = nx && ny ? Z.n : 0;   // (a column outside the source reads nothing)
       double acc[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
@@ -426,13 +427,29 @@ cudaError_t launch_remap(tde_mesh *dst, double *Udst, const tde_mesh *src, const
     ProfScope _ps(dst->ctx, TDE_K_REMAP);
     // columns: target cells at most twice as wide (with a margin for roundings: up to
     // three consecutive entries per direction; one along a direction that is not
-    // sampled twice), 32-bit source offsets
-    bool columns = !d.coinc && nc < (1LL << 31);
+    // sampled twice), 32-bit source offsets, more than one plane of target cells (512^2
+    // cells: 34 us by cells, 39 by columns)
+    bool columns = !d.coinc && nc < (1LL << 31) && D.N[2] > 1;
     for (int a = 0; a < 3; ++a) columns = columns && D.dx[a] <= 1.999 * S.dx[a];
     if (columns) {
-      int64_t mc = 1;
-      for (const DevBlock &B : dst->hblocks) mc = std::max<int64_t>(mc, (int64_t)B.n[0] * B.n[1]);
-      k_remap_columns<<<dim3((unsigned)((mc + RT - 1) / RT), (unsigned)dst->nb), RT, 0, st>>>(d, s, G, tab);
+      // Cells of a column per thread: each run of zs cells averages up to two planes more
+      // than zs, so long runs, but threads enough: one and a half waves (zs = 32 / 16 / 8
+      // for 4.1 M cells 496 / 516 / 531 us, for 2.1 M 160 / 150 / 162), down to runs of
+      // four, which are worth idle SMs (262 k cells, zs = 8 / 4 / 2: 39 / 39 / 43); and no
+      // CTA left part empty by small blocks (8^3: 156 us at 8, 129 at 4).  Whole calls, a
+      // thread per column against per cell before: 48^3 cells 68 and 33, now 29 us; 17^3
+      // 72 and 24, now 22; 128^3 160 and 250, now 150.
+      int64_t total = 0, mcol = 1, mz = 1;
+      for (const DevBlock &B : dst->hblocks) {
+        total += (int64_t)B.n[0] * B.n[1] * B.n[2];
+        mcol = std::max<int64_t>(mcol, (int64_t)B.n[0] * B.n[1]);
+        mz = std::max<int64_t>(mz, B.n[2]);
+      }
+      const int64_t wave = 4LL * RT * n_sm();
+      int zs = 32;
+      while (zs > 1 && (total / zs < (zs > 4 ? 3 * wave / 2 : 4 * wave / 5) || mcol * ((mz + zs - 1) / zs) < RT)) zs /= 2;
+      const int64_t mt = mcol * ((mz + zs - 1) / zs);
+      k_remap_columns<<<dim3((unsigned)((mt + RT - 1) / RT), (unsigned)dst->nb), RT, 0, st>>>(d, s, G, tab, zs);
     } else {
       const dim3 grid((unsigned)std::min<int64_t>((dst->max_interior + RT - 1) / RT, 64), (unsigned)dst->nb);
       k_remap<<<grid, RT, 0, st>>>(d, s, G, tab);

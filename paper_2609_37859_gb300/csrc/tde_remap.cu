@@ -274,15 +274,16 @@ __global__ void __launch_bounds__(RT) k_remap(RemapDst d, RemapSrc s, const doub
 // needs 31: a 128^3 source onto 8.4 M cells went from 0.91 ms to 0.48 ms (the FP64
 // pipe still 86 % busy).
 constexpr int RC = 3;
-// the x-y average of one source plane over N x N entries (unused ones have weight
-// zero and the offset of a used one)
+// the x-y average of one source plane over the used ones of N x N entries (bit 4 cy + cx
+// of use; N = 2: all four, so nothing is tested)
 template <int N>
 __device__ __forceinline__ void remap_plane(const double *__restrict__ g, const int off[RC][RC], const double w[RC][RC],
-                                            long long nc, double t[5]) {
+                                            unsigned use, long long nc, double t[5]) {
 #pragma unroll
   for (int cy = 0; cy < N; ++cy)
 #pragma unroll
     for (int cx = 0; cx < N; ++cx) {
+      if (N > 2 && cx + cy > 0 && !(use >> (4 * cy + cx) & 1)) continue;
       const double *r = g + off[cy][cx];
 #pragma unroll
       for (int q = 0; q < 5; ++q) {
@@ -303,15 +304,17 @@ __global__ void __launch_bounds__(RT, 4) k_remap_columns(RemapDst d, RemapSrc s,
     const int nx = X.n, ny = Y.n;
     double w[RC][RC];
     int off[RC][RC];
+    unsigned use = 0;
 #pragma unroll
     for (int cy = 0; cy < RC; ++cy)
 #pragma unroll
       for (int cx = 0; cx < RC; ++cx) {
-        const bool used = cy < ny && cx < nx;
-        w[cy][cx] = used ? Y.w[cy] * X.w[cx] : 0.0;
-        off[cy][cx] = (int)((cy < ny ? Y.off[cy] : Y.off[0]) + (cx < nx ? X.off[cx] : X.off[0]));
+        if (cy < ny && cx < nx) use |= 1u << (4 * cy + cx);
+        w[cy][cx] = Y.w[cy] * X.w[cx];
+        off[cy][cx] = (int)(Y.off[cy] + X.off[cx]);
       }
-    const bool pairs = __all_sync(__activemask(), nx <= 2 && ny <= 2);   // two entries at most in x and y
+    // two entries in x and y on every lane that reads (a vote, so that a warp takes one form)
+    const bool pairs = __all_sync(__activemask(), !use || (nx == 2 && ny == 2));
     const double fxy = X.f * Y.f;
     double v[RC][5];   // the averages of source planes base, base + 1, base + 2
     int base = 0, have = 0;
@@ -344,8 +347,8 @@ __global__ void __launch_bounds__(RT, 4) k_remap_columns(RemapDst d, RemapSrc s,
         for (int p = 0; p < RC; ++p) {
           if (p < have || p >= nz) continue;
           const double *g = G + Z.off[p];
-          if (pairs) remap_plane<2>(g, off, w, nc, v[p]);
-          else remap_plane<RC>(g, off, w, nc, v[p]);
+          if (pairs) remap_plane<2>(g, off, w, use, nc, v[p]);
+          else remap_plane<RC>(g, off, w, use, nc, v[p]);
         }
         if (have < nz) have = nz;
         const double z0 = Z.w[0], z1 = nz > 1 ? Z.w[1] : 0.0;

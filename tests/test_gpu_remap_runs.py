@@ -29,3 +29,18 @@ def test_matches_oracle(oracle, tde, ctx, N, block):
     U = S.om.prim_to_cons(wl.random_smooth(src, seed=9, drho=0.4))
     got, want = remap_both(oracle, tde, S, D, U, tde.REMAP_THERMAL)
     assert_parity(got, want, TOL)   # the remap tests' bound
+
+
+@pytest.mark.parametrize("N,half", [((40, 40, 40), 0.5), ((21, 21, 21), 0.5), ((16, 16, 16), 0.46875), ((64, 20, 20), 0.5)])
+def test_an_infinite_source_cell(oracle, tde, ctx, N, half):
+    """Target cells that sample an infinite density have an infinite density, as the sum of
+    the used entries gives it; the others are untouched."""
+    src = wl.uniform_layout((16, 16, 16), (8, 8, 8), ((-0.5, 0.5),) * 3, bc=(0, 0, 0), ng=2)
+    dst = wl.uniform_layout(N, (8, 8, 8), ((-half, half),) * 3, bc=(0, 0, 0), ng=2)
+    S, D = Side(oracle, tde, ctx, src, 1), Side(oracle, tde, ctx, dst, 1)
+    G = src.to_global(S.om.prim_to_cons(wl.random_smooth(src, seed=9)))
+    G[0, 5, 7, 9] = np.inf
+    with np.errstate(invalid="ignore"):
+        got, want = remap_both(oracle, tde, S, D, src.from_global(G), tde.REMAP_THERMAL)
+    assert np.isinf(got[0]).any() and np.array_equal(np.isposinf(got[0]), np.isposinf(want[0]))
+    assert not np.isnan(got[0]).any() and not np.isnan(want[0]).any()

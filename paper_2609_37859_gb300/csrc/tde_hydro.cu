@@ -969,8 +969,9 @@ cudaError_t launch_sweeps(tde_mesh *m, int stage, const double *U0, const double
 // Time every tile shape that fits in shared memory on each active direction
 // (one warm-up and `reps` timed launches over all blocks, CUDA events on the
 // context's stream) and keep the fastest.  The sweeps read the bound state and
-// the primitives computed from it here, and write only scratch arrays: the
-// state, the counters and the workspaces the next step reads are untouched.
+// the primitives computed from it here, and write only scratch arrays and the
+// counters, which are put back: the state and the workspaces the next step reads are
+// untouched.
 cudaError_t autotune_sweeps(tde_mesh *m, const BH &bh, int reps, float ms_out[3][N_TILE_SHAPES]) {
   tde_ctx *c = m->ctx;
   cudaStream_t s = c->stream;
@@ -1001,7 +1002,6 @@ cudaError_t autotune_sweeps(tde_mesh *m, const BH &bh, int reps, float ms_out[3]
       if (sweep_smem_for(m, D, t) > SWEEP_SMEM_LIMIT) continue;
       SweepArgs a = sweep_args(m, 0, m->U, m->U, Uo, m->d_allids, bh, ta, nullptr);
       a.dU = dU;
-      a.cnt = nullptr;
       err = sweep_dir(m, a, D, t, D == firstD, D == lastD, m->nb);
       if (err == cudaSuccess) err = cudaEventRecord(e0, s);
       for (int r = 0; r < reps && err == cudaSuccess; ++r)

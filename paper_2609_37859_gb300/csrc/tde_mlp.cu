@@ -1166,8 +1166,8 @@ extern "C" int tde_eos_surrogate_train(tde_eos *e, uint64_t seed, int n_samples,
   }
   c->launches[TDE_K_EOS] += (uint64_t)nbt + 1;
   if (rep) {
-    rep->loss_first = losses.front();
-    rep->loss_last = losses.back();
+    rep->loss_first = nbt ? losses.front() : 0.0;   // (fewer samples than a batch: nothing to train on)
+    rep->loss_last = nbt ? losses.back() : 0.0;
     rep->epochs = epochs;
     rep->samples = n_samples;
     rep->batches = nbt;

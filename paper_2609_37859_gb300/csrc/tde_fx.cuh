@@ -191,7 +191,8 @@ FX_HD ufx fx_frac(fx num, fx den) {
 //
 // The same trade as above for the refined reciprocals of the hydro kernels: an
 // FP32 seed of the significand (MUFU), a residual exact in 64 bits and a
-// second-order correction give the FP64 result within 0.51 ulp in about 40
+// second-order correction give the reciprocal within 0.51 ulp and the roots
+// within 0.52 (0.501, 0.516 and 0.514 over 4 M random arguments) in about 40
 // integer instructions (20 cycles per warp and SM), where the FP64 refinement
 // took 3 slots (48 cycles) for 1/d, 7 for sqrt(a/b), 5 for 1/sqrt(t).  For normal
 // arguments whose result is normal; *_ok says so from the exponent fields.

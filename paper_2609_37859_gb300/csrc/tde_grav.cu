@@ -597,7 +597,7 @@ __global__ void __launch_bounds__(GT) k_mg_prolong(Lev F, Lev C) {
 // each side; wrapped, or mirrored with a sign flip beyond an isolated face) and
 // applies the 4-tap weights one direction at a time (x, then y, then z), the same
 // weights summed in another order: 9.3 FMAs per fine cell at T = 16 and 12 at
-// T = 8 instead of 64.  T = 16 wherever the level has at least 152 such tiles.
+// T = 8 instead of 64.  T = 16 wherever the level has at least one such tile per SM.
 __device__ double full_value(const Lev &C, const MP &mp, int u0, int u1, int u2);
 // FULL = 0: the V-cycle's correction (C.tmp, odd mirror images, added to F.phi);
 // FULL = 1: the full-multigrid start's solution (C.phi with its boundary values,
@@ -674,7 +674,7 @@ __host__ __forceinline__ int prolong_tile(const Lev &F, const Lev &C) {
     ok16 = ok16 && F.n[a] % 16 == 0;
   }
   if (!ok8) return 0;
-  return ok16 && (long long)F.n[0] * F.n[1] * F.n[2] >= 152LL * 4096 ? 16 : 8;
+  return ok16 && (long long)F.n[0] * F.n[1] * F.n[2] >= 4096LL * n_sm() ? 16 : 8;
 }
 template <int FULL>
 void launch_prolong_tiled(const Lev &F, const Lev &C, const MP &mp, int T, cudaStream_t s) {
@@ -1017,7 +1017,7 @@ __global__ void __launch_bounds__(GT) k_mp_faces(FaceJob job, MP mp, double *out
 }
 
 unsigned grid_for(long long n) {
-  return (unsigned)std::max<long long>(1, std::min<long long>((n + GT - 1) / GT, 152LL * 8));
+  return (unsigned)std::max<long long>(1, std::min<long long>((n + GT - 1) / GT, 8LL * n_sm()));
 }
 
 }  // namespace
@@ -1227,7 +1227,7 @@ static void multipole_setup(GravState *g, int lmax, cudaStream_t s) {
   pdl_launch(k_mp_centroid, gr, GT, 0, s, L0, g->part);
   pdl_launch(k_mp_centre, 1, GT, 0, s, g->part, (int)gr, L0, g->mp);
   // (a warp's reduction of the 30 sums costs as much as several cells: few CTAs)
-  const unsigned grm = std::min(gr, 304u);
+  const unsigned grm = std::min(gr, 2u * (unsigned)n_sm());
   switch (lmax) {
     case 0: pdl_launch(k_mp_moments<0>, grm, GT, 0, s, L0, g->mp, g->mpart); break;
     case 1: pdl_launch(k_mp_moments<1>, grm, GT, 0, s, L0, g->mp, g->mpart); break;
@@ -1265,7 +1265,7 @@ static void full_multigrid(GravState *g, const tde_grav_params &gp, int lmax, cu
     if (const int T = prolong_tile(F, g->lev[l + 1]))
       launch_prolong_tiled<1>(F, g->lev[l + 1], mp, T, s);
     else
-      pdl_launch(k_mg_prolong_full, (unsigned)std::min<long long>((long long)F.n[0] * F.n[1] * F.n[2], 152LL * 32), 32, 0, s, F, g->lev[l + 1], mp);
+      pdl_launch(k_mg_prolong_full, (unsigned)std::min<long long>((long long)F.n[0] * F.n[1] * F.n[2], 32LL * n_sm()), 32, 0, s, F, g->lev[l + 1], mp);
     g->launches += 1;
     vcycle(g, l, gp, s);
     if (l == 0) smooth(g, F, gp.omega, s);

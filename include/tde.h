@@ -148,10 +148,11 @@ TDE_API int tde_eos_destroy(tde_eos *eos);
 
 /* Invert n cells (rho, e) -> (T, P, cs2), all cgs, device arrays of n doubles.
  * The logarithms, interpolations and the solve are in 64-bit fixed point (55
- * fraction bits of log2; finer than FP64 logarithms of this size); tables with
- * an entry of magnitude 38 or more (log10), and tables loaded without device memory
- * for their fixed-point form (88 bytes an entry beside the arrays' 28), take FP64
- * instead.
+ * fraction bits of log2; finer than FP64 logarithms of this size); a table with an
+ * entry of magnitude 38 or more (log10) at a corner is inverted in FP64 instead, as
+ * are the cells at such an entry elsewhere.  Loading prepares the fixed-point form
+ * (88 bytes an entry beside the arrays' 28) if every entry fits it and device memory
+ * allows; else values are converted as they are read, with the same results.
  * mode TDE_INVERT_BISECT: binary search of the interpolated log e column, on a
  * rounded 32-bit copy of the part of the table that log e bounds, confirmed by
  * the 64-bit bracket of the cell (64-bit bisection where it cannot decide);

@@ -213,8 +213,8 @@ __global__ void k_fx_buckets(const longlong2 *__restrict__ nd, int nr, int nt, f
 }
 
 // One allocation: the log2 / exp2 tables, then the above (about 88 bytes an entry).  A
-// table with an entry outside the format, or without room for that much, keeps none of it,
-// and every cell goes through the FP64 arrays.
+// table with an entry outside the format, or without room for that much, keeps the former
+// only, and its values are converted as they are read (eos_invert_views).
 static cudaError_t load_fx_table(tde_eos *e, double lr_max, const double *le, const double *lp, const double *lc) {
   DTable &t = e->tab;
   const int nr = t.nr, nt = t.nt;
@@ -223,17 +223,22 @@ static cudaError_t load_fx_table(tde_eos *e, double lr_max, const double *le, co
   bool ok = t.fa.valid;
   for (size_t k = 0; k < nn; ++k)
     ok = ok && fabs(le[k]) < FX_MAX_LOG10 && fabs(lp[k]) < FX_MAX_LOG10 && fabs(lc[k]) < FX_MAX_LOG10;
-  if (!ok) return cudaSuccess;
+  for (int k = 0; k < 4; ++k)
+    if (corner_outside(nr, nt, k, le, lp, lc)) t.fa.valid = 0;   // in FP64 as a whole
   // bucket width: the smallest power of two that needs at most 8 nt buckets (the columns
   // increase: the ends hold the extremes)
-  fx y0 = fx_of_log10(le[0]), y1 = fx_of_log10(le[nt - 1]);
-  for (int i = 1; i < nr; ++i) {
-    y0 = std::min(y0, fx_of_log10(le[(size_t)i * nt]));
-    y1 = std::max(y1, fx_of_log10(le[(size_t)i * nt + nt - 1]));
+  int sh = 32, nbk = 0;
+  fx y0 = 0;
+  if (ok) {
+    fx y1 = fx_of_log10(le[nt - 1]);
+    y0 = fx_of_log10(le[0]);
+    for (int i = 1; i < nr; ++i) {
+      y0 = std::min(y0, fx_of_log10(le[(size_t)i * nt]));
+      y1 = std::max(y1, fx_of_log10(le[(size_t)i * nt + nt - 1]));
+    }
+    while (((y1 - y0) >> sh) + 1 > 8LL * nt) ++sh;
+    nbk = (int)((y1 - y0) >> sh) + 1;
   }
-  int sh = 32;
-  while (((y1 - y0) >> sh) + 1 > 8LL * nt) ++sh;
-  const int nbk = (int)((y1 - y0) >> sh) + 1;
   size_t size = sizeof(FxMath);
   auto part = [&](size_t bytes) {
     const size_t o = (size + 15) / 16 * 16;
@@ -245,14 +250,16 @@ static cudaError_t load_fx_table(tde_eos *e, double lr_max, const double *le, co
   const size_t o_bk = buckets ? part(sizeof(ushort2) * (size_t)(nr - 1) * nbk) : 0;
   FxMath fm;
   fx_fill_math(&fm);
-  cudaError_t err = cudaMalloc(&e->d_fx, size);
+  cudaError_t err = ok ? cudaMalloc(&e->d_fx, size) : cudaErrorMemoryAllocation;
   if (err == cudaErrorMemoryAllocation) {
-    cudaGetLastError();
-    e->d_fx = nullptr;
-    return cudaSuccess;
+    if (ok) cudaGetLastError();
+    ok = false;
+    err = cudaMalloc(&e->d_fx, sizeof fm);
   }
   if (err == cudaSuccess) err = cudaMemcpy(e->d_fx, &fm, sizeof fm, cudaMemcpyHostToDevice);
   if (err != cudaSuccess) return err;
+  t.fm = reinterpret_cast<const FxMath *>(e->d_fx);
+  if (!ok) return cudaSuccess;
   longlong2 *node = reinterpret_cast<longlong2 *>(e->d_fx + o_node);
   int2 *n32 = reinterpret_cast<int2 *>(e->d_fx + o_n32);
   ushort2 *bk = buckets ? reinterpret_cast<ushort2 *>(e->d_fx + o_bk) : nullptr;
@@ -266,7 +273,6 @@ static cudaError_t load_fx_table(tde_eos *e, double lr_max, const double *le, co
   err = cudaGetLastError();
   if (err == cudaSuccess) err = cudaStreamSynchronize(s);   // (the handle may be used on another stream)
   if (err != cudaSuccess) return err;
-  t.fm = reinterpret_cast<const FxMath *>(e->d_fx);
   t.node = node;
   t.n32 = n32;
   t.bk = bk;

@@ -168,9 +168,8 @@ struct DTable {
   // fixed-point form (tde_fx.cuh; log2 units, Q55), built at load where every
   // entry fits it.  node: per (density cell i, temperature node j) the pairs
   // (row i, row i + 1) of log e, log P, log cs^2 in three 16-byte words, so an
-  // inversion's last lookups are two runs of 48 bytes; null: from the FP64
-  // arrays, in FP64 (a table with an entry outside the format) or, for arrays of a
-  // caller's own, in fixed point unless *outside says that they hold such an entry
+  // inversion's last lookups are two runs of 48 bytes; null: converted from the FP64
+  // arrays as they are read (eos_invert_views)
   FxAxes fa;
   const FxMath *__restrict__ fm;       // tables of fx_log2 / fx_exp2
   const longlong2 *__restrict__ node;  // [nr - 1][nt][3]
@@ -179,8 +178,8 @@ struct DTable {
     // node given: per density cell and bucket of log e (2^bshift wide from y0), the first
     // and last temperature cell the inversion can end in (null: search the column)
     const ushort2 *__restrict__ bk;
-    // node null: whether a caller's arrays hold an entry outside the format (null: a
-    // loaded table, which does)
+    // node null: a caller's arrays, where this says whether a corner entry is outside the
+    // format (null: a loaded table, whose fa says that)
     const int *outside;
   };
   fx y0;
@@ -417,9 +416,19 @@ __device__ __forceinline__ double cell_log10T(const DTable &t, int j, double s) 
 // the table's e at the clamped point.  WANT_CS2 = false computes P only (cs2, T
 // and e_used are left untouched).
 //
-// The FP64 form, for tables with an entry that the fixed-point format does not take:
-// every cell of such a table, so that the bits depend on the table alone.  The search
-// runs on the FP32 copy of log e (le32; null: in FP64), confirmed by the FP64 bracket.
+// The FP64 form, for entries that the fixed-point format does not take.  The search runs on
+// the FP32 copy of log e (le32; null: in FP64) and is confirmed by the FP64 bracket.
+template <bool WANT_CS2>
+__device__ __forceinline__ void fp64_cell(const DTable &t, int i, double w, int j, double s, bool cl, double e, double &P,
+                                          double &cs2, double &e_used, double *T) {
+  const int nt = t.nt;
+  P = texp10(t, bilin(t.lp, nt, i, w, j, s));
+  if (WANT_CS2) {
+    cs2 = texp10(t, bilin(t.lc, nt, i, w, j, s));
+    if (T) *T = texp10(t, cell_log10T(t, j, s));
+    e_used = cl ? texp10(t, bilin(t.le, nt, i, w, j, s)) : e;
+  }
+}
 template <bool WANT_CS2>
 __device__ __forceinline__ bool eos_invert_fp64(const DTable &t, double rho, double e, double &P,
                                                 double &cs2, double &e_used, double *T) {
@@ -464,65 +473,92 @@ __device__ __forceinline__ bool eos_invert_fp64(const DTable &t, double rho, dou
     }
     s = cell_solve(y, g0, g1);
   }
-  P = texp10(t, bilin(t.lp, nt, i, w, j, s));
-  if (WANT_CS2) {
-    cs2 = texp10(t, bilin(t.lc, nt, i, w, j, s));
-    if (T) *T = texp10(t, cell_log10T(t, j, s));
-    e_used = cl ? texp10(t, bilin(t.le, nt, i, w, j, s)) : e;
-  }
+  fp64_cell<WANT_CS2>(t, i, w, j, s, cl, e, P, cs2, e_used, T);
   return cl;
 }
 
-// Without the prepared table: the FP64 form, or, for the entry that may allocate nothing
-// (arrays of a caller's own, no entry outside the format), the fixed-point form with the
-// table values converted as they are read -- the same bits as eos_invert's.  The search
-// runs on their FP32 truncations (converting both values of each step put the time step of
-// a 32^3 mesh from 28 to 31 us), confirmed by the 64-bit bracket.
+// The fixed-point results in temperature cell j of density cell i, every table value
+// converted as it is read; false if the cell does not hold y (nor clamps it), or one of its
+// entries is outside the format (then out is set).  The same bits as eos_invert's.
+template <bool WANT_CS2>
+__device__ __forceinline__ bool fx_cell_views(const DTable &t, int i, ufx w, fx y, int j, bool &cl, bool &out, double e,
+                                              double &P, double &cs2, double &e_used, double *T) {
+  const size_t a = (size_t)i * t.nt + j, b = a + t.nt;
+  int top = 0;   // the largest high word of a magnitude (38 has a low word of zero)
+  auto g = [&](const double *f, int k) {
+    const double u = __ldg(f + a + k), v = __ldg(f + b + k);
+    top = max(top, max((int)(dmag(u) >> 32), (int)(dmag(v) >> 32)));
+    return fx_lerp(fx_of_log10_in(u), fx_of_log10_in(v), w);
+  };
+  auto outside = [&] { return top >= (int)(fx_bits(FX_MAX_LOG10) >> 32); };
+  const fx g0 = g(t.le, 0), g1 = g(t.le, 1);
+  out = outside();
+  if (out) return false;
+  ufx s;
+  bool c = true;
+  if (j == 0 && y <= g0) s = 0;
+  else if (j == t.nt - 2 && y >= g1) s = ~0ull;
+  else if (g0 <= y && y < g1) { s = fx_frac(y - g0, g1 - g0); c = false; }
+  else return false;
+  const bool clamped = cl || c;
+  P = fx_exp2(t.fm, fx_lerp(g(t.lp, 0), g(t.lp, 1), s));
+  if (WANT_CS2) {
+    cs2 = fx_exp2(t.fm, fx_lerp(g(t.lc, 0), g(t.lc, 1), s));
+    if (T) *T = fx_exp2(t.fm, fx_log2T(t.fa, j, s));
+    e_used = clamped ? fx_exp2(t.fm, fx_lerp(g0, g1, s)) : e;
+  }
+  out = outside();
+  if (!out) cl = clamped;
+  return !out;
+}
+
+// Without the prepared table.  One with an entry outside the format at a corner (where a
+// table that increases along both axes has its extremes) is inverted in FP64 as a whole: no
+// cell pays for both forms (2^22 inversions 0.73 ms; 0.89 to 0.98 with a choice per cell).
+// Others -- a caller's arrays, a table loaded without room for the prepared form, entries
+// outside elsewhere in the table -- cell by cell: in fixed point, with eos_invert's
+// bits, where the cell's entries are inside the format, else in FP64.  Which of the two
+// depends on the table and the input alone: where the cell of the FP32 search (on truncations
+// of log e) does not hold log e or an entry is outside, the 64-bit search decides, with
+// entries outside the format taken at its ends (the columns increase, so a cell inside is
+// found).
+// (Calls within calls, so that the kernels that never get here save no registers for it.)
+template <bool WANT_CS2>
+__device__ __forceinline__ int eos_invert_cells(const DTable &t, double rho, double e, double &P, double &cs2,
+                                             double &e_used, double *T) {   // -1: FP64
+  int i;
+  ufx w;
+  bool cl = fx_rho_cell(t.fm, t.fa, t.nr, rho, i, w), out;
+  const int nt = t.nt;
+  const double *__restrict__ a = t.le + (size_t)i * nt;
+  const double *__restrict__ b = a + nt;
+  const fx y = dgt0(e) ? fx_log2(t.fm, e) : -FX_SAT;
+  int lo = 0, hi = nt - 1;
+  bool all = !t.le32 && !t.outside;   // every step in 64 bits
+  if (!all) {
+    const float w32 = (float)(unsigned)(w >> 32) * 2.3283064e-10f;   // 2^-32
+    const float y32 = (float)(int)(y >> 32) * 3.5885572e-8f;         // 2^-23 log10(2)
+    while (hi - lo > 1) {
+      const int mid = (lo + hi) >> 1;
+      const float u = dguide(__ldg(a + mid));
+      if (fmaf(w32, dguide(__ldg(b + mid)) - u, u) <= y32) lo = mid; else hi = mid;
+    }
+    if (fx_cell_views<WANT_CS2>(t, i, w, y, lo, cl, out, e, P, cs2, e_used, T)) return cl;
+    lo = 0;
+    hi = nt - 1;
+  }
+  while (hi - lo > 1) {
+    const int mid = (lo + hi) >> 1;
+    if (fx_lerp(fx_of_log10_sat(__ldg(a + mid)), fx_of_log10_sat(__ldg(b + mid)), w) <= y) lo = mid; else hi = mid;
+  }
+  return fx_cell_views<WANT_CS2>(t, i, w, y, lo, cl, out, e, P, cs2, e_used, T) ? (int)cl : -1;
+}
 template <bool WANT_CS2>
 __device__ __noinline__ bool eos_invert_views(const DTable &t, double rho, double e, double &P, double &cs2,
                                               double &e_used, double *T) {
-  if (!t.outside || !t.fa.valid || *t.outside) return eos_invert_fp64<WANT_CS2>(t, rho, e, P, cs2, e_used, T);
-  int i;
-  ufx w;
-  bool cl = fx_rho_cell(t.fm, t.fa, t.nr, rho, i, w);
-  const int nt = t.nt;
-  const size_t a = (size_t)i * nt, b = a + nt;
-  auto g = [&](const double *f, int j) {
-    return fx_lerp(fx_of_log10(__ldg(f + a + j)), fx_of_log10(__ldg(f + b + j)), w);
-  };
-  const fx y = dgt0(e) ? fx_log2(t.fm, e) : -FX_SAT;
-  int lo = 0, hi = nt - 1;
-  // (log10 e from the high word, in units of 2^-23 log10(2))
-  const float w32 = (float)(unsigned)(w >> 32) * 2.3283064e-10f, y32 = (float)(int)(y >> 32) * 3.5885572e-8f;
-  while (hi - lo > 1) {
-    const int mid = (lo + hi) >> 1;
-    const float a0 = dguide(__ldg(t.le + a + mid));
-    if (fmaf(w32, dguide(__ldg(t.le + b + mid)) - a0, a0) <= y32) lo = mid; else hi = mid;
-  }
-  int j = lo;
-  fx g0 = g(t.le, j), g1 = g(t.le, j + 1);
-  ufx s;
-  for (;;) {   // at most twice
-    if (j == 0 && y <= g0) { s = 0; cl = true; break; }
-    if (j == nt - 2 && y >= g1) { s = ~0ull; cl = true; break; }
-    if (g0 <= y && y < g1) { s = fx_frac(y - g0, g1 - g0); break; }
-    lo = 0;
-    hi = nt - 1;
-    while (hi - lo > 1) {
-      const int mid = (lo + hi) >> 1;
-      if (g(t.le, mid) <= y) lo = mid; else hi = mid;
-    }
-    j = lo;
-    g0 = g(t.le, j);
-    g1 = g(t.le, j + 1);
-  }
-  P = fx_exp2(t.fm, fx_lerp(g(t.lp, j), g(t.lp, j + 1), s));
-  if (WANT_CS2) {
-    cs2 = fx_exp2(t.fm, fx_lerp(g(t.lc, j), g(t.lc, j + 1), s));
-    if (T) *T = fx_exp2(t.fm, fx_log2T(t.fa, j, s));
-    e_used = cl ? fx_exp2(t.fm, fx_lerp(g(t.le, j), g(t.le, j + 1), s)) : e;
-  }
-  return cl;
+  int r = -1;
+  if (t.fa.valid && !(t.outside && *t.outside)) r = eos_invert_cells<WANT_CS2>(t, rho, e, P, cs2, e_used, T);
+  return r < 0 ? eos_invert_fp64<WANT_CS2>(t, rho, e, P, cs2, e_used, T) : r > 0;
 }
 
 // a pair (row i, row i + 1) of the prepared table interpolated in density
@@ -552,9 +588,8 @@ __device__ __forceinline__ void eos_at(const DTable &t, const longlong2 *__restr
 // the buckets (1 or 2 search loads instead of 8) and the node pairs (6 loads for
 // all of a cell's 12 values) matter as much as the arithmetic.
 template <bool WANT_CS2 = true>
-__device__ __forceinline__ bool eos_invert(const DTable &t, double rho, double e, double &P,
-                                           double &cs2, double &e_used, double *T = nullptr) {
-  if (!t.node) return eos_invert_views<WANT_CS2>(t, rho, e, P, cs2, e_used, T);   // uniform
+__device__ __forceinline__ bool eos_invert_node(const DTable &t, double rho, double e, double &P,
+                                                double &cs2, double &e_used, double *T = nullptr) {
   int i;
   ufx w;
   bool cl = fx_rho_cell(t.fm, t.fa, t.nr, rho, i, w);
@@ -604,6 +639,14 @@ __device__ __forceinline__ bool eos_invert(const DTable &t, double rho, double e
   return cl;
 }
 
+// the inversion for whatever table the kernel got
+template <bool WANT_CS2 = true>
+__device__ __forceinline__ bool eos_invert(const DTable &t, double rho, double e, double &P,
+                                           double &cs2, double &e_used, double *T = nullptr) {
+  if (!t.node) return eos_invert_views<WANT_CS2>(t, rho, e, P, cs2, e_used, T);   // uniform
+  return eos_invert_node<WANT_CS2>(t, rho, e, P, cs2, e_used, T);
+}
+
 // The table's inputs (cgs density and specific internal energy) of a cell with
 // density rho and internal energy density U in code units.
 __device__ __forceinline__ void eos_inputs(const Phys &p, double rho, double U, double &rho_c,
@@ -620,8 +663,9 @@ struct EOSBuf {
 };
 
 // EOS closure in code units: internal energy density U at density rho ->
-// P, cs^2 and the internal energy the table actually represents.  EOSB: take
-// the table results of the cell at index flat from eb instead of inverting.
+// P, cs^2 and the internal energy the table actually represents.  EOSB = 1: take
+// the table results of the cell at index flat from eb instead of inverting; 2: the
+// table has the prepared form (no call that the kernel keeps registers for).
 template <int EOSK, int EOSB = 0>
 __device__ __forceinline__ void eos_closure(const Phys &p, double rho, double U, double &P,
                                             double &cs2, double &Uu, Counters *cnt,
@@ -633,7 +677,7 @@ __device__ __forceinline__ void eos_closure(const Phys &p, double rho, double U,
   } else {
     double Pc, c2c, eu;
     bool cl;
-    if (EOSB) {
+    if (EOSB == 1) {
       Pc = eb->P[flat];
       c2c = eb->cs2[flat];
       eu = eb->eu[flat];
@@ -641,7 +685,7 @@ __device__ __forceinline__ void eos_closure(const Phys &p, double rho, double U,
     } else {
       double rc, ec;
       eos_inputs(p, rho, U, rc, ec);
-      cl = eos_invert(p.tab, rc, ec, Pc, c2c, eu);
+      cl = EOSB == 2 ? eos_invert_node(p.tab, rc, ec, Pc, c2c, eu) : eos_invert(p.tab, rc, ec, Pc, c2c, eu);
     }
     if (cl && cnt) count(&cnt->table_clamp);
     P = Pc * p.inv_unit_p;
@@ -651,11 +695,14 @@ __device__ __forceinline__ void eos_closure(const Phys &p, double rho, double U,
 }
 
 // Pressure of internal energy density U at density rho (code units), table EOS
-// (the compression source of Eq. dual-tabulated-compression needs P only).
+// (the compression source of Eq. dual-tabulated-compression needs P only).  PREP: the
+// table has its prepared form.
+template <int PREP>
 __device__ __forceinline__ double table_pressure(const Phys &p, double rho, double U,
                                                  Counters *cnt) {
   double Pc, c2c, eu;
-  bool cl = eos_invert<false>(p.tab, rho * p.unit_rho, (U * rcp_nr(rho)) * p.unit_e, Pc, c2c, eu);
+  const double rc = rho * p.unit_rho, ec = (U * rcp_nr(rho)) * p.unit_e;
+  const bool cl = PREP ? eos_invert_node<false>(p.tab, rc, ec, Pc, c2c, eu) : eos_invert<false>(p.tab, rc, ec, Pc, c2c, eu);
   if (cl && cnt) count(&cnt->table_clamp);
   return Pc * p.inv_unit_p;
 }

@@ -98,18 +98,27 @@ FX_HD int fx_clz(ufx a) {
 #endif
 }
 
-// log10 value v (a table entry, FP64) in Q55 log2 units, rounded to nearest;
-// FX_BAD if it is not below FX_MAX_LOG10 in magnitude (or not a number)
-FX_HD fx fx_of_log10(double v) {
+// log10 value v (a table entry, FP64, below FX_MAX_LOG10 in magnitude) in Q55 log2 units,
+// rounded to nearest
+FX_HD fx fx_of_log10_in(double v) {
   const fx b = fx_bits(v), a = b & 0x7fffffffffffffffLL;
-  if (a >= fx_bits(FX_MAX_LOG10)) return FX_BAD;
   const int e = (int)(a >> 52);   // 2^(e - 1023) <= |v|; subnormals round to 0 below
   const ufx m = ((ufx)(a & 0xfffffffffffffLL) | 0x10000000000000ull) << 11;
   // |v| log2(10) = m 2^(e - 1086) LOG2_10 2^-62 = h 2^(e - 1084), wanted times 2^55
   const ufx h = fx_umulhi(m, FX_LOG2_10);
   const int s = 1029 - e;         // >= 1 for |v| < 64
-  const fx q = s < 64 ? (fx)((h >> s) + ((h >> (s - 1)) & 1)) : 0;
+  const fx q = s < 64 ? (fx)((h >> (s & 63)) + ((h >> ((s - 1) & 63)) & 1)) : 0;
   return b < 0 ? -q : q;
+}
+// FX_BAD if it is not (or not a number)
+FX_HD fx fx_of_log10(double v) {
+  return (fx_bits(v) & 0x7fffffffffffffffLL) >= fx_bits(FX_MAX_LOG10) ? FX_BAD : fx_of_log10_in(v);
+}
+
+// likewise, but the end of the range on its side
+FX_HD fx fx_of_log10_sat(double v) {
+  const fx b = fx_bits(v);
+  return (b & 0x7fffffffffffffffLL) >= fx_bits(FX_MAX_LOG10) ? (b < 0 ? -FX_SAT : FX_SAT) : fx_of_log10_in(v);
 }
 
 // log2 of x > 0 in Q55.  x above 2^127 (or infinite, or a positive NaN)
@@ -383,6 +392,13 @@ FX_HD bool fx_lap_group(const double q[8], const double o[24], double &sum) {
   const fx r = ((fx)(emax + 6 - z) << 52) + (fx)((w >> 11) + ((w >> 10) & 1));
   sum = fx_value(r | (s & (fx)0x8000000000000000ull));
   return true;
+}
+
+// Is an entry outside the format at a corner of an nr x nt table?  (k = 0 .. 3)
+FX_HD bool fx_outside(double v) { return (fx_bits(v) & 0x7fffffffffffffffLL) >= fx_bits(FX_MAX_LOG10); }
+FX_HD bool corner_outside(int nr, int nt, int k, const double *le, const double *lp, const double *lc) {
+  const long long at = ((k & 2) ? (long long)(nr - 1) * nt : 0) + ((k & 1) ? nt - 1 : 0);
+  return fx_outside(le[at]) || fx_outside(lp[at]) || fx_outside(lc[at]);
 }
 
 // The table's axes in fixed point (the same function of the FP64 axes for every

@@ -105,7 +105,8 @@ __device__ __forceinline__ void cta_bh_info(const BH &bh, double t, double dx, c
 // converts in its own kernel).  With the inversion on the integer pipe the pass waits on
 // its gathers, so four CTAs an SM (64 registers, a few spilled) instead of two (92): a
 // step of the 128^3 wave 2.405 -> 2.375 ms.
-template <int EOSK, int DUAL, int DT_ONLY = 0>
+// PREP: the table has its prepared form.
+template <int EOSK, int DUAL, int DT_ONLY = 0, int PREP = 0>
 __global__ void __launch_bounds__(NT, 4) k_c2p(Phys p, BH bh, TimeArgs ta,
                                             const DevBlock *blocks,
                                             const int32_t *ids,
@@ -146,7 +147,7 @@ __global__ void __launch_bounds__(NT, 4) k_c2p(Phys p, BH bh, TimeArgs ta,
     } else {
 #pragma unroll
       for (int v = 0; v < 5 + DUAL; ++v) u[v] = U[v * ntot + flat];
-      cons_to_prim<EOSK, DUAL>(p, u, w, cnt);
+      cons_to_prim<EOSK, DUAL, PREP ? 2 : 0>(p, u, w, cnt);
 #pragma unroll
       for (int v = 0; v < NWV; ++v) W[v * ntot + flat] = w[v];
     }
@@ -507,13 +508,14 @@ __global__ void k_set_dt(double *scal, double dt) {
 
 // ---------------------------------------------------------- EOS batch ----
 
+template <int PREP>
 __global__ void __launch_bounds__(NT) k_eos_invert(DTable t, long long n, const double *rho,
                                                    const double *en, double *T,
                                                    double *P, double *cs2, Counters *cnt) {
   pdl_begin();
   for (long long e = blockIdx.x * (long long)NT + threadIdx.x; e < n; e += (long long)gridDim.x * NT) {
     double Pv, cv, eu, Tv;
-    bool cl = eos_invert(t, rho[e], en[e], Pv, cv, eu, &Tv);
+    const bool cl = PREP ? eos_invert_node(t, rho[e], en[e], Pv, cv, eu, &Tv) : eos_invert(t, rho[e], en[e], Pv, cv, eu, &Tv);
     if (cl) count(&cnt->table_clamp);
     if (T) T[e] = Tv;
     if (P) P[e] = Pv;
@@ -693,6 +695,9 @@ cudaError_t launch_c2p(tde_mesh *m, const double *Uin, int nblk, const int32_t *
   } else if (p.eos == EOS_IDEAL) {
     if (p.dual) pdl_launch(k_c2p<EOS_IDEAL, 1>, C2P_ARGS);
     else pdl_launch(k_c2p<EOS_IDEAL, 0>, C2P_ARGS);
+  } else if (p.tab.node) {
+    if (p.dual) pdl_launch(k_c2p<EOS_TABLE, 1, 0, 1>, C2P_ARGS);
+    else pdl_launch(k_c2p<EOS_TABLE, 0, 0, 1>, C2P_ARGS);
   } else {
     if (p.dual) pdl_launch(k_c2p<EOS_TABLE, 1>, C2P_ARGS);
     else pdl_launch(k_c2p<EOS_TABLE, 0>, C2P_ARGS);
@@ -719,6 +724,9 @@ cudaError_t launch_c2p_padded(tde_mesh *m, const double *Uin, int nblk, const in
   } else if (surrogate_closure(m)) {
     if (p.dual) pdl_launch(k_c2p_padded<EOS_TABLE, 1, 1>, grid, NT, 0, m->ctx->stream, C2PP_ARGS);
     else pdl_launch(k_c2p_padded<EOS_TABLE, 0, 1>, grid, NT, 0, m->ctx->stream, C2PP_ARGS);
+  } else if (p.tab.node) {
+    if (p.dual) pdl_launch(k_c2p_padded<EOS_TABLE, 1, 2>, grid, NT, 0, m->ctx->stream, C2PP_ARGS);
+    else pdl_launch(k_c2p_padded<EOS_TABLE, 0, 2>, grid, NT, 0, m->ctx->stream, C2PP_ARGS);
   } else {
     if (p.dual) pdl_launch(k_c2p_padded<EOS_TABLE, 1>, grid, NT, 0, m->ctx->stream, C2PP_ARGS);
     else pdl_launch(k_c2p_padded<EOS_TABLE, 0>, grid, NT, 0, m->ctx->stream, C2PP_ARGS);
@@ -754,6 +762,9 @@ cudaError_t launch_c2p_list(tde_mesh *m, const double *Uin, const int32_t *list,
   } else if (surrogate_closure(m)) {
     if (p.dual) pdl_launch(k_c2p_list<EOS_TABLE, 1, 1>, grid, NT, 0, s, C2PL_ARGS);
     else pdl_launch(k_c2p_list<EOS_TABLE, 0, 1>, grid, NT, 0, s, C2PL_ARGS);
+  } else if (p.tab.node) {
+    if (p.dual) pdl_launch(k_c2p_list<EOS_TABLE, 1, 2>, grid, NT, 0, s, C2PL_ARGS);
+    else pdl_launch(k_c2p_list<EOS_TABLE, 0, 2>, grid, NT, 0, s, C2PL_ARGS);
   } else {
     if (p.dual) pdl_launch(k_c2p_list<EOS_TABLE, 1>, grid, NT, 0, s, C2PL_ARGS);
     else pdl_launch(k_c2p_list<EOS_TABLE, 0>, grid, NT, 0, s, C2PL_ARGS);
@@ -1083,7 +1094,7 @@ cudaError_t launch_eos_invert(tde_eos *e, int64_t n, const double *rho, const do
     t.n32 = nullptr;
     t.le32 = nullptr;
   }
-  pdl_launch(k_eos_invert, g, NT, 0, s, t, (long long)n, rho, en, T, P, cs2, e->d_cnt);
+  pdl_launch(t.node ? k_eos_invert<1> : k_eos_invert<0>, g, NT, 0, s, t, (long long)n, rho, en, T, P, cs2, e->d_cnt);
   return cudaGetLastError();
 }
 

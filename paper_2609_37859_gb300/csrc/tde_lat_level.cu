@@ -165,7 +165,7 @@ __device__ __forceinline__ long long interior_flat(const Phys &p, const DevBlock
 
 // One RK stage of the level (STAGE a template parameter, so that every access to
 // the kernel's argument block has a constant offset).
-template <int STAGE, int RECON, int EOSK, int DUAL>
+template <int STAGE, int RECON, int EOSK, int DUAL, int PREP>
 __device__ __forceinline__ bool level_stage(const LevelArgs &a, double *sm, unsigned long long *mbar,
                                             uint32_t *s_par) {
   constexpr unsigned B0 = 6 * STAGE;   // this stage's first grid barrier
@@ -220,7 +220,7 @@ __device__ __forceinline__ bool level_stage(const LevelArgs &a, double *sm, unsi
     double u[6], w[8];
 #pragma unroll
     for (int v = 0; v < NVAR; ++v) u[v] = Udst[v * ntot + flat];
-    cons_to_prim<EOSK, DUAL>(p, u, w, a.cnt);
+    cons_to_prim<EOSK, DUAL, PREP ? 2 : 0>(p, u, w, a.cnt);
 #pragma unroll
     for (int v = 0; v < NWV; ++v) a.W[v * ntot + flat] = w[v];
   });
@@ -229,7 +229,7 @@ __device__ __forceinline__ bool level_stage(const LevelArgs &a, double *sm, unsi
     double u[6], w[8];
 #pragma unroll
     for (int v = 0; v < NVAR; ++v) u[v] = Udst[v * ntot + flat];
-    cons_to_prim<EOSK, DUAL>(p, u, w, nullptr);
+    cons_to_prim<EOSK, DUAL, PREP ? 2 : 0>(p, u, w, nullptr);
 #pragma unroll
     for (int v = 0; v < NWV; ++v) a.W[v * ntot + flat] = w[v];
   }
@@ -254,24 +254,24 @@ __device__ __forceinline__ bool level_stage(const LevelArgs &a, double *sm, unsi
   if (!level_sweep<1, RECON, EOSK, DUAL, 0>(a.sw[STAGE][1], a.n, a.tiles[1], ctr + 1, sm, mbar, s_par))
     return false;
   if (!grid_barrier(a, B0 + 4, true)) return false;
-  return level_sweep<2, RECON, EOSK, DUAL, 1>(a.sw[STAGE][2], a.n, a.tiles[2], ctr + 2, sm, mbar, s_par);
+  return level_sweep<2, RECON, EOSK, DUAL, PREP ? 2 : 1>(a.sw[STAGE][2], a.n, a.tiles[2], ctr + 2, sm, mbar, s_par);
 }
 
-template <int RECON, int EOSK, int DUAL>
+template <int RECON, int EOSK, int DUAL, int PREP>
 __global__ void __launch_bounds__(LNTS, LMINB) k_lat_level(const LevelArgs a) {
   extern __shared__ __align__(128) double sm[];
   unsigned long long *mbar = reinterpret_cast<unsigned long long *>(reinterpret_cast<char *>(sm) + a.mbar_off);
   if (a.sw[0][0].tmap && threadIdx.x == 0) sweep_mbar_init(mbar);   // ordered by the first barrier
   __shared__ uint32_t s_par;
   if (threadIdx.x == 0) s_par = 0;   // ordered by the first barrier
-  if (!level_stage<0, RECON, EOSK, DUAL>(a, sm, mbar, &s_par)) return;
+  if (!level_stage<0, RECON, EOSK, DUAL, PREP>(a, sm, mbar, &s_par)) return;
   if (!grid_barrier(a, 5, true)) return;
-  level_stage<1, RECON, EOSK, DUAL>(a, sm, mbar, &s_par);
+  level_stage<1, RECON, EOSK, DUAL, PREP>(a, sm, mbar, &s_par);
 }
 
 template <int RECON, int EOSK, int DUAL>
 cudaError_t launch_level_kernel(const LevelArgs &a, size_t smem, int max_items, cudaStream_t s, int device) {
-  auto k = k_lat_level<RECON, EOSK, DUAL>;
+  auto k = a.sw[0][0].p.tab.node ? k_lat_level<RECON, EOSK, DUAL, EOSK == EOS_TABLE> : k_lat_level<RECON, EOSK, DUAL, 0>;
   cudaError_t err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   int per_sm = 0, sms = 0;
   if (err == cudaSuccess) err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, LNTS, smem);

@@ -444,8 +444,10 @@ __device__ __forceinline__ void cm_split(const CellMap &cm, long long t, long lo
 // brackets it.  An accepted cell is the one bisection finds (g_j <= y < g_{j+1}
 // is unique) and the state is evaluated with the same formulas (eos_at), so the
 // result is the bisection result bit for bit.  Returns false for the cells left
-// to bisection (clamped inputs, a step that misses).  FX: on the prepared table; else in
-// FP64 (tables with an entry outside the fixed-point format).
+// to bisection (clamped inputs, a step that misses).  FX: on the prepared table; else the
+// step is taken in FP64 and the results in the form that the cell's entries call for, as
+// eos_invert_views does (log e within 1e-12 of a node, where the two forms may see it in
+// different cells, is left to it).
 template <int FX>
 __device__ __forceinline__ bool newton_cell(const DTable &t, double rho_c, double e, float lTg, float idlt,
                                             double &P, double &cs2, double *T) {
@@ -472,10 +474,17 @@ __device__ __forceinline__ bool newton_cell(const DTable &t, double rho_c, doubl
       if (!(dle(g0, y) && dlt(y, g1))) return false;
       s = cell_solve(y, g0, g1);
     }
-    if (j == 0 && !dlt(g0, y)) return false;   // (bisection clamps at the coldest node)
-    P = texp10(t, bilin(t.lp, nt, i, w, j, s));
-    cs2 = texp10(t, bilin(t.lc, nt, i, w, j, s));
-    if (T) *T = texp10(t, cell_log10T(t, j, s));
+    if (!(y - g0 > 1e-12 && g1 - y > 1e-12)) return false;
+    double ev;
+    if (t.fa.valid) {
+      int ix;
+      ufx wx;
+      bool cl = false, out;
+      if (fx_rho_cell(t.fm, t.fa, t.nr, rho_c, ix, wx)) return false;
+      if (fx_cell_views<true>(t, ix, wx, fx_log2(t.fm, e), j, cl, out, e, P, cs2, ev, T)) return !cl;
+      if (!out) return false;
+    }
+    fp64_cell<true>(t, i, w, j, s, false, e, P, cs2, ev, T);
     return true;
   }
   int i;
@@ -773,6 +782,8 @@ __global__ void __launch_bounds__(IT, FX ? 8 : 6) k_eos_surrogate(const Surrogat
 // Table bisection for the cells the Newton step left (their indices in queue).
 // With eu (the hydro closure's buffers) the clamped table energy is returned
 // (0 inside the table) and the closure counts clamps; without, they are counted here.
+// PREP: the table has its prepared form.
+template <int PREP>
 __global__ void __launch_bounds__(256) k_eos_fallback(DTable t, const long long *queue,
                                                       const unsigned long long *qcount,
                                                       const double *rho,
@@ -784,7 +795,7 @@ __global__ void __launch_bounds__(256) k_eos_fallback(DTable t, const long long 
        q += (long long)gridDim.x * blockDim.x) {
     const long long c = queue[q];
     double Pv, cv, euv, Tv;
-    const bool cl = eos_invert(t, rho[c], e[c], Pv, cv, euv, &Tv);
+    const bool cl = PREP ? eos_invert_node(t, rho[c], e[c], Pv, cv, euv, &Tv) : eos_invert(t, rho[c], e[c], Pv, cv, euv, &Tv);
     if (cl && !eu) count(&cnt->table_clamp);
     if (T) T[c] = Tv;
     if (P) P[c] = Pv;
@@ -794,7 +805,7 @@ __global__ void __launch_bounds__(256) k_eos_fallback(DTable t, const long long 
 }
 
 // the primitives of the cells the hydro form left (their indices in queue)
-template <int DUAL>
+template <int DUAL, int PREP>
 __global__ void __launch_bounds__(256) k_fallback_c2p(Phys p, const long long *queue, const unsigned long long *qcount,
                                                       const double *U, double *W, long long ntot, Counters *cnt) {
   pdl_begin();
@@ -805,7 +816,7 @@ __global__ void __launch_bounds__(256) k_fallback_c2p(Phys p, const long long *q
     double u[6], w[8];
 #pragma unroll
     for (int v = 0; v < 5 + DUAL; ++v) u[v] = U[v * ntot + c];
-    cons_to_prim<EOS_TABLE, DUAL>(p, u, w, cnt);
+    cons_to_prim<EOS_TABLE, DUAL, PREP ? 2 : 0>(p, u, w, cnt);
 #pragma unroll
     for (int v = 0; v < 7 + DUAL; ++v) W[v * ntot + c] = w[v];
   }
@@ -973,7 +984,7 @@ cudaError_t surrogate_run(tde_eos *e, const CellMap &cm, long long n, const doub
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, e->ctx->device);
   const long long ncell = n * (cm.blocks ? cm.nblk : 1);
   const unsigned gf = (unsigned)std::min<long long>((ncell + 255) / 256, (long long)sms * 8);
-  pdl_launch(k_eos_fallback, gf, 256, 0, s, e->tab, queue, qcount, rho, en, T, P, cs2, eu, cnt);
+  pdl_launch(e->tab.node ? k_eos_fallback<1> : k_eos_fallback<0>, gf, 256, 0, s, e->tab, queue, qcount, rho, en, T, P, cs2, eu, cnt);
   return cudaGetLastError();
 }
 
@@ -1014,7 +1025,8 @@ cudaError_t launch_surrogate_c2p(tde_mesh *m, const CellMap &cm, int64_t nmax, c
   int sms = 152;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, e->ctx->device);
   const unsigned gf = (unsigned)std::min<long long>((nmax * cm.nblk + 255) / 256, (long long)sms * 8);
-  auto k = m->phys.dual ? k_fallback_c2p<1> : k_fallback_c2p<0>;
+  auto k = m->phys.dual ? k_fallback_c2p<1, 0> : k_fallback_c2p<0, 0>;
+  if (e->tab.node) k = m->phys.dual ? k_fallback_c2p<1, 1> : k_fallback_c2p<0, 1>;
   return pdl_launch(k, gf, 256, 0, s, m->phys, sb.queue, sb.qcount, U, m->d_W, (long long)m->ntot, m->d_cnt);
 }
 

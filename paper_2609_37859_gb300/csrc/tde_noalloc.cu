@@ -27,14 +27,12 @@ using namespace tde;
 
 constexpr int NA_MAX_BLOCKS = 4096;   // largest block count one call accepts
 constexpr int NA_NT = 256;
-constexpr int NA_SCAN = 256;   // CTAs that look a table over
 
 struct NAScratch {
   tde_block_desc blocks[NA_MAX_BLOCKS];      // copy of the caller's block list
   long long off[NA_MAX_BLOCKS + 1];          // first padded cell of each block
   unsigned long long minbits[NA_MAX_BLOCKS]; // per-block CFL minima (IEEE bits)
-  int bad[NA_SCAN], outside;                 // a table entry outside the fixed-point format: per CTA, any
-  unsigned done;                             // CTAs finished (zero between calls)
+  int outside;                               // an entry at a corner of the table outside the fixed-point format
 };
 
 // The only scratch of this entry point (about 176 KB per device).
@@ -55,9 +53,8 @@ __device__ __forceinline__ void na_bh_pos(const BH &bh, double t, double r[3]) {
   for (int a = 0; a < 3; ++a) r[a] = bh.x0[a] + bh.v0[a] * s + 0.5 * bh.a0[a] * s * s;
 }
 
-// padded sizes, offsets and the +inf initial minima of every block; whether the table in
-// the caller's arrays holds an entry outside the fixed-point format (then every cell takes
-// FP64, as with a loaded table)
+// padded sizes, offsets and the +inf initial minima of every block; the table's corners
+// looked at (a second CTA at least: the offsets keep the first one busy)
 __global__ void __launch_bounds__(NA_NT) k_na_setup(NAScratch *S, int nb, Phys p) {
   pdl_begin();
   if (threadIdx.x == 0 && blockIdx.x == 0) {
@@ -71,23 +68,11 @@ __global__ void __launch_bounds__(NA_NT) k_na_setup(NAScratch *S, int nb, Phys p
   }
   for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < nb; b += gridDim.x * blockDim.x)
     S->minbits[b] = (unsigned long long)__double_as_longlong(INFINITY);
-  if (p.eos != EOS_TABLE) return;
-  __shared__ int s_last;
-  const long long lim = dbits(FX_MAX_LOG10), n = (long long)p.tab.nr * p.tab.nt;
-  int bad = 0;
-  for (long long k = blockIdx.x * (long long)NA_NT + threadIdx.x; k < n; k += (long long)gridDim.x * NA_NT)
-    bad |= dmag(p.tab.le[k]) >= lim || dmag(p.tab.lp[k]) >= lim || dmag(p.tab.lc[k]) >= lim;
-  bad = __syncthreads_or(bad);
-  if (threadIdx.x == 0) {
-    S->bad[blockIdx.x] = bad;
-    __threadfence();
-    s_last = atomicInc(&S->done, gridDim.x - 1) == gridDim.x - 1;
+  if (p.eos == EOS_TABLE && blockIdx.x == gridDim.x - 1 && threadIdx.x < 32) {
+    const bool bad = threadIdx.x < 4 && corner_outside(p.tab.nr, p.tab.nt, threadIdx.x, p.tab.le, p.tab.lp, p.tab.lc);
+    const unsigned any = __ballot_sync(0xffffffffu, bad);
+    if (threadIdx.x == 0) S->outside = any != 0;
   }
-  __syncthreads();
-  if (!s_last) return;
-  __threadfence();
-  bad = __syncthreads_or(threadIdx.x < gridDim.x && __ldcg(&S->bad[threadIdx.x]));
-  if (threadIdx.x == 0) S->outside = bad;
 }
 
 // The CFL minimum of tde_compute_dt (k_c2p's want_dt path) with the same
@@ -331,8 +316,7 @@ extern "C" int tde_compute_dt_noalloc(tde_ctx *ctx, int nblocks, const tde_block
     ctx->err = std::string("tde_compute_dt_noalloc: ") + cudaGetErrorString(err);
     return TDE_ECUDA;
   }
-  const unsigned gs = p.eos == TDE_EOS_TABLE ? NA_SCAN : (unsigned)((nblocks + NA_NT - 1) / NA_NT);
-  pdl_launch(k_na_setup, gs, NA_NT, 0, s, S, nblocks, p);
+  pdl_launch(k_na_setup, (unsigned)((nblocks + NA_NT - 1) / NA_NT) + (p.eos == TDE_EOS_TABLE), NA_NT, 0, s, S, nblocks, p);
   const dim3 gc((unsigned)((max_int + NA_NT - 1) / NA_NT), (unsigned)nblocks);
   if (p.eos == TDE_EOS_IDEAL) {
     if (p.dual) pdl_launch(k_na_cfl<EOS_IDEAL, 1>, gc, NA_NT, 0, s, S, p, bh, U, ntot, t_block);

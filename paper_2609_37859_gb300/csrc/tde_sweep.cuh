@@ -137,7 +137,9 @@ __device__ __forceinline__ void sweep_mbar_init(unsigned long long *mbar) {
   asm volatile("fence.proxy.async.shared::cta;");
 }
 
-// One sweep tile: tile `tile` of block ids[qb].  The TMA barrier (at `mbar`,
+// One sweep tile: tile `tile` of block ids[qb].  LAST: the last direction, which completes the
+// update (2: with a table in its prepared form; the call for other tables costs a z sweep of
+// 8.4 M cells 0.8 % in registers kept for it).  The TMA barrier (at `mbar`,
 // initialised) completes once per staged tile with the parity `parity`, which
 // the caller flips after every tile that returns staged = true.  Returns false
 // if the bounded wait for the staging copy expired (the tile is skipped and the
@@ -522,7 +524,7 @@ __device__ __forceinline__ bool sweep_tile(const SweepArgs &a, int qb, int tile,
         if (EOSK == EOS_IDEAL) {
           un[5] = un[5] * exp(-p.gm1 * dv * dtl);
         } else {
-          const double Pa = table_pressure(p, un[0], un[5], a.cnt);
+          const double Pa = table_pressure<LAST == 2>(p, un[0], un[5], a.cnt);
           un[5] = un[5] - Pa * dv * dtl;
         }
         if (dlt(un[5], p.u_floor)) { un[5] = p.u_floor; count(&a.cnt->u_floor); }
@@ -558,7 +560,9 @@ cudaError_t sweep_one(const SweepArgs &a, bool last, dim3 grid, size_t smem, cud
   // the dynamic shared-memory limit is a per-function attribute (set to this
   // launch's size on every launch: cheap, and correct on whichever device is
   // current; the kernel's static shared memory counts against the same 227 KB)
+  constexpr int PREP = EOSK == EOS_TABLE && DUAL ? 2 : 1;
   auto k = last ? k_sweep<D, RECON, EOSK, DUAL, 1, M, NTS, MINB> : k_sweep<D, RECON, EOSK, DUAL, 0, M, NTS, MINB>;
+  if (last && a.p.tab.node) k = k_sweep<D, RECON, EOSK, DUAL, PREP, M, NTS, MINB>;
   cudaError_t err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (err != cudaSuccess) return err;
   return pdl_launch(k, grid, NTS, smem, s, a);

@@ -1,6 +1,6 @@
-"""Tables with an entry outside the fixed-point format (|log10| of 38 or more) are inverted
-in FP64 throughout: every search form gives the same bits, the learned form settles cells by
-its Newton step there too, and the time step without allocations equals the mesh's."""
+"""Tables with an entry outside the fixed-point format (|log10| of 38 or more): every search
+form gives the same bits, on and beside the nodes too, the learned form settles cells by its
+Newton step as on other tables, and the time step without allocations equals the mesh's."""
 import numpy as np
 import pytest
 
@@ -22,6 +22,10 @@ def _arrays(which):
     lc = 0.95 * le
     if which == "one":        # a single entry, in a corner no input comes near
         lc[NR - 1, NT - 1] = 38.5
+    elif which == "inner":    # away from the corners
+        lc[20, 30] = 38.5
+        lp[5:9, 40:50] += 40.0
+        le[30, 50:] += 30.0
     elif which == "P":
         lp = lp + 40.0
     elif which == "half":     # the hot half of the columns
@@ -29,7 +33,7 @@ def _arrays(which):
     return le, lp, lc
 
 
-@pytest.mark.parametrize("which", ["one", "P", "half"])
+@pytest.mark.parametrize("which", ["one", "inner", "P", "half"])
 def test_all_forms_agree(which):
     from paper_2609_37859_gb300 import tde
     le, lp, lc = _arrays(which)
@@ -37,8 +41,13 @@ def test_all_forms_agree(which):
     eos.train(seed=4, n_samples=1 << 16, epochs=10, batch=2048)
     rng = np.random.default_rng(8)
     n = 40000
-    rho = torch.tensor(10 ** rng.uniform(LRHO[0] - 0.2, LRHO[1] + 0.2, n), device="cuda")
-    e = torch.tensor(10 ** rng.uniform(le.min() - 0.2, le.max() + 0.2, n), device="cuda")
+    lr, ly = rng.uniform(LRHO[0] - 0.2, LRHO[1] + 0.2, n), rng.uniform(le.min() - 0.2, le.max() + 0.2, n)
+    i, j = rng.integers(0, NR, n // 2), rng.integers(0, NT, n // 2)
+    lr[: n // 2] = LRHO[0] + i * (LRHO[1] - LRHO[0]) / (NR - 1)   # nodes, and up to three roundings beside them
+    ly[: n // 2] = le[i, j]
+    e = 10.0 ** ly
+    e[: n // 2] += rng.integers(-3, 4, n // 2) * np.spacing(e[: n // 2])
+    rho, e = torch.from_numpy(10.0 ** lr).cuda(), torch.from_numpy(e).cuda()
     outs = []
     for mode in (tde.INVERT_BISECT, tde.INVERT_BISECT_PLAIN, tde.INVERT_SURROGATE):
         c0 = eos.counts()
@@ -53,7 +62,7 @@ def test_all_forms_agree(which):
     assert [x[2] for x in outs[:2]] == [0, 0] and outs[2][2] > 0
 
 
-@pytest.mark.parametrize("which", ["in", "one", "P", "half"])
+@pytest.mark.parametrize("which", ["in", "one", "inner", "P", "half"])
 def test_noalloc_dt_has_the_same_bits(which):
     from paper_2609_37859_gb300 import tde
     ctx = tde.Context(0)

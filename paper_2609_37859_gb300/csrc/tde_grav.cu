@@ -849,33 +849,67 @@ __device__ double full_value(const Lev &C, const MP &mp, int u0, int u1, int u2)
   return fma(sg, C.phi[lin(C, u[0], u[1], u[2])], acc);
 }
 
-// full multigrid: F.phi = P phi_C (the solution itself, tricubic), one warp per
-// fine cell with its taps (up to 64) over the lanes: beyond an isolated face a tap
-// evaluates the multipole expansion several times, and the levels that come here
-// have few cells, so a CTA is one warp (with one thread per cell a 4^3 level took
-// 1.9 ms)
-__global__ void __launch_bounds__(GT) k_mg_prolong_full(Lev F, Lev C, MP mp) {
+// full multigrid: F.phi = P phi_C (the solution itself, tricubic).  A warp takes per cells
+// in a row.  One by one with the taps (up to 64) over its lanes on small levels: beyond an
+// isolated face a tap evaluates the multipole expansion several times, and with one thread
+// per cell a 4^3 level took 1.9 ms.  On large ones (flat grids, thin boxes: the others are
+// tiled) a lane per cell whose taps lie inside the grid, and only the rest one by one: a
+// solve on 4096^2 cells 24.6 -> 15.0 ms (periodic), 32.2 -> 21.3 (isolated).  The line at
+// 400 cells an SM: with it at 4 k / 16 k / 64 k / 250 k / 1 M cells a 512^2 periodic solve
+// takes 1.197 / 1.195 / 1.205 / 1.240 / 1.362 ms, a 256^2 isolated one 1.74 / 1.70 / 1.65 /
+// 1.65 / 1.65.
+__global__ void __launch_bounds__(GT) k_mg_prolong_full(Lev F, Lev C, MP mp, int per) {
   pdl_begin();
   const unsigned n = (unsigned)F.n[0] * F.n[1] * F.n[2];
   const int lane = threadIdx.x & 31;
-  for (unsigned c = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; c < n; c += (gridDim.x * blockDim.x) >> 5) {
+  const unsigned step = ((gridDim.x * blockDim.x) >> 5) * per;
+  for (unsigned base = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * per; base < n; base += step) {
     int f[3];
-    decompose(F, c, f[0], f[1], f[2]);
     double w[3][4];
     int first[3], nt[3];
+    auto taps = [&](unsigned c) {
+      decompose(F, c, f[0], f[1], f[2]);
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      const bool h = F.n[a] != C.n[a];
-      first[a] = cubic_taps(f[a], h, w[a]);
-      nt[a] = h ? 4 : 1;
+      for (int a = 0; a < 3; ++a) {
+        const bool h = F.n[a] != C.n[a];
+        first[a] = cubic_taps(f[a], h, w[a]);
+        nt[a] = h ? 4 : 1;
+      }
+    };
+    unsigned todo = 1;   // the cells left to the whole warp
+    if (per > 1) {
+      const unsigned c = base + lane;
+      bool left = false;
+      if (c < n) {
+        taps(c);
+        if (C.iso)
+#pragma unroll
+          for (int a = 0; a < 3; ++a) left = left || first[a] < 0 || first[a] + nt[a] > C.n[a];
+        if (!left) {
+          double s = 0.0;
+          for (int cz = 0; cz < nt[2]; ++cz)
+            for (int by = 0; by < nt[1]; ++by) {
+              const double wyz = w[1][by] * w[2][cz];
+              for (int ax = 0; ax < nt[0]; ++ax)
+                s = fma(w[0][ax] * wyz, C.phi[wrap_idx(C, first[0] + ax, first[1] + by, first[2] + cz)], s);
+            }
+          F.phi[c] = s;
+        }
+      }
+      todo = __ballot_sync(0xffffffffu, left);
     }
-    double s = 0.0;
-    for (int q = lane; q < nt[0] * nt[1] * nt[2]; q += 32) {
-      const int ax = q % nt[0], r = q / nt[0], by = r % nt[1], cz = r / nt[1];
-      s = fma(w[0][ax] * w[1][by] * w[2][cz], full_value(C, mp, first[0] + ax, first[1] + by, first[2] + cz), s);
+    while (todo) {
+      const unsigned c = base + __ffs(todo) - 1;
+      todo &= todo - 1;
+      taps(c);
+      double s = 0.0;
+      for (int q = lane; q < nt[0] * nt[1] * nt[2]; q += 32) {
+        const int ax = q % nt[0], r = q / nt[0], by = r % nt[1], cz = r / nt[1];
+        s = fma(w[0][ax] * w[1][by] * w[2][cz], full_value(C, mp, first[0] + ax, first[1] + by, first[2] + cz), s);
+      }
+      for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+      if (lane == 0) F.phi[c] = s;
     }
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) F.phi[c] = s;
   }
 }
 
@@ -1262,10 +1296,13 @@ static void full_multigrid(GravState *g, const tde_grav_params &gp, int lmax, cu
   const MP mp{lmax, g->mp};
   for (int l = g->nl - 2; l >= 0; --l) {
     const Lev &F = g->lev[l];
+    const long long nf = (long long)F.n[0] * F.n[1] * F.n[2];
     if (const int T = prolong_tile(F, g->lev[l + 1]))
       launch_prolong_tiled<1>(F, g->lev[l + 1], mp, T, s);
+    else if (nf < 400LL * n_sm())
+      pdl_launch(k_mg_prolong_full, (unsigned)std::min<long long>(nf, 32LL * n_sm()), 32, 0, s, F, g->lev[l + 1], mp, 1);
     else
-      pdl_launch(k_mg_prolong_full, (unsigned)std::min<long long>((long long)F.n[0] * F.n[1] * F.n[2], 32LL * n_sm()), 32, 0, s, F, g->lev[l + 1], mp);
+      pdl_launch(k_mg_prolong_full, grid_for(nf), GT, 0, s, F, g->lev[l + 1], mp, 32);
     g->launches += 1;
     vcycle(g, l, gp, s);
     if (l == 0) smooth(g, F, gp.omega, s);

@@ -16,22 +16,34 @@ using namespace tde;
 
 // tables of the table-driven log10 / exp10 (tde_device.cuh), computed in
 // extended precision on the host
-void tde::fill_math_tables(MathTables *h) {
-  for (int j = 0; j < 182; ++j) {
-    const long double F = j / 128.0L;
-    h->logF[j] = j > 0 ? (double)logl(F) : 0.0;
-    h->invF[j] = j > 0 ? (double)(1.0L / F) : 0.0;
-    h->F[j] = j / 128.0;
-  }
-  for (int j = 0; j < 128; ++j) h->exp2j[j] = (double)exp2l(j / 128.0L);
+// (computed once per process: about 1000 logarithms and exponentials in extended precision,
+// 0.4 ms of every table load on a machine that has no such arithmetic in hardware)
+const MathTables &tde::math_tables() {
+  static const MathTables t = [] {
+    MathTables h;
+    for (int j = 0; j < 182; ++j) {
+      const long double F = j / 128.0L;
+      h.logF[j] = j > 0 ? (double)logl(F) : 0.0;
+      h.invF[j] = j > 0 ? (double)(1.0L / F) : 0.0;
+      h.F[j] = j / 128.0;
+    }
+    for (int j = 0; j < 128; ++j) h.exp2j[j] = (double)exp2l(j / 128.0L);
+    return h;
+  }();
+  return t;
 }
 
-void tde::fx_fill_math(FxMath *h) {
-  for (int j = 0; j < 256; ++j) {
-    h->c[j] = (unsigned)floorl(1024.0L / (1.0L + (j + 0.5L) / 256.0L) + 0.5L);
-    h->lg[j] = (fx)floorl(-log2l(h->c[j] / 1024.0L) * 36028797018963968.0L + 0.5L);
-    h->ex[j] = (unsigned long long)floorl(exp2l((j + 0.5L) / 256.0L) * 4611686018427387904.0L + 0.5L);
-  }
+const FxMath &tde::fx_math() {
+  static const FxMath t = [] {
+    FxMath h;
+    for (int j = 0; j < 256; ++j) {
+      h.c[j] = (unsigned)floorl(1024.0L / (1.0L + (j + 0.5L) / 256.0L) + 0.5L);
+      h.lg[j] = (fx)floorl(-log2l(h.c[j] / 1024.0L) * 36028797018963968.0L + 0.5L);
+      h.ex[j] = (unsigned long long)floorl(exp2l((j + 0.5L) / 256.0L) * 4611686018427387904.0L + 0.5L);
+    }
+    return h;
+  }();
+  return t;
 }
 
 namespace {
@@ -215,14 +227,13 @@ __global__ void k_fx_buckets(const longlong2 *__restrict__ nd, int nr, int nt, f
 // One allocation: the log2 / exp2 tables, then the above (about 88 bytes an entry).  A
 // table with an entry outside the format, or without room for that much, keeps the former
 // only, and its values are converted as they are read (eos_invert_views).
-static cudaError_t load_fx_table(tde_eos *e, double lr_max, const double *le, const double *lp, const double *lc) {
+static cudaError_t load_fx_table(tde_eos *e, double lr_max, bool outside, const double *le, const double *lp,
+                                 const double *lc) {
   DTable &t = e->tab;
   const int nr = t.nr, nt = t.nt;
-  const size_t nn = (size_t)nr * nt, npair = (size_t)(nr - 1) * nt;
+  const size_t npair = (size_t)(nr - 1) * nt;
   t.fa = fx_axes(nr, nt, t.lr0, lr_max, t.inv_dlr, t.lt0, t.dlt);
-  bool ok = t.fa.valid;
-  for (size_t k = 0; k < nn; ++k)
-    ok = ok && fabs(le[k]) < FX_MAX_LOG10 && fabs(lp[k]) < FX_MAX_LOG10 && fabs(lc[k]) < FX_MAX_LOG10;
+  bool ok = t.fa.valid && !outside;
   for (int k = 0; k < 4; ++k)
     if (corner_outside(nr, nt, k, le, lp, lc)) t.fa.valid = 0;   // in FP64 as a whole
   // bucket width: the smallest power of two that needs at most 8 nt buckets (the columns
@@ -248,8 +259,7 @@ static cudaError_t load_fx_table(tde_eos *e, double lr_max, const double *le, co
   const bool buckets = nt <= 65535;
   const size_t o_node = part(sizeof(longlong2) * 3 * npair), o_n32 = part(sizeof(int2) * npair);
   const size_t o_bk = buckets ? part(sizeof(ushort2) * (size_t)(nr - 1) * nbk) : 0;
-  FxMath fm;
-  fx_fill_math(&fm);
+  const FxMath &fm = fx_math();
   cudaError_t err = ok ? cudaMalloc(&e->d_fx, size) : cudaErrorMemoryAllocation;
   if (err == cudaErrorMemoryAllocation) {
     if (ok) cudaGetLastError();
@@ -292,7 +302,10 @@ extern "C" int tde_eos_load_table(tde_ctx *ctx, int n_rho, int n_T, double lr_mi
   if (!(lr_max > lr_min) || !(lT_max > lT_min))
     return fail(ctx, TDE_EINVAL, "tde_eos_load_table: empty range");
   const size_t nn = (size_t)n_rho * n_T;
+  unsigned outside = 0;   // an entry the fixed-point format does not take (or not finite)
   for (size_t k = 0; k < nn; ++k)
+    outside |= (unsigned)fx_outside(log10_e[k]) | (unsigned)fx_outside(log10_P[k]) | (unsigned)fx_outside(log10_cs2[k]);
+  for (size_t k = 0; outside && k < nn; ++k)
     if (!isfinite(log10_e[k]) || !isfinite(log10_P[k]) || !isfinite(log10_cs2[k]))
       return fail(ctx, TDE_EINVAL, "tde_eos_load_table: non-finite entry");
   for (int i = 0; i < n_rho; ++i)
@@ -354,8 +367,7 @@ extern "C" int tde_eos_load_table(tde_ctx *ctx, int n_rho, int n_T, double lr_mi
   t.lc = e->d_data + 2 * nn;
   t.le32 = reinterpret_cast<const float *>(e->d_data + 3 * nn);
   {   // tables of the table-driven log10 / exp10, computed in extended precision
-    MathTables h;
-    fill_math_tables(&h);
+    const MathTables &h = math_tables();
     err = cudaMalloc(&e->d_mt, sizeof(MathTables));
     if (err == cudaSuccess) err = cudaMemcpy(e->d_mt, &h, sizeof h, cudaMemcpyHostToDevice);
     if (err != cudaSuccess) {
@@ -367,7 +379,7 @@ extern "C" int tde_eos_load_table(tde_ctx *ctx, int n_rho, int n_T, double lr_mi
     }
     t.mt = e->d_mt;
   }
-  err = load_fx_table(e, lr_max, log10_e, log10_P, log10_cs2);
+  err = load_fx_table(e, lr_max, outside != 0, log10_e, log10_P, log10_cs2);
   if (err != cudaSuccess) {
     tde_eos_destroy(e);
     return cuda_fail(ctx, err, "tde_eos_load_table: fixed-point table");

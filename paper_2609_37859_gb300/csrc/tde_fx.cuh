@@ -464,6 +464,6 @@ FX_HD fx fx_log2T(const FxAxes &A, int j, ufx s) {
 }
 
 // tables of fx_log2 and fx_exp2 (host, extended precision)
-void fx_fill_math(FxMath *h);
+const FxMath &fx_math();
 
 }  // namespace tde

@@ -25,8 +25,8 @@ struct tde_ctx {
 };
 
 namespace tde {
-// fills the tables of fast_log10 / fast_exp10 (host, extended precision)
-void fill_math_tables(MathTables *h);
+// the tables of fast_log10 / fast_exp10 (host, extended precision)
+const MathTables &math_tables();
 // SMs of the current device
 int n_sm();
 

@@ -215,10 +215,8 @@ extern "C" int tde_compute_dt_noalloc(tde_ctx *ctx, int nblocks, const tde_block
   // device addresses, and the log10 / exp10 tables copied into the others
   cudaError_t err = cudaSetDevice(ctx->device);
   if (err == cudaSuccess && !g_scratch_ptr[ctx->device]) {
-    MathTables h;
-    fill_math_tables(&h);
-    FxMath hf;
-    fx_fill_math(&hf);
+    const MathTables &h = math_tables();
+    const FxMath &hf = fx_math();
     void *ps = nullptr, *pm = nullptr, *pf = nullptr;
     err = cudaMemcpyToSymbol(g_noalloc_mt, &h, sizeof h);
     if (err == cudaSuccess) err = cudaMemcpyToSymbol(g_noalloc_fm, &hf, sizeof hf);

@@ -421,8 +421,9 @@ def autotune_report(tiles, ms):
 
 def closure_bench(mesh, U_init, tde, torch, dev, args):
     """The bench step with each way of inverting the table in cons -> prim
-    (same results, checked bitwise): FP32-guided bisection (the headline), plain
-    FP64 bisection, and the learned guess + one FP64 Newton step."""
+    (same results, checked bitwise), in 64-bit fixed point: bisection with the 32-bit
+    search (the headline), plain bisection (every step in 64 bits), and the learned guess
+    + one Newton step."""
     out, ref = {}, None
     nsteps = 10
     for name, mode in (("bisect_fp32_guided", tde.INVERT_BISECT), ("bisect_plain", tde.INVERT_BISECT_PLAIN),
@@ -584,7 +585,7 @@ def lat_bench(ctx, eos, tde, torch, dev, args):
         c["surrogate_accepted"] //= 2   # per window
         return ms, U1w, c
 
-    # LAT with tiles autotuned on this mesh: FP32-guided bisection (the GB300
+    # LAT with tiles autotuned on this mesh: bisection with the 32-bit search (the GB300
     # form) and the learned guess (the learned + batched form)
     tiles, tile_ms = mesh.autotune(bh=bh, reps=2)
     ms_lat, U_lat, lat_counts = lat_arm(tde.INVERT_BISECT)
@@ -613,7 +614,7 @@ def lat_bench(ctx, eos, tde, torch, dev, args):
     flat = torch.from_numpy(lay.interior_flat()).to(dev)
     vs_sync = lat_vs_sync_metrics(torch, U_lat[0][flat], mesh.U[0][flat], params.rho_floor)
     del U_lat, flat
-    # plain form: plain FP64 table bisection, the default tile shape, one launch
+    # plain form: table bisection with every step in 64 bits, the default tile shape, one launch
     # sequence per block and stage; one step of dt0
     set_mode(tde.INVERT_BISECT_PLAIN)
     mesh.set_tiles((0, 0, 0))
@@ -653,8 +654,8 @@ def lat_bench(ctx, eos, tde, torch, dev, args):
             "effective_cell_updates_per_s": {"lat": upd / (ms_lat * 1e-3), "sync": upd / (ms_sync * 1e-3),
                                              "learned_batched": upd / (ms_lat_sur * 1e-3),
                                              "plain": ncell / (ms_plain_step * 1e-3)},
-            "plain_form": "plain FP64 table bisection, default tiles, one launch sequence per block and stage",
-            "learned_batched_form": "learned guess + one FP64 Newton step, autotuned tiles, per-level batched "
+            "plain_form": "plain table bisection (every step in 64 bits), default tiles, one launch sequence per block and stage",
+            "learned_batched_form": "learned guess + one Newton step, autotuned tiles, per-level batched "
                                     "launches replayed as a CUDA graph",
             "lat_counters": lat_counts}
 
@@ -905,7 +906,7 @@ C5_WORKLOAD = ("production-shaped: stretched n=1.5 polytrope (1 Msun, 1 Rsun, 4:
                "point mass with excision passing at the parabolic speed through free-falling ambient gas; "
                "2048 MeshBlocks of 32^3 (512x512x256 = 67,108,864 cells), ghost width 3, PPM+HLLC+SSP-RK2, "
                "Saha H/He 256x256 table in the code units of Table 1, learned-guess closure (BF16 tensor-core "
-               "MLP + FP64 Newton, bisection fallback), dual energy, floors 100x Table 1's, CFL 0.3")
+               "MLP + Newton step, bisection fallback), dual energy, floors 100x Table 1's, CFL 0.3")
 
 
 def build_c5(ctx, eos, tde, torch, dev, floors=C5_FLOORS, grid=(16, 16, 8)):

@@ -778,7 +778,11 @@ __device__ __forceinline__ void plm(double q0, double dl, double dr, double &lef
     }
   }
 }
-// a - b, without the subtraction where a = b on every lane of the warp
+// a - b, without the subtraction where a = b on every lane that votes.  (The votes of the
+// reconstruction are over whichever lanes are still in the loop: a vote only skips work whose
+// outcome is known, so no result depends on who votes.  But for equal infinities, whose
+// difference is not a number: whether their face values are infinite or none depends on it,
+// and the cells beside them are non-finite, and counted as such, either way.)
 __device__ __forceinline__ double diff_or_zero(double a, double b) {
   double d = 0.0;
   if (__any_sync(__activemask(), dbits(a) != dbits(b))) d = a - b;
@@ -801,7 +805,7 @@ __device__ __forceinline__ double ppm_iface(double q0, double q1, double D0, dou
   const long long bt = dbits(t), b1 = dbits(D1);
   const long long m1 = b1 & 0x7fffffffffffffffLL;
   const bool over = (bt & 0x7fffffffffffffffLL) >= m1 + 0x10000000000000LL && (bt ^ b1) >= 0;   // |t| >= 2 |D1|
-  if ((bt ^ b1) < 0 || m1 < 0x10000000000000LL) t = 0.0;   // the other sign, or D1 = 0
+  if ((bt ^ b1) < 0 || m1 < 0x10000000000000LL) t = 0.0;   // the other sign, or D1 zero (or subnormal)
   T = t;
   V = fma(2.0, D1, -t);
   double a = fma(0.5, t, q0);
@@ -856,7 +860,7 @@ struct FState {
 // contact: mass m = r chi S_M with chi = sigma / (S - S_M), momentum m v plus
 // P* = P + r sigma w, energy (E* + P*) S_M, auxiliary A chi S_M, instead of
 // F_K + S (U*_K - U_K).  Outside the wave fan chi = 1, w = 0 and S_M = u give the
-// side's own flux by the same expressions.  About 40 FP64 operations a face
+// side's own flux by the same expressions.  33 FP64 operations a face
 // instead of 73 (the square roots and reciprocals are integer arithmetic).
 template <int D, int EOSK, int DUAL>
 __device__ __forceinline__ void hllc(const Phys &p, const FState &L, const FState &R, double *F,

@@ -7,7 +7,7 @@
 // slots (1600 cycles per warp); here it is a few hundred integer instructions
 // and no FP64 at all: 2^24 inversions of (T, P, cs^2) with densities and energies
 // scattered over the 256 x 256 table went from 3.10 ms to 0.63 ms (1.06 TB/s of
-// input and output), the learned-guess form on 6 million from 1.86 to 0.78 ms, a
+// input and output), the learned-guess form on 6 million from 1.86 to 0.78 ms (0.72 since), a
 // step of the 8.4 M-cell star mesh from 25.6 to 21.4 ms.  A fixed-point logarithm of 55 fraction bits resolves
 // 2.8e-17 in log2, an FP64 one of size 40 (log10 of size 12) only 7e-15, so the
 // results are nearer to the exact ones than the FP64 form's.

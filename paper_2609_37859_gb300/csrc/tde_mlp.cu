@@ -524,7 +524,7 @@ __device__ __forceinline__ bool newton_cell(const DTable &t, double rho_c, doubl
 // state and the primitives of accepted cells written, so the FP64 work of the
 // conversion runs beside the network's integer and MUFU work and the state is read by
 // one kernel; the queued cells are converted by k_fallback_c2p.  A step of 8.4 M cells:
-// 14.3 -> 13.4 ms against separate kernels for inputs, inversion and conversion.
+// 14.3 -> 13.2 ms against separate kernels for inputs, inversion and conversion.
 // What bounds it is instruction issue (two thirds of its slots): the layers go two
 // units at a time through the packed FP32 FMA, and the output the inversion does not
 // use is left out (5.9 M cells 780 -> 728 us; one 16-byte record of weights per unit

@@ -9,9 +9,9 @@
 // this entry point takes the block list, the grid and the state directly and
 // keeps all of its scratch -- a copy of the block list, the padded-block
 // offsets and the per-block CFL minima -- in one fixed file-scope device array
-// that exists in every process that loads the library.  A second, constant
-// file-scope array holds the log10 / exp10 tables of the EOS lookups, so the
-// results equal tde_compute_dt's bit for bit.
+// that exists in every process that loads the library.  Two constant
+// file-scope arrays hold the logarithms' and exponentials' tables of the EOS lookups, so
+// the results equal tde_compute_dt's bit for bit.
 //
 // The scratch array is shared by every call in the process: calls whose GPU
 // work overlaps (on two streams, or from two threads) race on it and must be

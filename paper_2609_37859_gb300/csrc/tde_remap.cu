@@ -17,7 +17,7 @@
 // as a separable stencil of at most 4 x 4 x 4 staged cells: by a thread per target
 // column that keeps the x- and y-averaged source planes along z where a target cell is
 // less than twice as wide as a source cell (k_remap_columns: 31 FP64 operations a cell
-// and variable instead of 64; a 128^3 source onto 8.4 M cells 1.00 -> 0.59 ms), by a
+// and variable instead of 64; a 128^3 source onto 8.4 M cells, whole call, 1.00 -> 0.56 ms), by a
 // thread per target cell elsewhere.  Coincident cells are
 // copied from the source's own layout through its owner lattice.  32-bit index
 // division only (a 64-bit integer division would issue on the FP64 pipe).
@@ -271,8 +271,7 @@ __global__ void __launch_bounds__(RT) k_remap(RemapDst d, RemapSrc s, const doub
 // source planes, so a plane is averaged once for all of them that use it, with
 // the products of the x and y weights formed once per run.  The direct form is
 // bound by the FP64 pipe (64 operations per cell of a twofold refinement); this one
-// needs 31: a 128^3 source onto 8.4 M cells went from 0.91 ms to 0.48 ms (the FP64
-// pipe still 86 % busy).
+// needs 31 (the FP64 pipe still 86 % busy).
 constexpr int RC = 3;
 // the x-y average of one source plane over the used ones of N x N entries (bit 4 cy + cx
 // of use; N = 2: all four, so nothing is tested)

@@ -374,7 +374,7 @@ __device__ __forceinline__ bool sweep_tile(const SweepArgs &a, int qb, int tile,
         double D1 = q0 - qm, D2 = q1 - q0, T, V;
         double a = ppm_iface(qm, q0, qm - w[-2 * ws], D1, D2, T, V);   // the run's lowest interface
         // the last pairs of neighbours with equal values: where the four cells of an
-        // interface are equal on every lane of the warp (floor gas, a variable that
+        // interface are equal on every lane that votes (floor gas, a variable that
         // does not vary) its value is theirs and the cell below it is flat
         int same = dbits(q1) != dbits(q0) ? 0 : (dbits(q0) == dbits(qm) ? 2 : 1);
         for (int c = c0; c < c1; ++c) {
@@ -598,7 +598,8 @@ cudaError_t sweep_launch_shape(const SweepArgs &a, int D, bool last, dim3 grid, 
 }
 
 // The tile shapes offered to the autotuner: lanes per tile, CTA width, and the
-// CTAs per SM the register budget is sized for.  Index 0 is the default.
+// CTAs per SM the register budget is sized for.  Index 0 is the default, 1 along directions
+// of 9 to 16 cells a block (tde_mesh_create).
 struct TileShape {
   int M, NTS, MINB;
 };
